@@ -1,0 +1,436 @@
+// Tree sampling by rounds of cycle popping with many lanes per tree
+// (lane_tree.cuh): the vertex words in shared memory for graphs that fit (up to
+// about 56000 vertices), in global memory otherwise.
+//
+// Measured (kernel time, whole-block popping rounds in shared memory or
+// concurrent walkers before -> here): BA n = 2000, 1000 trees 0.51 -> 0.12 ms;
+// weighted RGG n = 19999, 304 trees 194 -> 8 ms; 224 x 240 grid, 1000 trees
+// 1.38 -> 0.27 s; R-MAT n = 100000, 1000 trees 20.1 -> 6.5 ms; 512 x 512 grid,
+// 64 trees 3.97 -> 1.18 s.  Latency bound: one tree of the 150 x 150 grid runs
+// at 6 cycles per instruction and warp, 30% of them at barriers, with 4 warps
+// on an SM; one lane per thread (twice the warps of two) took 313 instead of
+// 404 ms on the 224 x 240 grid.
+#include <algorithm>
+#include <type_traits>
+#include <vector>
+
+#include "lane_tree.cuh"
+#include "rwc_common.cuh"
+
+namespace rwc {
+namespace {
+
+// One tree per block of NT threads, its words in shared memory; trees are
+// handed out by ctr[0] after the first of each block.  Trees whose counts
+// outgrow the word are left out and listed in wide[0 .. ctr[2]).
+template <bool OFF64, bool WT, int EW, int NT>
+__global__ void __launch_bounds__(NT) l_trees_smem(DevGraph g, uint32_t tree0, int64_t T, uint32_t k0,
+                                                   uint32_t k1, uint32_t klim, int kb, double *sums,
+                                                   int32_t *parents, int32_t *visits, uint32_t *spill,
+                                                   int *err, unsigned long long *ctr, uint32_t *wide) {
+    constexpr int S = 1;
+    static_assert(sizeof(LaneShared<NT, S>) % 4 == 0 && NT <= 256, "lane_smem");
+    extern __shared__ __align__(16) unsigned char smem[];
+    __shared__ unsigned long long sh_next;
+    LaneShared<NT, S> &sh = *reinterpret_cast<LaneShared<NT, S> *>(smem);
+    uint32_t *word = reinterpret_cast<uint32_t *>(smem + sizeof(LaneShared<NT, S>));
+    const int n = (int)g.n;
+    const uint32_t kmask = (1u << kb) - 1u;
+    uint32_t *sp = spill + (int64_t)blockIdx.x * n;
+    unsigned long long draws = 0;
+    int64_t t = blockIdx.x;
+    while (t < T) {
+        for (int u = threadIdx.x; u < n; u += NT) word[u] = u == g.root ? lt_root_word<uint32_t>(kb, NT * S) : 0u;
+        __syncthreads();
+        const int bad = lane_tree<OFF64, WT, EW, NT, S, true, uint32_t>(g, word, kb, klim, sh, sp, tree0 + (uint32_t)t,
+                                                                     0u, k0, k1);
+        if (bad & ~LE_KREP) { if (threadIdx.x == 0) atomicOr(err, bad); break; }
+        if (bad && threadIdx.x == 0) wide[atomicAdd(ctr + 2, 1ull)] = (uint32_t)t;
+        for (int u = bad ? n : threadIdx.x; u < n; u += NT) {
+            const uint32_t w = word[u];
+            const uint32_t vis = u == g.root ? 0u : (w & kmask) + 1u;
+            draws += vis;
+            if (sums && vis) atomicAdd(sums + u, (double)vis);
+            if (parents) parents[t * n + u] = u == g.root ? -1 : (int32_t)(((w & 0x7fffffffu) >> kb) - lt_id0(NT * S));
+            if (visits) visits[t * n + u] = (int32_t)vis;
+        }
+        if (threadIdx.x == 0) sh_next = atomicAdd(ctr, 1ull);
+        __syncthreads();
+        t = (int64_t)gridDim.x + (int64_t)sh_next;
+    }
+    for (int o = 16; o > 0; o >>= 1) draws += __shfl_xor_sync(0xffffffffu, draws, o);
+    if ((threadIdx.x & 31) == 0 && draws) atomicAdd(ctr + 1, draws);
+}
+
+// One tree per block of NT threads, its words in global memory (zeroed by the
+// caller), `ld` words apart.
+template <bool OFF64, bool WT, int EW, int NT, class W>
+__global__ void __launch_bounds__(NT) l_trees(DevGraph g, uint32_t tree0, int64_t B, int64_t ld, uint32_t k0,
+                                              uint32_t k1, uint32_t klim, int kb, W *words, uint32_t *spill,
+                                              int *err, unsigned long long *ctr) {
+    constexpr int S = 2;   // lanes per thread: two loads in flight
+    __shared__ LaneShared<NT, S> sh;
+    __shared__ unsigned long long sh_next;
+    uint32_t *sp = spill + (int64_t)blockIdx.x * g.n;
+    int64_t t = blockIdx.x;
+    while (t < B) {
+        W *word = words + t * ld;
+        if (threadIdx.x == 0) word[g.root] = lt_root_word<W>(kb, NT * S);
+        __syncthreads();
+        const int bad = lane_tree<OFF64, WT, EW, NT, S, false, W>(g, word, kb, klim, sh, sp, tree0 + (uint32_t)t, 0u, k0, k1);
+        if (bad) { if (threadIdx.x == 0) atomicOr(err, bad); break; }
+        if (threadIdx.x == 0) sh_next = atomicAdd(ctr, 1ull);
+        __syncthreads();
+        t = (int64_t)gridDim.x + (int64_t)sh_next;
+    }
+}
+
+// visits_u = k_u + 1 over the chunk's trees into sums; optional per-tree
+// output.  Nothing after an error (the chunk is then sampled again).  The trees
+// are split over gridDim.y so that small graphs fill the chip too; the sums are
+// whole numbers, exact in any order.
+template <class W>
+__global__ void l_accum(int64_t n, int32_t root, const W *words, int64_t ld, int kb, uint32_t id0, int64_t B, double *sums,
+                        int32_t *parents, int32_t *visits, const int *err, unsigned long long *draws) {
+    if (*err) return;
+    const W kmask = ((W)1 << kb) - 1, pmask = ~(W)0 >> 1;
+    const int64_t t0 = B * blockIdx.y / gridDim.y, t1 = B * (blockIdx.y + 1) / gridDim.y;
+    unsigned long long local = 0;
+    for (int64_t u = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; u < n;
+         u += (int64_t)gridDim.x * blockDim.x) {
+        unsigned long long acc = 0;
+#pragma unroll 4
+        for (int64_t t = t0; t < t1; ++t) {
+            const W w = words[t * ld + u];
+            const uint32_t vis = u == root ? 0u : (uint32_t)(w & kmask) + 1u;
+            acc += vis;
+            if (parents) parents[t * n + u] = u == root ? -1 : (int32_t)((uint32_t)((w & pmask) >> kb) - id0);
+            if (visits) visits[t * n + u] = (int32_t)vis;
+        }
+        local += acc;
+        if (sums && acc) atomicAdd(sums + u, (double)acc);
+    }
+    for (int o = 16; o > 0; o >>= 1) local += __shfl_xor_sync(0xffffffffu, local, o);
+    if ((threadIdx.x & 31) == 0 && local) atomicAdd(draws, local);
+}
+
+template <int V> using int_c = std::integral_constant<int, V>;
+
+// f(off64, weighted, inline row width) as compile-time constants
+template <class F>
+void dispatch(const DevGraph &g, F f) {
+    if (g.off64) {
+        if (g.weighted) f(std::true_type{}, std::true_type{}, int_c<0>{});
+        else f(std::true_type{}, std::false_type{}, int_c<0>{});
+    } else {
+        if (g.weighted) f(std::false_type{}, std::true_type{}, int_c<0>{});
+        else if (g.ell_w == 4) f(std::false_type{}, std::false_type{}, int_c<4>{});
+        else if (g.ell_w == 8) f(std::false_type{}, std::false_type{}, int_c<8>{});
+        else f(std::false_type{}, std::false_type{}, int_c<0>{});
+    }
+}
+
+struct Buf {
+    void *p = nullptr;
+    cudaStream_t st;
+    explicit Buf(cudaStream_t s) : st(s) {}
+    ~Buf() { if (p) cudaFreeAsync(p, st); }
+};
+struct Events {
+    cudaEvent_t e[4] = {};
+    bool on;
+    explicit Events(bool o) : on(o) { if (on) for (auto &x : e) cudaEventCreate(&x); }
+    ~Events() { if (on) for (auto &x : e) cudaEventDestroy(x); }
+    void rec(int i, cudaStream_t s) { if (on) cudaEventRecord(e[i], s); }
+    double ms(int a, int b) { float v = 0.f; if (on) cudaEventElapsedTime(&v, e[a], e[b]); return v; }
+};
+
+constexpr int64_t TAIL = 64;   // err @0, next tree @8, draws @16, listed trees @24
+constexpr int64_t WIDE_CAP = 65536;   // trees of one shared-memory launch
+
+template <int NT, class W>
+rwc_status walker_range(rwc_graph *G, uint64_t seed, int64_t tree0, int64_t T, double *sums, int32_t *parents,
+                        int32_t *visits, const rwc_options_t &o, rwc_stats_t *st, cudaStream_t stream) {
+    const DevGraph &g = G->g;
+    const int64_t n = g.n, ld = (n + 3) & ~(int64_t)3;
+    const uint32_t klim = (1u << 20) - 1u;
+    constexpr int NL = 2 * NT;
+    const int kb = lt_kbits<W>(n, NL);
+    const int sms = num_sms();
+    const uint32_t k0 = (uint32_t)seed, k1 = (uint32_t)(seed >> 32);
+    int64_t B = o.trees_per_chunk;
+    if (B <= 0) {
+        const size_t per_tree = (size_t)ld * (sizeof(W) + 4) + 256;
+        size_t budget = (size_t)std::max<int64_t>(0, o.memory_budget);
+        if (!budget) {
+            size_t fr = 0, tot = 0;
+            RWC_CUDA_TRY(cudaMemGetInfo(&fr, &tot));
+            budget = (size_t)(fr * 0.6);
+        }
+        B = (int64_t)std::max<size_t>(1, budget / per_tree);
+    }
+    B = std::min(B, T);
+    rwc_status status = RWC_OK;
+    int per_sm = 0;
+    dispatch(g, [&](auto o64, auto wt, auto ew) {
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(
+            &per_sm, l_trees<decltype(o64)::value, decltype(wt)::value, decltype(ew)::value, NT, W>, NT, 0);
+    });
+    if (per_sm < 1) return set_error(RWC_ERR_UNSUPPORTED, "walker block does not fit");
+    const int64_t slots = std::min<int64_t>(B, (int64_t)sms * per_sm);
+    Buf buf(stream);
+    const size_t wbytes = (size_t)B * ld * sizeof(W);
+    RWC_CUDA_TRY(cudaMallocAsync(&buf.p, wbytes + (size_t)slots * n * 4 + TAIL + 64, stream));
+    W *words = (W *)buf.p;
+    uint32_t *spill = (uint32_t *)((char *)buf.p + wbytes);
+    char *tail = (char *)(spill + slots * n);
+    tail = (char *)(((uintptr_t)tail + 63) & ~(uintptr_t)63);
+    int *err = (int *)tail;
+    unsigned long long *ctr = (unsigned long long *)(tail + 8);
+    Events ev(o.profile != 0);
+    int64_t *h = G->host_scalars;
+    for (int64_t c0 = 0; c0 < T; c0 += B) {
+        const int64_t Bc = std::min(B, T - c0);
+        int32_t *par = parents ? parents + c0 * n : nullptr, *vis = visits ? visits + c0 * n : nullptr;
+        RWC_CUDA_TRY(cudaMemsetAsync(tail, 0, TAIL, stream));
+        ev.rec(0, stream);
+        RWC_CUDA_TRY(cudaMemsetAsync(words, 0, (size_t)Bc * ld * sizeof(W), stream));
+        ev.rec(1, stream);
+        dispatch(g, [&](auto o64, auto wt, auto ew) {
+            ::rwc::count_launches(1);
+            l_trees<decltype(o64)::value, decltype(wt)::value, decltype(ew)::value, NT, W>
+                <<<(unsigned)std::min(Bc, slots), NT, 0, stream>>>(g, (uint32_t)(tree0 + c0), Bc, ld, k0, k1, klim,
+                                                                   kb, words, spill, err, ctr);
+        });
+        ev.rec(2, stream);
+        const int64_t bx = std::min<int64_t>((n + 255) / 256, (int64_t)sms * 8);
+        const int64_t by = std::max<int64_t>(1, std::min<int64_t>((int64_t)sms * 8 / bx, Bc / 8));
+        ::rwc::count_launches(1);
+        l_accum<W><<<dim3((unsigned)bx, (unsigned)by), 256, 0, stream>>>(n, g.root, words, ld, kb, lt_id0(NL), Bc, sums, par,
+                                                                         vis, err, ctr + 1);
+        ev.rec(3, stream);
+        RWC_CUDA_TRY(cudaGetLastError());
+        if (o.async_status) {
+            ::rwc::count_launches(1);
+            fold_lane_status<<<1, 1, 0, stream>>>(err, G->dev_status);
+            RWC_CUDA_TRY(cudaGetLastError());
+            continue;
+        }
+        RWC_CUDA_TRY(cudaMemcpyAsync(h, tail, 24, cudaMemcpyDeviceToHost, stream));
+        RWC_CUDA_TRY(cudaStreamSynchronize(stream));
+        const int e = (int)(h[0] & 0xffffffff);
+        if (e & LE_KOVF) return set_error(RWC_ERR_UNSUPPORTED, "a vertex was popped more than 2^20 - 1 times");
+        if (e & LE_LOOP) return set_error(RWC_ERR_CUDA, "sampler internal check failed");
+        if (e & LE_KREP) {
+            // a count outgrew the 32-bit word: this chunk again with 64-bit words
+            if (sizeof(W) == 8) return set_error(RWC_ERR_CUDA, "sampler internal check failed");
+            RWC_TRY((walker_range<NT, uint64_t>(G, seed, tree0 + c0, Bc, sums, par, vis, o, st, stream)));
+            continue;
+        }
+        if (st) {
+            const int64_t draws = h[2];
+            st->chunks += 1;
+            st->draws += draws;
+            st->marked += draws;
+            st->block_threads = NL;
+            st->phase_units[RWC_PHASE_INIT] += Bc * n;
+            st->phase_units[RWC_PHASE_WALK] += draws;
+            st->phase_units[RWC_PHASE_ACCUM] += Bc * n;
+            if (ev.on) {
+                st->phase_ms[RWC_PHASE_INIT] += ev.ms(0, 1);
+                st->phase_ms[RWC_PHASE_WALK] += ev.ms(1, 2);
+                st->phase_ms[RWC_PHASE_ACCUM] += ev.ms(2, 3);
+                st->phase_launches[RWC_PHASE_WALK] += 1;
+                st->phase_launches[RWC_PHASE_ACCUM] += 1;
+            }
+        }
+    }
+    if (st) st->mode = RWC_MODE_WALKER;
+    return status;
+}
+
+}  // namespace
+
+// Shared memory of one tree with nt threads.
+static size_t lane_smem(int64_t n, int nt) {
+    const size_t head = nt == 32 ? sizeof(LaneShared<32, 1>) : nt == 64 ? sizeof(LaneShared<64, 1>)
+                      : nt == 128 ? sizeof(LaneShared<128, 1>) : sizeof(LaneShared<256, 1>);
+    return head + (size_t)n * 4;
+}
+
+namespace {
+template <int NT>
+rwc_status smem_range(rwc_graph *G, uint64_t seed, int64_t tree0, int64_t T, double *sums, int32_t *parents,
+                      int32_t *visits, uint32_t klim, const rwc_options_t &o, rwc_stats_t *st,
+                      std::vector<uint32_t> &redo, int *h_err, cudaStream_t stream) {
+    const DevGraph &g = G->g;
+    const int64_t n = g.n;
+    const size_t smem = lane_smem(n, NT);
+    const int kb = lt_kbits<uint32_t>(n, NT);
+    const int sms = num_sms();
+    const uint32_t k0 = (uint32_t)seed, k1 = (uint32_t)(seed >> 32);
+    const bool need_spill = n > LT_STACK;
+    Buf buf(stream);
+    Events ev(o.profile != 0);
+    rwc_status status = RWC_OK;
+    int *err = nullptr;
+    *h_err = 0;
+    dispatch(g, [&](auto o64, auto wt, auto ew) {
+        auto kern = l_trees_smem<decltype(o64)::value, decltype(wt)::value, decltype(ew)::value, NT>;
+        auto launch = [&]() -> rwc_status {
+            RWC_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+            int per_sm = 0;
+            RWC_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, NT, smem));
+            if (per_sm < 1) return set_error(RWC_ERR_UNSUPPORTED, "graph too large for shared mode");
+            const int64_t blocks = std::min<int64_t>(T, (int64_t)sms * per_sm);
+            RWC_CUDA_TRY(cudaMallocAsync(&buf.p, TAIL + (size_t)T * 4 + (need_spill ? (size_t)blocks * n * 4 : 0), stream));
+            RWC_CUDA_TRY(cudaMemsetAsync(buf.p, 0, TAIL, stream));
+            err = (int *)buf.p;
+            ev.rec(0, stream);
+            ::rwc::count_launches(1);
+            kern<<<(unsigned)blocks, NT, smem, stream>>>(
+                g, (uint32_t)tree0, T, k0, k1, klim, kb, sums, parents, visits,
+                need_spill ? (uint32_t *)((char *)buf.p + TAIL) + T : nullptr, err,
+                (unsigned long long *)((char *)buf.p + 8), (uint32_t *)((char *)buf.p + TAIL));
+            ev.rec(1, stream);
+            RWC_CUDA_TRY(cudaGetLastError());
+            return RWC_OK;
+        };
+        status = launch();
+    });
+    RWC_TRY(status);
+    if (o.async_status) {
+        ::rwc::count_launches(1);
+        fold_lane_status<<<1, 1, 0, stream>>>(err, G->dev_status);
+        RWC_CUDA_TRY(cudaGetLastError());
+        return RWC_OK;
+    }
+    int64_t *h = G->host_scalars;
+    RWC_CUDA_TRY(cudaMemcpyAsync(h, buf.p, 32, cudaMemcpyDeviceToHost, stream));
+    RWC_CUDA_TRY(cudaStreamSynchronize(stream));
+    *h_err = (int)(h[0] & 0xffffffff);
+    if (*h_err) return RWC_OK;
+    if (h[3]) {
+        redo.resize((size_t)h[3]);
+        RWC_CUDA_TRY(cudaMemcpyAsync(redo.data(), (char *)buf.p + TAIL, redo.size() * 4, cudaMemcpyDeviceToHost, stream));
+        RWC_CUDA_TRY(cudaStreamSynchronize(stream));
+    }
+    if (st) {
+        st->draws += h[2];
+        st->marked += h[2];
+        st->chunks += 1;
+        st->phase_units[RWC_PHASE_WALK] += h[2];
+        if (ev.on) {
+            st->phase_ms[RWC_PHASE_WALK] += ev.ms(0, 1);
+            st->phase_launches[RWC_PHASE_WALK] += 1;
+        }
+    }
+    return RWC_OK;
+}
+}  // namespace
+
+namespace {
+// Trees tree0 .. tree0 + T - 1 with their words in shared memory; status is
+// the caller's message.
+rwc_status sample_smem(rwc_graph *G, uint64_t seed, int64_t tree0, int64_t T, double *sums, int32_t *parents,
+                       int32_t *visits, uint32_t klim, const rwc_options_t &o, rwc_stats_t *st, int *err,
+                       cudaStream_t stream) {
+    const int64_t n = G->g.n;
+    const int64_t chunk = std::min(T, o.trees_per_chunk > 0 ? std::min(o.trees_per_chunk, WIDE_CAP) : WIDE_CAP);
+    // threads per tree: 1024 on an SM, over the trees that it holds at once (BA
+    // n = 12000, 1000 trees: 1.0, 0.65 and 0.50 ms with 64, 128 and 256 threads;
+    // n = 2000, 1000 trees: 0.142, 0.122 and 0.135 ms)
+    int NTs = 256;
+    while (NTs > 64 && NTs * std::min<int64_t>((227 * 1024) / (int64_t)(lane_smem(n, NTs) + 1024),
+                                               (chunk + num_sms() - 1) / num_sms()) > 1024)
+        NTs /= 2;
+    for (int64_t c0 = 0; c0 < T; c0 += chunk) {
+        const int64_t Tc = std::min(chunk, T - c0);
+        int32_t *par = parents ? parents + c0 * n : nullptr, *vis = visits ? visits + c0 * n : nullptr;
+        std::vector<uint32_t> redo;
+        if (NTs == 256) RWC_TRY(smem_range<256>(G, seed, tree0 + c0, Tc, sums, par, vis, klim, o, st, redo, err, stream));
+        else if (NTs == 128) RWC_TRY(smem_range<128>(G, seed, tree0 + c0, Tc, sums, par, vis, klim, o, st, redo, err, stream));
+        else RWC_TRY(smem_range<64>(G, seed, tree0 + c0, Tc, sums, par, vis, klim, o, st, redo, err, stream));
+        if (*err) return RWC_OK;
+        // trees whose counts outgrew 32-bit words, again with 64-bit ones
+        for (uint32_t t : redo)
+            RWC_TRY((walker_range<256, uint64_t>(G, seed, tree0 + c0 + t, 1, sums, par ? par + (int64_t)t * n : nullptr,
+                                                 vis ? vis + (int64_t)t * n : nullptr, o, st, stream)));
+        if (st) {
+            st->chunks -= (int64_t)redo.size();
+            st->block_threads = NTs;
+        }
+    }
+    return RWC_OK;
+}
+}  // namespace
+
+namespace {
+constexpr size_t SMEM_MAX = 226 * 1024;   // dynamic shared memory of one block beside 1 KB of its own
+
+// Whether walker mode keeps this graph's words in shared memory: a lane's hop
+// is 45 cycles there against 150 to 230 in global memory, where some lane of a
+// warp nearly always misses L1 (RGG n = 40000, 300 trees: 14 against 41 ms).  An
+// asynchronous call cannot list trees for wider words, so there every allowed
+// count has to fit.
+bool walker_in_smem(int64_t n, const rwc_options_t &o) {
+    return lane_smem(n, 256) <= SMEM_MAX && (!o.async_status || lt_kbits<uint32_t>(n, 256) >= 20);
+}
+}  // namespace
+
+// The concurrent walkers (sample_walker) keep calls that ask for their options
+// and, with words in global memory, graphs of unbounded degree above 400000
+// vertices: there every access goes to HBM and the walkers' fewer words per
+// draw count (R-MAT n = 262144, 500 trees: 24.4 -> 13.6 ms here; n = 524288:
+// 36.8 and 33.2; n = 1048576: 69 and 80).
+bool lane_walker_takes(const rwc_graph *G, const rwc_options_t &o) {
+    const DevGraph &g = G->g;
+    if (o.walker_policy || o.block_threads || o.max_wait_ns || o.profile >= 2) return false;
+    if (g.n >= ((int64_t)1 << 31) - 4096) return false;
+    return walker_in_smem(g.n, o) || g.ell || g.n <= 400000;
+}
+
+rwc_status sample_lane_walker(rwc_graph *G, uint64_t seed, int64_t tree0, int64_t T, double *sums,
+                              int32_t *parents, int32_t *visits, const rwc_options_t &o, rwc_stats_t *st,
+                              cudaStream_t stream) {
+    const int64_t n = G->g.n;
+    if (walker_in_smem(n, o)) {
+        int e = 0;
+        RWC_TRY(sample_smem(G, seed, tree0, T, sums, parents, visits, (1u << 20) - 1u, o, st, &e, stream));
+        if (e & LE_KOVF) return set_error(RWC_ERR_UNSUPPORTED, "a vertex was popped more than 2^20 - 1 times");
+        if (e) return set_error(RWC_ERR_CUDA, "sampler internal check failed");
+        if (st) st->mode = RWC_MODE_WALKER;
+        return RWC_OK;
+    }
+    auto run = [&](auto nt) -> rwc_status {
+        constexpr int NT = decltype(nt)::value;
+        // 64-bit words at once where 32 bits leave less than 8 for the count,
+        // and for asynchronous calls unless every allowed count fits
+        const int kb = n < ((int64_t)1 << 30) ? lt_kbits<uint32_t>(n, 2 * NT) : 0;
+        if (kb < (o.async_status ? 20 : 8))
+            return walker_range<NT, uint64_t>(G, seed, tree0, T, sums, parents, visits, o, st, stream);
+        return walker_range<NT, uint32_t>(G, seed, tree0, T, sums, parents, visits, o, st, stream);
+    };
+    // threads per tree by the trees that an SM gets: 32 (64 lanes) when they
+    // fill it, more when few are left to it (300 x 300 grid, 300 trees: 572, 429
+    // and 449 ms with 32, 128 and 512; 512 x 512, 64 trees: 2.01, 1.44, 1.18 s);
+    // graphs of unbounded degree have ends for 1024 lanes (R-MAT n = 262144, 2000
+    // trees: 101, 60 and 48 ms)
+    const int64_t share = (T + num_sms() - 1) / num_sms();
+    if (G->g.ell && share >= 8) return run(int_c<32>{});
+    if (G->g.ell && share >= 2) return run(int_c<128>{});
+    return run(int_c<512>{});
+}
+
+rwc_status sample_lane_shared(rwc_graph *G, uint64_t seed, int64_t tree0, int64_t T, double *sums,
+                              int32_t *parents, int32_t *visits, const rwc_options_t &o, rwc_stats_t *st,
+                              cudaStream_t stream) {
+    int e = 0;
+    RWC_TRY(sample_smem(G, seed, tree0, T, sums, parents, visits, 65535u, o, st, &e, stream));
+    if (e & LE_KOVF) return set_error(RWC_ERR_UNSUPPORTED, "a vertex was popped more than 65535 times; use RWC_MODE_GLOBAL");
+    if (e) return set_error(RWC_ERR_CUDA, "sampler internal check failed");
+    if (st) st->mode = RWC_MODE_SHARED;
+    return RWC_OK;
+}
+
+}  // namespace rwc

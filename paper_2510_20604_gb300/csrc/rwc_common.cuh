@@ -103,6 +103,15 @@ rwc_status sample_walker(rwc_graph *G, uint64_t seed, int64_t tree0, int64_t T, 
 rwc_status sample_park(rwc_graph *G, uint64_t seed, int64_t tree0, int64_t T, double *sums,
                        int32_t *parents, int32_t *visits, const rwc_options_t &o,
                        rwc_stats_t *st, cudaStream_t stream);
+// One warp per tree (lane.cu): words in shared memory, or in global memory.
+rwc_status sample_lane_shared(rwc_graph *G, uint64_t seed, int64_t tree0, int64_t T, double *sums,
+                              int32_t *parents, int32_t *visits, const rwc_options_t &o,
+                              rwc_stats_t *st, cudaStream_t stream);
+// Whether sample_lane_walker serves a walker-mode call (else sample_walker).
+bool lane_walker_takes(const rwc_graph *G, const rwc_options_t &o);
+rwc_status sample_lane_walker(rwc_graph *G, uint64_t seed, int64_t tree0, int64_t T, double *sums,
+                              int32_t *parents, int32_t *visits, const rwc_options_t &o,
+                              rwc_stats_t *st, cudaStream_t stream);
 // The walkers' start order (a fixed permutation of the non-root vertices, on
 // the device, made on first use and kept with the graph).
 rwc_status walker_order(rwc_graph *G, const int32_t **out);

@@ -620,8 +620,12 @@ extern "C" rwc_status rwc_sample_trees(rwc_graph_t *G, uint64_t seed, int64_t tr
     }
     rwc_status s;
     try {
-        if (mode == RWC_MODE_SHARED)
+        if (mode == RWC_MODE_SHARED && !o.max_rounds && !o.block_threads)
+            s = sample_lane_shared(G, seed, tree0, T, sums, parents, visits, o, stats, (cudaStream_t)stream);
+        else if (mode == RWC_MODE_SHARED)
             s = sample_shared(G, seed, tree0, T, sums, parents, visits, o, stats, (cudaStream_t)stream);
+        else if (mode == RWC_MODE_WALKER && lane_walker_takes(G, o))
+            s = sample_lane_walker(G, seed, tree0, T, sums, parents, visits, o, stats, (cudaStream_t)stream);
         else if (mode == RWC_MODE_WALKER)
             s = sample_walker(G, seed, tree0, T, sums, parents, visits, o, stats, (cudaStream_t)stream);
         else if (mode == RWC_MODE_GLOBAL)

@@ -34,6 +34,7 @@
 #include <type_traits>
 #include <vector>
 
+#include "lane_tree.cuh"
 #include "rwc_common.cuh"
 
 namespace rwc {
@@ -135,44 +136,6 @@ enum : int { S_IDLE = 0, S_WALK, S_POP, S_REL, S_SET, S_WAITK, S_WAITV, S_WAITH,
 #ifndef RWC_WALKER_MAXNREG
 #define RWC_WALKER_MAXNREG 64
 #endif
-
-// The row of a vertex that may be drawn: its CSR bounds (EW = 0), or, for
-// graphs whose degrees are at most EW (4 or 8), its inline neighbour list
-// (heads in arc order, -1 after the last), read with one or two 16-byte loads.
-template <bool OFF64, int EW>
-struct DrawRow {
-    int4 e[EW / 4];
-    __device__ __forceinline__ void load(const DevGraph &g, int32_t u) {
-#pragma unroll
-        for (int i = 0; i < EW / 4; ++i) e[i] = __ldg(g.ell + (int64_t)u * (EW / 4) + i);
-    }
-    // head of the arc picked by the 32-bit uniform x: arc floor(x deg / 2^32)
-    __device__ __forceinline__ int32_t pick(uint32_t x) const {
-        uint32_t deg = 0;
-#pragma unroll
-        for (int i = 0; i < EW / 4; ++i)
-            deg += (e[i].x >= 0) + (e[i].y >= 0) + (e[i].z >= 0) + (e[i].w >= 0);
-        const uint32_t j = __umulhi(x, deg);
-        const int4 q = (EW == 4 || j < 4) ? e[0] : e[EW / 4 - 1];
-        const uint32_t jj = j & 3u;
-        return jj < 2 ? (jj == 0 ? q.x : q.y) : (jj == 2 ? q.z : q.w);
-    }
-};
-template <bool OFF64>
-struct DrawRow<OFF64, 0> {
-    int64_t rb;
-    uint32_t deg;
-    __device__ __forceinline__ void load(const DevGraph &g, int32_t u) { row_bounds<OFF64>(g, u, rb, deg); }
-    template <bool WT>
-    __device__ __forceinline__ int32_t pick_csr(const DevGraph &g, uint32_t x, uint32_t y) const {
-        const uint32_t j = __umulhi(x, deg);
-        if (WT) {
-            const WArc arc = g.warc[rb + j];
-            return (y < arc.thr) ? arc.col : arc.alias_col;
-        }
-        return __ldg(g.col + rb + j);
-    }
-};
 
 template <bool OFF64, bool WT, int EW, bool DIAG>
 __global__ void __maxnreg__(RWC_WALKER_MAXNREG) w_trees(DevGraph g, WState s, int64_t B, uint32_t tree0,

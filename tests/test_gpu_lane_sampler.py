@@ -1,0 +1,88 @@
+"""The lane sampler (one tree per warp or block, cycle popping in rounds)
+where it can go wrong: the edges of its word layout, of its shared-memory and
+global-memory variants and of the stack of pending ends.  Trees are compared
+with the oracle's sequential Wilson bit for bit."""
+import numpy as np
+import pytest
+import torch
+
+import paper_2510_20604_gb300 as rwc
+import synth
+from oracle import wilson as ow
+
+pytestmark = pytest.mark.gpu
+
+
+def _exact(g, T, opt=None, seed=1, tree0=0, flags=0, root=-1):
+    G = rwc.Graph.from_synth(g, root=root, flags=flags)
+    sums, st, par, vis = G.sample(T, seed=seed, tree0=tree0, want_trees=True, opt=opt)
+    ref = ow.Sampler(g, root=G.root, seed=seed).sample(tree0, T, want_trees=True, nthreads=min(T, 8))
+    assert np.array_equal(par.cpu().numpy(), ref["parents"])
+    assert np.array_equal(vis.cpu().numpy(), ref["visits"])
+    assert np.array_equal(sums.cpu().numpy(), ref["sums"])
+    return st
+
+
+def _heavy_pair(n, ratio):
+    """A BA graph with one edge `ratio` times heavier than the others, between
+    two vertices of small degree: a walk that enters the pair goes to and fro
+    about `ratio` times, so two counts are large.  Returns (graph, hub)."""
+    b = synth.ba(n, 2, seed=9)
+    deg = np.diff(b.row_ptr)
+    u, v, _ = b.undirected()
+    w = np.ones(len(u), np.float32)
+    w[np.argmin(deg[u] + deg[v])] = ratio
+    return synth.from_edges(n, u, v, w), int(np.argmax(deg))
+
+
+@pytest.mark.parametrize("n", [61, 62, 63, 126, 127, 190, 192, 193, 255, 256, 257, 1023])
+def test_sizes_around_the_word_layout_and_the_stack(n):
+    # p' takes one more bit at n + lanes + 2 = 2^b; the stack of pending ends
+    # spills to global memory only for n > 192
+    _exact(synth.ba(n, 2, seed=n), 40)
+    _exact(synth.cycle(n), 6)
+
+
+@pytest.mark.parametrize("mode", [rwc.MODE_AUTO, rwc.MODE_WALKER])
+@pytest.mark.parametrize("T", [1, 3, 160, 700])
+def test_threads_per_tree_follow_the_trees_per_sm(mode, T):
+    _exact(synth.rgg(1500, 9.0, seed=3, sigma=0.5), T, rwc.Options(mode=mode), tree0=5)
+
+
+@pytest.mark.parametrize("n", [55000, 57000, 58000])
+@pytest.mark.parametrize("sigma", [None, 0.7])
+def test_shared_and_global_words_meet(n, sigma):
+    _exact(synth.rmat(16, 8, seed=2, sigma=sigma) if n == 57000 else synth.rgg(n, 8.0, seed=n, sigma=sigma), 3,
+           flags=rwc.GRAPH_INT64_OFFSETS if sigma else 0)
+
+
+def test_long_chains_spill_the_stack():
+    # a grid above the shared-memory size (global words, inline rows) and a
+    # path: long popped cycles fill the stack of pending ends
+    _exact(synth.grid2d(250, 245), 2)
+    _exact(synth.path(900), 5)
+
+
+def test_counts_beyond_the_word_are_sampled_again():
+    # 40000 vertices leave 15 bits for the count in a 32-bit word
+    g, hub = _heavy_pair(40000, 300000.0)
+    opt = rwc.Options(mode=rwc.MODE_WALKER)
+    st = _exact(g, 3, opt, root=hub)
+    assert st.chunks == 1
+    G = rwc.Graph.from_synth(g, root=hub)
+    ref, _, _, vis = G.sample(3, want_trees=True, opt=opt)
+    assert int(vis.max()) > 32768
+    s = torch.zeros(g.n, dtype=torch.float64, device="cuda")
+    rwc.rwc_sample_trees(G.handle, 1, 0, 3, s, None, None, rwc.Options(mode=rwc.MODE_WALKER, async_status=1))
+    rwc.rwc_sync_status(G.handle)
+    assert torch.equal(s, ref)
+
+
+@pytest.mark.parametrize("mode,ratio", [(rwc.MODE_SHARED, 1e6), (rwc.MODE_WALKER, 2e7)])
+def test_count_limits_are_reported(mode, ratio):
+    # SHARED allows 65535 pops of a vertex, WALKER 2^20 - 1
+    g, hub = _heavy_pair(300, ratio)
+    G = rwc.Graph.from_synth(g, root=hub)
+    with pytest.raises(rwc.RWCError) as e:
+        G.sample(16, opt=rwc.Options(mode=mode))
+    assert e.value.status == 6 and "popped more than" in str(e.value)
