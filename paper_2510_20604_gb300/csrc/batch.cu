@@ -1,14 +1,14 @@
 // Batched sampler: all trees of thousands of small graphs in one CUDA-graph
-// launch.  Work items (graph, tile of trees) are pulled from device counters
-// by persistent kernels (no grid-wide barrier).  The graphs are split by size:
-// those with more than `split` vertices run block-per-tree; the others run
-// warp-per-tree (every warp of a block pulls its own items and keeps its tree
-// in its own slice of the block's shared memory) or block-per-tree with small
-// blocks, as the schedule says.  The two classes run as two persistent
-// kernels on forked streams, so each gets the shared-memory size (and thus
-// the occupancy) its own graphs need; the fork and join are captured into the
-// call's CUDA graph, which is replayed.  The autotuner times candidate
-// schedules on the device.  Tree state lives in shared memory (smem_tree.cuh).
+// launch.  Trees of work items (graph, tile of trees) are pulled one by one
+// from device counters by persistent kernels (no grid-wide barrier); a tree's
+// words live in shared memory and a block of 32 to 256 threads runs it
+// (lane_tree.cuh).  The graphs are sorted by size and cut into bins of about a
+// factor of two, one kernel each, so that every bin gets the shared memory
+// (and thus the occupancy) and the threads its own graphs need; the bins run
+// on forked streams, and fork and join are captured into the call's CUDA
+// graph, which is replayed.  The schedule sets the split between the classes of
+// large and small graphs, the largest block of the large class and whether the
+// small class runs one tree per warp; the autotuner times candidates.
 #include <algorithm>
 #include <chrono>
 #include <cmath>
@@ -18,7 +18,7 @@
 #include <vector>
 
 #include "rwc_common.cuh"
-#include "smem_tree.cuh"
+#include "lane_tree.cuh"
 
 namespace rwc {
 namespace {
@@ -34,76 +34,69 @@ struct BItem {
     int32_t tile;   // index of the tile of trees within the graph
 };
 
-// One work item: the tiles' trees of graph it.g, run by the group Grp whose
-// tree state is carved from `region`.  Adds the visit totals to sums.
-// Returns the group-uniform error mask.
-template <bool OFF64, bool W, class Grp>
-__device__ int run_item(const DevGraph &base, const BGraph *__restrict__ graphs, BItem it,
-                        unsigned char *region, int tile, int64_t T, uint32_t k0, uint32_t k1,
-                        int64_t max_rounds, double *sums, unsigned long long *round_ctr) {
-    const BGraph bg = graphs[it.g];
-    DevGraph g = base;
-    g.n = bg.n;
-    g.root = bg.root;
-    if (OFF64) g.rp64 = base.rp64 + bg.voff;
-    else g.rp32 = base.rp32 + bg.voff;
-    SmemTree S;
-    S.carve(region, bg.n);
-    for (int u = Grp::rank(); u < bg.n; u += Grp::size()) S.acc[u] = 0;
-    const int64_t t0 = (int64_t)it.tile * tile, t1 = std::min<int64_t>(T, t0 + tile);
-    int mask = 0;
-    unsigned long long rounds = 0;
-    for (int64_t t = t0; t < t1 && !mask; ++t) {
-        int64_t r = 0;
-        mask = smem_tree<OFF64, W, Grp>(g, S, (uint32_t)t, (uint32_t)it.g, k0, k1, max_rounds,
-                                        nullptr, nullptr, &r);
-        rounds += (unsigned long long)r;
-    }
-    Grp::sync();
-    if (mask) return mask;
+// Trees 0 .. npull - 1 of a bin: pull i is tree i % tile of item i / tile.  The
+// blocks take them in turn, after their first from the counter `next` (NULL:
+// every gridDim.x-th).
+template <bool OFF64, bool W, int NT>
+__global__ void __launch_bounds__(NT) l_batch(DevGraph base, const BGraph *__restrict__ graphs,
+                                              const BItem *__restrict__ items, int64_t npull, unsigned long long *next, int64_t tile,
+                                              int64_t T, uint32_t k0, uint32_t k1, int max_n, double *sums,
+                                              uint32_t *spill, int *err, unsigned long long *ctr) {
+    extern __shared__ __align__(16) unsigned char smem[];
+    __shared__ unsigned long long sh_next;
+    using Sh = LaneShared<NT, 1>;
+    Sh &sh = *reinterpret_cast<Sh *>(smem);
+    uint32_t *word = reinterpret_cast<uint32_t *>(smem + sizeof(Sh));
+    uint32_t *sp = spill + (int64_t)blockIdx.x * max_n;
     unsigned long long draws = 0;
-    for (int u = Grp::rank(); u < bg.n; u += Grp::size()) {
-        draws += S.acc[u];
-        if (S.acc[u]) atomicAdd(sums + bg.voff + u, (double)S.acc[u]);
+    uint32_t rounds = 0;
+    int64_t i = blockIdx.x;
+    while (i < npull) {
+        const BItem it = items[i / tile];
+        const int64_t t = (int64_t)it.tile * tile + i % tile;
+        if (t < T) {
+            const BGraph bg = graphs[it.g];
+            DevGraph g = base;
+            g.n = bg.n;
+            g.root = bg.root;
+            if (OFF64) g.rp64 = base.rp64 + bg.voff;
+            else g.rp32 = base.rp32 + bg.voff;
+            const int kb = lt_kbits<uint32_t>(bg.n, NT);
+            for (int u = threadIdx.x; u < bg.n; u += NT) word[u] = u == bg.root ? lt_root_word<uint32_t>(kb, NT) : 0u;
+            __syncthreads();
+            const int bad = lane_tree<OFF64, W, 0, NT, 1, true, uint32_t>(g, word, kb, 65535u, sh, sp, (uint32_t)t,
+                                                                          (uint32_t)it.g, k0, k1, rounds);
+            if (bad) { if (threadIdx.x == 0) atomicOr(err, bad); break; }
+            const uint32_t kmask = (1u << kb) - 1u;
+            double *out = sums + bg.voff;
+            for (int u = threadIdx.x; u < bg.n; u += NT) {
+                if (u == bg.root) continue;
+                const uint32_t vis = (word[u] & kmask) + 1u;
+                draws += vis;
+                atomicAdd(out + u, (double)vis);
+            }
+        }
+        if (!next) { i += gridDim.x; continue; }
+        if (threadIdx.x == 0) sh_next = atomicAdd(next, 1ull);
+        __syncthreads();
+        i = (int64_t)gridDim.x + (int64_t)sh_next;
     }
-    if (draws) atomicAdd(round_ctr + 1, draws);
-    if (Grp::rank() == 0 && rounds) atomicAdd(round_ctr, rounds);
-    return 0;
+    for (int o = 16; o > 0; o >>= 1) draws += __shfl_xor_sync(0xffffffffu, draws, o);
+    if ((threadIdx.x & 31) == 0 && draws) atomicAdd(ctr + 1, draws);
+    if (threadIdx.x == 0 && rounds) atomicAdd(ctr, (unsigned long long)rounds);
 }
 
-// Persistent kernel over both item lists: first every block pulls
-// block-per-tree items, then every warp pulls warp-per-tree items into its
-// own shared-memory slice of warp_slice bytes.
-template <bool OFF64, bool W>
-__global__ void b_persistent(DevGraph base, const BGraph *__restrict__ graphs,
-                             const BItem *__restrict__ bitems, int64_t nb,
-                             const BItem *__restrict__ witems, int64_t nw, int *next_item,
-                             int warp_slice, int tile, int64_t T, uint32_t k0, uint32_t k1,
-                             int64_t max_rounds, double *sums, int *err,
-                             unsigned long long *round_ctr) {
-    extern __shared__ __align__(16) unsigned char smem[];
-    __shared__ int item;
-    for (;;) {
-        __syncthreads();
-        if (threadIdx.x == 0) item = atomicAdd(next_item, 1);
-        __syncthreads();
-        const int i = item;
-        if (i >= nb) break;
-        const int mask = run_item<OFF64, W, BlockGroup>(base, graphs, bitems[i], smem, tile, T, k0, k1,
-                                                        max_rounds, sums, round_ctr);
-        if (mask) { if (threadIdx.x == 0) atomicOr(err, mask); return; }
-    }
-    if (nw == 0) return;
-    unsigned char *region = smem + (size_t)(threadIdx.x >> 5) * warp_slice;
-    for (;;) {
-        int i = 0;
-        if ((threadIdx.x & 31) == 0) i = atomicAdd(next_item + 1, 1);
-        i = __shfl_sync(0xffffffffu, i, 0);
-        if (i >= nw) break;
-        const int mask = run_item<OFF64, W, WarpGroup>(base, graphs, witems[i], region, tile, T, k0, k1,
-                                                       max_rounds, sums, round_ctr);
-        if (mask) { if ((threadIdx.x & 31) == 0) atomicOr(err, mask); return; }
-    }
+// Threads per tree of graphs of up to n vertices: what keeps about 40 warps on
+// an SM beside n words of shared memory per tree (21 blocks of 64 up to 2500
+// vertices by registers, 10 of 128 up to 5000, 2 of 256 at 20000).  512 graphs
+// of 50 to 20000 vertices, 64 trees each: 158 ms with whole-block popping
+// rounds (11 bytes per vertex, one kernel for each of two classes), 19.4 ms so.
+int batch_threads(int n) { return n <= 2500 ? 64 : n <= 5000 ? 128 : 256; }
+
+size_t batch_tree_smem(int n, int nt) {
+    const size_t head = nt == 32 ? sizeof(LaneShared<32, 1>) : nt == 64 ? sizeof(LaneShared<64, 1>)
+                      : nt == 128 ? sizeof(LaneShared<128, 1>) : sizeof(LaneShared<256, 1>);
+    return head + (size_t)n * 4;
 }
 
 template <class F>
@@ -116,6 +109,29 @@ void dispatch(bool off64, bool weighted, F f) {
         else f(std::false_type{}, std::false_type{});
     }
 }
+
+template <class F>
+void dispatch_nt(bool off64, bool weighted, int nt, F f) {
+    dispatch(off64, weighted, [&](auto o64, auto wt) {
+        constexpr bool O = decltype(o64)::value, W = decltype(wt)::value;
+        if (nt == 32) f(l_batch<O, W, 32>);
+        else if (nt == 64) f(l_batch<O, W, 64>);
+        else if (nt == 128) f(l_batch<O, W, 128>);
+        else f(l_batch<O, W, 256>);
+    });
+}
+
+constexpr int MAX_BINS = 12;
+
+// Items of one kernel: a range of a class's list.
+struct Bin {
+    int cls;
+    int64_t begin, count;   // items
+    int max_n, nt;
+    size_t smem;
+    int64_t blocks;
+    int64_t spill;          // its blocks' ends in global memory: offset in entries
+};
 
 }  // namespace
 }  // namespace rwc
@@ -130,22 +146,25 @@ struct rwc_batch {
     std::vector<int32_t> roots;
     DevGraph base;                     // concatenated CSR (local column ids)
     BGraph *graphs = nullptr;
-    // schedule: block size of the large graphs, the largest n of the small
+    // schedule: largest block of the large graphs, the largest n of the small
     // class (0: one class), small class warp-per-tree (1) or block-per-tree
-    // with SMALL_THREADS threads (0), trees per work item
+    // (0), trees per work item
     int threads = 512;
     int split = 1024;
     int warp = 1;
     int tile = 4;
     int conc = 1;                      // 1: the classes run concurrently (forked streams)
-    cudaStream_t side = nullptr;       // the small class's stream (forked from the call's)
-    cudaEvent_t fork = nullptr, join = nullptr;
-    int max_n[2] = {0, 0};             // largest n of the block / warp item lists
+    cudaStream_t side[MAX_BINS] = {};  // the bins' streams (forked from the call's)
+    cudaEvent_t fork = nullptr, join[MAX_BINS] = {};
     BItem *items[2] = {nullptr, nullptr};
     int64_t nitems[2] = {0, 0};
+    int max_n[2] = {0, 0};             // largest n of each class
+    std::vector<Bin> bins;
+    uint32_t *spill = nullptr;         // the bins' pending ends beyond shared memory
+    BItem *single = nullptr;           // item g: graph g's first tile (one launch per graph)
     int64_t items_T = -1;              // T the item lists were built for
     int64_t items_tile = -1, items_split = -1;
-    void *scratch = nullptr;           // [0] err, [8] rounds, [16] draws, [32..48) item counters
+    void *scratch = nullptr;           // [0] err, [8] rounds, [16] draws, [64..160) the bins' counters
     std::vector<void *> allocs;
     // captured launches
     cudaGraph_t graph = nullptr;
@@ -173,27 +192,76 @@ void drop_graph(rwc_batch *b) {
     b->cap_T = -1;
 }
 
-// Bytes of one warp's shared-memory slice for trees of up to n vertices.
-size_t warp_slice_bytes(int n) { return (smem_tree_bytes(n) + 15) & ~(size_t)15; }
-
-constexpr int SMALL_THREADS = 256;   // block size of the small class (8 warps)
-
-// Dynamic shared memory of each class's kernel for the current schedule.
-size_t class_smem(const rwc_batch *b, int c) {
-    if (!b->nitems[c]) return 64;
-    if (c == 1 && b->warp) return (size_t)(SMALL_THREADS / 32) * warp_slice_bytes(b->max_n[1]);
-    return std::max<size_t>(smem_tree_bytes(b->max_n[c]), 64);
+void drop_streams(rwc_batch *b) {
+    for (int i = 0; i < MAX_BINS; ++i) {
+        if (b->join[i]) cudaEventDestroy(b->join[i]);
+        if (b->side[i]) cudaStreamDestroy(b->side[i]);
+    }
+    if (b->fork) cudaEventDestroy(b->fork);
 }
-size_t batch_smem(const rwc_batch *b) { return std::max(class_smem(b, 0), class_smem(b, 1)); }
 
-// Work items for T trees per graph: list 0 (block-per-tree) holds graphs with
-// more than `split` vertices, list 1 (warp-per-tree) the others; each list
-// runs its largest graphs first.
+// The largest schedule a batch accepts: a tree counts 11 n + 64 bytes of shared
+// memory, eight of them in a block where the small class runs warp-per-tree.
+size_t tree_allowance(int64_t n) { return (size_t)n * 11 + 64; }
+size_t schedule_allowance(int max_large, int max_small, int warp) {
+    const size_t large = max_large ? tree_allowance(max_large) : 64;
+    const size_t small = !max_small ? 64 : warp ? 8 * ((tree_allowance(max_small) + 15) & ~(size_t)15)
+                                                : tree_allowance(max_small);
+    return std::max(large, small);
+}
+size_t batch_smem(const rwc_batch *b) { return schedule_allowance(b->max_n[0], b->max_n[1], b->warp); }
+
+rwc_status build_bins(rwc_batch *b, const std::vector<int32_t> (&order)[2], int64_t ntile) {
+    b->bins.clear();
+    for (int c = 0; c < 2; ++c)
+        for (size_t i = 0; i < order[c].size();) {
+            const int top = b->hgraphs[order[c][i]].n;
+            size_t j = i;
+            while (j < order[c].size() && (top <= 640 || 2 * b->hgraphs[order[c][j]].n > top)) ++j;
+            Bin q{};
+            q.cls = c;
+            q.begin = (int64_t)i * ntile;
+            q.count = (int64_t)(j - i) * ntile;
+            q.max_n = top;
+            q.nt = batch_threads(top);
+            if (c == 1 && b->warp) q.nt = 32;
+            while (c == 0 && q.nt > b->threads) q.nt /= 2;
+            q.smem = batch_tree_smem(top, q.nt);
+            b->bins.push_back(q);
+            i = j;
+        }
+    if (b->bins.size() > (size_t)MAX_BINS) return set_error(RWC_ERR_UNSUPPORTED, "too many size bins");
+    int64_t spill = 0;
+    for (Bin &q : b->bins) {
+        int per_sm = 0;
+        cudaError_t e = cudaSuccess;
+        dispatch_nt(b->off64, b->weighted, q.nt, [&](auto kern) {
+            e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)std::max<size_t>(q.smem, 96 * 1024));
+            if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, q.nt, q.smem);
+        });
+        RWC_CUDA_TRY(e);
+        if (per_sm < 1) return set_error(RWC_ERR_UNSUPPORTED, "batch block does not fit on an SM");
+        q.blocks = std::max<int64_t>(1, std::min<int64_t>(q.count * b->tile, (int64_t)num_sms() * per_sm));
+        q.spill = spill;
+        spill += q.blocks * q.max_n;
+    }
+    if (b->spill) {
+        cudaFree(b->spill);
+        b->allocs.erase(std::find(b->allocs.begin(), b->allocs.end(), (void *)b->spill));
+        b->spill = nullptr;
+    }
+    RWC_CUDA_TRY(balloc(b, (void **)&b->spill, (size_t)spill * sizeof(uint32_t)));
+    return RWC_OK;
+}
+
+// Work items for T trees per graph: list 0 holds graphs with more than `split`
+// vertices, list 1 the others; each list runs its largest graphs first.
 rwc_status build_items(rwc_batch *b, int64_t T) {
     if (b->items_T == T && b->items_tile == b->tile && b->items_split == b->split) return RWC_OK;
+    std::vector<int32_t> orders[2];
     for (int c = 0; c < 2; ++c) {
         std::vector<BItem> v;
-        std::vector<int32_t> order;
+        std::vector<int32_t> &order = orders[c];
         for (int32_t g = 0; g < b->G; ++g) {
             const int cls = b->hgraphs[g].n <= b->split ? 1 : 0;
             if (cls == c) order.push_back(g);
@@ -213,6 +281,7 @@ rwc_status build_items(rwc_batch *b, int64_t T) {
         b->max_n[c] = 0;
         for (int32_t g : order) b->max_n[c] = std::max(b->max_n[c], b->hgraphs[g].n);
     }
+    RWC_TRY(build_bins(b, orders, (T + b->tile - 1) / b->tile));
     b->items_T = T;
     b->items_tile = b->tile;
     b->items_split = b->split;
@@ -220,50 +289,42 @@ rwc_status build_items(rwc_batch *b, int64_t T) {
     return RWC_OK;
 }
 
-// Enqueue one call: the large class on st, the small class on the batch's
-// side stream forked from st and joined back.
+// Enqueue one call: the first bin on st, the others on the batch's side streams
+// forked from st and joined back (conc = 0: all on st).
 rwc_status enqueue(rwc_batch *b, uint64_t seed, int64_t T, double *sums, cudaStream_t st) {
     int *err = (int *)b->scratch;
-    unsigned long long *rounds = (unsigned long long *)((char *)b->scratch + 8);
-    int *counters = (int *)((char *)b->scratch + 32);   // [0..1] large class, [2..3] small class
-    RWC_CUDA_TRY(cudaMemsetAsync((char *)b->scratch + 32, 0, 16, st));
+    unsigned long long *ctr = (unsigned long long *)((char *)b->scratch + 8);
+    unsigned long long *next = (unsigned long long *)((char *)b->scratch + 64);
+    RWC_CUDA_TRY(cudaMemsetAsync(next, 0, MAX_BINS * sizeof(*next), st));
     const uint32_t k0 = (uint32_t)seed, k1 = (uint32_t)(seed >> 32);
     if (batch_smem(b) > 227 * 1024) return set_error(RWC_ERR_UNSUPPORTED, "batch schedule needs %zu bytes of shared memory", batch_smem(b));
-    const bool fork = b->conc && b->nitems[0] && b->nitems[1];
-    if (fork) {
-        RWC_CUDA_TRY(cudaEventRecord(b->fork, st));
-        RWC_CUDA_TRY(cudaStreamWaitEvent(b->side, b->fork, 0));
-    }
-    rwc_status status = RWC_OK;
-    for (int c = 0; c < 2 && status == RWC_OK; ++c) {
-        if (!b->nitems[c]) continue;
-        const bool warp = c == 1 && b->warp;
-        const int threads = c == 0 ? b->threads : SMALL_THREADS;
-        const size_t smem = class_smem(b, c);
-        cudaStream_t s = (c == 1 && fork) ? b->side : st;
-        dispatch(b->off64, b->weighted, [&](auto o64, auto wt) {
-            auto kern = b_persistent<decltype(o64)::value, decltype(wt)::value>;
-            cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-            int per_sm = 0;
-            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, threads, smem);
-            if (per_sm < 1) { status = set_error(RWC_ERR_UNSUPPORTED, "batch block does not fit on an SM"); return; }
-            const int64_t per_block = warp ? threads / 32 : 1;
-            const int64_t want = (b->nitems[c] + per_block - 1) / per_block;
-            const int64_t blocks = std::max<int64_t>(1, std::min<int64_t>(want, (int64_t)num_sms() * per_sm));
-            ::rwc::count_launches(1);
-            kern<<<(unsigned)blocks, threads, smem, s>>>(
-                b->base, b->graphs, warp ? nullptr : b->items[c], warp ? 0 : b->nitems[c],
-                warp ? b->items[c] : nullptr, warp ? b->nitems[c] : 0, counters + 2 * c,
-                warp ? (int)warp_slice_bytes(b->max_n[c]) : 0, b->tile, T, k0, k1, (int64_t)1 << 22,
-                sums, err, rounds);
+    const bool fork = b->conc && b->bins.size() > 1;
+    if (fork) RWC_CUDA_TRY(cudaEventRecord(b->fork, st));
+    cudaError_t e = cudaSuccess;
+    size_t forked = 0;
+    for (size_t i = 0; i < b->bins.size() && e == cudaSuccess; ++i) {
+        const Bin &q = b->bins[i];
+        cudaStream_t s = st;
+        if (fork && i > 0) {
+            s = b->side[i];
+            if ((e = cudaStreamWaitEvent(s, b->fork, 0)) != cudaSuccess) break;
+            forked = i;
+        }
+        ::rwc::count_launches(1);
+        dispatch_nt(b->off64, b->weighted, q.nt, [&](auto kern) {
+            kern<<<(unsigned)q.blocks, q.nt, q.smem, s>>>(b->base, b->graphs, b->items[q.cls] + q.begin,
+                                                          q.count * b->tile, next + i, b->tile, T, k0, k1, q.max_n,
+                                                          sums, b->spill + q.spill, err, ctr);
         });
+        e = cudaGetLastError();
     }
-    if (fork) {
-        RWC_CUDA_TRY(cudaEventRecord(b->join, b->side));
-        RWC_CUDA_TRY(cudaStreamWaitEvent(st, b->join, 0));
+    // every forked stream joins st again, after an error too
+    for (size_t i = 1; i <= forked; ++i) {
+        const cudaError_t e1 = cudaEventRecord(b->join[i], b->side[i]);
+        const cudaError_t e2 = cudaStreamWaitEvent(st, b->join[i], 0);
+        if (e == cudaSuccess) e = e1 != cudaSuccess ? e1 : e2;
     }
-    RWC_TRY(status);
-    RWC_CUDA_TRY(cudaGetLastError());
+    RWC_CUDA_TRY(e);
     return RWC_OK;
 }
 
@@ -271,9 +332,8 @@ rwc_status finish(rwc_batch *b, rwc_stats_t *stats, int mode, int64_t T, cudaStr
     RWC_CUDA_TRY(cudaMemcpyAsync(b->host, b->scratch, 24, cudaMemcpyDeviceToHost, st));
     RWC_CUDA_TRY(cudaStreamSynchronize(st));
     const int e = (int)(b->host[0] & 0xffffffff);
-    if (e & SM_ERR_KOVF) return set_error(RWC_ERR_UNSUPPORTED, "a vertex was popped more than 65535 times");
-    if (e & SM_ERR_LOOP) return set_error(RWC_ERR_CUDA, "sampler internal check failed");
-    if (e) return set_error(RWC_ERR_NOT_CONVERGED, "cycle popping exceeded max_rounds");
+    if (e & LE_KOVF) return set_error(RWC_ERR_UNSUPPORTED, "a vertex was popped more than 65535 times");
+    if (e) return set_error(RWC_ERR_CUDA, "sampler internal check failed");
     if (stats) {
         stats->trees = T * b->G;
         stats->rounds = b->host[1];
@@ -374,13 +434,21 @@ extern "C" rwc_status rwc_batch_create(int32_t G, const int64_t *voff, const int
     }
     if ((e = balloc(b, (void **)&b->graphs, G * sizeof(BGraph))) != cudaSuccess) return fail(e);
     if ((e = cudaMemcpy(b->graphs, hg.data(), G * sizeof(BGraph), cudaMemcpyHostToDevice)) != cudaSuccess) return fail(e);
-    if ((e = balloc(b, &b->scratch, 128)) != cudaSuccess) return fail(e);
+    {
+        std::vector<BItem> one(G);
+        for (int32_t g = 0; g < G; ++g) one[g] = BItem{g, 0};
+        if ((e = balloc(b, (void **)&b->single, G * sizeof(BItem))) != cudaSuccess) return fail(e);
+        if ((e = cudaMemcpy(b->single, one.data(), G * sizeof(BItem), cudaMemcpyHostToDevice)) != cudaSuccess) return fail(e);
+    }
+    if ((e = balloc(b, &b->scratch, 256)) != cudaSuccess) return fail(e);
     if ((e = cudaMallocHost((void **)&b->host, 64)) != cudaSuccess) return fail(e);
-    if ((e = cudaStreamCreateWithFlags(&b->side, cudaStreamNonBlocking)) != cudaSuccess ||
-        (e = cudaEventCreateWithFlags(&b->fork, cudaEventDisableTiming)) != cudaSuccess ||
-        (e = cudaEventCreateWithFlags(&b->join, cudaEventDisableTiming)) != cudaSuccess) {
-        if (b->fork) cudaEventDestroy(b->fork);
-        if (b->side) cudaStreamDestroy(b->side);
+    e = cudaEventCreateWithFlags(&b->fork, cudaEventDisableTiming);
+    for (int i = 1; i < MAX_BINS && e == cudaSuccess; ++i) {
+        e = cudaStreamCreateWithFlags(&b->side[i], cudaStreamNonBlocking);
+        if (e == cudaSuccess) e = cudaEventCreateWithFlags(&b->join[i], cudaEventDisableTiming);
+    }
+    if (e != cudaSuccess) {
+        drop_streams(b);
         return fail(e);
     }
     *out = b;
@@ -402,30 +470,37 @@ extern "C" rwc_status rwc_batch_sample(rwc_batch_t *b, uint64_t seed, int64_t T,
     cudaStream_t st = (cudaStream_t)stream;
     RWC_CUDA_TRY(cudaMemsetAsync(b->scratch, 0, 32, st));
     if (per_graph_launch) {
-        // baseline: one launch per graph, same per-tree kernel
+        // baseline: one launch per graph, same per-tree code
         int *err = (int *)b->scratch;
-        unsigned long long *rounds = (unsigned long long *)((char *)b->scratch + 8);
+        unsigned long long *ctr = (unsigned long long *)((char *)b->scratch + 8);
         const uint32_t k0 = (uint32_t)seed, k1 = (uint32_t)(seed >> 32);
-        for (int32_t g = 0; g < b->G; ++g) {
-            const BGraph &bg = b->hgraphs[g];
-            DevGraph dg = b->base;
-            dg.n = bg.n; dg.root = bg.root;
-            if (b->off64) dg.rp64 = b->base.rp64 + bg.voff; else dg.rp32 = b->base.rp32 + bg.voff;
-            const int thr = bg.n <= 2048 ? 256 : 512;   // the block sizes of a plain per-graph launch
-            const size_t smem = smem_tree_bytes(bg.n);
-            rwc_status status = RWC_OK;
-            dispatch(b->off64, b->weighted, [&](auto o64, auto wt) {
-                auto kern = s_trees<decltype(o64)::value, decltype(wt)::value>;
-                cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-                int per_sm = 0;
-                cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, thr, smem);
-                if (per_sm < 1) { status = set_error(RWC_ERR_UNSUPPORTED, "graph %d does not fit", g); return; }
-                const int64_t blocks = std::min<int64_t>(T, (int64_t)num_sms() * per_sm);
-                ::rwc::count_launches(1); kern<<<(unsigned)blocks, thr, smem, st>>>(dg, 0u, T, k0, k1, (uint32_t)g, (int64_t)1 << 22,
-                                                           sums + bg.voff, nullptr, nullptr, err, rounds);
+        std::vector<int64_t> blocks(b->G);
+        int64_t spill = 0;
+        cudaError_t e = cudaSuccess;
+        for (int32_t g = 0; g < b->G && e == cudaSuccess; ++g) {
+            const int n = b->hgraphs[g].n, nt = batch_threads(n);
+            const size_t smem = batch_tree_smem(n, nt);
+            int per_sm = 0;
+            dispatch_nt(b->off64, b->weighted, nt, [&](auto kern) {
+                e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)std::max<size_t>(smem, 96 * 1024));
+                if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, nt, smem);
             });
-            RWC_TRY(status);
+            if (e == cudaSuccess && per_sm < 1) return set_error(RWC_ERR_UNSUPPORTED, "graph %d does not fit", g);
+            blocks[g] = std::min<int64_t>(T, (int64_t)num_sms() * per_sm);
+            spill = std::max(spill, blocks[g] * n);
         }
+        RWC_CUDA_TRY(e);
+        uint32_t *sp = nullptr;
+        RWC_CUDA_TRY(cudaMallocAsync((void **)&sp, (size_t)spill * sizeof(uint32_t), st));
+        for (int32_t g = 0; g < b->G; ++g) {
+            const int n = b->hgraphs[g].n, nt = batch_threads(n);
+            ::rwc::count_launches(1);
+            dispatch_nt(b->off64, b->weighted, nt, [&](auto kern) {
+                kern<<<(unsigned)blocks[g], nt, batch_tree_smem(n, nt), st>>>(
+                    b->base, b->graphs, b->single + g, T, nullptr, T, T, k0, k1, n, sums, sp, err, ctr);
+            });
+        }
+        cudaFreeAsync(sp, st);
         RWC_CUDA_TRY(cudaGetLastError());
         return finish(b, stats, 3, T, st);
     }
@@ -488,8 +563,7 @@ extern "C" rwc_status rwc_batch_set_schedule(rwc_batch_t *b, int32_t threads, in
         if (g.n <= split) wmax = std::max(wmax, g.n);
         else bmax = std::max(bmax, g.n);
     }
-    const size_t small = wmax ? (warp ? (size_t)(SMALL_THREADS / 32) * warp_slice_bytes(wmax) : smem_tree_bytes(wmax)) : 0;
-    const size_t need = std::max(bmax ? smem_tree_bytes(bmax) : 0, small);
+    const size_t need = schedule_allowance(bmax, wmax, warp);
     if (need > 227 * 1024)
         return set_error(RWC_ERR_UNSUPPORTED, "schedule needs %zu bytes of shared memory per block", need);
     b->threads = threads;
@@ -592,12 +666,11 @@ done:
 extern "C" rwc_status rwc_batch_destroy(rwc_batch_t *b) {
     if (!b) return RWC_OK;
     drop_graph(b);
-    if (b->side) cudaStreamSynchronize(b->side);
+    for (cudaStream_t s : b->side)
+        if (s) cudaStreamSynchronize(s);
     for (void *p : b->allocs) cudaFree(p);
     if (b->host) cudaFreeHost(b->host);
-    if (b->join) cudaEventDestroy(b->join);
-    if (b->fork) cudaEventDestroy(b->fork);
-    if (b->side) cudaStreamDestroy(b->side);
+    drop_streams(b);
     delete b;
     return RWC_OK;
 }

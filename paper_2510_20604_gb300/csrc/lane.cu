@@ -38,12 +38,13 @@ __global__ void __launch_bounds__(NT) l_trees_smem(DevGraph g, uint32_t tree0, i
     const uint32_t kmask = (1u << kb) - 1u;
     uint32_t *sp = spill + (int64_t)blockIdx.x * n;
     unsigned long long draws = 0;
+    uint32_t rounds = 0;
     int64_t t = blockIdx.x;
     while (t < T) {
         for (int u = threadIdx.x; u < n; u += NT) word[u] = u == g.root ? lt_root_word<uint32_t>(kb, NT * S) : 0u;
         __syncthreads();
         const int bad = lane_tree<OFF64, WT, EW, NT, S, true, uint32_t>(g, word, kb, klim, sh, sp, tree0 + (uint32_t)t,
-                                                                     0u, k0, k1);
+                                                                     0u, k0, k1, rounds);
         if (bad & ~LE_KREP) { if (threadIdx.x == 0) atomicOr(err, bad); break; }
         if (bad && threadIdx.x == 0) wide[atomicAdd(ctr + 2, 1ull)] = (uint32_t)t;
         for (int u = bad ? n : threadIdx.x; u < n; u += NT) {
@@ -60,6 +61,7 @@ __global__ void __launch_bounds__(NT) l_trees_smem(DevGraph g, uint32_t tree0, i
     }
     for (int o = 16; o > 0; o >>= 1) draws += __shfl_xor_sync(0xffffffffu, draws, o);
     if ((threadIdx.x & 31) == 0 && draws) atomicAdd(ctr + 1, draws);
+    if (threadIdx.x == 0 && rounds) atomicAdd(ctr + 3, (unsigned long long)rounds);
 }
 
 // One tree per block of NT threads, its words in global memory (zeroed by the
@@ -77,7 +79,9 @@ __global__ void __launch_bounds__(NT) l_trees(DevGraph g, uint32_t tree0, int64_
         W *word = words + t * ld;
         if (threadIdx.x == 0) word[g.root] = lt_root_word<W>(kb, NT * S);
         __syncthreads();
-        const int bad = lane_tree<OFF64, WT, EW, NT, S, false, W>(g, word, kb, klim, sh, sp, tree0 + (uint32_t)t, 0u, k0, k1);
+        uint32_t rounds = 0;
+        const int bad = lane_tree<OFF64, WT, EW, NT, S, false, W>(g, word, kb, klim, sh, sp, tree0 + (uint32_t)t, 0u,
+                                                                  k0, k1, rounds);
         if (bad) { if (threadIdx.x == 0) atomicOr(err, bad); break; }
         if (threadIdx.x == 0) sh_next = atomicAdd(ctr, 1ull);
         __syncthreads();
@@ -145,7 +149,7 @@ struct Events {
     double ms(int a, int b) { float v = 0.f; if (on) cudaEventElapsedTime(&v, e[a], e[b]); return v; }
 };
 
-constexpr int64_t TAIL = 64;   // err @0, next tree @8, draws @16, listed trees @24
+constexpr int64_t TAIL = 64;   // err @0, next tree @8, draws @16, listed trees @24, rounds @32
 constexpr int64_t WIDE_CAP = 65536;   // trees of one shared-memory launch
 
 template <int NT, class W>
@@ -306,7 +310,7 @@ rwc_status smem_range(rwc_graph *G, uint64_t seed, int64_t tree0, int64_t T, dou
         return RWC_OK;
     }
     int64_t *h = G->host_scalars;
-    RWC_CUDA_TRY(cudaMemcpyAsync(h, buf.p, 32, cudaMemcpyDeviceToHost, stream));
+    RWC_CUDA_TRY(cudaMemcpyAsync(h, buf.p, 40, cudaMemcpyDeviceToHost, stream));
     RWC_CUDA_TRY(cudaStreamSynchronize(stream));
     *h_err = (int)(h[0] & 0xffffffff);
     if (*h_err) return RWC_OK;
@@ -319,6 +323,7 @@ rwc_status smem_range(rwc_graph *G, uint64_t seed, int64_t tree0, int64_t T, dou
         st->draws += h[2];
         st->marked += h[2];
         st->chunks += 1;
+        st->rounds += h[4];
         st->phase_units[RWC_PHASE_WALK] += h[2];
         if (ev.on) {
             st->phase_ms[RWC_PHASE_WALK] += ev.ms(0, 1);
@@ -399,7 +404,7 @@ rwc_status sample_lane_walker(rwc_graph *G, uint64_t seed, int64_t tree0, int64_
         RWC_TRY(sample_smem(G, seed, tree0, T, sums, parents, visits, (1u << 20) - 1u, o, st, &e, stream));
         if (e & LE_KOVF) return set_error(RWC_ERR_UNSUPPORTED, "a vertex was popped more than 2^20 - 1 times");
         if (e) return set_error(RWC_ERR_CUDA, "sampler internal check failed");
-        if (st) st->mode = RWC_MODE_WALKER;
+        if (st) { st->mode = RWC_MODE_WALKER; st->rounds = 0; }
         return RWC_OK;
     }
     auto run = [&](auto nt) -> rwc_status {

@@ -190,12 +190,12 @@ __host__ __device__ inline W lt_root_word(int kb, int nl) { return (W)lt_id0(nl)
 // the whole block), S lanes per thread.  word: [n] state, zero but for the root's lt_root_word
 // (made visible to the group), in shared memory if SM; spill: [n] entries of global memory for the
 // stack's overflow.  kb: bits of k; klim: largest pop count allowed.  Returns
-// a group-uniform error mask; on success every word holds its vertex's
-// successor and count.
+// a group-uniform error mask and adds the tree's rounds to `rounds`; on success
+// every word holds its vertex's successor and count.
 template <bool OFF64, bool WT, int EW, int NT, int S, bool SM, class W>
 __device__ __forceinline__ int lane_tree(const DevGraph &g, W *word, int kb, uint32_t klim, LaneShared<NT, S> &sh,
                                          uint32_t *spill, uint32_t tree, uint32_t gid, uint32_t k0,
-                                         uint32_t k1) {
+                                         uint32_t k1, uint32_t &rounds) {
     constexpr unsigned FULL = 0xffffffffu;
     constexpr bool WARP = NT == 32;
     constexpr int NW = NT / 32;
@@ -307,6 +307,7 @@ __device__ __forceinline__ int lane_tree(const DevGraph &g, W *word, int kb, uin
         }
         // every lane asked and there was nothing to give: the tree is done
         if (want == NT * S && total == 0 && scan == nstart) break;
+        ++rounds;
         {
             const uint32_t fresh = want > total ? want - total : 0u, used = want < total ? want : total;
             scan = nstart - scan < fresh ? nstart : scan + fresh;

@@ -86,3 +86,24 @@ def test_count_limits_are_reported(mode, ratio):
     with pytest.raises(rwc.RWCError) as e:
         G.sample(16, opt=rwc.Options(mode=mode))
     assert e.value.status == 6 and "popped more than" in str(e.value)
+
+
+@pytest.mark.parametrize("sched", [None, (128, 2600, 2, 0, 0), (64, 700, 3, 1, 1)])
+def test_batch_bins_and_block_sizes(sched):
+    # sizes on both sides of the bins' and block sizes' bounds, one kernel per
+    # bin on forked streams or one after the other, and one launch per graph
+    ns = [2, 3, 191, 193, 640, 641, 1281, 2500, 2501, 5000, 5001]
+    gs = [synth.path(2) if n == 2 else synth.ba(n, 2, seed=n) if n > 5 else synth.cycle(n) for n in ns]
+    B = rwc.Batch(gs)
+    if sched:
+        B.set_schedule(*sched)
+    T = 5
+    s, st = B.sample(T, seed=7)
+    one, _ = B.sample(T, seed=7, per_graph_launch=1)
+    assert torch.equal(s, one)
+    roots, o = B.roots(), B.offsets
+    sums = s.cpu().numpy()
+    for i, g in enumerate(gs):
+        ref = ow.Sampler(g, root=int(roots[i]), seed=7, graph_id=i).sample(0, T)
+        assert np.array_equal(sums[o[i]:o[i + 1]], ref["sums"]), ns[i]
+    assert st.trees == T * len(gs) and st.draws == int(sums.sum()) and st.rounds > 0
