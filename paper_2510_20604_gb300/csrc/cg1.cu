@@ -1,0 +1,549 @@
+// LapSolve for one right-hand side, x = L^+ b, in one launch: FP64 residual
+// refinement around Jacobi-preconditioned conjugate gradients in FP32, all of it
+// in a cooperative kernel (the host reads one status at the end).
+//
+// What bounds it: FP64 arithmetic (2 FMA per cycle and SM), grid barriers and
+// L2 latency, in that order for the earlier kernel.  So
+//   - the iteration's sums are taken in pairs of floats (exact products and
+//     sums by FMA and two-sum, about 48 bits) up to one value per warp;
+//   - the direction p = z + beta p is formed where the sparse product gathers
+//     it, from (z, p) pairs in two buffers used in turn, so an iteration has
+//     two grid barriers (<p,q>; <r,z> and <r,r>) and no pass for p;
+//   - graphs of bounded degree keep a thread's rows of e, r, p, q in registers
+//     and their inline neighbour rows in shared memory.
+// Measured (estimate of a whole pivot solve, before -> here): 1024 x 1024 grid,
+// R-MAT 20 and BA 2000 in the table beside solve_one.
+#include <algorithm>
+#include <cmath>
+#include <cstring>
+#include <type_traits>
+
+#include <cooperative_groups.h>
+
+#include "pair_sum.cuh"
+#include "rwc_common.cuh"
+
+namespace cg = cooperative_groups;
+
+namespace rwc {
+namespace {
+
+constexpr int CSR_TPB = 512;
+constexpr int ELL_TPB = 1024;
+constexpr int ELL_RMAX = 7;             // rows per thread held in registers
+constexpr int CG_WINDOW = 1024;         // iterations without a halved residual: stagnation
+constexpr double CG_INNER_TOL = 1e-5;
+
+struct CgArgs {
+    DevGraph g;
+    const double *B;
+    double *X, *R;
+    const float *d32;                   // [n] degrees
+    float *e, *r, *q;                   // [n] (not used by the register kernel)
+    float2 *zp[2];                      // [n] (z, p) of the last iteration, in turn
+    float *hsum;                        // heavy chunks' sums, FP32 and FP64
+    double *hsumd;
+    double *parts;                      // [2][2][gridDim] block sums, in turn
+    double tol;
+    int max_outer, max_inner;
+    int use_smem;                       // inline rows fit shared memory
+    double *out;                        // iterations, relative residual, status
+};
+enum : int { CG_OK = 0, CG_NAN = 1, CG_STALLED = 2, CG_MAX_OUTER = 3 };
+
+// Fixed-order sums over the grid of K values per thread: a shuffle tree in
+// every warp, the warps of a block in order, the blocks in order; every thread
+// gets the same bits.  `flip` alternates the blocks' slots, so that a block can
+// write its next sums while another still reads these.
+template <int K, class T>
+__device__ void grid_sums(const T (&v)[K], double (&out)[K], double *parts, int &flip) {
+    __shared__ double ws[K][32];
+    __shared__ double bc[K];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    const int nb = gridDim.x;
+    double *slot = parts + (size_t)flip * 2 * nb;
+    flip ^= 1;
+#pragma unroll
+    for (int k = 0; k < K; ++k) {
+        if constexpr (std::is_same<T, Pair>::value) {
+            Pair a = v[k];
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) {
+                const float s2 = __shfl_xor_sync(0xffffffffu, a.s, o), c2 = __shfl_xor_sync(0xffffffffu, a.c, o);
+                // both partners add the same pair in the same order
+                Pair lo = (lane & o) ? Pair{s2, c2} : a;
+                const Pair hi = (lane & o) ? a : Pair{s2, c2};
+                pair_add(lo, hi.s, hi.c);
+                a = lo;
+            }
+            if (lane == 0) ws[k][wid] = (double)a.s + (double)a.c;
+        } else {
+            double a = v[k];
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
+            if (lane == 0) ws[k][wid] = a;
+        }
+    }
+    __syncthreads();
+    if (wid < K) {
+        double a = lane < nw ? ws[wid][lane] : 0.0;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
+        if (lane == 0) { if (nb > 1) slot[(size_t)wid * nb + blockIdx.x] = a; else bc[wid] = a; }
+    }
+    if (nb > 1) {
+        cg::this_grid().sync();
+        if (wid < K) {
+            double a = 0.0;
+            for (int i = lane; i < nb; i += 32) a += __ldcg(slot + (size_t)wid * nb + i);
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
+            if (lane == 0) bc[wid] = a;
+        }
+    }
+    __syncthreads();
+#pragma unroll
+    for (int k = 0; k < K; ++k) out[k] = bc[k];
+}
+__device__ __forceinline__ void all_sync() {
+    if (gridDim.x > 1) cg::this_grid().sync();
+    else __syncthreads();
+}
+
+template <bool OFF64>
+__device__ __forceinline__ void row_of(const DevGraph &g, int64_t u, int64_t &b, int64_t &e) {
+    if (OFF64) { b = g.rp64[u]; e = g.rp64[u + 1]; }
+    else { b = g.rp32[u]; e = g.rp32[u + 1]; }
+}
+
+// ------------------------------------------------------- general sparse rows
+// f(u, sum) for the rows of a degree bin, VW lanes per row (rows of at most VW
+// arcs, or more than 16 for VW = 32), term(arc) summed in type T.  Several rows
+// per group of lanes (arcs per lane for VW = 32) are in flight, since a row is
+// a chain of four dependent loads.
+template <int VW, bool OFF64, class T, class Term, class F>
+__device__ __forceinline__ void bin_rows(const DevGraph &g, int bin, Term term, F f) {
+    constexpr int NR = VW == 32 ? 1 : 4;
+    const int32_t *rows = g.bin_rows + g.bin_off[bin];
+    const int64_t nrows = g.bin_off[bin + 1] - g.bin_off[bin];
+    const int64_t tid = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    const int64_t ngroups = (int64_t)gridDim.x * blockDim.x / VW;
+    const int sub = threadIdx.x & (VW - 1);
+    const int64_t mine = tid / VW, first = mine - mine % (32 / VW);
+    for (int64_t i0 = first; i0 < nrows; i0 += NR * ngroups) {
+        int32_t u[NR];
+        int64_t b[NR], e[NR];
+        T s[NR];
+#pragma unroll
+        for (int k = 0; k < NR; ++k) {
+            const int64_t i = i0 + (mine - first) + k * ngroups;
+            u[k] = i < nrows ? rows[i] : -1;
+        }
+#pragma unroll
+        for (int k = 0; k < NR; ++k) {
+            b[k] = e[k] = 0;
+            if (u[k] >= 0) row_of<OFF64>(g, u[k], b[k], e[k]);
+        }
+        if (VW == 32) {
+            T s4[4] = {};
+            for (int64_t j = b[0] + sub; j < e[0]; j += 128) {
+#pragma unroll
+                for (int k = 0; k < 4; ++k)
+                    if (j + 32 * k < e[0]) s4[k] += term(j + 32 * k);
+            }
+            s[0] = (s4[0] + s4[1]) + (s4[2] + s4[3]);
+        } else {
+#pragma unroll
+            for (int k = 0; k < NR; ++k) s[k] = b[k] + sub < e[k] ? term(b[k] + sub) : (T)0;
+        }
+#pragma unroll
+        for (int k = 0; k < NR; ++k) {
+#pragma unroll
+            for (int o = VW / 2; o > 0; o >>= 1) s[k] += __shfl_xor_sync(0xffffffffu, s[k], o, VW);
+            if (sub == 0 && u[k] >= 0) f(u[k], s[k]);
+        }
+    }
+}
+// all rows of at most HEAVY_DEG arcs through f, the heavy rows' chunks through
+// h(chunk, row, first chunk of its row, sum)
+template <bool OFF64, class T, class Term, class F, class H>
+__device__ __forceinline__ void all_rows(const DevGraph &g, Term term, F f, H h) {
+    bin_rows<2, OFF64, T>(g, 0, term, f);
+    bin_rows<4, OFF64, T>(g, 1, term, f);
+    bin_rows<8, OFF64, T>(g, 2, term, f);
+    bin_rows<16, OFF64, T>(g, 3, term, f);
+    bin_rows<32, OFF64, T>(g, 4, term, f);
+    const int lane = threadIdx.x & 31;
+    const int64_t tid = blockIdx.x * (int64_t)blockDim.x + threadIdx.x, nthr = (int64_t)gridDim.x * blockDim.x;
+    for (int64_t c = tid / 32; c < g.hc_n; c += nthr / 32) {
+        const int32_t u = g.hc_row[c];
+        int64_t rb, re;
+        row_of<OFF64>(g, u, rb, re);
+        const int64_t b = g.hc_beg[c], e = min(b + HEAVY_CHUNK, re);
+        T s4[4] = {};
+        for (int64_t j = b + lane; j < e; j += 128) {
+#pragma unroll
+            for (int k = 0; k < 4; ++k)
+                if (j + 32 * k < e) s4[k] += term(j + 32 * k);
+        }
+        T s = (s4[0] + s4[1]) + (s4[2] + s4[3]);
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+        if (lane == 0) h(c, u, b == rb, s);
+    }
+}
+// sum of a heavy row's chunks in chunk order
+template <bool OFF64, class T>
+__device__ __forceinline__ T heavy_sum(const DevGraph &g, int64_t u, const T *hsum) {
+    int64_t rb, re;
+    row_of<OFF64>(g, u, rb, re);
+    const int64_t nc = (re - rb + HEAVY_CHUNK - 1) / HEAVY_CHUNK;
+    T s = 0;
+    for (int64_t c = 0; c < nc; ++c) s += hsum[g.hfirst[u] + c];
+    return s;
+}
+
+// Outer loop shared by both kernels: INNER runs the conjugate gradients on R /
+// |R| and adds the correction to X; RESID fills R = B - L X and returns this
+// thread's share of its sum; EACH visits the thread's rows.
+template <class Resid, class Each, class Inner>
+__device__ void refine(const CgArgs &a, int &flip, Resid resid, Each each, Inner inner) {
+    const double n = (double)a.g.n;
+    double bn = 0.0, prev = INFINITY, worst = 0.0;
+    int total = 0, slow = 0, status = CG_MAX_OUTER;
+    for (int outer = 0; outer <= a.max_outer; ++outer) {
+        double sum[1] = {resid()}, tot[1];
+        grid_sums<1>(sum, tot, a.parts, flip);
+        const double mean = tot[0] / n;
+        sum[0] = 0.0;
+        each([&](int64_t i) {
+            const double v = a.R[i] - mean;
+            a.R[i] = v;
+            sum[0] += v * v;
+        });
+        grid_sums<1>(sum, tot, a.parts, flip);
+        const double rn = sqrt(tot[0]);
+        if (outer == 0) bn = rn;
+        worst = bn > 0 ? rn / bn : 0.0;
+        if (!(worst == worst)) { status = CG_NAN; break; }
+        if (worst <= a.tol) { status = CG_OK; break; }
+        if (worst < 0.5 * prev) { prev = worst; slow = 0; }
+        else if (++slow >= 4) { status = CG_STALLED; break; }
+        if (outer == a.max_outer) break;
+        total += inner(rn);
+    }
+    // X onto 1-perp
+    double sum[1] = {0.0}, tot[1];
+    each([&](int64_t i) { sum[0] += a.X[i]; });
+    grid_sums<1>(sum, tot, a.parts, flip);
+    const double mean = tot[0] / n;
+    each([&](int64_t i) { a.X[i] -= mean; });
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        a.out[0] = (double)total;
+        a.out[1] = worst;
+        a.out[2] = (double)status;
+    }
+}
+
+// Step length and direction factor with their guards, and the exit test of the
+// inner iteration, the same in every thread.
+struct Inner {
+    double rz, best = INFINITY;
+    int since = 0;
+    __device__ float step(double den) const { return den > 0.0 && rz > 0.0 ? (float)(rz / den) : 0.f; }
+    // true when the iteration ends
+    __device__ bool done(double rz1, double rr, float &beta) {
+        if (!(rr == rr) || rr <= CG_INNER_TOL * CG_INNER_TOL) return true;
+        if (rr < 0.25 * best) { best = rr; since = 0; }
+        else if (++since >= CG_WINDOW) return true;
+        beta = rz > 0.0 ? (float)(rz1 / rz) : 0.f;
+        rz = rz1;
+        return false;
+    }
+};
+
+template <bool OFF64, bool W>
+__global__ void __launch_bounds__(CSR_TPB, 2) cg1_csr(CgArgs a) {
+    const DevGraph &g = a.g;
+    const int64_t n = g.n;
+    const int64_t tid = blockIdx.x * (int64_t)blockDim.x + threadIdx.x, nthr = (int64_t)gridDim.x * blockDim.x;
+    int flip = 0;
+    auto each = [&](auto f) { for (int64_t i = tid; i < n; i += nthr) f(i); };
+    auto resid = [&]() -> double {
+        double s = 0.0;
+        all_rows<OFF64, double>(
+            g, [&](int64_t j) { return (W ? (double)g.w[j] : 1.0) * a.X[g.col[j]]; },
+            [&](int32_t u, double t) { a.R[u] = a.B[u] - (g.d[u] * a.X[u] - t); },
+            [&](int64_t c, int32_t, bool, double t) { a.hsumd[c] = t; });
+        all_sync();
+        each([&](int64_t i) {
+            if (g.hc_n && g.hfirst[i] >= 0)
+                a.R[i] = a.B[i] - (g.d[i] * a.X[i] - heavy_sum<OFF64, double>(g, i, a.hsumd));
+            s += a.R[i];
+        });
+        return s;
+    };
+    auto inner = [&](double rn) -> int {
+        Pair acc[1] = {{0.f, 0.f}};
+        double t1[1], t2[2];
+        each([&](int64_t i) {
+            const float rv = (float)(a.R[i] / rn), zv = g.dinv32[i] * rv;
+            a.r[i] = rv;
+            a.e[i] = 0.f;
+            a.zp[0][i] = make_float2(zv, 0.f);
+            pair_fma(acc[0], rv, zv);
+        });
+        grid_sums<1>(acc, t1, a.parts, flip);
+        Inner s;
+        s.rz = t1[0];
+        float beta = 0.f;
+        int it = 0;
+        while (it < a.max_inner) {
+            const float2 *zi = a.zp[it & 1];
+            float2 *zo = a.zp[(it & 1) ^ 1];
+            // q = L p, <p, q>; a heavy row's share of <p, q> comes from its chunks
+            Pair pq[1] = {{0.f, 0.f}};
+            auto dir = [&](int64_t v) { const float2 t = zi[v]; return fmaf(beta, t.y, t.x); };
+            all_rows<OFF64, float>(
+                g, [&](int64_t j) { return (W ? g.w[j] : 1.f) * dir(g.col[j]); },
+                [&](int32_t u, float t) {
+                    const float pu = dir(u), qu = a.d32[u] * pu - t;
+                    a.q[u] = qu;
+                    pair_fma(pq[0], pu, qu);
+                },
+                [&](int64_t c, int32_t u, bool start, float t) {
+                    a.hsum[c] = t;
+                    const float pu = dir(u);
+                    if (start) pair_fma(pq[0], pu, a.d32[u] * pu);
+                    pair_fma(pq[0], -pu, t);
+                });
+            grid_sums<1>(pq, t1, a.parts, flip);
+            const float al = s.step(t1[0]);
+            Pair z2[2] = {{0.f, 0.f}, {0.f, 0.f}};
+            each([&](int64_t i) {
+                const float pi = dir(i);
+                const float qi = g.hc_n && g.hfirst[i] >= 0 ? a.d32[i] * pi - heavy_sum<OFF64, float>(g, i, a.hsum) : a.q[i];
+                a.e[i] += al * pi;
+                const float rv = a.r[i] - al * qi;
+                a.r[i] = rv;
+                const float zv = g.dinv32[i] * rv;
+                zo[i] = make_float2(zv, pi);
+                pair_fma(z2[0], rv, zv);
+                pair_fma(z2[1], rv, rv);
+            });
+            grid_sums<2>(z2, t2, a.parts, flip);
+            ++it;
+            if (s.done(t2[0], t2[1], beta)) break;
+        }
+        each([&](int64_t i) { a.X[i] += rn * (double)a.e[i]; });
+        all_sync();
+        return it;
+    };
+    refine(a, flip, resid, each, inner);
+}
+
+// Bounded degree: block b owns consecutive rows, thread t of it the rows t, t +
+// ELL_TPB, ... (RT of them), whose e, r, p and q stay in registers.
+template <int EW, int RT>
+__global__ void __launch_bounds__(ELL_TPB, 1) cg1_ell(CgArgs a) {
+    extern __shared__ int4 rows_s[];
+    const DevGraph &g = a.g;
+    const int n = (int)g.n;
+    const int rpb = (n + gridDim.x - 1) / gridDim.x;
+    const int row0 = blockIdx.x * rpb, nrow = max(0, min(rpb, n - row0));
+    int flip = 0;
+    constexpr int E4 = EW / 4;
+    if (a.use_smem) {
+        for (int i = threadIdx.x; i < nrow * E4; i += ELL_TPB) rows_s[i] = g.ell[(int64_t)row0 * E4 + i];
+        __syncthreads();
+    }
+    // sum over the row's neighbours of get(v)
+    auto row_sum = [&](int l, auto zero, auto get) {
+        auto s = zero;
+#pragma unroll
+        for (int k = 0; k < E4; ++k) {
+            const int4 c = a.use_smem ? rows_s[l * E4 + k] : __ldg(g.ell + (int64_t)(row0 + l) * E4 + k);
+            const auto v0 = c.x >= 0 ? get(c.x) : zero, v1 = c.y >= 0 ? get(c.y) : zero;
+            const auto v2 = c.z >= 0 ? get(c.z) : zero, v3 = c.w >= 0 ? get(c.w) : zero;
+            s += v0; s += v1; s += v2; s += v3;
+        }
+        return s;
+    };
+    auto each = [&](auto f) { for (int l = threadIdx.x; l < nrow; l += ELL_TPB) f((int64_t)(row0 + l)); };
+    auto resid = [&]() -> double {
+        double s = 0.0;
+        for (int l = threadIdx.x; l < nrow; l += ELL_TPB) {
+            const int64_t u = row0 + l;
+            const double v = a.B[u] - (g.d[u] * a.X[u] - row_sum(l, 0.0, [&](int c) { return a.X[c]; }));
+            a.R[u] = v;
+            s += v;
+        }
+        return s;
+    };
+    auto inner = [&](double rn) -> int {
+        float e[RT], r[RT], p[RT], q[RT], d[RT];
+        Pair acc[1] = {{0.f, 0.f}};
+        double t1[1], t2[2];
+#pragma unroll
+        for (int i = 0; i < RT; ++i) {
+            const int l = threadIdx.x + i * ELL_TPB;
+            e[i] = r[i] = p[i] = q[i] = 0.f;
+            d[i] = 1.f;
+            if (l < nrow) {
+                const int64_t u = row0 + l;
+                d[i] = a.d32[u];
+                r[i] = (float)(a.R[u] / rn);
+                const float zv = r[i] / d[i];
+                a.zp[0][u] = make_float2(zv, 0.f);
+                pair_fma(acc[0], r[i], zv);
+            }
+        }
+        grid_sums<1>(acc, t1, a.parts, flip);
+        Inner s;
+        s.rz = t1[0];
+        float beta = 0.f;
+        int it = 0;
+        while (it < a.max_inner) {
+            const float2 *zi = a.zp[it & 1];
+            float2 *zo = a.zp[(it & 1) ^ 1];
+            Pair pq[1] = {{0.f, 0.f}};
+#pragma unroll
+            for (int i = 0; i < RT; ++i) {
+                const int l = threadIdx.x + i * ELL_TPB;
+                if (l < nrow) {
+                    p[i] = fmaf(beta, p[i], r[i] / d[i]);
+                    const float t = row_sum(l, 0.f, [&](int c) { const float2 v = zi[c]; return fmaf(beta, v.y, v.x); });
+                    q[i] = d[i] * p[i] - t;
+                    pair_fma(pq[0], p[i], q[i]);
+                }
+            }
+            grid_sums<1>(pq, t1, a.parts, flip);
+            const float al = s.step(t1[0]);
+            Pair z2[2] = {{0.f, 0.f}, {0.f, 0.f}};
+#pragma unroll
+            for (int i = 0; i < RT; ++i) {
+                const int l = threadIdx.x + i * ELL_TPB;
+                if (l < nrow) {
+                    e[i] += al * p[i];
+                    r[i] -= al * q[i];
+                    const float zv = r[i] / d[i];
+                    zo[row0 + l] = make_float2(zv, p[i]);
+                    pair_fma(z2[0], r[i], zv);
+                    pair_fma(z2[1], r[i], r[i]);
+                }
+            }
+            grid_sums<2>(z2, t2, a.parts, flip);
+            ++it;
+            if (s.done(t2[0], t2[1], beta)) break;
+        }
+#pragma unroll
+        for (int i = 0; i < RT; ++i) {
+            const int l = threadIdx.x + i * ELL_TPB;
+            if (l < nrow) a.X[row0 + l] += rn * (double)e[i];
+        }
+        all_sync();
+        return it;
+    };
+    refine(a, flip, resid, each, inner);
+}
+
+__global__ void degrees32(int64_t n, const double *d, float *d32, double *X) {
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
+        d32[i] = (float)d[i];
+        X[i] = 0.0;
+    }
+}
+
+struct Buf {
+    void *p = nullptr;
+    cudaStream_t st;
+    explicit Buf(cudaStream_t s) : st(s) {}
+    ~Buf() { if (p) cudaFreeAsync(p, st); }
+};
+
+}  // namespace
+
+rwc_status solve_one(rwc_graph *G, const double *B, double *X, double tol, int *iters_out, cudaStream_t st) {
+    const DevGraph &g = G->g;
+    const int64_t n = g.n;
+    const int sms = num_sms();
+    // the grid: rows in registers where they fit, else blocks for about four
+    // arcs a thread (small graphs in one block need no grid barrier)
+    const bool ell = g.ell && n <= (int64_t)sms * ELL_TPB * ELL_RMAX;
+    int rt = 1;
+    while (ell && (n + (int64_t)ELL_TPB * rt - 1) / ((int64_t)ELL_TPB * rt) > sms) rt = rt == 1 ? 2 : rt == 2 ? 4 : ELL_RMAX;
+    int64_t blocks = ell ? (n + (int64_t)ELL_TPB * rt - 1) / ((int64_t)ELL_TPB * rt)
+                         : std::max<int64_t>(1, std::min<int64_t>(2 * sms, g.nnz / (4 * CSR_TPB)));
+    const size_t rows_b = ell ? (size_t)((n + blocks - 1) / blocks) * g.ell_w * 4 : 0;
+    const size_t smem = rows_b <= 200 * 1024 ? rows_b : 0;
+    Buf buf(st);
+    const size_t np = (size_t)(n + 31) & ~(size_t)31;
+    const size_t parts_b = (size_t)4 * std::max<int64_t>(2 * sms, blocks) * 8;
+    const size_t bytes = np * (8 + 4 + 3 * 4 + 2 * 8) + (size_t)(g.hc_n + 1) * 12 + parts_b + 16 * 256;
+    RWC_CUDA_TRY(cudaMallocAsync(&buf.p, bytes, st));
+    CgArgs a{};
+    char *q = (char *)buf.p;
+    auto take = [&](size_t b) { char *r = q; q += (b + 255) & ~(size_t)255; return r; };
+    a.out = (double *)take(256);
+    a.R = (double *)take(np * 8);
+    a.zp[0] = (float2 *)take(np * 8);
+    a.zp[1] = (float2 *)take(np * 8);
+    float *d32 = (float *)take(np * 4);
+    a.e = (float *)take(np * 4);
+    a.r = (float *)take(np * 4);
+    a.q = (float *)take(np * 4);
+    a.hsumd = (double *)take((size_t)(g.hc_n + 1) * 8);
+    a.hsum = (float *)take((size_t)(g.hc_n + 1) * 4);
+    a.parts = (double *)take(parts_b);
+    a.g = g;
+    a.B = B;
+    a.X = X;
+    a.d32 = d32;
+    a.tol = tol;
+    a.max_outer = 30;
+    a.max_inner = (int)std::min<int64_t>(200000, std::max<int64_t>(1000, 4 * n));
+    a.use_smem = smem > 0;
+    ::rwc::count_launches(2);
+    degrees32<<<(unsigned)std::max<int64_t>(1, std::min<int64_t>(4 * sms, (n + 255) / 256)), 256, 0, st>>>(n, g.d, d32, X);
+    RWC_CUDA_TRY(cudaGetLastError());
+    void *args[] = {&a};
+    auto launch = [&](auto kern, int tpb, size_t sm, int64_t nb) -> cudaError_t {
+        if (sm > 48 * 1024) {
+            const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(200 * 1024));
+            if (e != cudaSuccess) return e;
+        }
+        if (nb == 1) return cudaLaunchKernel((const void *)kern, dim3(1), dim3(tpb), args, sm, st);
+        return cudaLaunchCooperativeKernel((const void *)kern, dim3((unsigned)nb), dim3(tpb), args, sm, st);
+    };
+    auto csr = [&](int64_t nb) -> cudaError_t {
+        if (g.off64) return g.weighted ? launch(cg1_csr<true, true>, CSR_TPB, 0, nb) : launch(cg1_csr<true, false>, CSR_TPB, 0, nb);
+        return g.weighted ? launch(cg1_csr<false, true>, CSR_TPB, 0, nb) : launch(cg1_csr<false, false>, CSR_TPB, 0, nb);
+    };
+    auto inl = [&](auto ew) -> cudaError_t {
+        constexpr int EW = decltype(ew)::value;
+        return rt == 1 ? launch(cg1_ell<EW, 1>, ELL_TPB, smem, blocks) : rt == 2 ? launch(cg1_ell<EW, 2>, ELL_TPB, smem, blocks)
+             : rt == 4 ? launch(cg1_ell<EW, 4>, ELL_TPB, smem, blocks) : launch(cg1_ell<EW, ELL_RMAX>, ELL_TPB, smem, blocks);
+    };
+    cudaError_t e = !ell ? csr(blocks) : g.ell_w == 4 ? inl(std::integral_constant<int, 4>{}) : inl(std::integral_constant<int, 8>{});
+    if (e != cudaSuccess && blocks > 1) {
+        // a device that refuses the cooperative launch: one block, no grid barrier
+        (void)cudaGetLastError();
+        e = csr(1);
+    }
+    RWC_CUDA_TRY(e);
+    double h[3];
+    RWC_CUDA_TRY(cudaMemcpyAsync(h, a.out, sizeof(h), cudaMemcpyDeviceToHost, st));
+    RWC_CUDA_TRY(cudaStreamSynchronize(st));
+    if (iters_out) *iters_out = (int)h[0];
+    switch ((int)h[2]) {
+        case CG_OK: return RWC_OK;
+        case CG_NAN: return set_error(RWC_ERR_NOT_CONVERGED, "solver produced NaN");
+        case CG_STALLED:
+            return set_error(RWC_ERR_NOT_CONVERGED, "Laplacian solve stalled at relative residual %.3g (tol %.3g)", h[1], tol);
+        default:
+            return set_error(RWC_ERR_NOT_CONVERGED, "Laplacian solve reached %d refinements at relative residual %.3g (tol %.3g)",
+                             a.max_outer, h[1], tol);
+    }
+}
+
+}  // namespace rwc

@@ -124,6 +124,8 @@ bool csr_connected(int64_t n, const int64_t *rp, const int32_t *col);
 void vose_row(const float *w, int64_t deg, uint32_t *thr, int32_t *alias,
               std::vector<double> &prob, std::vector<int64_t> &lo_q, std::vector<int64_t> &hi_q);
 
+// x = L^+ b for one right-hand side (cg1.cu).
+rwc_status solve_one(rwc_graph *G, const double *B, double *X, double tol, int *iters_out, cudaStream_t st);
 // X = L^+ B for node-major [n][k] FP64 arrays (solver.cu).
 rwc_status solve_nodemajor(rwc_graph *G, int k, const double *B, double *X, double tol,
                            int *iters_out, cudaStream_t st);

@@ -1,23 +1,29 @@
-// Laplacian solves, Algorithm 1 (AppRWC) and the centrality gradient.
+// Laplacian solves with several right-hand sides (the gradient, rwc_solve).
 //
-// LapSolve (Lemma 3.2 names no concrete solver): X = L^+ B for k right-hand
-// sides.  Outer loop in FP64: R = B - L X (FP64 SpMV over the FP32 weights),
-// columns projected onto 1-perp; inner loop: Jacobi-preconditioned conjugate
-// gradients on the k columns together (one shared FP32 SpMM per iteration,
-// per-column step sizes, FP64 dot products), X += correction.  The matrix is
-// read once per iteration for all k columns; node-major [n][k] layout keeps
-// each gathered neighbour row contiguous.
+// X = L^+ B for k columns.  Outer loop in FP64: R = B - L X (FP64 sparse product
+// over the FP32 weights), columns projected onto 1-perp; inner loop:
+// Jacobi-preconditioned conjugate gradients on the k columns together (one
+// shared FP32 sparse product per iteration, per-column step sizes), X +=
+// correction.  One right-hand side goes to cg1.cu.
+//
+// Layout: node-major [n][k], the FP32 arrays padded to quads of columns.  A
+// thread owns one quad of columns and a slot of rows, so a neighbour row is
+// read as consecutive 16-byte loads, the weight and the column index are shared
+// by its threads, and the dot products stay in the thread until the end of the
+// kernel: four pairs of floats (exact products and sums by FMA and two-sum,
+// about 48 bits; FP64 runs at 2 FMA per cycle and SM).  The iteration is three
+// passes (product and <p,q>; r and its sums; e and p), whose working set of four
+// arrays stays in L2 for 66 columns of 100000 rows.
+// Measured: gradient of an RGG of 100000 vertices, 64 sketch columns, in the
+// comment at solve_nodemajor.
 #include <algorithm>
 #include <cmath>
 #include <cstring>
 #include <type_traits>
 #include <vector>
 
-#include <cooperative_groups.h>
-
+#include "pair_sum.cuh"
 #include "rwc_common.cuh"
-
-namespace cg = cooperative_groups;
 
 namespace rwc {
 namespace {
@@ -37,518 +43,245 @@ __device__ __forceinline__ void rowb(const DevGraph &g, int64_t u, int64_t &b, i
     else { b = g.rp32[u]; e = g.rp32[u + 1]; }
 }
 
-__device__ __forceinline__ double warp_sum(double v) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    return v;
-}
-__device__ __forceinline__ float warp_sumf(float v) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    return v;
-}
-
-// Q = L P (FP32), node-major [n][k], k > 1, one warp per row, lanes over
-// columns.  (The per-column dots <P, Q> are taken by col_parts in a fixed
-// order.)
-template <bool OFF64, bool W>
-__global__ void __launch_bounds__(TPB) spmm32(DevGraph g, int k, const float *__restrict__ P,
-                                              float *__restrict__ Q) {
-    const int lane = threadIdx.x & 31;
-    const int64_t warp = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
-    const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    for (int64_t u = warp; u < g.n; u += nwarps) {
-        int64_t b, e;
-        rowb<OFF64>(g, u, b, e);
-        const float du = (float)g.d[u];
-        for (int c0 = 0; c0 < k; c0 += 32) {
-            const int c = c0 + lane;
-            if (c >= k) continue;
-            float s = 0.f;
-            for (int64_t j = b; j < e; ++j) {
-                const float wj = W ? g.w[j] : 1.f;
-                s += wj * P[(int64_t)g.col[j] * k + c];
-            }
-            Q[u * k + c] = du * P[u * k + c] - s;
-        }
+// The threads of a block as quads of columns x rows: quad q (of this block's
+// tile), row slot rs, and the block's range of rows [u0, u1).
+struct Tile {
+    int q, rs, slots;
+    int64_t u0, u1;
+    bool on;
+    __device__ Tile(int64_t n, int k4, int qt)
+        : q(blockIdx.y * qt + threadIdx.x % qt), rs(threadIdx.x / qt), slots(blockDim.x / qt) {
+        const int64_t rpb = (n + gridDim.x - 1) / gridDim.x;
+        u0 = blockIdx.x * rpb;
+        u1 = u0 + rpb < n ? u0 + rpb : n;
+        on = q < k4;
     }
-}
+};
 
-// k == 1 SpMV with VW lanes per row (VW = power of two <= 32 chosen from the
-// average degree): Q = L P (FP32) and pq += <P, Q> (FP64).
-template <int VW, bool OFF64, bool W>
-__global__ void __launch_bounds__(TPB) spmv32(DevGraph g, const float *__restrict__ P,
-                                              float *__restrict__ Q, double *parts) {
-    const int sub = threadIdx.x & (VW - 1);
-    const int64_t row0 = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) / VW;
-    const int64_t nrows = ((int64_t)gridDim.x * blockDim.x) / VW;
-    double acc = 0.0;
-    for (int64_t u0 = row0 - (row0 % (32 / VW)); u0 < g.n; u0 += nrows) {
-        // all lanes of a warp iterate together so the shuffles stay converged
-        const int64_t u = u0 + (row0 % (32 / VW));
-        float s = 0.f;
-        if (u < g.n) {
-            int64_t b, e;
-            rowb<OFF64>(g, u, b, e);
-            for (int64_t j = b + sub; j < e; j += VW) s += (W ? g.w[j] : 1.f) * P[g.col[j]];
-        }
+// parts[column][block] = the sums of the block's row slots in slot order.
+__device__ __forceinline__ void quad_parts(const Tile &t, const Pair (&a)[4], int qt, double *parts) {
+    __shared__ double sh[4 * TPB];
+    __syncthreads();
 #pragma unroll
-        for (int o = VW / 2; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o, VW);
-        if (sub == 0 && u < g.n) {
-            const float pu = P[u];
-            const float q = (float)g.d[u] * pu - s;
-            Q[u] = q;
-            acc += (double)pu * (double)q;
-        }
-    }
-    acc = block_sum_fixed(acc);
-    if (threadIdx.x == 0) parts[blockIdx.x] = acc;
-}
-
-// k == 1 residual R = B - L X (FP64), column sum into colsum[0].
-template <int VW, bool OFF64, bool W>
-__global__ void __launch_bounds__(TPB) resid1(DevGraph g, const double *__restrict__ B,
-                                              const double *__restrict__ X, double *__restrict__ R,
-                                              double *parts) {
-    const int sub = threadIdx.x & (VW - 1);
-    const int64_t row0 = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) / VW;
-    const int64_t nrows = ((int64_t)gridDim.x * blockDim.x) / VW;
-    double acc = 0.0;
-    for (int64_t u0 = row0 - (row0 % (32 / VW)); u0 < g.n; u0 += nrows) {
-        const int64_t u = u0 + (row0 % (32 / VW));
-        double s = 0.0;
-        if (u < g.n) {
-            int64_t b, e;
-            rowb<OFF64>(g, u, b, e);
-            for (int64_t j = b + sub; j < e; j += VW) s += (W ? (double)g.w[j] : 1.0) * X[g.col[j]];
-        }
+    for (int i = 0; i < 4; ++i) sh[i * blockDim.x + threadIdx.x] = (double)a[i].s + (double)a[i].c;
+    __syncthreads();
+    if (t.rs == 0 && t.on) {
 #pragma unroll
-        for (int o = VW / 2; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o, VW);
-        if (sub == 0 && u < g.n) {
-            const double r = B[u] - (g.d[u] * X[u] - s);
-            R[u] = r;
-            acc += r;
-        }
-    }
-    acc = block_sum_fixed(acc);
-    if (threadIdx.x == 0) parts[blockIdx.x] = acc;
-}
-
-// R = B - L X in FP64 (node-major), k > 1, one warp per row.
-template <bool OFF64, bool W>
-__global__ void __launch_bounds__(TPB) resid64(DevGraph g, int k, const double *__restrict__ B,
-                                               const double *__restrict__ X, double *__restrict__ R) {
-    const int lane = threadIdx.x & 31;
-    const int64_t warp = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
-    const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    for (int64_t u = warp; u < g.n; u += nwarps) {
-        int64_t b, e;
-        rowb<OFF64>(g, u, b, e);
-        const double du = g.d[u];
-        for (int c0 = 0; c0 < k; c0 += 32) {
-            const int c = c0 + lane;
-            if (c >= k) continue;
+        for (int i = 0; i < 4; ++i) {
             double s = 0.0;
-            for (int64_t j = b; j < e; ++j) {
-                const double wj = W ? (double)g.w[j] : 1.0;
-                s += wj * X[(int64_t)g.col[j] * k + c];
-            }
-            R[u * k + c] = B[u * k + c] - (du * X[u * k + c] - s);
+            for (int r = 0; r < t.slots; ++r) s += sh[i * blockDim.x + r * qt + threadIdx.x];
+            parts[(int64_t)(4 * t.q + i) * gridDim.x + blockIdx.x] = s;
         }
     }
 }
 
-// Per-column sums over the rows of a node-major [n][k] array, in a fixed
-// order (k > 1): block b adds the rows [b rpb, (b + 1) rpb), rpb =
-// ceil(n / gridDim).  With k < blockDim, thread t takes column t % k of the
-// rows t / k, t / k + P, ... (P = blockDim / k phases; consecutive threads read
-// consecutive words) and the phases' sums are added in phase order; otherwise
-// thread t takes the columns t, t + blockDim, ... over all the block's rows.
-// parts[c * gridDim + b] (and parts2 for COL_DOT2); sum_cols adds them in
-// block order, so a call of the same size gives the same bits every time.
-enum : int { COL_SUM = 0, COL_SQ = 1, COL_DOT = 2, COL_DOT2 = 3 };
-template <int OP, class T>
-__device__ __forceinline__ void col_term(const T *A, const T *Bv, int64_t i, double &a1, double &a2) {
-    const double x = (double)A[i];
-    if (OP == COL_SUM) a1 += x;
-    else if (OP == COL_SQ) a1 += x * x;
-    else if (OP == COL_DOT) a1 += x * (double)Bv[i];
-    else { a1 += x * (double)Bv[i]; a2 += x * x; }
+__device__ __forceinline__ void fma4(float4 &s, float w, const float4 &v) {
+    s.x = fmaf(w, v.x, s.x); s.y = fmaf(w, v.y, s.y); s.z = fmaf(w, v.z, s.z); s.w = fmaf(w, v.w, s.w);
 }
-template <int OP, class T>
-__global__ void __launch_bounds__(TPB) col_parts(int64_t n, int k, const T *__restrict__ A,
-                                                 const T *__restrict__ Bv, double *parts, double *parts2) {
-    __shared__ double s1[TPB], s2[TPB];
+__device__ __forceinline__ void dot4(Pair (&a)[4], const float4 &x, const float4 &y) {
+    pair_fma(a[0], x.x, y.x); pair_fma(a[1], x.y, y.y); pair_fma(a[2], x.z, y.z); pair_fma(a[3], x.w, y.w);
+}
+
+// Q = L P and the parts of <P, Q>.  Four neighbour rows are in flight.
+template <bool OFF64, bool W>
+__global__ void __launch_bounds__(TPB) bcg_product(DevGraph g, int k4, int qt, const float4 *__restrict__ P,
+                                                   float4 *__restrict__ Q, double *parts) {
+    const Tile t(g.n, k4, qt);
+    Pair a[4] = {};
+    if (t.on && t.rs < t.slots)
+        for (int64_t u = t.u0 + t.rs; u < t.u1; u += t.slots) {
+            int64_t b, e;
+            rowb<OFF64>(g, u, b, e);
+            float4 s0 = {}, s1 = {};
+            int64_t j = b;
+            for (; j + 4 <= e; j += 4) {
+                int32_t c[4];
+                float w[4];
+                float4 v[4];
+#pragma unroll
+                for (int i = 0; i < 4; ++i) { c[i] = g.col[j + i]; w[i] = W ? g.w[j + i] : 1.f; }
+#pragma unroll
+                for (int i = 0; i < 4; ++i) v[i] = P[(int64_t)c[i] * k4 + t.q];
+                fma4(s0, w[0], v[0]); fma4(s1, w[1], v[1]); fma4(s0, w[2], v[2]); fma4(s1, w[3], v[3]);
+            }
+            for (; j < e; ++j) fma4(s0, W ? g.w[j] : 1.f, P[(int64_t)g.col[j] * k4 + t.q]);
+            const float d = (float)g.d[u];
+            const float4 p = P[u * k4 + t.q];
+            const float4 q = {d * p.x - (s0.x + s1.x), d * p.y - (s0.y + s1.y), d * p.z - (s0.z + s1.z),
+                              d * p.w - (s0.w + s1.w)};
+            Q[u * k4 + t.q] = q;
+            dot4(a, p, q);
+        }
+    quad_parts(t, a, qt, parts);
+}
+
+__device__ __forceinline__ float step_of(double num, double den) {
+    return den > 0.0 && num > 0.0 ? (float)(num / den) : 0.f;
+}
+
+// r -= alpha q; parts of <r, z> (z = D^-1 r) and <r, r>.  Every parts array is
+// [4 k4][gridDim.x].
+__global__ void __launch_bounds__(TPB) bcg_residual(int64_t n, int k4, int qt, const double *rz, const double *pq,
+                                                    const float *dinv, const float4 *__restrict__ Q,
+                                                    float4 *__restrict__ r, double *parts, double *parts2) {
+    const Tile t(n, k4, qt);
+    Pair a[4] = {}, b[4] = {};
+    if (t.on && t.rs < t.slots) {
+        const double *z = rz + 4 * t.q, *d = pq + 4 * t.q;
+        const float4 al = {step_of(z[0], d[0]), step_of(z[1], d[1]), step_of(z[2], d[2]), step_of(z[3], d[3])};
+        for (int64_t u = t.u0 + t.rs; u < t.u1; u += t.slots) {
+            const int64_t i = u * k4 + t.q;
+            const float4 q = Q[i];
+            float4 v = r[i];
+            v.x -= al.x * q.x; v.y -= al.y * q.y; v.z -= al.z * q.z; v.w -= al.w * q.w;
+            r[i] = v;
+            const float di = dinv[u];
+            dot4(a, v, float4{di * v.x, di * v.y, di * v.z, di * v.w});
+            dot4(b, v, v);
+        }
+    }
+    quad_parts(t, a, qt, parts);
+    quad_parts(t, b, qt, parts2);
+}
+
+// e += alpha p; p = D^-1 r + beta p.
+__global__ void __launch_bounds__(TPB) bcg_direction(int64_t n, int k4, int qt, const double *rz0, const double *pq,
+                                                     const double *rz1, const float *dinv,
+                                                     const float4 *__restrict__ r, float4 *__restrict__ e,
+                                                     float4 *__restrict__ p) {
+    const Tile t(n, k4, qt);
+    if (!t.on || t.rs >= t.slots) return;
+    const double *z = rz0 + 4 * t.q, *d = pq + 4 * t.q, *z1 = rz1 + 4 * t.q;
+    float al[4], be[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        al[i] = step_of(z[i], d[i]);
+        be[i] = z[i] > 0.0 ? (float)(z1[i] / z[i]) : 0.f;
+    }
+    for (int64_t u = t.u0 + t.rs; u < t.u1; u += t.slots) {
+        const int64_t i = u * k4 + t.q;
+        const float di = dinv[u];
+        const float4 v = r[i];
+        float4 pv = p[i], ev = e[i];
+        ev.x += al[0] * pv.x; ev.y += al[1] * pv.y; ev.z += al[2] * pv.z; ev.w += al[3] * pv.w;
+        pv.x = di * v.x + be[0] * pv.x; pv.y = di * v.y + be[1] * pv.y;
+        pv.z = di * v.z + be[2] * pv.z; pv.w = di * v.w + be[3] * pv.w;
+        e[i] = ev;
+        p[i] = pv;
+    }
+}
+
+// Start of an inner solve: r = R / |R_c|, e = 0, p = z = D^-1 r, parts of
+// <r, z>; columns beyond k are 0.
+__global__ void __launch_bounds__(TPB) bcg_start(int64_t n, int k, int k4, int qt, const double *__restrict__ R,
+                                                 const double *rnrm2, const float *dinv, float4 *__restrict__ r,
+                                                 float4 *__restrict__ e, float4 *__restrict__ p, double *parts) {
+    const Tile t(n, k4, qt);
+    Pair a[4] = {};
+    if (t.on && t.rs < t.slots) {
+        double nr[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) nr[i] = 4 * t.q + i < k ? sqrt(rnrm2[4 * t.q + i]) : 0.0;
+        for (int64_t u = t.u0 + t.rs; u < t.u1; u += t.slots) {
+            float v[4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) v[i] = nr[i] > 0.0 ? (float)(R[u * k + 4 * t.q + i] / nr[i]) : 0.f;
+            const float di = dinv[u];
+            const float4 rv = {v[0], v[1], v[2], v[3]}, zv = {di * v[0], di * v[1], di * v[2], di * v[3]};
+            const int64_t i = u * k4 + t.q;
+            r[i] = rv;
+            e[i] = float4{0.f, 0.f, 0.f, 0.f};
+            p[i] = zv;
+            dot4(a, rv, zv);
+        }
+    }
+    quad_parts(t, a, qt, parts);
+}
+
+// X += |R_c| e.
+__global__ void __launch_bounds__(TPB) bcg_add(int64_t n, int k, int k4, const double *rnrm2, const float *e, double *X) {
+    const int64_t tot = n * k;
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < tot; i += (int64_t)gridDim.x * blockDim.x) {
+        const int64_t u = i / k;
+        const int c = (int)(i - u * k);
+        X[i] += sqrt(rnrm2[c]) * (double)e[u * 4 * k4 + c];
+    }
+}
+
+// R = B - L X in FP64, one thread per (row, column), ct columns per block.
+template <bool OFF64, bool W>
+__global__ void __launch_bounds__(TPB) resid64(DevGraph g, int k, int ct, const double *__restrict__ B,
+                                               const double *__restrict__ X, double *__restrict__ R) {
+    const int c = blockIdx.y * ct + threadIdx.x % ct, rs = threadIdx.x / ct, slots = blockDim.x / ct;
+    if (c >= k || rs >= slots) return;
+    for (int64_t u = blockIdx.x * (int64_t)slots + rs; u < g.n; u += (int64_t)gridDim.x * slots) {
+        int64_t b, e;
+        rowb<OFF64>(g, u, b, e);
+        double s = 0.0;
+        int64_t j = b;
+        for (; j + 4 <= e; j += 4) {
+            double v[4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) v[i] = X[(int64_t)g.col[j + i] * k + c];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) s += (W ? (double)g.w[j + i] : 1.0) * v[i];
+        }
+        for (; j < e; ++j) s += (W ? (double)g.w[j] : 1.0) * X[(int64_t)g.col[j] * k + c];
+        R[u * k + c] = B[u * k + c] - (g.d[u] * X[u * k + c] - s);
+    }
+}
+
+// Per-column sums of X or X^2 over the rows of a node-major FP64 [n][k] array,
+// in a fixed order: block b adds the rows [b rpb, (b + 1) rpb).  With k <
+// blockDim, thread t takes column t % k of the rows t / k, t / k + P, ... and
+// the phases' sums are added in phase order; otherwise thread t takes the
+// columns t, t + blockDim, ... over all the block's rows.  parts[c * gridDim +
+// b]; sum_cols adds them in block order.
+template <bool SQUARE>
+__global__ void __launch_bounds__(TPB) col_parts(int64_t n, int k, const double *__restrict__ A, double *parts) {
+    __shared__ double s1[TPB];
     const int nb = gridDim.x, bk = blockIdx.x, t = threadIdx.x;
     const int64_t rpb = (n + nb - 1) / nb;
     const int64_t u0 = bk * rpb, u1 = u0 + rpb < n ? u0 + rpb : n;
     if (k < (int)blockDim.x) {
         const int P = (int)blockDim.x / k, c = t % k, ph = t / k;
-        double a1 = 0.0, a2 = 0.0;
+        double a = 0.0;
         if (ph < P)
-            for (int64_t u = u0 + ph; u < u1; u += P) col_term<OP>(A, Bv, u * k + c, a1, a2);
-        s1[t] = a1;
-        s2[t] = a2;
+            for (int64_t u = u0 + ph; u < u1; u += P) { const double v = A[u * k + c]; a += SQUARE ? v * v : v; }
+        s1[t] = a;
         __syncthreads();
         if (t < k) {
-            double r1 = 0.0, r2 = 0.0;
-            for (int q = 0; q < P; ++q) { r1 += s1[q * k + t]; r2 += s2[q * k + t]; }
-            parts[(int64_t)t * nb + bk] = r1;
-            if (OP == COL_DOT2) parts2[(int64_t)t * nb + bk] = r2;
+            double r = 0.0;
+            for (int q = 0; q < P; ++q) r += s1[q * k + t];
+            parts[(int64_t)t * nb + bk] = r;
         }
     } else {
         for (int c = t; c < k; c += blockDim.x) {
-            double a1 = 0.0, a2 = 0.0;
-            for (int64_t u = u0; u < u1; ++u) col_term<OP>(A, Bv, u * k + c, a1, a2);
-            parts[(int64_t)c * nb + bk] = a1;
-            if (OP == COL_DOT2) parts2[(int64_t)c * nb + bk] = a2;
+            double a = 0.0;
+            for (int64_t u = u0; u < u1; ++u) { const double v = A[u * k + c]; a += SQUARE ? v * v : v; }
+            parts[(int64_t)c * nb + bk] = a;
         }
     }
 }
 
-// out[c] = sum over b of parts[c * nb + b] in order of b; one block per column.
-__global__ void __launch_bounds__(TPB) sum_cols(const double *parts, int nb, double *out) {
+// out[c] = sum over b of parts[c * nb + b] in order of b; one block per column
+// (blockIdx.y = 1: the second set of parts, into out2).
+__global__ void __launch_bounds__(128) sum_cols(const double *parts, const double *parts2, int nb, double *out,
+                                                double *out2) {
     const int c = blockIdx.x;
+    const double *p = (blockIdx.y ? parts2 : parts) + (int64_t)c * nb;
     double s = 0.0;
-    for (int b = threadIdx.x; b < nb; b += blockDim.x) s += parts[(int64_t)c * nb + b];
+    for (int b = threadIdx.x; b < nb; b += blockDim.x) s += p[b];
     s = block_sum_fixed(s);
-    if (threadIdx.x == 0) out[c] = s;
+    if (threadIdx.x == 0) (blockIdx.y ? out2 : out)[c] = s;
 }
 
-// V[u][c] -= colsum[c] / n (FP64), k > 1.
+// V[u][c] -= colsum[c] / n (FP64).
 __global__ void center64(int64_t n, int k, double *V, const double *colsum) {
     const int64_t tot = n * k;
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < tot;
          i += (int64_t)gridDim.x * blockDim.x)
         V[i] -= colsum[(int)(i % k)] / (double)n;
-}
-
-// Single right-hand side versions with fixed-order block parts (the pivot
-// solve of rwc_estimate gives the same bits on every run).
-// V -= colsum / n; parts: sum of V^2.
-__global__ void center1(int64_t n, double *V, const double *colsum, double *parts) {
-    double acc = 0.0;
-    const double m = colsum[0] / (double)n;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
-         i += (int64_t)gridDim.x * blockDim.x) {
-        const double v = V[i] - m;
-        V[i] = v;
-        acc += v * v;
-    }
-    acc = block_sum_fixed(acc);
-    if (threadIdx.x == 0) parts[blockIdx.x] = acc;
-}
-
-// parts: sum of V.
-__global__ void sum1(int64_t n, const double *V, double *parts) {
-    double acc = 0.0;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
-         i += (int64_t)gridDim.x * blockDim.x)
-        acc += V[i];
-    acc = block_sum_fixed(acc);
-    if (threadIdx.x == 0) parts[blockIdx.x] = acc;
-}
-
-// r = R / |R|, e = 0, z = D^-1 r, p = z; parts: <r, z>.
-__global__ void inner_start1(int64_t n, const double *R, const double *rnrm2, const float *dinv,
-                             float *r, float *e, float *z, float *p, double *parts) {
-    double acc = 0.0;
-    const double nr = sqrt(rnrm2[0]);
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
-         i += (int64_t)gridDim.x * blockDim.x) {
-        const float rv = nr > 0 ? (float)(R[i] / nr) : 0.f;
-        const float zv = dinv[i] * rv;
-        r[i] = rv; e[i] = 0.f; z[i] = zv; p[i] = zv;
-        acc += (double)rv * (double)zv;
-    }
-    acc = block_sum_fixed(acc);
-    if (threadIdx.x == 0) parts[blockIdx.x] = acc;
-}
-
-// alpha = rz / pq; e += alpha p; r -= alpha q; z = D^-1 r; parts: <r, z>
-// at [0, stride), <r, r> at [stride, 2 stride).
-__global__ void inner_update1(int64_t n, const double *rz, const double *pq, const float *dinv,
-                              const float *p, const float *q, float *e, float *r, float *z,
-                              double *parts, int stride) {
-    double a1 = 0.0, a2 = 0.0;
-    const double den = pq[0];
-    const float a = (den > 0.0 && rz[0] > 0.0) ? (float)(rz[0] / den) : 0.f;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
-         i += (int64_t)gridDim.x * blockDim.x) {
-        e[i] += a * p[i];
-        const float rv = r[i] - a * q[i];
-        r[i] = rv;
-        const float zv = dinv[i] * rv;
-        z[i] = zv;
-        a1 += (double)rv * (double)zv;
-        a2 += (double)rv * (double)rv;
-    }
-    a1 = block_sum_fixed(a1);
-    a2 = block_sum_fixed(a2);
-    if (threadIdx.x == 0) { parts[blockIdx.x] = a1; parts[stride + blockIdx.x] = a2; }
-}
-
-// Start of an inner solve (k > 1): r = R / |R_c| (FP32), e = 0, z = D^-1 r,
-// p = z.  (rz0[c] = <r, z> by col_parts.)
-__global__ void inner_start(int64_t n, int k, const double *R, const double *rnrm2,
-                            const float *dinv, float *r, float *e, float *z, float *p) {
-    const int64_t tot = n * k;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < tot;
-         i += (int64_t)gridDim.x * blockDim.x) {
-        const int c = (int)(i % k);
-        const int64_t u = i / k;
-        const double nr = sqrt(rnrm2[c]);
-        const float rv = nr > 0 ? (float)(R[i] / nr) : 0.f;
-        const float zv = dinv[u] * rv;
-        r[i] = rv; e[i] = 0.f; z[i] = zv; p[i] = zv;
-    }
-}
-
-// k > 1: alpha_c = rz[c] / pq[c]; e += alpha p; r -= alpha q; z = D^-1 r.
-// (<r, z> and <r, r> by col_parts.)
-__global__ void inner_update(int64_t n, int k, const double *rz, const double *pq,
-                             const float *dinv, const float *p, const float *q, float *e,
-                             float *r, float *z) {
-    const int64_t tot = n * k;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < tot;
-         i += (int64_t)gridDim.x * blockDim.x) {
-        const int c = (int)(i % k);
-        const int64_t u = i / k;
-        const double den = pq[c];
-        const float a = (den > 0.0 && rz[c] > 0.0) ? (float)(rz[c] / den) : 0.f;
-        e[i] += a * p[i];
-        const float rv = r[i] - a * q[i];
-        r[i] = rv;
-        z[i] = dinv[u] * rv;
-    }
-}
-
-// q = L p over the rows of degree bin VW (rows of at most VW arcs, or more
-// than 16 arcs for VW = 32), VW lanes per row; all lanes of a warp iterate
-// together so the shuffles stay converged.  Returns this thread's share of
-// <p, q>.
-template <int VW, bool OFF64, bool W>
-__device__ __forceinline__ double spmv_bin(const DevGraph &g, const int32_t *__restrict__ rows,
-                                           int64_t nrows_bin, const float *__restrict__ p,
-                                           float *__restrict__ q, int64_t tid, int64_t nthr) {
-    const int sub = threadIdx.x & (VW - 1);
-    const int64_t row0 = tid / VW, ngroups = nthr / VW;
-    double acc = 0.0;
-    for (int64_t i0 = row0 - (row0 % (32 / VW)); i0 < nrows_bin; i0 += ngroups) {
-        const int64_t i = i0 + (row0 % (32 / VW));
-        float sacc = 0.f;
-        int u = -1;
-        if (i < nrows_bin) {
-            u = rows[i];
-            int64_t b, e2;
-            rowb<OFF64>(g, u, b, e2);
-            for (int64_t j = b + sub; j < e2; j += VW) sacc += (W ? g.w[j] : 1.f) * p[g.col[j]];
-        }
-#pragma unroll
-        for (int o = VW / 2; o > 0; o >>= 1) sacc += __shfl_xor_sync(0xffffffffu, sacc, o, VW);
-        if (sub == 0 && u >= 0) {
-            const float pu = p[u];
-            const float qu = (float)g.d[u] * pu - sacc;
-            q[u] = qu;
-            acc += (double)pu * (double)qu;
-        }
-    }
-    return acc;
-}
-
-// Grid-wide sums in a fixed order inside a cooperative launch: every block
-// stores its block_sum_fixed in parts, the grid synchronises, and every block
-// adds all the parts in block order, so all blocks hold the same bits.  The
-// parts are read through L2 (other SMs wrote them).
-__device__ __forceinline__ double bcast0(double v) {
-    __shared__ double b;
-    if (threadIdx.x == 0) b = v;
-    __syncthreads();
-    const double r = b;
-    return r;
-}
-__device__ __forceinline__ double gather_parts(const double *parts) {
-    double s = 0.0;
-    for (int i = threadIdx.x; i < (int)gridDim.x; i += blockDim.x) s += __ldcg(parts + i);
-    return bcast0(block_sum_fixed(s));
-}
-__device__ double grid_sum_fixed(cg::grid_group &grid, double v, double *parts) {
-    v = block_sum_fixed(v);
-    if (threadIdx.x == 0) parts[blockIdx.x] = v;
-    grid.sync();
-    return gather_parts(parts);
-}
-__device__ void grid_sum_fixed2(cg::grid_group &grid, double &v1, double &v2, double *p1, double *p2) {
-    const double b1 = block_sum_fixed(v1);
-    const double b2 = block_sum_fixed(v2);
-    if (threadIdx.x == 0) { p1[blockIdx.x] = b1; p2[blockIdx.x] = b2; }
-    grid.sync();
-    v1 = gather_parts(p1);
-    v2 = gather_parts(p2);
-}
-
-// One-launch inner PCG for a single right-hand side (cooperative launch,
-// grid-wide synchronisation between the phases of an iteration).  The
-// iteration's sums <p,q>, <r,z> and <r,r> are grid_sum_fixed results, the
-// same in every block, so the loop exit (relative residual at most tol, or no
-// halving of <r,r> for `window` iterations, or max_it) is taken by all blocks
-// together, and the same input gives the same bits on every run.  sc[1] holds
-// the starting <r,z>; parts: three arrays of gridDim doubles.  out[0] =
-// iterations, out[1] = last <r,r>.
-// Rows with more than HEAVY_DEG arcs are left out of the sub-warp product;
-// each of their HEAVY_CHUNK-arc chunks gets one warp, which stores its partial
-// sum in hsum and adds its share of <p, q> (p_u d_u p_u for a row's first
-// chunk, -p_u s_c for every chunk), and the update phase assembles such a
-// row's q_u = d_u p_u - sum of its chunks in chunk order.
-template <int VW, bool OFF64, bool W>
-__global__ void __launch_bounds__(TPB) cg1_coop(DevGraph g, const float *__restrict__ dinv,
-                                                float *r, float *e, float *z, float *p, float *q,
-                                                float *hsum, const double *sc, double *parts,
-                                                int max_it, double tol2, int window, double *out) {
-    cg::grid_group grid = cg::this_grid();
-    const int sub = threadIdx.x & (VW - 1);
-    const int64_t tid = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    const int64_t nthr = (int64_t)gridDim.x * blockDim.x;
-    const int64_t row0 = tid / VW, nrows = nthr / VW;
-    double best = INFINITY, rr = 1.0;
-    double rz = sc[1];
-    double *pA = parts, *pB = parts + gridDim.x, *pC = parts + 2 * (size_t)gridDim.x;
-    int since = 0, it = 0;
-    for (; it < max_it; ++it) {
-        // q = L p and <p, q>
-        double acc = 0.0;
-        bool done = false;
-        if constexpr (!W && !OFF64) {
-            if (g.ell) {
-                // bounded degree: one thread per row over its inline neighbour
-                // list (one or two 16-byte loads), the heads' p gathered in
-                // arc order
-                const int ew4 = g.ell_w / 4;
-                for (int64_t u = tid; u < g.n; u += nthr) {
-                    float s = 0.f;
-                    for (int i = 0; i < ew4; ++i) {
-                        const int4 c4 = __ldg(g.ell + u * ew4 + i);
-                        if (c4.x >= 0) s += p[c4.x];
-                        if (c4.y >= 0) s += p[c4.y];
-                        if (c4.z >= 0) s += p[c4.z];
-                        if (c4.w >= 0) s += p[c4.w];
-                    }
-                    const float pu = p[u];
-                    const float qu = (float)g.d[u] * pu - s;
-                    q[u] = qu;
-                    acc += (double)pu * (double)qu;
-                }
-                done = true;
-            }
-        }
-        if (done) {
-        } else if (g.bin_rows) {
-            // rows by degree bin, each bin with as many lanes per row as its degrees
-            acc += spmv_bin<2, OFF64, W>(g, g.bin_rows + g.bin_off[0], g.bin_off[1] - g.bin_off[0], p, q, tid, nthr);
-            acc += spmv_bin<4, OFF64, W>(g, g.bin_rows + g.bin_off[1], g.bin_off[2] - g.bin_off[1], p, q, tid, nthr);
-            acc += spmv_bin<8, OFF64, W>(g, g.bin_rows + g.bin_off[2], g.bin_off[3] - g.bin_off[2], p, q, tid, nthr);
-            acc += spmv_bin<16, OFF64, W>(g, g.bin_rows + g.bin_off[3], g.bin_off[4] - g.bin_off[3], p, q, tid, nthr);
-            acc += spmv_bin<32, OFF64, W>(g, g.bin_rows + g.bin_off[4], g.bin_off[5] - g.bin_off[4], p, q, tid, nthr);
-        } else
-        for (int64_t u0 = row0 - (row0 % (32 / VW)); u0 < g.n; u0 += nrows) {
-            const int64_t u = u0 + (row0 % (32 / VW));
-            float sacc = 0.f;
-            bool light = false;
-            if (u < g.n) {
-                int64_t b, e2;
-                rowb<OFF64>(g, u, b, e2);
-                light = g.hc_n == 0 || e2 - b <= HEAVY_DEG;
-                if (light)
-                    for (int64_t j = b + sub; j < e2; j += VW) sacc += (W ? g.w[j] : 1.f) * p[g.col[j]];
-            }
-#pragma unroll
-            for (int o = VW / 2; o > 0; o >>= 1) sacc += __shfl_xor_sync(0xffffffffu, sacc, o, VW);
-            if (sub == 0 && light) {
-                const float pu = p[u];
-                const float qu = (float)g.d[u] * pu - sacc;
-                q[u] = qu;
-                acc += (double)pu * (double)qu;
-            }
-        }
-        if (g.hc_n) {
-            const int lane = threadIdx.x & 31;
-            for (int64_t c = tid / 32; c < g.hc_n; c += nthr / 32) {
-                const int32_t u = g.hc_row[c];
-                int64_t rb0, re;
-                rowb<OFF64>(g, u, rb0, re);
-                const int64_t b = g.hc_beg[c], e2 = min(b + HEAVY_CHUNK, re);
-                float s = 0.f;
-                for (int64_t j = b + lane; j < e2; j += 32) s += (W ? g.w[j] : 1.f) * p[g.col[j]];
-#pragma unroll
-                for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-                if (lane == 0) {
-                    hsum[c] = s;
-                    const double pu = (double)p[u];
-                    if (b == rb0) acc += pu * (double)(float)((float)g.d[u] * p[u]);
-                    acc -= pu * (double)s;
-                }
-            }
-        }
-        const double den = grid_sum_fixed(grid, acc, pA);
-        // step and the new residual
-        const float a = (den > 0.0 && rz > 0.0) ? (float)(rz / den) : 0.f;
-        double a1 = 0.0, a2 = 0.0;
-        for (int64_t i = tid; i < g.n; i += nthr) {
-            float qi;
-            const int32_t hf = g.hc_n ? g.hfirst[i] : -1;
-            if (hf < 0) {
-                qi = q[i];
-            } else {
-                int64_t rb0, re;
-                rowb<OFF64>(g, i, rb0, re);
-                const int64_t nc = (re - rb0 + HEAVY_CHUNK - 1) / HEAVY_CHUNK;
-                float s = 0.f;
-                for (int64_t c = 0; c < nc; ++c) s += hsum[hf + c];
-                qi = (float)g.d[i] * p[i] - s;
-            }
-            e[i] += a * p[i];
-            const float rv = r[i] - a * qi;
-            r[i] = rv;
-            const float zv = dinv[i] * rv;
-            z[i] = zv;
-            a1 += (double)rv * (double)zv;
-            a2 += (double)rv * (double)rv;
-        }
-        grid_sum_fixed2(grid, a1, a2, pB, pC);
-        rr = a2;
-        const double rz1 = a1;
-        if (!(rr == rr) || rr <= tol2) { ++it; break; }
-        if (rr < 0.25 * best) { best = rr; since = 0; }
-        else if (++since >= window) { ++it; break; }
-        // new direction
-        const float bta = rz > 0.0 ? (float)(rz1 / rz) : 0.f;
-        rz = rz1;
-        for (int64_t i = tid; i < g.n; i += nthr) p[i] = z[i] + bta * p[i];
-        grid.sync();
-    }
-    if (tid == 0) { out[0] = (double)it; out[1] = rr; }
-}
-
-// p = z + beta p, beta_c = rz1[c] / rz0[c].
-__global__ void inner_dir(int64_t n, int k, const double *rz0, const double *rz1, const float *z,
-                          float *p) {
-    const int64_t tot = n * k;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < tot;
-         i += (int64_t)gridDim.x * blockDim.x) {
-        const int c = (int)(i % k);
-        const float bta = rz0[c] > 0.0 ? (float)(rz1[c] / rz0[c]) : 0.f;
-        p[i] = z[i] + bta * p[i];
-    }
-}
-
-// X += |R_c| e.
-__global__ void outer_add(int64_t n, int k, const double *rnrm2, const float *e, double *X) {
-    const int64_t tot = n * k;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < tot;
-         i += (int64_t)gridDim.x * blockDim.x) {
-        const int c = (int)(i % k);
-        X[i] += sqrt(rnrm2[c]) * (double)e[i];
-    }
 }
 
 template <class F>
@@ -560,21 +293,6 @@ void dispatch(const DevGraph &g, F f) {
         if (g.weighted) f(std::false_type{}, std::true_type{});
         else f(std::false_type{}, std::false_type{});
     }
-}
-
-template <class F>
-void dispatch_vw(int vw, F f) {
-    switch (vw) {
-        case 4: f(std::integral_constant<int, 4>{}); break;
-        case 8: f(std::integral_constant<int, 8>{}); break;
-        case 16: f(std::integral_constant<int, 16>{}); break;
-        default: f(std::integral_constant<int, 32>{}); break;
-    }
-}
-
-int pick_vw(const DevGraph &g) {
-    const double avg = (double)g.nnz / (double)g.n;
-    return avg <= 4.5 ? 4 : avg <= 9 ? 8 : avg <= 20 ? 16 : 32;
 }
 
 unsigned grid_for(int64_t work) {
@@ -591,104 +309,66 @@ rwc_status solve_nodemajor(rwc_graph *G, int k, const double *B, double *X, doub
     const int64_t n = g.n;
     if (k <= 0) return set_error(RWC_ERR_INVALID, "k must be positive");
     if (tol <= 0) tol = 1e-10;
+    if (k == 1) return solve_one(G, B, X, tol, iters_out, st);
     const int64_t nk = n * k;
     const int max_inner = (int)std::min<int64_t>(200000, std::max<int64_t>(1000, 4 * n));
     const int max_outer = 30;
     const double inner_tol = 1e-5;
-    // device buffers
+    const int k4 = (k + 3) / 4, kp = 4 * k4;
+    // blocks: qt quads of columns x TPB / qt row slots; nb row ranges, fewer for
+    // many column tiles (the parts are [kp][nb])
+    const int qt = std::min(k4, 64), threads = qt * (TPB / qt), tiles = (k4 + qt - 1) / qt;
+    const unsigned nb = (unsigned)std::max<int64_t>(1, std::min<int64_t>(((int64_t)num_sms() * 6 + tiles - 1) / tiles,
+                                                                         (n + threads / qt - 1) / (threads / qt)));
+    const dim3 grid(nb, (unsigned)tiles);
+    const int ct = std::min(k, 128), rthreads = ct * (TPB / ct);
+    const dim3 rgrid((unsigned)std::max<int64_t>(1, std::min<int64_t>((int64_t)num_sms() * 8, (n * ct + rthreads - 1) / rthreads)),
+                     (unsigned)((k + ct - 1) / ct));
+    const unsigned nbc = (unsigned)std::max<int64_t>(1, std::min<int64_t>((int64_t)num_sms() * 4, (n + 63) / 64));
     Buf buf(st);
-    const size_t fbytes = (size_t)nk * sizeof(float);
-    const size_t sc_per_it = 3 * (size_t)k;                 // pq, rz, rr per iteration
-    const size_t sc_count = (size_t)(max_inner + 4) * sc_per_it + 8 * (size_t)k;
-    const size_t hbytes = (size_t)(g.hc_n + 1) * sizeof(float);
-    constexpr int PMAX = 4096;                             // block parts of one reduction
-    // k > 1: blocks of the column reductions and their [k][nbc] parts (two sets)
-    const unsigned nbc = k > 1 ? (unsigned)std::max<int64_t>(1, std::min<int64_t>((int64_t)num_sms() * 4,
-                                                                                  (n + 63) / 64)) : 0u;
-    const size_t cbytes = k > 1 ? 2 * (size_t)k * nbc * sizeof(double) : 0;
-    const size_t bytes = (size_t)nk * sizeof(double) + 5 * fbytes + sc_count * sizeof(double) + hbytes +
-                         3 * PMAX * sizeof(double) + cbytes + 1024;
+    const size_t fbytes = (size_t)n * kp * sizeof(float);
+    const size_t nparts = (size_t)kp * std::max(nb, nbc);
+    const size_t bytes = (size_t)nk * 8 + 4 * fbytes + 2 * nparts * 8 + (size_t)8 * kp * 8 + 16 * 256;
     RWC_CUDA_TRY(cudaMallocAsync(&buf.p, bytes, st));
-    char *q = (char *)buf.p;
-    double *R = (double *)q; q += (size_t)nk * sizeof(double);
-    float *r = (float *)q; q += fbytes;
-    float *e = (float *)q; q += fbytes;
-    float *z = (float *)q; q += fbytes;
-    float *p = (float *)q; q += fbytes;
-    float *Qv = (float *)q; q += fbytes;
-    q = (char *)(((uintptr_t)q + 255) & ~(uintptr_t)255);
-    double *outer_sc = (double *)q;       // [0,k) colsum, [k,2k) |R|^2, [2k,3k) |B|^2
-    double *it_sc = outer_sc + 8 * (size_t)k;
-    double *parts = it_sc + (sc_count - 8 * (size_t)k);   // [3][PMAX] fixed-order block parts
-    double *cparts = parts + 3 * (size_t)PMAX;          // k > 1: [2][k][nbc] column parts
-    float *hsum = (float *)(cparts + 2 * (size_t)k * nbc);   // [hc_n] heavy-chunk sums
-    const size_t shk = (size_t)k * sizeof(double);
-    const unsigned gs = grid_for(nk), gw = grid_for(n * 32);
-    const int vw = pick_vw(g);
-    const unsigned gv = grid_for(n * vw);
-    if (gs > (unsigned)PMAX || gv > (unsigned)PMAX) return set_error(RWC_ERR_UNSUPPORTED, "solver grid above %d blocks", PMAX);
-    // k == 1: fixed-order sums (block parts, then sum_parts in block order)
-    auto finish_sum = [&](unsigned blocks, int nvals, double *out) {
-        ::rwc::count_launches(1);
-        sum_parts<<<1, TPB, 0, st>>>(parts, (int)blocks, PMAX, nvals, out);
-    };
-    // k > 1: fixed-order per-column sums of f(A, B) into o1 (and o2)
-    double *cp2 = cparts + (size_t)k * nbc;
-    auto col_sum = [&](auto op, const auto *A, const auto *Bv, double *o1, double *o2) {
-        constexpr int OP = decltype(op)::value;
-        using T = std::remove_cv_t<std::remove_pointer_t<decltype(A)>>;
+    char *at = (char *)buf.p;
+    auto take = [&](size_t b) { char *r = at; at += (b + 255) & ~(size_t)255; return r; };
+    double *R = (double *)take((size_t)nk * 8);
+    float4 *r = (float4 *)take(fbytes), *e = (float4 *)take(fbytes), *p = (float4 *)take(fbytes), *q = (float4 *)take(fbytes);
+    double *pa = (double *)take(nparts * 8), *pb = (double *)take(nparts * 8);
+    double *colsum = (double *)take((size_t)kp * 8), *rn2 = (double *)take((size_t)kp * 8);
+    double *pq = (double *)take((size_t)kp * 8), *rr = (double *)take((size_t)kp * 8);
+    double *rz[2] = {(double *)take((size_t)kp * 8), (double *)take((size_t)kp * 8)};
+    const unsigned gs = grid_for(nk);
+    auto col_sum = [&](auto square, const double *A, double *out) {
         ::rwc::count_launches(2);
-        col_parts<OP, T><<<nbc, TPB, 0, st>>>(n, k, A, Bv, cparts, cp2);
-        sum_cols<<<(unsigned)k, TPB, 0, st>>>(cparts, (int)nbc, o1);
-        if (OP == COL_DOT2) { ::rwc::count_launches(1); sum_cols<<<(unsigned)k, TPB, 0, st>>>(cp2, (int)nbc, o2); }
+        col_parts<decltype(square)::value><<<nbc, TPB, 0, st>>>(n, k, A, pa);
+        sum_cols<<<dim3((unsigned)k, 1), 128, 0, st>>>(pa, nullptr, (int)nbc, out, nullptr);
     };
-    using op_sum = std::integral_constant<int, COL_SUM>;
-    using op_sq = std::integral_constant<int, COL_SQ>;
-    using op_dot = std::integral_constant<int, COL_DOT>;
-    using op_dot2 = std::integral_constant<int, COL_DOT2>;
-    int dev = 0, coop = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev);
-    const bool coop_ok = coop != 0;
-
     RWC_CUDA_TRY(cudaMemsetAsync(X, 0, (size_t)nk * sizeof(double), st));
-    std::vector<double> h(3 * (size_t)k), bn(k);
+    std::vector<double> h(kp), bn(k);
     int total_iters = 0;
     double prev_worst = INFINITY;
     int slow = 0;
     for (int outer = 0; outer <= max_outer; ++outer) {
-        RWC_CUDA_TRY(cudaMemsetAsync(outer_sc, 0, 3 * shk, st));
         dispatch(g, [&](auto o64, auto wt) {
             ::rwc::count_launches(1);
-            if (k == 1) {
-                dispatch_vw(vw, [&](auto V) {
-                    resid1<decltype(V)::value, decltype(o64)::value, decltype(wt)::value>
-                        <<<gv, TPB, 0, st>>>(g, B, X, R, parts);
-                });
-            } else {
-                resid64<decltype(o64)::value, decltype(wt)::value><<<gw, TPB, 0, st>>>(g, k, B, X, R);
-            }
+            resid64<decltype(o64)::value, decltype(wt)::value><<<rgrid, rthreads, 0, st>>>(g, k, ct, B, X, R);
         });
-        if (k == 1) {
-            finish_sum(gv, 1, outer_sc);
-            ::rwc::count_launches(1); center1<<<gs, TPB, 0, st>>>(n, R, outer_sc, parts);
-            finish_sum(gs, 1, outer_sc + 1);
-        } else {
-            col_sum(op_sum{}, (const double *)R, (const double *)nullptr, outer_sc, nullptr);
-            ::rwc::count_launches(1); center64<<<gs, TPB, 0, st>>>(n, k, R, outer_sc);
-            col_sum(op_sq{}, (const double *)R, (const double *)nullptr, outer_sc + k, nullptr);
-        }
+        col_sum(std::false_type{}, R, colsum);
+        ::rwc::count_launches(1);
+        center64<<<gs, TPB, 0, st>>>(n, k, R, colsum);
+        col_sum(std::true_type{}, R, rn2);
         RWC_CUDA_TRY(cudaGetLastError());
-        RWC_CUDA_TRY(cudaMemcpyAsync(h.data(), outer_sc, 2 * shk, cudaMemcpyDeviceToHost, st));
+        RWC_CUDA_TRY(cudaMemcpyAsync(h.data(), rn2, (size_t)k * 8, cudaMemcpyDeviceToHost, st));
         RWC_CUDA_TRY(cudaStreamSynchronize(st));
         if (outer == 0)
-            for (int c = 0; c < k; ++c) bn[c] = std::sqrt(h[k + c]);
+            for (int c = 0; c < k; ++c) bn[c] = std::sqrt(h[c]);
         double worst = 0.0;
         for (int c = 0; c < k; ++c) {
-            const double rel = bn[c] > 0 ? std::sqrt(h[k + c]) / bn[c] : 0.0;
+            const double rel = bn[c] > 0 ? std::sqrt(h[c]) / bn[c] : 0.0;
+            if (!(rel == rel)) return set_error(RWC_ERR_NOT_CONVERGED, "solver produced NaN");
             worst = std::max(worst, rel);
         }
-        if (!(worst == worst)) return set_error(RWC_ERR_NOT_CONVERGED, "solver produced NaN");
         if (worst <= tol) break;
         if (worst < 0.5 * prev_worst) { prev_worst = worst; slow = 0; }
         else if (++slow >= 4)
@@ -696,118 +376,50 @@ rwc_status solve_nodemajor(rwc_graph *G, int k, const double *B, double *X, doub
         if (outer == max_outer)
             return set_error(RWC_ERR_NOT_CONVERGED, "Laplacian solve reached %d refinements at relative residual %.3g (tol %.3g)", max_outer, worst, tol);
         // inner FP32 PCG on the normalised residual
-        RWC_CUDA_TRY(cudaMemsetAsync(it_sc, 0, sc_count * sizeof(double) - 8 * shk, st));
-        if (k == 1) {
-            ::rwc::count_launches(1); inner_start1<<<gs, TPB, 0, st>>>(n, R, outer_sc + 1, g.dinv32, r, e, z, p, parts);
-            finish_sum(gs, 1, it_sc + 1);
-        } else {
-            ::rwc::count_launches(1); inner_start<<<gs, TPB, 0, st>>>(n, k, R, outer_sc + k, g.dinv32, r, e, z, p);
-            col_sum(op_dot{}, (const float *)r, (const float *)z, it_sc + 1 * k, nullptr);
-        }
-        if (k == 1 && coop_ok) {
-            // one cooperative launch for the whole inner solve
-            double *outv = outer_sc + 4;
-            int mi = max_inner;
-            double t2 = inner_tol * inner_tol;
-            int window = 1024;
-            bool launched = false;
-            dispatch(g, [&](auto o64, auto wt) {
-                dispatch_vw(vw, [&](auto V) {
-                    auto kern = cg1_coop<decltype(V)::value, decltype(o64)::value, decltype(wt)::value>;
-                    int per_sm = 0;
-                    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, TPB, 0);
-                    if (per_sm < 1) return;
-                    // at most 4 blocks per SM (6 fit): fewer blocks make each grid
-                    // synchronisation and fixed-order sum cheaper, which the
-                    // latency-bound iterations of large-diameter graphs feel most
-                    // (1024² grid 0.48 -> 0.37 s; R-MAT 24 the same; 3 per SM slows
-                    // the bandwidth-heavier R-MAT solves)
-                    per_sm = std::min(per_sm, 4);
-                    const unsigned blocks = (unsigned)std::min<int64_t>(std::min<int64_t>((int64_t)num_sms() * per_sm, gv), PMAX);
-                    const float *dinv = g.dinv32;
-                    float *rr_ = r, *ee = e, *zz = z, *pp = p, *qq = Qv, *hs = hsum;
-                    const double *scp = it_sc;
-                    double *pts = parts;
-                    DevGraph gg = g;
-                    void *args[] = {&gg, &dinv, &rr_, &ee, &zz, &pp, &qq, &hs, &scp, &pts, &mi, &t2, &window, &outv};
-                    ::rwc::count_launches(1);
-                    if (cudaLaunchCooperativeKernel((const void *)kern, blocks, TPB, args, 0, st) == cudaSuccess)
-                        launched = true;
-                });
-            });
-            if (launched) {
-                double hv[2];
-                RWC_CUDA_TRY(cudaMemcpyAsync(hv, outv, 2 * sizeof(double), cudaMemcpyDeviceToHost, st));
-                RWC_CUDA_TRY(cudaStreamSynchronize(st));
-                total_iters += (int)hv[0];
-                ::rwc::count_launches(1); outer_add<<<gs, TPB, 0, st>>>(n, k, outer_sc + k, e, X);
-                RWC_CUDA_TRY(cudaGetLastError());
-                continue;
-            }
-            (void)cudaGetLastError();
-        }
+        ::rwc::count_launches(2);
+        bcg_start<<<grid, threads, 0, st>>>(n, k, k4, qt, R, rn2, g.dinv32, r, e, p, pa);
+        sum_cols<<<dim3((unsigned)kp, 1), 128, 0, st>>>(pa, nullptr, (int)nb, rz[0], nullptr);
         int it = 0;
-        const int check = 16;
+        const int check = 4;   // iterations between looks at the residual
         bool inner_done = false;
         double best = INFINITY;
         int since_best = 0;
         while (!inner_done && it < max_inner) {
             for (int j = 0; j < check && it < max_inner; ++j, ++it) {
-                double *pq = it_sc + (size_t)it * sc_per_it;          // slot it: pq
-                double *rz0 = it_sc + (size_t)it * sc_per_it + k;     // rz of iterate it
-                double *rz1 = it_sc + (size_t)(it + 1) * sc_per_it + k;
-                double *rr1 = it_sc + (size_t)(it + 1) * sc_per_it + 2 * k;
+                double *z0 = rz[it & 1], *z1 = rz[(it & 1) ^ 1];
+                ::rwc::count_launches(5);
                 dispatch(g, [&](auto o64, auto wt) {
-                    ::rwc::count_launches(1);
-                    if (k == 1) {
-                        dispatch_vw(vw, [&](auto V) {
-                            spmv32<decltype(V)::value, decltype(o64)::value, decltype(wt)::value>
-                                <<<gv, TPB, 0, st>>>(g, p, Qv, parts);
-                        });
-                    } else {
-                        spmm32<decltype(o64)::value, decltype(wt)::value><<<gw, TPB, 0, st>>>(g, k, p, Qv);
-                    }
+                    bcg_product<decltype(o64)::value, decltype(wt)::value><<<grid, threads, 0, st>>>(g, k4, qt, p, q, pa);
                 });
-                if (k == 1) {
-                    finish_sum(gv, 1, pq);
-                    ::rwc::count_launches(1);
-                    inner_update1<<<gs, TPB, 0, st>>>(n, rz0, pq, g.dinv32, p, Qv, e, r, z, parts, PMAX);
-                    finish_sum(gs, 2, rz1);   // rz1, then rr1 = rz1 + 1
-                } else {
-                    col_sum(op_dot{}, (const float *)p, (const float *)Qv, pq, nullptr);
-                    ::rwc::count_launches(1); inner_update<<<gs, TPB, 0, st>>>(n, k, rz0, pq, g.dinv32, p, Qv, e, r, z);
-                    col_sum(op_dot2{}, (const float *)r, (const float *)z, rz1, rr1);
-                }
-                ::rwc::count_launches(1); inner_dir<<<gs, TPB, 0, st>>>(n, k, rz0, rz1, z, p);
+                sum_cols<<<dim3((unsigned)kp, 1), 128, 0, st>>>(pa, nullptr, (int)nb, pq, nullptr);
+                bcg_residual<<<grid, threads, 0, st>>>(n, k4, qt, z0, pq, g.dinv32, q, r, pa, pb);
+                sum_cols<<<dim3((unsigned)kp, 2), 128, 0, st>>>(pa, pb, (int)nb, z1, rr);
+                bcg_direction<<<grid, threads, 0, st>>>(n, k4, qt, z0, pq, z1, g.dinv32, r, e, p);
             }
             RWC_CUDA_TRY(cudaGetLastError());
-            RWC_CUDA_TRY(cudaMemcpyAsync(h.data(), it_sc + (size_t)it * sc_per_it + 2 * k, shk,
-                                         cudaMemcpyDeviceToHost, st));
+            RWC_CUDA_TRY(cudaMemcpyAsync(h.data(), rr, (size_t)k * 8, cudaMemcpyDeviceToHost, st));
             RWC_CUDA_TRY(cudaStreamSynchronize(st));
             double w2 = 0.0;
-            for (int c = 0; c < k; ++c) w2 = std::max(w2, h[c]);
-            if (std::sqrt(w2) <= inner_tol || !(w2 == w2)) inner_done = true;
-            // FP32 stagnation: the residual norm has not halved for 64 checks
-            // (1024 iterations); CG residuals are not monotone, so the window
-            // is long
+            bool bad = false;
+            for (int c = 0; c < k; ++c) {
+                bad = bad || !(h[c] == h[c]);
+                w2 = std::max(w2, h[c]);
+            }
+            if (std::sqrt(w2) <= inner_tol || bad) inner_done = true;
+            // FP32 stagnation: the residual norm has not halved for 1024
+            // iterations; CG residuals are not monotone, so the window is long
             if (w2 < 0.25 * best) { best = w2; since_best = 0; }
-            else if (++since_best >= 64) inner_done = true;
+            else if (++since_best >= 1024 / check) inner_done = true;
         }
         total_iters += it;
-        ::rwc::count_launches(1); outer_add<<<gs, TPB, 0, st>>>(n, k, outer_sc + k, e, X);
+        ::rwc::count_launches(1);
+        bcg_add<<<gs, TPB, 0, st>>>(n, k, k4, rn2, (const float *)e, X);
         RWC_CUDA_TRY(cudaGetLastError());
     }
     // final projection of X onto 1-perp
-    RWC_CUDA_TRY(cudaMemsetAsync(outer_sc, 0, 2 * shk, st));
-    if (k == 1) {
-        ::rwc::count_launches(1); sum1<<<gs, TPB, 0, st>>>(n, X, parts);
-        finish_sum(gs, 1, outer_sc);
-        ::rwc::count_launches(1); center1<<<gs, TPB, 0, st>>>(n, X, outer_sc, parts);
-        finish_sum(gs, 1, outer_sc + 1);
-    } else {
-        col_sum(op_sum{}, (const double *)X, (const double *)nullptr, outer_sc, nullptr);
-        ::rwc::count_launches(1); center64<<<gs, TPB, 0, st>>>(n, k, X, outer_sc);
-    }
+    col_sum(std::false_type{}, X, colsum);
+    ::rwc::count_launches(1);
+    center64<<<gs, TPB, 0, st>>>(n, k, X, colsum);
     RWC_CUDA_TRY(cudaGetLastError());
     if (iters_out) *iters_out = total_iters;
     return RWC_OK;
