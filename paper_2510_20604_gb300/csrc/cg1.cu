@@ -47,18 +47,32 @@ struct CgArgs {
     double tol;
     int max_outer, max_inner;
     int use_smem;                       // inline rows fit shared memory
+    bool clustered;                     // the blocks are one cluster
     double *out;                        // iterations, relative residual, status
 };
 enum : int { CG_OK = 0, CG_NAN = 1, CG_STALLED = 2, CG_MAX_OUTER = 3 };
 
+// All blocks: one cluster (its barrier is a few hundred cycles) or the grid.
+__device__ __forceinline__ void blocks_sync(bool clustered) {
+    if (clustered) cg::this_cluster().sync();
+    else cg::this_grid().sync();
+}
+__device__ __forceinline__ void all_sync(bool clustered) {
+    if (gridDim.x > 1) blocks_sync(clustered);
+    else __syncthreads();
+}
+
 // Fixed-order sums over the grid of K values per thread: a shuffle tree in
-// every warp, the warps of a block in order, the blocks in order; every thread
-// gets the same bits.  `flip` alternates the blocks' slots, so that a block can
-// write its next sums while another still reads these.
-template <int K, class T>
-__device__ void grid_sums(const T (&v)[K], double (&out)[K], double *parts, int &flip) {
+// every warp, the warps of a block in order, the blocks in order.  Thread 0 of
+// every block passes them to post(sums), which gets the same bits in every
+// block and returns what all threads get: scalar FP64 work (a division is a
+// dozen instructions of 16 cycles each) is done once per block, not once per
+// warp.  `flip` alternates the blocks' slots, so that a block can write its next
+// sums while another still reads these.
+template <int K, class Out, class T, class Post>
+__device__ Out grid_sums(const T (&v)[K], double *parts, int &flip, bool clustered, Post post) {
     __shared__ double ws[K][32];
-    __shared__ double bc[K];
+    __shared__ Out bc;
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
     const int nb = gridDim.x;
     double *slot = parts + (size_t)flip * 2 * nb;
@@ -85,29 +99,35 @@ __device__ void grid_sums(const T (&v)[K], double (&out)[K], double *parts, int 
         }
     }
     __syncthreads();
-    if (wid < K) {
-        double a = lane < nw ? ws[wid][lane] : 0.0;
+    double t[K];
+    if (wid == 0) {
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
-        if (lane == 0) { if (nb > 1) slot[(size_t)wid * nb + blockIdx.x] = a; else bc[wid] = a; }
+        for (int k = 0; k < K; ++k) t[k] = lane < nw ? ws[k][lane] : 0.0;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+            for (int k = 0; k < K; ++k) t[k] += __shfl_xor_sync(0xffffffffu, t[k], o);
+        if (nb > 1 && lane == 0)
+#pragma unroll
+            for (int k = 0; k < K; ++k) slot[(size_t)k * nb + blockIdx.x] = t[k];
     }
     if (nb > 1) {
-        cg::this_grid().sync();
-        if (wid < K) {
-            double a = 0.0;
-            for (int i = lane; i < nb; i += 32) a += __ldcg(slot + (size_t)wid * nb + i);
+        blocks_sync(clustered);
+        if (wid == 0) {
 #pragma unroll
-            for (int o = 16; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
-            if (lane == 0) bc[wid] = a;
+            for (int k = 0; k < K; ++k) t[k] = 0.0;
+            for (int i = lane; i < nb; i += 32)
+#pragma unroll
+                for (int k = 0; k < K; ++k) t[k] += __ldcg(slot + (size_t)k * nb + i);
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+                for (int k = 0; k < K; ++k) t[k] += __shfl_xor_sync(0xffffffffu, t[k], o);
         }
     }
+    if (threadIdx.x == 0) bc = post(t);
     __syncthreads();
-#pragma unroll
-    for (int k = 0; k < K; ++k) out[k] = bc[k];
-}
-__device__ __forceinline__ void all_sync() {
-    if (gridDim.x > 1) cg::this_grid().sync();
-    else __syncthreads();
+    return bc;
 }
 
 template <bool OFF64>
@@ -164,15 +184,63 @@ __device__ __forceinline__ void bin_rows(const DevGraph &g, int bin, Term term, 
         }
     }
 }
+// The same rows where there are few: a warp takes units of 32 / VW rows of any
+// bin in turn, so that the bins' chains of loads run side by side.
+template <int VW, bool OFF64, class T, class Term, class F>
+__device__ __forceinline__ void one_unit(const DevGraph &g, int bin, int64_t unit, Term term, F f) {
+    const int lane = threadIdx.x & 31, sub = lane & (VW - 1);
+    const int64_t i = unit * (32 / VW) + lane / VW;
+    const int64_t nrows = g.bin_off[bin + 1] - g.bin_off[bin];
+    int32_t u = -1;
+    int64_t b = 0, e = 0;
+    if (i < nrows) { u = g.bin_rows[g.bin_off[bin] + i]; row_of<OFF64>(g, u, b, e); }
+    T s = 0;
+    if (VW == 32) {
+        T s4[4] = {};
+        for (int64_t j = b + sub; j < e; j += 128) {
+#pragma unroll
+            for (int k = 0; k < 4; ++k)
+                if (j + 32 * k < e) s4[k] += term(j + 32 * k);
+        }
+        s = (s4[0] + s4[1]) + (s4[2] + s4[3]);
+    } else if (b + sub < e) {
+        s = term(b + sub);
+    }
+#pragma unroll
+    for (int o = VW / 2; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o, VW);
+    if (sub == 0 && u >= 0) f(u, s);
+}
+template <bool OFF64, class T, class Term, class F>
+__device__ __forceinline__ bool few_rows(const DevGraph &g, Term term, F f) {
+    const int64_t warps = (int64_t)gridDim.x * blockDim.x / 32;
+    int64_t end[5], total = 0;
+#pragma unroll
+    for (int b = 0; b < 5; ++b) {
+        const int rows = 16 >> b;
+        total += (g.bin_off[b + 1] - g.bin_off[b] + rows - 1) / rows;
+        end[b] = total;
+    }
+    if (total > 8 * warps) return false;
+    for (int64_t w = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) / 32; w < total; w += warps) {
+        if (w < end[0]) one_unit<2, OFF64, T>(g, 0, w, term, f);
+        else if (w < end[1]) one_unit<4, OFF64, T>(g, 1, w - end[0], term, f);
+        else if (w < end[2]) one_unit<8, OFF64, T>(g, 2, w - end[1], term, f);
+        else if (w < end[3]) one_unit<16, OFF64, T>(g, 3, w - end[2], term, f);
+        else one_unit<32, OFF64, T>(g, 4, w - end[3], term, f);
+    }
+    return true;
+}
 // all rows of at most HEAVY_DEG arcs through f, the heavy rows' chunks through
 // h(chunk, row, first chunk of its row, sum)
 template <bool OFF64, class T, class Term, class F, class H>
 __device__ __forceinline__ void all_rows(const DevGraph &g, Term term, F f, H h) {
-    bin_rows<2, OFF64, T>(g, 0, term, f);
-    bin_rows<4, OFF64, T>(g, 1, term, f);
-    bin_rows<8, OFF64, T>(g, 2, term, f);
-    bin_rows<16, OFF64, T>(g, 3, term, f);
-    bin_rows<32, OFF64, T>(g, 4, term, f);
+    if (!few_rows<OFF64, T>(g, term, f)) {
+        bin_rows<2, OFF64, T>(g, 0, term, f);
+        bin_rows<4, OFF64, T>(g, 1, term, f);
+        bin_rows<8, OFF64, T>(g, 2, term, f);
+        bin_rows<16, OFF64, T>(g, 3, term, f);
+        bin_rows<32, OFF64, T>(g, 4, term, f);
+    }
     const int lane = threadIdx.x & 31;
     const int64_t tid = blockIdx.x * (int64_t)blockDim.x + threadIdx.x, nthr = (int64_t)gridDim.x * blockDim.x;
     for (int64_t c = tid / 32; c < g.hc_n; c += nthr / 32) {
@@ -212,17 +280,15 @@ __device__ void refine(const CgArgs &a, int &flip, Resid resid, Each each, Inner
     double bn = 0.0, prev = INFINITY, worst = 0.0;
     int total = 0, slow = 0, status = CG_MAX_OUTER;
     for (int outer = 0; outer <= a.max_outer; ++outer) {
-        double sum[1] = {resid()}, tot[1];
-        grid_sums<1>(sum, tot, a.parts, flip);
-        const double mean = tot[0] / n;
+        double sum[1] = {resid()};
+        const double mean = grid_sums<1, double>(sum, a.parts, flip, a.clustered, [&](const double *t) { return t[0] / n; });
         sum[0] = 0.0;
         each([&](int64_t i) {
             const double v = a.R[i] - mean;
             a.R[i] = v;
             sum[0] += v * v;
         });
-        grid_sums<1>(sum, tot, a.parts, flip);
-        const double rn = sqrt(tot[0]);
+        const double rn = grid_sums<1, double>(sum, a.parts, flip, a.clustered, [&](const double *t) { return sqrt(t[0]); });
         if (outer == 0) bn = rn;
         worst = bn > 0 ? rn / bn : 0.0;
         if (!(worst == worst)) { status = CG_NAN; break; }
@@ -233,10 +299,9 @@ __device__ void refine(const CgArgs &a, int &flip, Resid resid, Each each, Inner
         total += inner(rn);
     }
     // X onto 1-perp
-    double sum[1] = {0.0}, tot[1];
+    double sum[1] = {0.0};
     each([&](int64_t i) { sum[0] += a.X[i]; });
-    grid_sums<1>(sum, tot, a.parts, flip);
-    const double mean = tot[0] / n;
+    const double mean = grid_sums<1, double>(sum, a.parts, flip, a.clustered, [&](const double *t) { return t[0] / n; });
     each([&](int64_t i) { a.X[i] -= mean; });
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         a.out[0] = (double)total;
@@ -245,20 +310,27 @@ __device__ void refine(const CgArgs &a, int &flip, Resid resid, Each each, Inner
     }
 }
 
+// num / den rounded to float: a float quotient corrected by its FP64 residual
+// (the FP64 division is a long dependent chain on the iteration's path).
+__device__ __forceinline__ float quotient(double num, double den) {
+    const float d = (float)den, q = __fdiv_rn((float)num, d);
+    return q + __fdiv_rn((float)fma(-(double)q, den, num), d);
+}
+
 // Step length and direction factor with their guards, and the exit test of the
-// inner iteration, the same in every thread.
+// inner iteration: thread 0's, the same in every block.
 struct Inner {
-    double rz, best = INFINITY;
+    double rz = 0.0, best = INFINITY;
     int since = 0;
-    __device__ float step(double den) const { return den > 0.0 && rz > 0.0 ? (float)(rz / den) : 0.f; }
-    // true when the iteration ends
-    __device__ bool done(double rz1, double rr, float &beta) {
-        if (!(rr == rr) || rr <= CG_INNER_TOL * CG_INNER_TOL) return true;
+    __device__ float step(double den) const { return den > 0.0 && rz > 0.0 ? quotient(rz, den) : 0.f; }
+    // the direction factor, and whether the iteration ends
+    __device__ float2 next(double rz1, double rr) {
+        if (!(rr == rr) || rr <= CG_INNER_TOL * CG_INNER_TOL) return make_float2(0.f, 1.f);
         if (rr < 0.25 * best) { best = rr; since = 0; }
-        else if (++since >= CG_WINDOW) return true;
-        beta = rz > 0.0 ? (float)(rz1 / rz) : 0.f;
+        else if (++since >= CG_WINDOW) return make_float2(0.f, 1.f);
+        const float beta = rz > 0.0 ? quotient(rz1, rz) : 0.f;
         rz = rz1;
-        return false;
+        return make_float2(beta, 0.f);
     }
 };
 
@@ -275,7 +347,7 @@ __global__ void __launch_bounds__(CSR_TPB, 2) cg1_csr(CgArgs a) {
             g, [&](int64_t j) { return (W ? (double)g.w[j] : 1.0) * a.X[g.col[j]]; },
             [&](int32_t u, double t) { a.R[u] = a.B[u] - (g.d[u] * a.X[u] - t); },
             [&](int64_t c, int32_t, bool, double t) { a.hsumd[c] = t; });
-        all_sync();
+        all_sync(a.clustered);
         each([&](int64_t i) {
             if (g.hc_n && g.hfirst[i] >= 0)
                 a.R[i] = a.B[i] - (g.d[i] * a.X[i] - heavy_sum<OFF64, double>(g, i, a.hsumd));
@@ -285,7 +357,6 @@ __global__ void __launch_bounds__(CSR_TPB, 2) cg1_csr(CgArgs a) {
     };
     auto inner = [&](double rn) -> int {
         Pair acc[1] = {{0.f, 0.f}};
-        double t1[1], t2[2];
         each([&](int64_t i) {
             const float rv = (float)(a.R[i] / rn), zv = g.dinv32[i] * rv;
             a.r[i] = rv;
@@ -293,10 +364,8 @@ __global__ void __launch_bounds__(CSR_TPB, 2) cg1_csr(CgArgs a) {
             a.zp[0][i] = make_float2(zv, 0.f);
             pair_fma(acc[0], rv, zv);
         });
-        grid_sums<1>(acc, t1, a.parts, flip);
         Inner s;
-        s.rz = t1[0];
-        float beta = 0.f;
+        float beta = grid_sums<1, float>(acc, a.parts, flip, a.clustered, [&](const double *t) { s.rz = t[0]; return 0.f; });
         int it = 0;
         while (it < a.max_inner) {
             const float2 *zi = a.zp[it & 1];
@@ -317,8 +386,7 @@ __global__ void __launch_bounds__(CSR_TPB, 2) cg1_csr(CgArgs a) {
                     if (start) pair_fma(pq[0], pu, a.d32[u] * pu);
                     pair_fma(pq[0], -pu, t);
                 });
-            grid_sums<1>(pq, t1, a.parts, flip);
-            const float al = s.step(t1[0]);
+            const float al = grid_sums<1, float>(pq, a.parts, flip, a.clustered, [&](const double *t) { return s.step(t[0]); });
             Pair z2[2] = {{0.f, 0.f}, {0.f, 0.f}};
             each([&](int64_t i) {
                 const float pi = dir(i);
@@ -331,12 +399,13 @@ __global__ void __launch_bounds__(CSR_TPB, 2) cg1_csr(CgArgs a) {
                 pair_fma(z2[0], rv, zv);
                 pair_fma(z2[1], rv, rv);
             });
-            grid_sums<2>(z2, t2, a.parts, flip);
+            const float2 nx = grid_sums<2, float2>(z2, a.parts, flip, a.clustered, [&](const double *t) { return s.next(t[0], t[1]); });
             ++it;
-            if (s.done(t2[0], t2[1], beta)) break;
+            beta = nx.x;
+            if (nx.y != 0.f) break;
         }
         each([&](int64_t i) { a.X[i] += rn * (double)a.e[i]; });
-        all_sync();
+        all_sync(a.clustered);
         return it;
     };
     refine(a, flip, resid, each, inner);
@@ -383,7 +452,6 @@ __global__ void __launch_bounds__(ELL_TPB, 1) cg1_ell(CgArgs a) {
     auto inner = [&](double rn) -> int {
         float e[RT], r[RT], p[RT], q[RT], d[RT];
         Pair acc[1] = {{0.f, 0.f}};
-        double t1[1], t2[2];
 #pragma unroll
         for (int i = 0; i < RT; ++i) {
             const int l = threadIdx.x + i * ELL_TPB;
@@ -393,15 +461,13 @@ __global__ void __launch_bounds__(ELL_TPB, 1) cg1_ell(CgArgs a) {
                 const int64_t u = row0 + l;
                 d[i] = a.d32[u];
                 r[i] = (float)(a.R[u] / rn);
-                const float zv = r[i] / d[i];
+                const float zv = r[i] * __fdividef(1.f, d[i]);
                 a.zp[0][u] = make_float2(zv, 0.f);
                 pair_fma(acc[0], r[i], zv);
             }
         }
-        grid_sums<1>(acc, t1, a.parts, flip);
         Inner s;
-        s.rz = t1[0];
-        float beta = 0.f;
+        float beta = grid_sums<1, float>(acc, a.parts, flip, a.clustered, [&](const double *t) { s.rz = t[0]; return 0.f; });
         int it = 0;
         while (it < a.max_inner) {
             const float2 *zi = a.zp[it & 1];
@@ -411,14 +477,13 @@ __global__ void __launch_bounds__(ELL_TPB, 1) cg1_ell(CgArgs a) {
             for (int i = 0; i < RT; ++i) {
                 const int l = threadIdx.x + i * ELL_TPB;
                 if (l < nrow) {
-                    p[i] = fmaf(beta, p[i], r[i] / d[i]);
+                    p[i] = fmaf(beta, p[i], r[i] * __fdividef(1.f, d[i]));
                     const float t = row_sum(l, 0.f, [&](int c) { const float2 v = zi[c]; return fmaf(beta, v.y, v.x); });
                     q[i] = d[i] * p[i] - t;
                     pair_fma(pq[0], p[i], q[i]);
                 }
             }
-            grid_sums<1>(pq, t1, a.parts, flip);
-            const float al = s.step(t1[0]);
+            const float al = grid_sums<1, float>(pq, a.parts, flip, a.clustered, [&](const double *t) { return s.step(t[0]); });
             Pair z2[2] = {{0.f, 0.f}, {0.f, 0.f}};
 #pragma unroll
             for (int i = 0; i < RT; ++i) {
@@ -426,22 +491,23 @@ __global__ void __launch_bounds__(ELL_TPB, 1) cg1_ell(CgArgs a) {
                 if (l < nrow) {
                     e[i] += al * p[i];
                     r[i] -= al * q[i];
-                    const float zv = r[i] / d[i];
+                    const float zv = r[i] * __fdividef(1.f, d[i]);
                     zo[row0 + l] = make_float2(zv, p[i]);
                     pair_fma(z2[0], r[i], zv);
                     pair_fma(z2[1], r[i], r[i]);
                 }
             }
-            grid_sums<2>(z2, t2, a.parts, flip);
+            const float2 nx = grid_sums<2, float2>(z2, a.parts, flip, a.clustered, [&](const double *t) { return s.next(t[0], t[1]); });
             ++it;
-            if (s.done(t2[0], t2[1], beta)) break;
+            beta = nx.x;
+            if (nx.y != 0.f) break;
         }
 #pragma unroll
         for (int i = 0; i < RT; ++i) {
             const int l = threadIdx.x + i * ELL_TPB;
             if (l < nrow) a.X[row0 + l] += rn * (double)e[i];
         }
-        all_sync();
+        all_sync(a.clustered);
         return it;
     };
     refine(a, flip, resid, each, inner);
@@ -473,7 +539,8 @@ rwc_status solve_one(rwc_graph *G, const double *B, double *X, double tol, int *
     int rt = 1;
     while (ell && (n + (int64_t)ELL_TPB * rt - 1) / ((int64_t)ELL_TPB * rt) > sms) rt = rt == 1 ? 2 : rt == 2 ? 4 : ELL_RMAX;
     int64_t blocks = ell ? (n + (int64_t)ELL_TPB * rt - 1) / ((int64_t)ELL_TPB * rt)
-                         : std::max<int64_t>(1, std::min<int64_t>(2 * sms, g.nnz / (4 * CSR_TPB)));
+                         : g.nnz <= 2048 ? 1 : g.nnz <= 65536 ? std::min<int64_t>(8, (g.nnz + 2047) / 2048)
+                         : std::min<int64_t>(2 * sms, g.nnz / (4 * CSR_TPB));
     const size_t rows_b = ell ? (size_t)((n + blocks - 1) / blocks) * g.ell_w * 4 : 0;
     const size_t smem = rows_b <= 200 * 1024 ? rows_b : 0;
     Buf buf(st);
@@ -507,12 +574,28 @@ rwc_status solve_one(rwc_graph *G, const double *B, double *X, double tol, int *
     degrees32<<<(unsigned)std::max<int64_t>(1, std::min<int64_t>(4 * sms, (n + 255) / 256)), 256, 0, st>>>(n, g.d, d32, X);
     RWC_CUDA_TRY(cudaGetLastError());
     void *args[] = {&a};
+    // up to eight blocks are one cluster
+    a.clustered = blocks > 1 && blocks <= 8;
     auto launch = [&](auto kern, int tpb, size_t sm, int64_t nb) -> cudaError_t {
         if (sm > 48 * 1024) {
             const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(200 * 1024));
             if (e != cudaSuccess) return e;
         }
         if (nb == 1) return cudaLaunchKernel((const void *)kern, dim3(1), dim3(tpb), args, sm, st);
+        if (nb <= 8) {
+            cudaLaunchConfig_t cfg{};
+            cfg.gridDim = dim3((unsigned)nb);
+            cfg.blockDim = dim3(tpb);
+            cfg.dynamicSmemBytes = sm;
+            cfg.stream = st;
+            cudaLaunchAttribute at[1];
+            at[0].id = cudaLaunchAttributeClusterDimension;
+            at[0].val.clusterDim.x = (unsigned)nb;
+            at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+            cfg.attrs = at;
+            cfg.numAttrs = 1;
+            return cudaLaunchKernelExC(&cfg, (const void *)kern, args);
+        }
         return cudaLaunchCooperativeKernel((const void *)kern, dim3((unsigned)nb), dim3(tpb), args, sm, st);
     };
     auto csr = [&](int64_t nb) -> cudaError_t {
@@ -528,6 +611,7 @@ rwc_status solve_one(rwc_graph *G, const double *B, double *X, double tol, int *
     if (e != cudaSuccess && blocks > 1) {
         // a device that refuses the cooperative launch: one block, no grid barrier
         (void)cudaGetLastError();
+        a.clustered = false;
         e = csr(1);
     }
     RWC_CUDA_TRY(e);
