@@ -62,51 +62,66 @@ __device__ __forceinline__ void all_sync(bool clustered) {
     else __syncthreads();
 }
 
-// Fixed-order sums over the grid of K values per thread: a shuffle tree in
-// every warp, the warps of a block in order, the blocks in order.  Thread 0 of
-// every block passes them to post(sums), which gets the same bits in every
-// block and returns what all threads get: scalar FP64 work (a division is a
-// dozen instructions of 16 cycles each) is done once per block, not once per
-// warp.  `flip` alternates the blocks' slots, so that a block can write its next
-// sums while another still reads these.
+// a + b over the lanes of a warp by a shuffle tree, the same bits in every lane.
+__device__ __forceinline__ double warp_tree(double a) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
+    return a;
+}
+template <int K>
+__device__ __forceinline__ void warp_tree(Pair (&v)[K]) {
+    const int lane = threadIdx.x & 31;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+        for (int k = 0; k < K; ++k) {
+            const float s2 = __shfl_xor_sync(0xffffffffu, v[k].s, o), c2 = __shfl_xor_sync(0xffffffffu, v[k].c, o);
+            // both partners add the same pair in the same order
+            Pair lo = (lane & o) ? Pair{s2, c2} : v[k];
+            const Pair hi = (lane & o) ? v[k] : Pair{s2, c2};
+            pair_add(lo, hi.s, hi.c);
+            v[k] = lo;
+        }
+}
+template <int K>
+__device__ __forceinline__ void warp_tree(double (&v)[K]) {
+#pragma unroll
+    for (int k = 0; k < K; ++k) v[k] = warp_tree(v[k]);
+}
+__device__ __forceinline__ Pair load_part(const Pair *p) {
+    const float2 v = __ldcg(reinterpret_cast<const float2 *>(p));
+    return {v.x, v.y};
+}
+__device__ __forceinline__ double load_part(const double *p) { return __ldcg(p); }
+__device__ __forceinline__ void add_part(Pair &a, const Pair &b) { pair_add(a, b.s, b.c); }
+__device__ __forceinline__ void add_part(double &a, double b) { a += b; }
+
+// Fixed-order sums over the grid of K values per thread (FP64, or pairs of
+// floats on the iteration's path: an FP64 addition costs ten times a pair's
+// there): a shuffle tree in every warp, the warps of a block, then the blocks.
+// Thread 0 of every block passes them to post(sums), which gets the same bits in
+// every block and returns what all threads get.  `flip` alternates the blocks'
+// slots, so that a block can write its next sums while another still reads
+// these.
 template <int K, class Out, class T, class Post>
-__device__ Out grid_sums(const T (&v)[K], double *parts, int &flip, bool clustered, Post post) {
-    __shared__ double ws[K][32];
+__device__ Out grid_sums(T (&v)[K], double *parts, int &flip, bool clustered, Post post) {
+    static_assert(sizeof(T) == 8, "a slot");
+    __shared__ T ws[K][32];
     __shared__ Out bc;
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
     const int nb = gridDim.x;
-    double *slot = parts + (size_t)flip * 2 * nb;
+    T *slot = reinterpret_cast<T *>(parts) + (size_t)flip * 2 * nb;
     flip ^= 1;
+    warp_tree(v);
+    if (lane == 0)
 #pragma unroll
-    for (int k = 0; k < K; ++k) {
-        if constexpr (std::is_same<T, Pair>::value) {
-            Pair a = v[k];
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) {
-                const float s2 = __shfl_xor_sync(0xffffffffu, a.s, o), c2 = __shfl_xor_sync(0xffffffffu, a.c, o);
-                // both partners add the same pair in the same order
-                Pair lo = (lane & o) ? Pair{s2, c2} : a;
-                const Pair hi = (lane & o) ? a : Pair{s2, c2};
-                pair_add(lo, hi.s, hi.c);
-                a = lo;
-            }
-            if (lane == 0) ws[k][wid] = (double)a.s + (double)a.c;
-        } else {
-            double a = v[k];
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
-            if (lane == 0) ws[k][wid] = a;
-        }
-    }
+        for (int k = 0; k < K; ++k) ws[k][wid] = v[k];
     __syncthreads();
-    double t[K];
+    T t[K];
     if (wid == 0) {
 #pragma unroll
-        for (int k = 0; k < K; ++k) t[k] = lane < nw ? ws[k][lane] : 0.0;
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1)
-#pragma unroll
-            for (int k = 0; k < K; ++k) t[k] += __shfl_xor_sync(0xffffffffu, t[k], o);
+        for (int k = 0; k < K; ++k) t[k] = lane < nw ? ws[k][lane] : T{};
+        warp_tree(t);
         if (nb > 1 && lane == 0)
 #pragma unroll
             for (int k = 0; k < K; ++k) slot[(size_t)k * nb + blockIdx.x] = t[k];
@@ -115,14 +130,11 @@ __device__ Out grid_sums(const T (&v)[K], double *parts, int &flip, bool cluster
         blocks_sync(clustered);
         if (wid == 0) {
 #pragma unroll
-            for (int k = 0; k < K; ++k) t[k] = 0.0;
+            for (int k = 0; k < K; ++k) t[k] = T{};
             for (int i = lane; i < nb; i += 32)
 #pragma unroll
-                for (int k = 0; k < K; ++k) t[k] += __ldcg(slot + (size_t)k * nb + i);
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1)
-#pragma unroll
-                for (int k = 0; k < K; ++k) t[k] += __shfl_xor_sync(0xffffffffu, t[k], o);
+                for (int k = 0; k < K; ++k) add_part(t[k], load_part(slot + (size_t)k * nb + i));
+            warp_tree(t);
         }
     }
     if (threadIdx.x == 0) bc = post(t);
@@ -230,6 +242,82 @@ __device__ __forceinline__ bool few_rows(const DevGraph &g, Term term, F f) {
     }
     return true;
 }
+// A warp's units of rows held in registers for the whole solve (small systems):
+// row, first arc and weight of every lane.  An iteration then waits for one
+// gather instead of a chain of four loads per unit, which the barrier's acquire
+// sends to L2 each time (BA 2000: 13500 -> 4700 cycles per product).
+constexpr int RES_UNITS = 4, RES_TPB = 1024;
+template <bool OFF64, bool W>
+struct ResidentRows {
+    int32_t u[RES_UNITS], c[RES_UNITS];
+    float w[RES_UNITS];
+    int32_t more[RES_UNITS];               // arcs of the lane beyond the first, 32 apart
+    int vw[RES_UNITS];
+    __device__ void load(const DevGraph &g) {
+        const int64_t warps = (int64_t)gridDim.x * blockDim.x / 32;
+        const int64_t w0 = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) / 32;
+        const int lane = threadIdx.x & 31;
+#pragma unroll
+        for (int q = 0; q < RES_UNITS; ++q) {
+            int64_t unit = w0 + q * warps;
+            u[q] = c[q] = -1;
+            w[q] = 0.f;
+            more[q] = 0;
+            vw[q] = 0;
+            for (int b = 0; b < 5; ++b) {
+                const int rows = 16 >> b, v = 2 << b;
+                const int64_t nrows = g.bin_off[b + 1] - g.bin_off[b], nu = (nrows + rows - 1) / rows;
+                if (unit < nu) {
+                    vw[q] = v;
+                    const int64_t i = unit * rows + lane / v;
+                    if (i < nrows) {
+                        u[q] = g.bin_rows[g.bin_off[b] + i];
+                        int64_t rb, re;
+                        row_of<OFF64>(g, u[q], rb, re);
+                        const int64_t j = rb + (lane & (v - 1));
+                        if (j < re) {
+                            c[q] = g.col[j];
+                            w[q] = W ? g.w[j] : 1.f;
+                            more[q] = (int32_t)((re - 1 - j) / 32);
+                        }
+                    }
+                    break;
+                }
+                unit -= nu;
+            }
+        }
+    }
+    // f(row, sum over its arcs of weight times dir(head))
+    template <class Dir, class F>
+    __device__ __forceinline__ void rows(const DevGraph &g, Dir dir, F f) const {
+        const int lane = threadIdx.x & 31;
+        float s[RES_UNITS];
+#pragma unroll
+        for (int q = 0; q < RES_UNITS; ++q) s[q] = c[q] >= 0 ? w[q] * dir(c[q]) : 0.f;
+#pragma unroll
+        for (int q = 0; q < RES_UNITS; ++q) {
+            if (vw[q] == 32) {
+                int64_t rb = 0, re;
+                if (more[q]) row_of<OFF64>(g, u[q], rb, re);
+                for (int k = 1; k <= more[q]; ++k) {
+                    const int64_t j = rb + lane + 32 * (int64_t)k;
+                    s[q] += (W ? g.w[j] : 1.f) * dir(g.col[j]);
+                }
+                __syncwarp();
+            }
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1)
+                if (o < vw[q]) s[q] += __shfl_xor_sync(0xffffffffu, s[q], o);
+            if (u[q] >= 0 && (lane & (vw[q] - 1)) == 0) f(u[q], s[q]);
+        }
+    }
+};
+// Units of a graph's rows.
+inline int64_t row_units(const DevGraph &g) {
+    int64_t t = 0;
+    for (int b = 0; b < 5; ++b) t += (g.bin_off[b + 1] - g.bin_off[b] + (16 >> b) - 1) / (16 >> b);
+    return t;
+}
 // all rows of at most HEAVY_DEG arcs through f, the heavy rows' chunks through
 // h(chunk, row, first chunk of its row, sum)
 template <bool OFF64, class T, class Term, class F, class H>
@@ -310,32 +398,43 @@ __device__ void refine(const CgArgs &a, int &flip, Resid resid, Each each, Inner
     }
 }
 
-// num / den rounded to float: a float quotient corrected by its FP64 residual
-// (the FP64 division is a long dependent chain on the iteration's path).
-__device__ __forceinline__ float quotient(double num, double den) {
-    const float d = (float)den, q = __fdiv_rn((float)num, d);
-    return q + __fdiv_rn((float)fma(-(double)q, den, num), d);
+// num / den to float precision: a float quotient corrected by its residual.
+__device__ __forceinline__ float quotient(Pair num, Pair den) {
+    const float q = __fdiv_rn(num.s, den.s);
+    const float r = __fadd_rn(__fmaf_rn(-q, den.s, num.s), __fmaf_rn(-q, den.c, num.c));
+    return __fadd_rn(q, __fdividef(r, den.s));
+}
+// the pair's value as its leading float, the rest in c
+__device__ __forceinline__ Pair normal(Pair a) {
+    const float t = __fadd_rn(a.s, a.c);
+    return {t, __fsub_rn(a.c, __fsub_rn(t, a.s))};
 }
 
 // Step length and direction factor with their guards, and the exit test of the
 // inner iteration: thread 0's, the same in every block.
 struct Inner {
-    double rz = 0.0, best = INFINITY;
+    Pair rz = {0.f, 0.f};
+    float best = INFINITY;
     int since = 0;
-    __device__ float step(double den) const { return den > 0.0 && rz > 0.0 ? quotient(rz, den) : 0.f; }
+    __device__ float step(Pair den) const {
+        den = normal(den);
+        return den.s > 0.f && rz.s > 0.f ? quotient(rz, den) : 0.f;
+    }
     // the direction factor, and whether the iteration ends
-    __device__ float2 next(double rz1, double rr) {
-        if (!(rr == rr) || rr <= CG_INNER_TOL * CG_INNER_TOL) return make_float2(0.f, 1.f);
-        if (rr < 0.25 * best) { best = rr; since = 0; }
+    __device__ float2 next(Pair rz1, Pair rr2) {
+        rz1 = normal(rz1);
+        const float rr = normal(rr2).s;
+        if (!(rr == rr) || rr <= (float)(CG_INNER_TOL * CG_INNER_TOL)) return make_float2(0.f, 1.f);
+        if (rr < 0.25f * best) { best = rr; since = 0; }
         else if (++since >= CG_WINDOW) return make_float2(0.f, 1.f);
-        const float beta = rz > 0.0 ? quotient(rz1, rz) : 0.f;
+        const float beta = rz.s > 0.f ? quotient(rz1, rz) : 0.f;
         rz = rz1;
         return make_float2(beta, 0.f);
     }
 };
 
-template <bool OFF64, bool W>
-__global__ void __launch_bounds__(CSR_TPB, 2) cg1_csr(CgArgs a) {
+template <bool OFF64, bool W, bool RES>
+__global__ void __launch_bounds__(RES ? RES_TPB : CSR_TPB, RES ? 1 : 2) cg1_csr(CgArgs a) {
     const DevGraph &g = a.g;
     const int64_t n = g.n;
     const int64_t tid = blockIdx.x * (int64_t)blockDim.x + threadIdx.x, nthr = (int64_t)gridDim.x * blockDim.x;
@@ -355,6 +454,8 @@ __global__ void __launch_bounds__(CSR_TPB, 2) cg1_csr(CgArgs a) {
         });
         return s;
     };
+    ResidentRows<OFF64, W> held;
+    if constexpr (RES) held.load(g);
     auto inner = [&](double rn) -> int {
         Pair acc[1] = {{0.f, 0.f}};
         each([&](int64_t i) {
@@ -365,7 +466,7 @@ __global__ void __launch_bounds__(CSR_TPB, 2) cg1_csr(CgArgs a) {
             pair_fma(acc[0], rv, zv);
         });
         Inner s;
-        float beta = grid_sums<1, float>(acc, a.parts, flip, a.clustered, [&](const double *t) { s.rz = t[0]; return 0.f; });
+        float beta = grid_sums<1, float>(acc, a.parts, flip, a.clustered, [&](const Pair *t) { s.rz = normal(t[0]); return 0.f; });
         int it = 0;
         while (it < a.max_inner) {
             const float2 *zi = a.zp[it & 1];
@@ -373,20 +474,21 @@ __global__ void __launch_bounds__(CSR_TPB, 2) cg1_csr(CgArgs a) {
             // q = L p, <p, q>; a heavy row's share of <p, q> comes from its chunks
             Pair pq[1] = {{0.f, 0.f}};
             auto dir = [&](int64_t v) { const float2 t = zi[v]; return fmaf(beta, t.y, t.x); };
-            all_rows<OFF64, float>(
-                g, [&](int64_t j) { return (W ? g.w[j] : 1.f) * dir(g.col[j]); },
-                [&](int32_t u, float t) {
-                    const float pu = dir(u), qu = a.d32[u] * pu - t;
-                    a.q[u] = qu;
-                    pair_fma(pq[0], pu, qu);
-                },
-                [&](int64_t c, int32_t u, bool start, float t) {
-                    a.hsum[c] = t;
-                    const float pu = dir(u);
-                    if (start) pair_fma(pq[0], pu, a.d32[u] * pu);
-                    pair_fma(pq[0], -pu, t);
-                });
-            const float al = grid_sums<1, float>(pq, a.parts, flip, a.clustered, [&](const double *t) { return s.step(t[0]); });
+            auto row = [&](int32_t u, float t) {
+                const float pu = dir(u), qu = a.d32[u] * pu - t;
+                a.q[u] = qu;
+                pair_fma(pq[0], pu, qu);
+            };
+            auto chunk = [&](int64_t c, int32_t u, bool start, float t) {
+                a.hsum[c] = t;
+                const float pu = dir(u);
+                if (start) pair_fma(pq[0], pu, a.d32[u] * pu);
+                pair_fma(pq[0], -pu, t);
+            };
+            auto term = [&](int64_t j) { return (W ? g.w[j] : 1.f) * dir(g.col[j]); };
+            if constexpr (RES) held.rows(g, dir, row);
+            else all_rows<OFF64, float>(g, term, row, chunk);
+            const float al = grid_sums<1, float>(pq, a.parts, flip, a.clustered, [&](const Pair *t) { return s.step(t[0]); });
             Pair z2[2] = {{0.f, 0.f}, {0.f, 0.f}};
             each([&](int64_t i) {
                 const float pi = dir(i);
@@ -399,7 +501,7 @@ __global__ void __launch_bounds__(CSR_TPB, 2) cg1_csr(CgArgs a) {
                 pair_fma(z2[0], rv, zv);
                 pair_fma(z2[1], rv, rv);
             });
-            const float2 nx = grid_sums<2, float2>(z2, a.parts, flip, a.clustered, [&](const double *t) { return s.next(t[0], t[1]); });
+            const float2 nx = grid_sums<2, float2>(z2, a.parts, flip, a.clustered, [&](const Pair *t) { return s.next(t[0], t[1]); });
             ++it;
             beta = nx.x;
             if (nx.y != 0.f) break;
@@ -467,7 +569,7 @@ __global__ void __launch_bounds__(ELL_TPB, 1) cg1_ell(CgArgs a) {
             }
         }
         Inner s;
-        float beta = grid_sums<1, float>(acc, a.parts, flip, a.clustered, [&](const double *t) { s.rz = t[0]; return 0.f; });
+        float beta = grid_sums<1, float>(acc, a.parts, flip, a.clustered, [&](const Pair *t) { s.rz = normal(t[0]); return 0.f; });
         int it = 0;
         while (it < a.max_inner) {
             const float2 *zi = a.zp[it & 1];
@@ -483,7 +585,7 @@ __global__ void __launch_bounds__(ELL_TPB, 1) cg1_ell(CgArgs a) {
                     pair_fma(pq[0], p[i], q[i]);
                 }
             }
-            const float al = grid_sums<1, float>(pq, a.parts, flip, a.clustered, [&](const double *t) { return s.step(t[0]); });
+            const float al = grid_sums<1, float>(pq, a.parts, flip, a.clustered, [&](const Pair *t) { return s.step(t[0]); });
             Pair z2[2] = {{0.f, 0.f}, {0.f, 0.f}};
 #pragma unroll
             for (int i = 0; i < RT; ++i) {
@@ -497,7 +599,7 @@ __global__ void __launch_bounds__(ELL_TPB, 1) cg1_ell(CgArgs a) {
                     pair_fma(z2[1], r[i], r[i]);
                 }
             }
-            const float2 nx = grid_sums<2, float2>(z2, a.parts, flip, a.clustered, [&](const double *t) { return s.next(t[0], t[1]); });
+            const float2 nx = grid_sums<2, float2>(z2, a.parts, flip, a.clustered, [&](const Pair *t) { return s.next(t[0], t[1]); });
             ++it;
             beta = nx.x;
             if (nx.y != 0.f) break;
@@ -538,8 +640,13 @@ rwc_status solve_one(rwc_graph *G, const double *B, double *X, double tol, int *
     const bool ell = g.ell && n <= (int64_t)sms * ELL_TPB * ELL_RMAX;
     int rt = 1;
     while (ell && (n + (int64_t)ELL_TPB * rt - 1) / ((int64_t)ELL_TPB * rt) > sms) rt = rt == 1 ? 2 : rt == 2 ? 4 : ELL_RMAX;
+    // small systems: rows in registers, up to a cluster of blocks (the smallest
+    // take one block of half the threads: ER 100 178 against 215 us)
+    const int64_t units = row_units(g);
+    const bool held = !ell && g.hc_n == 0 && units > 64 && units <= 8 * (RES_TPB / 32) * RES_UNITS;
     int64_t blocks = ell ? (n + (int64_t)ELL_TPB * rt - 1) / ((int64_t)ELL_TPB * rt)
-                         : g.nnz <= 2048 ? 1 : g.nnz <= 65536 ? std::min<int64_t>(8, (g.nnz + 2047) / 2048)
+                         : held ? (units <= RES_TPB / 32 * RES_UNITS ? 1 : std::min<int64_t>(8, (units + 63) / 64))
+                         : units <= 64 ? 1
                          : std::min<int64_t>(2 * sms, g.nnz / (4 * CSR_TPB));
     const size_t rows_b = ell ? (size_t)((n + blocks - 1) / blocks) * g.ell_w * 4 : 0;
     const size_t smem = rows_b <= 200 * 1024 ? rows_b : 0;
@@ -598,9 +705,13 @@ rwc_status solve_one(rwc_graph *G, const double *B, double *X, double tol, int *
         }
         return cudaLaunchCooperativeKernel((const void *)kern, dim3((unsigned)nb), dim3(tpb), args, sm, st);
     };
+    auto csr_of = [&](auto res, int tpb, int64_t nb) -> cudaError_t {
+        constexpr bool RES = decltype(res)::value;
+        if (g.off64) return g.weighted ? launch(cg1_csr<true, true, RES>, tpb, 0, nb) : launch(cg1_csr<true, false, RES>, tpb, 0, nb);
+        return g.weighted ? launch(cg1_csr<false, true, RES>, tpb, 0, nb) : launch(cg1_csr<false, false, RES>, tpb, 0, nb);
+    };
     auto csr = [&](int64_t nb) -> cudaError_t {
-        if (g.off64) return g.weighted ? launch(cg1_csr<true, true>, CSR_TPB, 0, nb) : launch(cg1_csr<true, false>, CSR_TPB, 0, nb);
-        return g.weighted ? launch(cg1_csr<false, true>, CSR_TPB, 0, nb) : launch(cg1_csr<false, false>, CSR_TPB, 0, nb);
+        return held ? csr_of(std::true_type{}, RES_TPB, nb) : csr_of(std::false_type{}, CSR_TPB, nb);
     };
     auto inl = [&](auto ew) -> cudaError_t {
         constexpr int EW = decltype(ew)::value;
@@ -612,7 +723,7 @@ rwc_status solve_one(rwc_graph *G, const double *B, double *X, double tol, int *
         // a device that refuses the cooperative launch: one block, no grid barrier
         (void)cudaGetLastError();
         a.clustered = false;
-        e = csr(1);
+        e = csr_of(std::false_type{}, CSR_TPB, 1);
     }
     RWC_CUDA_TRY(e);
     double h[3];

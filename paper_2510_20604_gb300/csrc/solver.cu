@@ -44,35 +44,49 @@ __device__ __forceinline__ void rowb(const DevGraph &g, int64_t u, int64_t &b, i
 }
 
 // The threads of a block as quads of columns x rows: quad q (of this block's
-// tile), row slot rs, and the block's range of rows [u0, u1).
+// tile) and row slot rs; the slots of all blocks take rows u0, u0 + step, ... in
+// turn, so that neighbouring ids, which often are the hubs, fall to different
+// blocks.
 struct Tile {
     int q, rs, slots;
-    int64_t u0, u1;
+    int64_t u0, step;
     bool on;
-    __device__ Tile(int64_t n, int k4, int qt)
+    __device__ Tile(int k4, int qt)
         : q(blockIdx.y * qt + threadIdx.x % qt), rs(threadIdx.x / qt), slots(blockDim.x / qt) {
-        const int64_t rpb = (n + gridDim.x - 1) / gridDim.x;
-        u0 = blockIdx.x * rpb;
-        u1 = u0 + rpb < n ? u0 + rpb : n;
+        u0 = (int64_t)blockIdx.x * slots + rs;
+        step = (int64_t)gridDim.x * slots;
         on = q < k4;
     }
 };
 
-// parts[column][block] = the sums of the block's row slots in slot order.
+// parts[column][block] = the sums over the block's row slots by a fixed tree, in
+// pairs (a serial FP64 sum of 85 slots took longer than the rest of a small
+// system's pass).
 __device__ __forceinline__ void quad_parts(const Tile &t, const Pair (&a)[4], int qt, double *parts) {
-    __shared__ double sh[4 * TPB];
+    __shared__ Pair sh[4][TPB];
     __syncthreads();
 #pragma unroll
-    for (int i = 0; i < 4; ++i) sh[i * blockDim.x + threadIdx.x] = (double)a[i].s + (double)a[i].c;
+    for (int i = 0; i < 4; ++i) sh[i][threadIdx.x] = a[i];
+    int h = 1;
+    while (h < t.slots) h *= 2;
+    for (h /= 2; h > 0; h /= 2) {
+        __syncthreads();
+        if (t.rs < h && t.rs + h < t.slots)
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                Pair x = sh[i][threadIdx.x];
+                const Pair y = sh[i][threadIdx.x + h * qt];
+                pair_add(x, y.s, y.c);
+                sh[i][threadIdx.x] = x;
+            }
+    }
     __syncthreads();
-    if (t.rs == 0 && t.on) {
+    if (t.rs == 0 && t.on)
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
-            double s = 0.0;
-            for (int r = 0; r < t.slots; ++r) s += sh[i * blockDim.x + r * qt + threadIdx.x];
-            parts[(int64_t)(4 * t.q + i) * gridDim.x + blockIdx.x] = s;
+            const Pair x = sh[i][threadIdx.x];
+            parts[(int64_t)(4 * t.q + i) * gridDim.x + blockIdx.x] = (double)x.s + (double)x.c;
         }
-    }
 }
 
 __device__ __forceinline__ void fma4(float4 &s, float w, const float4 &v) {
@@ -86,12 +100,13 @@ __device__ __forceinline__ void dot4(Pair (&a)[4], const float4 &x, const float4
 template <bool OFF64, bool W>
 __global__ void __launch_bounds__(TPB) bcg_product(DevGraph g, int k4, int qt, const float4 *__restrict__ P,
                                                    float4 *__restrict__ Q, double *parts) {
-    const Tile t(g.n, k4, qt);
+    const Tile t(k4, qt);
     Pair a[4] = {};
-    if (t.on && t.rs < t.slots)
-        for (int64_t u = t.u0 + t.rs; u < t.u1; u += t.slots) {
+    if (t.on)
+        for (int64_t u = t.u0; u < g.n; u += t.step) {
             int64_t b, e;
             rowb<OFF64>(g, u, b, e);
+            if (g.hc_n && e - b > HEAVY_DEG) continue;
             float4 s0 = {}, s1 = {};
             int64_t j = b;
             for (; j + 4 <= e; j += 4) {
@@ -112,6 +127,29 @@ __global__ void __launch_bounds__(TPB) bcg_product(DevGraph g, int k4, int qt, c
             Q[u * k4 + t.q] = q;
             dot4(a, p, q);
         }
+    // rows of more than HEAVY_DEG arcs: a block's slots share the arcs of one
+    __shared__ float4 hs[TPB];
+    for (int64_t c = blockIdx.x; c < g.hc_n; c += gridDim.x) {
+        const int64_t u = g.hc_row[c];
+        int64_t b, e;
+        rowb<OFF64>(g, u, b, e);
+        if (g.hc_beg[c] != b) continue;          // the row's first chunk only
+        float4 s = {};
+        if (t.on)
+#pragma unroll 4
+            for (int64_t j = b + t.rs; j < e; j += t.slots) fma4(s, W ? g.w[j] : 1.f, P[(int64_t)g.col[j] * k4 + t.q]);
+        __syncthreads();
+        hs[threadIdx.x] = s;
+        __syncthreads();
+        if (t.rs == 0 && t.on) {
+            for (int r = 1; r < t.slots; ++r) fma4(s, 1.f, hs[r * qt + threadIdx.x]);
+            const float d = (float)g.d[u];
+            const float4 p = P[u * k4 + t.q];
+            const float4 q = {d * p.x - s.x, d * p.y - s.y, d * p.z - s.z, d * p.w - s.w};
+            Q[u * k4 + t.q] = q;
+            dot4(a, p, q);
+        }
+    }
     quad_parts(t, a, qt, parts);
 }
 
@@ -124,12 +162,12 @@ __device__ __forceinline__ float step_of(double num, double den) {
 __global__ void __launch_bounds__(TPB) bcg_residual(int64_t n, int k4, int qt, const double *rz, const double *pq,
                                                     const float *dinv, const float4 *__restrict__ Q,
                                                     float4 *__restrict__ r, double *parts, double *parts2) {
-    const Tile t(n, k4, qt);
+    const Tile t(k4, qt);
     Pair a[4] = {}, b[4] = {};
-    if (t.on && t.rs < t.slots) {
+    if (t.on) {
         const double *z = rz + 4 * t.q, *d = pq + 4 * t.q;
         const float4 al = {step_of(z[0], d[0]), step_of(z[1], d[1]), step_of(z[2], d[2]), step_of(z[3], d[3])};
-        for (int64_t u = t.u0 + t.rs; u < t.u1; u += t.slots) {
+        for (int64_t u = t.u0; u < n; u += t.step) {
             const int64_t i = u * k4 + t.q;
             const float4 q = Q[i];
             float4 v = r[i];
@@ -149,8 +187,8 @@ __global__ void __launch_bounds__(TPB) bcg_direction(int64_t n, int k4, int qt, 
                                                      const double *rz1, const float *dinv,
                                                      const float4 *__restrict__ r, float4 *__restrict__ e,
                                                      float4 *__restrict__ p) {
-    const Tile t(n, k4, qt);
-    if (!t.on || t.rs >= t.slots) return;
+    const Tile t(k4, qt);
+    if (!t.on) return;
     const double *z = rz0 + 4 * t.q, *d = pq + 4 * t.q, *z1 = rz1 + 4 * t.q;
     float al[4], be[4];
 #pragma unroll
@@ -158,7 +196,7 @@ __global__ void __launch_bounds__(TPB) bcg_direction(int64_t n, int k4, int qt, 
         al[i] = step_of(z[i], d[i]);
         be[i] = z[i] > 0.0 ? (float)(z1[i] / z[i]) : 0.f;
     }
-    for (int64_t u = t.u0 + t.rs; u < t.u1; u += t.slots) {
+    for (int64_t u = t.u0; u < n; u += t.step) {
         const int64_t i = u * k4 + t.q;
         const float di = dinv[u];
         const float4 v = r[i];
@@ -176,13 +214,13 @@ __global__ void __launch_bounds__(TPB) bcg_direction(int64_t n, int k4, int qt, 
 __global__ void __launch_bounds__(TPB) bcg_start(int64_t n, int k, int k4, int qt, const double *__restrict__ R,
                                                  const double *rnrm2, const float *dinv, float4 *__restrict__ r,
                                                  float4 *__restrict__ e, float4 *__restrict__ p, double *parts) {
-    const Tile t(n, k4, qt);
+    const Tile t(k4, qt);
     Pair a[4] = {};
-    if (t.on && t.rs < t.slots) {
+    if (t.on) {
         double nr[4];
 #pragma unroll
         for (int i = 0; i < 4; ++i) nr[i] = 4 * t.q + i < k ? sqrt(rnrm2[4 * t.q + i]) : 0.0;
-        for (int64_t u = t.u0 + t.rs; u < t.u1; u += t.slots) {
+        for (int64_t u = t.u0; u < n; u += t.step) {
             float v[4];
 #pragma unroll
             for (int i = 0; i < 4; ++i) v[i] = nr[i] > 0.0 ? (float)(R[u * k + 4 * t.q + i] / nr[i]) : 0.f;
@@ -380,7 +418,8 @@ rwc_status solve_nodemajor(rwc_graph *G, int k, const double *B, double *X, doub
         bcg_start<<<grid, threads, 0, st>>>(n, k, k4, qt, R, rn2, g.dinv32, r, e, p, pa);
         sum_cols<<<dim3((unsigned)kp, 1), 128, 0, st>>>(pa, nullptr, (int)nb, rz[0], nullptr);
         int it = 0;
-        const int check = 4;   // iterations between looks at the residual
+        // iterations between looks at the residual (a host round trip each)
+        const int check = (int64_t)n * kp >= 1000000 ? 4 : 8;
         bool inner_done = false;
         double best = INFINITY;
         int since_best = 0;
