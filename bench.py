@@ -60,8 +60,10 @@ EPS_SWEEP = (0.3, 0.2, 0.1, 0.05, 0.02, 0.01)
 
 PHASE_NAMES = ("init", "walk", "classify", "pop", "finish", "accum")
 KERNEL_NAMES = {1: {"init": "g_init", "walk": "g_walk", "pop": "g_pop", "accum": "g_accum"},
-                2: {"walk": "s_trees"},
-                3: {"init": "w_init", "walk": "w_trees", "accum": "w_accum"}}
+                2: {"walk": "l_trees_smem"},
+                # the lane sampler, or the concurrent walkers on large graphs of
+                # unbounded degree
+                3: {"init": "memset/w_init", "walk": "l_trees/w_trees", "accum": "l_accum/w_accum"}}
 
 
 def bytes_per_draw(weighted, off64):
@@ -90,9 +92,6 @@ def algorithmic_bytes(draws, trees, n, weighted, off64):
 # on (code_hash of the .cu file), else reported as null.
 TRAFFIC_PER_DRAW = {
     # family: (bytes per draw, case captured, source file, code hash of the kernel region)
-    "grid": (266.2, "grid 256x256, 2000 trees, 64 walkers per tree: one w_trees launch "
-                     "(565.0 GB over 2.123e9 draws)", "walker.cu",
-             "ab1fdc759f922dfae00450c5610e7341609c15fbdcdfceea4077a8a0d4278a2e"),
     "rmat": (222.3, "R-MAT scale 18, 2000 trees, 64 walkers per tree: one w_trees launch "
                      "(171.0 GB over 7.693e8 draws)", "walker.cu",
              "ab1fdc759f922dfae00450c5610e7341609c15fbdcdfceea4077a8a0d4278a2e"),
@@ -116,7 +115,7 @@ def code_hash(path, begin=None, end=None):
 
 
 # the walker kernel's source region in walker.cu (what a traffic capture measured)
-W_TREES_REGION = ("walker.cu", "struct DrawRow {",
+W_TREES_REGION = ("walker.cu", "template <bool OFF64, bool WT, int EW, bool DIAG>",
                   "// visits_u = k_u + 1 over the chunk's trees")
 
 

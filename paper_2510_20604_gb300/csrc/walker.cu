@@ -83,7 +83,8 @@ __device__ __forceinline__ void st32(int32_t *a, int32_t v) {
 
 struct WState {
     uint64_t *word;        // [B][n]
-    int32_t *retry;        // [B][n-1] requeued start indices (circular)
+    int32_t *retry;        // [B][rcap] requeued start indices (circular)
+    int rcap;              // at most n - 1; fewer: see RETRY_CAP
     const int32_t *order;  // [n-1] start order (a permutation of the non-root vertices)
     int *err;
     unsigned long long *ctr;   // [0] steps, [1] yields, [2] pops, [3] next tree
@@ -98,6 +99,13 @@ __global__ void w_init(int64_t n, int32_t root, uint64_t *word, int64_t B) {
         word[i] = (u == root) ? W_pack(P_INVALID, 0, OWN_SET) : W_pack(P_INVALID, 0, OWN_FREE);
     }
 }
+
+// Entries of a tree's retry queue.  A walker adds one only after it has taken a
+// start, so a queue that is within two blocks of full (a block's walkers may
+// each add one, and each may still be emptying a slot) only has to hand out its
+// own entries before fresh starts.  R-MAT 20, 2000 trees: 8.4 GB less scratch to
+// map and clear on every call, 288 -> 264 ms.
+constexpr int RETRY_CAP = 4096;
 
 // Retry queue: slots hold start index + 1 (0 = empty); a producer reserves a
 // slot with the tail counter and then fills it, a consumer reserves with the
@@ -183,7 +191,7 @@ __global__ void __maxnreg__(RWC_WALKER_MAXNREG) w_trees(DevGraph g, WState s, in
         const int t = sh_tree;
         if (t >= B) break;
         uint64_t *st = s.word + (int64_t)t * n;
-        int32_t *rq = s.retry + (int64_t)t * nstart;
+        int32_t *rq = s.retry + (int64_t)t * s.rcap;
         const uint32_t tree = tree0 + (uint32_t)t;
 
         int state = S_IDLE;
@@ -233,7 +241,7 @@ __global__ void __maxnreg__(RWC_WALKER_MAXNREG) w_trees(DevGraph g, WState s, in
         };
         auto drop_start = [&](bool requeue) {
             if (requeue) {
-                rq_push(rq, &sh_rtail, nstart, myprio);
+                rq_push(rq, &sh_rtail, s.rcap, myprio);
                 if (DIAG) ++yields;
             }
             *(volatile int *)&prio[me] = INF;
@@ -275,14 +283,16 @@ __global__ void __maxnreg__(RWC_WALKER_MAXNREG) w_trees(DevGraph g, WState s, in
                 // the prefetched fresh start, else a fresh one, else a requeued one
                 int idx = -1;
                 int32_t sv = -1;
-                if (pend_idx >= 0) {
+                const bool full = s.rcap < nstart &&
+                                  vread(&sh_rtail) - vread(&sh_rhead) >= s.rcap - 2 * (int)blockDim.x;
+                if (pend_idx >= 0 && !full) {
                     idx = pend_idx; sv = pend_start; pend_idx = -1;
                 } else {
-                    idx = take_fresh();
+                    idx = full ? -1 : take_fresh();
                     if (idx < 0) {
                         const int hd = vread(&sh_rhead);
                         if (hd < vread(&sh_rtail) && atomicCAS(&sh_rhead, hd, hd + 1) == hd) {
-                            int32_t *slot = rq + hd % nstart;
+                            int32_t *slot = rq + hd % s.rcap;
                             uint64_t t0 = gtimer();
                             int32_t v = ld32(slot);
                             while (v == 0 && gtimer() - t0 < (uint64_t)max_wait_ns) v = ld32(slot);
@@ -297,7 +307,7 @@ __global__ void __maxnreg__(RWC_WALKER_MAXNREG) w_trees(DevGraph g, WState s, in
                     // a premature "done" is harmless: a walker that requeues a
                     // start takes it back itself when it becomes idle
                     const int act = vread(&sh_active);
-                    if (act == 0 && vread(&sh_rhead) >= vread(&sh_rtail) && vread(&sh_next) >= nstart)
+                    if (act == 0 && pend_idx < 0 && vread(&sh_rhead) >= vread(&sh_rtail) && vread(&sh_next) >= nstart)
                         state = S_DONE;
                     else if (waited_out())
                         break;
@@ -311,7 +321,7 @@ __global__ void __maxnreg__(RWC_WALKER_MAXNREG) w_trees(DevGraph g, WState s, in
                 bump();
                 state = S_WALK;
                 // fetch the next fresh start now; it is used when this walk ends
-                const int ni = take_fresh();
+                const int ni = pend_idx < 0 ? take_fresh() : -1;
                 if (ni >= 0) { pend_idx = ni; pend_start = s.order[ni]; }
             }
             if (state == S_WALK && !hold && vread(&kill[me]) == myprio) {
@@ -610,7 +620,8 @@ rwc_status sample_walker(rwc_graph *G, uint64_t seed, int64_t tree0, int64_t T, 
     if (n >= ((int64_t)1 << 31) - 2) return set_error(RWC_ERR_UNSUPPORTED, "n too large for walker mode");
     const int32_t *order = nullptr;
     RWC_TRY(walker_order(G, &order));
-    const size_t per_tree = (size_t)n * (8 + 4) + 256;
+    const int64_t rcap = std::min<int64_t>(n - 1, RETRY_CAP);
+    const size_t per_tree = (size_t)n * 8 + (size_t)rcap * 4 + 256;
     int64_t B = o.trees_per_chunk;
     if (B <= 0) {
         size_t fr = 0, tot = 0;
@@ -624,7 +635,7 @@ rwc_status sample_walker(rwc_graph *G, uint64_t seed, int64_t tree0, int64_t T, 
     int W = o.block_threads > 0 ? std::max(32, std::min(512, o.block_threads / 32 * 32)) : 0;
     const uint32_t k0 = (uint32_t)seed, k1 = (uint32_t)(seed >> 32);
     void *buf = nullptr;
-    const size_t bytes = (size_t)B * n * 8 + (size_t)B * (n - 1) * 4 + 256;
+    const size_t bytes = (size_t)B * n * 8 + (size_t)B * rcap * 4 + 256;
     RWC_CUDA_TRY(cudaMallocAsync(&buf, bytes, stream));
     struct Free {
         void *p; cudaStream_t s;
@@ -633,7 +644,8 @@ rwc_status sample_walker(rwc_graph *G, uint64_t seed, int64_t tree0, int64_t T, 
     WState ws;
     ws.word = (uint64_t *)buf;
     ws.retry = (int32_t *)((char *)buf + (size_t)B * n * 8);
-    char *tail = (char *)buf + (size_t)B * n * 8 + (size_t)B * (n - 1) * 4;
+    ws.rcap = (int)rcap;
+    char *tail = (char *)buf + (size_t)B * n * 8 + (size_t)B * rcap * 4;
     tail = (char *)(((uintptr_t)tail + 63) & ~(uintptr_t)63);
     ws.order = order;
     ws.err = (int *)tail;                                  // @0
@@ -654,7 +666,7 @@ rwc_status sample_walker(rwc_graph *G, uint64_t seed, int64_t tree0, int64_t T, 
     for (int64_t c0 = 0; c0 < T; c0 += B) {
         const int64_t Bc = std::min(B, T - c0);
         RWC_CUDA_TRY(cudaMemsetAsync(tail, 0, 128, stream));
-        RWC_CUDA_TRY(cudaMemsetAsync(ws.retry, 0, (size_t)Bc * (n - 1) * 4, stream));
+        RWC_CUDA_TRY(cudaMemsetAsync(ws.retry, 0, (size_t)Bc * rcap * 4, stream));
         if (prof) cudaEventRecord(ev[0], stream);
         ::rwc::count_launches(1);
         w_init<<<sms * 8, 256, 0, stream>>>(n, g.root, ws.word, Bc);
@@ -834,6 +846,7 @@ extern "C" rwc_status rwc_sample_trees_noalloc(rwc_graph_t *G, uint64_t seed, in
     WState ws;
     ws.word = (uint64_t *)trees;
     ws.retry = (int32_t *)(trees + (size_t)B * n * 8);
+    ws.rcap = (int)(n - 1);
     ws.order = order;
     ws.err = (int *)tail;
     ws.ctr = (unsigned long long *)(tail + 8);
