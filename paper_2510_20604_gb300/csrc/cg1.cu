@@ -31,6 +31,7 @@ namespace {
 constexpr int CSR_TPB = 512;
 constexpr int ELL_TPB = 1024;
 constexpr int ELL_RMAX = 7;             // rows per thread held in registers
+constexpr int64_t CG_FUSED_MAX = 8000000;
 constexpr int CG_WINDOW = 1024;         // iterations without a halved residual: stagnation
 constexpr double CG_INNER_TOL = 1e-5;
 
@@ -433,7 +434,10 @@ struct Inner {
     }
 };
 
-template <bool OFF64, bool W, bool RES>
+// FUSED: the direction is formed from (z, p) pairs as it is gathered; else it is
+// an array of its own with a pass and a barrier per iteration, for systems whose
+// pairs do not stay in L2 while the directions do.
+template <bool OFF64, bool W, bool RES, bool FUSED>
 __global__ void __launch_bounds__(RES ? RES_TPB : CSR_TPB, RES ? 1 : 2) cg1_csr(CgArgs a) {
     const DevGraph &g = a.g;
     const int64_t n = g.n;
@@ -454,6 +458,7 @@ __global__ void __launch_bounds__(RES ? RES_TPB : CSR_TPB, RES ? 1 : 2) cg1_csr(
         });
         return s;
     };
+    float *p1 = reinterpret_cast<float *>(a.zp[0]), *z1 = reinterpret_cast<float *>(a.zp[1]);   // !FUSED
     ResidentRows<OFF64, W> held;
     if constexpr (RES) held.load(g);
     auto inner = [&](double rn) -> int {
@@ -462,7 +467,8 @@ __global__ void __launch_bounds__(RES ? RES_TPB : CSR_TPB, RES ? 1 : 2) cg1_csr(
             const float rv = (float)(a.R[i] / rn), zv = g.dinv32[i] * rv;
             a.r[i] = rv;
             a.e[i] = 0.f;
-            a.zp[0][i] = make_float2(zv, 0.f);
+            if (FUSED) a.zp[0][i] = make_float2(zv, 0.f);
+            else p1[i] = zv;
             pair_fma(acc[0], rv, zv);
         });
         Inner s;
@@ -473,7 +479,11 @@ __global__ void __launch_bounds__(RES ? RES_TPB : CSR_TPB, RES ? 1 : 2) cg1_csr(
             float2 *zo = a.zp[(it & 1) ^ 1];
             // q = L p, <p, q>; a heavy row's share of <p, q> comes from its chunks
             Pair pq[1] = {{0.f, 0.f}};
-            auto dir = [&](int64_t v) { const float2 t = zi[v]; return fmaf(beta, t.y, t.x); };
+            auto dir = [&](int64_t v) -> float {
+                if (!FUSED) return p1[v];
+                const float2 t = zi[v];
+                return fmaf(beta, t.y, t.x);
+            };
             auto row = [&](int32_t u, float t) {
                 const float pu = dir(u), qu = a.d32[u] * pu - t;
                 a.q[u] = qu;
@@ -497,7 +507,8 @@ __global__ void __launch_bounds__(RES ? RES_TPB : CSR_TPB, RES ? 1 : 2) cg1_csr(
                 const float rv = a.r[i] - al * qi;
                 a.r[i] = rv;
                 const float zv = g.dinv32[i] * rv;
-                zo[i] = make_float2(zv, pi);
+                if (FUSED) zo[i] = make_float2(zv, pi);
+                else z1[i] = zv;
                 pair_fma(z2[0], rv, zv);
                 pair_fma(z2[1], rv, rv);
             });
@@ -505,6 +516,10 @@ __global__ void __launch_bounds__(RES ? RES_TPB : CSR_TPB, RES ? 1 : 2) cg1_csr(
             ++it;
             beta = nx.x;
             if (nx.y != 0.f) break;
+            if (!FUSED) {
+                each([&](int64_t i) { p1[i] = z1[i] + beta * p1[i]; });
+                all_sync(a.clustered);
+            }
         }
         each([&](int64_t i) { a.X[i] += rn * (double)a.e[i]; });
         all_sync(a.clustered);
@@ -705,13 +720,18 @@ rwc_status solve_one(rwc_graph *G, const double *B, double *X, double tol, int *
         }
         return cudaLaunchCooperativeKernel((const void *)kern, dim3((unsigned)nb), dim3(tpb), args, sm, st);
     };
-    auto csr_of = [&](auto res, int tpb, int64_t nb) -> cudaError_t {
-        constexpr bool RES = decltype(res)::value;
-        if (g.off64) return g.weighted ? launch(cg1_csr<true, true, RES>, tpb, 0, nb) : launch(cg1_csr<true, false, RES>, tpb, 0, nb);
-        return g.weighted ? launch(cg1_csr<false, true, RES>, tpb, 0, nb) : launch(cg1_csr<false, false, RES>, tpb, 0, nb);
+    // pairs of 8 bytes in half of the 126 MB L2 or not
+    const bool fused = n <= CG_FUSED_MAX;
+    auto csr_of = [&](auto res, auto fu, int tpb, int64_t nb) -> cudaError_t {
+        constexpr bool RES = decltype(res)::value, FU = decltype(fu)::value;
+        if (g.off64)
+            return g.weighted ? launch(cg1_csr<true, true, RES, FU>, tpb, 0, nb) : launch(cg1_csr<true, false, RES, FU>, tpb, 0, nb);
+        return g.weighted ? launch(cg1_csr<false, true, RES, FU>, tpb, 0, nb) : launch(cg1_csr<false, false, RES, FU>, tpb, 0, nb);
     };
     auto csr = [&](int64_t nb) -> cudaError_t {
-        return held ? csr_of(std::true_type{}, RES_TPB, nb) : csr_of(std::false_type{}, CSR_TPB, nb);
+        if (held && nb == blocks) return csr_of(std::true_type{}, std::true_type{}, RES_TPB, nb);
+        if (fused) return csr_of(std::false_type{}, std::true_type{}, CSR_TPB, nb);
+        return csr_of(std::false_type{}, std::false_type{}, CSR_TPB, nb);
     };
     auto inl = [&](auto ew) -> cudaError_t {
         constexpr int EW = decltype(ew)::value;
@@ -723,7 +743,7 @@ rwc_status solve_one(rwc_graph *G, const double *B, double *X, double tol, int *
         // a device that refuses the cooperative launch: one block, no grid barrier
         (void)cudaGetLastError();
         a.clustered = false;
-        e = csr_of(std::false_type{}, CSR_TPB, 1);
+        e = csr(1);
     }
     RWC_CUDA_TRY(e);
     double h[3];

@@ -96,6 +96,11 @@ __device__ __forceinline__ void dot4(Pair (&a)[4], const float4 &x, const float4
     pair_fma(a[0], x.x, y.x); pair_fma(a[1], x.y, y.y); pair_fma(a[2], x.z, y.z); pair_fma(a[3], x.w, y.w);
 }
 
+// Rows of more arcs are shared by a block's slots: one slot takes about 150 cycles
+// per arc, so the hub of a BA graph of 9000 vertices alone took longer than the
+// rest of the product.
+constexpr int WIDE_ROW = 128;
+
 // Q = L P and the parts of <P, Q>.  Four neighbour rows are in flight.
 template <bool OFF64, bool W>
 __global__ void __launch_bounds__(TPB) bcg_product(DevGraph g, int k4, int qt, const float4 *__restrict__ P,
@@ -106,7 +111,7 @@ __global__ void __launch_bounds__(TPB) bcg_product(DevGraph g, int k4, int qt, c
         for (int64_t u = t.u0; u < g.n; u += t.step) {
             int64_t b, e;
             rowb<OFF64>(g, u, b, e);
-            if (g.hc_n && e - b > HEAVY_DEG) continue;
+            if (e - b > WIDE_ROW) continue;
             float4 s0 = {}, s1 = {};
             int64_t j = b;
             for (; j + 4 <= e; j += 4) {
@@ -127,27 +132,37 @@ __global__ void __launch_bounds__(TPB) bcg_product(DevGraph g, int k4, int qt, c
             Q[u * k4 + t.q] = q;
             dot4(a, p, q);
         }
-    // rows of more than HEAVY_DEG arcs: a block's slots share the arcs of one
+    // longer rows: the block's slots share the arcs of one
     __shared__ float4 hs[TPB];
-    for (int64_t c = blockIdx.x; c < g.hc_n; c += gridDim.x) {
-        const int64_t u = g.hc_row[c];
-        int64_t b, e;
-        rowb<OFF64>(g, u, b, e);
-        if (g.hc_beg[c] != b) continue;          // the row's first chunk only
-        float4 s = {};
-        if (t.on)
+    for (int64_t base = (int64_t)blockIdx.x * t.slots; base < g.n; base += t.step) {
+        int64_t b = 0, e = 0;
+        if (base + t.rs < g.n) rowb<OFF64>(g, base + t.rs, b, e);
+        if (!__syncthreads_or(e - b > WIDE_ROW)) continue;
+        for (int r = 0; r < t.slots && base + r < g.n; ++r) {
+            const int64_t u = base + r;
+            rowb<OFF64>(g, u, b, e);
+            if (e - b <= WIDE_ROW) continue;
+            float4 s = {};
+            if (t.on)
 #pragma unroll 4
-            for (int64_t j = b + t.rs; j < e; j += t.slots) fma4(s, W ? g.w[j] : 1.f, P[(int64_t)g.col[j] * k4 + t.q]);
-        __syncthreads();
-        hs[threadIdx.x] = s;
-        __syncthreads();
-        if (t.rs == 0 && t.on) {
-            for (int r = 1; r < t.slots; ++r) fma4(s, 1.f, hs[r * qt + threadIdx.x]);
-            const float d = (float)g.d[u];
-            const float4 p = P[u * k4 + t.q];
-            const float4 q = {d * p.x - s.x, d * p.y - s.y, d * p.z - s.z, d * p.w - s.w};
-            Q[u * k4 + t.q] = q;
-            dot4(a, p, q);
+                for (int64_t j = b + t.rs; j < e; j += t.slots) fma4(s, W ? g.w[j] : 1.f, P[(int64_t)g.col[j] * k4 + t.q]);
+            hs[threadIdx.x] = s;
+            int h = 1;
+            while (h < t.slots) h *= 2;
+            for (h /= 2; h > 0; h /= 2) {
+                __syncthreads();
+                if (t.rs < h && t.rs + h < t.slots) fma4(hs[threadIdx.x], 1.f, hs[threadIdx.x + h * qt]);
+            }
+            __syncthreads();
+            if (t.rs == 0 && t.on) {
+                s = hs[threadIdx.x];
+                const float d = (float)g.d[u];
+                const float4 p = P[u * k4 + t.q];
+                const float4 q = {d * p.x - s.x, d * p.y - s.y, d * p.z - s.z, d * p.w - s.w};
+                Q[u * k4 + t.q] = q;
+                dot4(a, p, q);
+            }
+            __syncthreads();
         }
     }
     quad_parts(t, a, qt, parts);
