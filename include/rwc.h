@@ -79,17 +79,23 @@ typedef struct {
 #define RWC_MODE_AUTO 0
 #define RWC_MODE_GLOBAL 1   /* rounds over tree chunks, state in HBM */
 #define RWC_MODE_SHARED 2   /* one thread block per tree, state in shared memory */
-#define RWC_MODE_WALKER 3   /* concurrent Wilson walkers, one block per tree, state in HBM */
+#define RWC_MODE_WALKER 3   /* many concurrent walks per tree: rounds of lanes with the
+                               state in shared memory (up to about 55000 vertices) or
+                               HBM, or, above 400000 vertices of unbounded degree and
+                               for calls that set block_threads, walker_policy,
+                               max_wait_ns or profile = 2, walkers that claim paths */
 
 typedef struct {
     int32_t mode;             /* RWC_MODE_*; AUTO picks SHARED when the tree fits in
                                  shared memory, WALKER otherwise */
-    int32_t max_rounds;       /* cap on popping rounds per chunk (0 = 1<<22) */
+    int32_t max_rounds;       /* GLOBAL, SHARED: cap on popping rounds per chunk (0 = 1<<22 in
+                                 GLOBAL mode; no cap in SHARED mode, whose rounds are then
+                                 those of the lanes) */
     int64_t trees_per_chunk;  /* GLOBAL/WALKER: trees resident at once (0 = auto) */
     int32_t use_jumps;        /* GLOBAL mode: 1 = jump pointers (default), 0 = off,
                                  -1 = default */
     int32_t block_threads;    /* SHARED: block size; WALKER: walkers per tree, at most
-                                 512 (0 = auto) */
+                                 512 (0 = auto: by the trees that an SM gets) */
     int64_t memory_budget;    /* GLOBAL/WALKER: bytes of scratch to use (0 = auto) */
     int32_t profile;          /* 1 = time every kernel launch with CUDA events on
                                  the call's stream (fills rwc_stats_t.phase_*);
@@ -136,7 +142,8 @@ typedef struct {
     int64_t trees;        /* trees sampled by the last call */
     int64_t draws;        /* successor draws (= sum of visits over all trees) */
     int64_t rounds;       /* GLOBAL/SHARED: popping rounds; WALKER: yielded walks
-                             (counted with rwc_options_t.profile = 2 only) */
+                             (counted with rwc_options_t.profile = 2 only); SHARED and
+                             batch: summed over the trees */
     int64_t walk_steps;   /* GLOBAL: pointer-chasing steps; WALKER: walker steps
                              (profile = 2 only) */
     int64_t chunks;       /* tree chunks processed */
@@ -344,8 +351,8 @@ rwc_status rwc_grad(rwc_graph_t *g, const double *c, int32_t k,
  * Batched sampler: many independent small graphs, all trees of all graphs in
  * one persistent launch (captured in a CUDA graph when use_graph != 0).
  * Graphs with more vertices than the schedule's split run one tree per thread
- * block, the others one tree per warp (several trees per block) or per small
- * block; see rwc_batch_set_schedule and rwc_autotune.
+ * block, the others one tree per warp or per small block, in one persistent
+ * kernel per bin of similar sizes; see rwc_batch_set_schedule and rwc_autotune.
  * host_graph_offsets: int64 [G+1] vertex offsets of each graph inside the
  * concatenated CSR; host_row_ptr: int64 [N+1] with global arc offsets;
  * host_col_idx: int32 [nnz] LOCAL vertex ids (0..n_g-1); host_w NULL (unit
@@ -371,13 +378,13 @@ rwc_status rwc_batch_roots(const rwc_batch_t *b, int32_t *host_roots);
  * the device; the choice is cached in cache_path (JSON, may be NULL) under a
  * signature of the batch's sizes.  Synchronises stream. */
 rwc_status rwc_autotune(rwc_batch_t *b, const char *cache_path, rwc_stream_t stream);
-/* The batch's schedule.  threads: block size of the large class (graphs with
- * more than split vertices, one tree per block; a multiple of 32, <= 1024);
- * split: the largest n of the small class (0: one class); warp: 1 = the small
- * class runs one tree per warp (8 trees per 256-thread block), 0 = one tree
- * per 256-thread block; tile: trees per work item; concurrent: 1 = the two
- * classes' persistent kernels run on forked streams at the same time, 0 = one
- * after the other (both inside the call's one CUDA graph).  set returns
+/* The batch's schedule.  threads: largest block of the large class (graphs with
+ * more than split vertices, one tree per block of 64 to 256 threads by its
+ * size; a multiple of 32, <= 1024); split: the largest n of the small class (0:
+ * one class); warp: 1 = the small class runs one tree per warp, 0 = one tree
+ * per block as the large class; tile: trees per work item; concurrent: 1 = the
+ * size bins' persistent kernels run on forked streams at the same time, 0 = one
+ * after the other (all inside the call's one CUDA graph).  set returns
  * RWC_ERR_UNSUPPORTED when a class needs more than 227 KB of shared memory
  * per block (a tree of n vertices takes 11 n + 64 bytes).  host_sched: int32
  * [5] = {threads, split, tile, warp, concurrent}.  Schedules do not change the
@@ -474,7 +481,7 @@ rwc_status rwc_predict_mre(rwc_graph_t *g, const double *sums, int64_t num_trees
  * tau-a).  a, b: device FP64 [n], no NaN (-0.0 equals +0.0).  out_diff:
  * device int64 scalar, written with alpha - beta (exact).  host_tau: NULL, or
  * a host double receiving K (then the call synchronises stream).  Every pair
- * is compared, O(n^2) work: 0 <= n <= 2^26.
+ * is counted (sorting and inversions above 8192 elements): 0 <= n <= 2^26.
  */
 rwc_status rwc_kendall(int64_t n, const double *a, const double *b, int64_t *out_diff,
                        double *host_tau, rwc_stream_t stream);
