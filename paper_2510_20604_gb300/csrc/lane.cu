@@ -149,6 +149,7 @@ struct Events {
     double ms(int a, int b) { float v = 0.f; if (on) cudaEventElapsedTime(&v, e[a], e[b]); return v; }
 };
 
+constexpr size_t SMEM_MAX = 226 * 1024;   // dynamic shared memory of one block beside 1 KB of its own
 constexpr int64_t TAIL = 64;   // err @0, next tree @8, draws @16, listed trees @24, rounds @32
 constexpr int64_t WIDE_CAP = 65536;   // trees of one shared-memory launch
 
@@ -282,7 +283,8 @@ rwc_status smem_range(rwc_graph *G, uint64_t seed, int64_t tree0, int64_t T, dou
     dispatch(g, [&](auto o64, auto wt, auto ew) {
         auto kern = l_trees_smem<decltype(o64)::value, decltype(wt)::value, decltype(ew)::value, NT>;
         auto launch = [&]() -> rwc_status {
-            RWC_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+            // the same value on every call: other threads launch the kernel too
+            RWC_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_MAX));
             int per_sm = 0;
             RWC_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, NT, smem));
             if (per_sm < 1) return set_error(RWC_ERR_UNSUPPORTED, "graph too large for shared mode");
@@ -371,7 +373,6 @@ rwc_status sample_smem(rwc_graph *G, uint64_t seed, int64_t tree0, int64_t T, do
 }  // namespace
 
 namespace {
-constexpr size_t SMEM_MAX = 226 * 1024;   // dynamic shared memory of one block beside 1 KB of its own
 
 // Whether walker mode keeps this graph's words in shared memory: a lane's hop
 // is 45 cycles there against 150 to 230 in global memory, where some lane of a

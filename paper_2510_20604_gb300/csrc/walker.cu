@@ -104,7 +104,7 @@ __global__ void w_init(int64_t n, int32_t root, uint64_t *word, int64_t B) {
 // start, so a queue that is within two blocks of full (a block's walkers may
 // each add one, and each may still be emptying a slot) only has to hand out its
 // own entries before fresh starts.  R-MAT 20, 2000 trees: 8.4 GB less scratch to
-// map and clear on every call, 288 -> 264 ms.
+// map and clear on every call, 292 -> 275 ms (281 ms with 65536 entries).
 constexpr int RETRY_CAP = 4096;
 
 // Retry queue: slots hold start index + 1 (0 = empty); a producer reserves a
