@@ -1,8 +1,7 @@
 // Batched sampler: all trees of thousands of small graphs in one CUDA-graph
-// launch.  Trees of work items (graph, tile of trees) are pulled one by one
-// from device counters by persistent kernels (no grid-wide barrier); a tree's
-// words live in shared memory and a block of 32 to 256 threads runs it
-// (lane_tree.cuh).  The graphs are sorted by size and cut into bins of about a
+// launch.  Trees are pulled one by one from device counters by persistent
+// kernels (no grid-wide barrier); a tree's words live in shared memory and a
+// block of 32 to 256 threads runs it (lane_tree.cuh).  The graphs are sorted by size and cut into bins of about a
 // factor of two, one kernel each, so that every bin gets the shared memory
 // (and thus the occupancy) and the threads its own graphs need; the bins run
 // on forked streams, and fork and join are captured into the call's CUDA
@@ -29,17 +28,13 @@ struct BGraph {
     int32_t root;
 };
 
-struct BItem {
-    int32_t g;
-    int32_t tile;   // index of the tile of trees within the graph
-};
-
-// Trees 0 .. npull - 1 of a bin: pull i is tree i % tile of item i / tile.  The
-// blocks take them in turn, after their first from the counter `next` (NULL:
-// every gridDim.x-th).
+// Trees 0 .. npull - 1 of a bin, T of each of its graphs: pull i is tree i % T of
+// graph order[i / T].  The blocks take them in turn, after their first from the
+// counter `next` (NULL: every gridDim.x-th).  Every pull is a tree, so
+// lane_tree's barriers lie between the reads of sh_next and its next write.
 template <bool OFF64, bool W, int NT>
 __global__ void __launch_bounds__(NT) l_batch(DevGraph base, const BGraph *__restrict__ graphs,
-                                              const BItem *__restrict__ items, int64_t npull, unsigned long long *next, int64_t tile,
+                                              const int32_t *__restrict__ order, int64_t npull, unsigned long long *next,
                                               int64_t T, uint32_t k0, uint32_t k1, int max_n, double *sums,
                                               uint32_t *spill, int *err, unsigned long long *ctr) {
     extern __shared__ __align__(16) unsigned char smem[];
@@ -52,29 +47,27 @@ __global__ void __launch_bounds__(NT) l_batch(DevGraph base, const BGraph *__res
     uint32_t rounds = 0;
     int64_t i = blockIdx.x;
     while (i < npull) {
-        const BItem it = items[i / tile];
-        const int64_t t = (int64_t)it.tile * tile + i % tile;
-        if (t < T) {
-            const BGraph bg = graphs[it.g];
-            DevGraph g = base;
-            g.n = bg.n;
-            g.root = bg.root;
-            if (OFF64) g.rp64 = base.rp64 + bg.voff;
-            else g.rp32 = base.rp32 + bg.voff;
-            const int kb = lt_kbits<uint32_t>(bg.n, NT);
-            for (int u = threadIdx.x; u < bg.n; u += NT) word[u] = u == bg.root ? lt_root_word<uint32_t>(kb, NT) : 0u;
-            __syncthreads();
-            const int bad = lane_tree<OFF64, W, 0, NT, 1, true, uint32_t>(g, word, kb, 65535u, sh, sp, (uint32_t)t,
-                                                                          (uint32_t)it.g, k0, k1, rounds);
-            if (bad) { if (threadIdx.x == 0) atomicOr(err, bad); break; }
-            const uint32_t kmask = (1u << kb) - 1u;
-            double *out = sums + bg.voff;
-            for (int u = threadIdx.x; u < bg.n; u += NT) {
-                if (u == bg.root) continue;
-                const uint32_t vis = (word[u] & kmask) + 1u;
-                draws += vis;
-                atomicAdd(out + u, (double)vis);
-            }
+        const int32_t gid = order[i / T];
+        const int64_t t = i % T;
+        const BGraph bg = graphs[gid];
+        DevGraph g = base;
+        g.n = bg.n;
+        g.root = bg.root;
+        if (OFF64) g.rp64 = base.rp64 + bg.voff;
+        else g.rp32 = base.rp32 + bg.voff;
+        const int kb = lt_kbits<uint32_t>(bg.n, NT);
+        for (int u = threadIdx.x; u < bg.n; u += NT) word[u] = u == bg.root ? lt_root_word<uint32_t>(kb, NT) : 0u;
+        __syncthreads();
+        const int bad = lane_tree<OFF64, W, 0, NT, 1, true, uint32_t>(g, word, kb, 65535u, sh, sp, (uint32_t)t,
+                                                                      (uint32_t)gid, k0, k1, rounds);
+        if (bad) { if (threadIdx.x == 0) atomicOr(err, bad); break; }
+        const uint32_t kmask = (1u << kb) - 1u;
+        double *out = sums + bg.voff;
+        for (int u = threadIdx.x; u < bg.n; u += NT) {
+            if (u == bg.root) continue;
+            const uint32_t vis = (word[u] & kmask) + 1u;
+            draws += vis;
+            atomicAdd(out + u, (double)vis);
         }
         if (!next) { i += gridDim.x; continue; }
         if (threadIdx.x == 0) sh_next = atomicAdd(next, 1ull);
@@ -123,10 +116,10 @@ void dispatch_nt(bool off64, bool weighted, int nt, F f) {
 
 constexpr int MAX_BINS = 12;
 
-// Items of one kernel: a range of a class's list.
+// Graphs of one kernel: a range of a class's list.
 struct Bin {
     int cls;
-    int64_t begin, count;   // items
+    int64_t begin, count;   // graphs
     int max_n, nt;
     size_t smem;
     int64_t blocks;
@@ -148,7 +141,7 @@ struct rwc_batch {
     BGraph *graphs = nullptr;
     // schedule: largest block of the large graphs, the largest n of the small
     // class (0: one class), small class warp-per-tree (1) or block-per-tree
-    // (0), trees per work item
+    // (0); tile is kept for saved schedules, trees are pulled one by one
     int threads = 512;
     int split = 1024;
     int warp = 1;
@@ -156,14 +149,13 @@ struct rwc_batch {
     int conc = 1;                      // 1: the classes run concurrently (forked streams)
     cudaStream_t side[MAX_BINS] = {};  // the bins' streams (forked from the call's)
     cudaEvent_t fork = nullptr, join[MAX_BINS] = {};
-    BItem *items[2] = {nullptr, nullptr};
-    int64_t nitems[2] = {0, 0};
+    int32_t *items[2] = {nullptr, nullptr};   // each class's graphs, the largest first
     int max_n[2] = {0, 0};             // largest n of each class
     std::vector<Bin> bins;
     uint32_t *spill = nullptr;         // the bins' pending ends beyond shared memory
-    BItem *single = nullptr;           // item g: graph g's first tile (one launch per graph)
-    int64_t items_T = -1;              // T the item lists were built for
-    int64_t items_tile = -1, items_split = -1;
+    int32_t *single = nullptr;         // graph ids 0 .. G - 1 (one launch per graph)
+    int64_t items_T = -1;              // T the bins were built for
+    int64_t items_split = -1;
     void *scratch = nullptr;           // [0] err, [8] rounds, [16] draws, [64..160) the bins' counters
     std::vector<void *> allocs;
     // captured launches
@@ -211,7 +203,7 @@ size_t schedule_allowance(int max_large, int max_small, int warp) {
 }
 size_t batch_smem(const rwc_batch *b) { return schedule_allowance(b->max_n[0], b->max_n[1], b->warp); }
 
-rwc_status build_bins(rwc_batch *b, const std::vector<int32_t> (&order)[2], int64_t ntile) {
+rwc_status build_bins(rwc_batch *b, const std::vector<int32_t> (&order)[2], int64_t T) {
     b->bins.clear();
     for (int c = 0; c < 2; ++c)
         for (size_t i = 0; i < order[c].size();) {
@@ -220,8 +212,8 @@ rwc_status build_bins(rwc_batch *b, const std::vector<int32_t> (&order)[2], int6
             while (j < order[c].size() && (top <= 640 || 2 * b->hgraphs[order[c][j]].n > top)) ++j;
             Bin q{};
             q.cls = c;
-            q.begin = (int64_t)i * ntile;
-            q.count = (int64_t)(j - i) * ntile;
+            q.begin = (int64_t)i;
+            q.count = (int64_t)(j - i);
             q.max_n = top;
             q.nt = batch_threads(top);
             if (c == 1 && b->warp) q.nt = 32;
@@ -241,7 +233,7 @@ rwc_status build_bins(rwc_batch *b, const std::vector<int32_t> (&order)[2], int6
         });
         RWC_CUDA_TRY(e);
         if (per_sm < 1) return set_error(RWC_ERR_UNSUPPORTED, "batch block does not fit on an SM");
-        q.blocks = std::max<int64_t>(1, std::min<int64_t>(q.count * b->tile, (int64_t)num_sms() * per_sm));
+        q.blocks = std::max<int64_t>(1, std::min<int64_t>(q.count * T, (int64_t)num_sms() * per_sm));
         q.spill = spill;
         spill += q.blocks * q.max_n;
     }
@@ -254,13 +246,12 @@ rwc_status build_bins(rwc_batch *b, const std::vector<int32_t> (&order)[2], int6
     return RWC_OK;
 }
 
-// Work items for T trees per graph: list 0 holds graphs with more than `split`
+// Bins for T trees per graph: list 0 holds graphs with more than `split`
 // vertices, list 1 the others; each list runs its largest graphs first.
 rwc_status build_items(rwc_batch *b, int64_t T) {
-    if (b->items_T == T && b->items_tile == b->tile && b->items_split == b->split) return RWC_OK;
+    if (b->items_T == T && b->items_split == b->split) return RWC_OK;
     std::vector<int32_t> orders[2];
     for (int c = 0; c < 2; ++c) {
-        std::vector<BItem> v;
         std::vector<int32_t> &order = orders[c];
         for (int32_t g = 0; g < b->G; ++g) {
             const int cls = b->hgraphs[g].n <= b->split ? 1 : 0;
@@ -268,22 +259,17 @@ rwc_status build_items(rwc_batch *b, int64_t T) {
         }
         std::stable_sort(order.begin(), order.end(),
                          [&](int32_t x, int32_t y) { return b->hgraphs[x].n > b->hgraphs[y].n; });
-        const int64_t ntile = (T + b->tile - 1) / b->tile;
-        for (int32_t g : order)
-            for (int64_t t = 0; t < ntile; ++t) v.push_back(BItem{g, (int32_t)t});
         if (b->items[c]) { cudaFree(b->items[c]); b->allocs.erase(std::find(b->allocs.begin(), b->allocs.end(), (void *)b->items[c])); }
         b->items[c] = nullptr;
-        b->nitems[c] = (int64_t)v.size();
-        if (!v.empty()) {
-            RWC_CUDA_TRY(balloc(b, (void **)&b->items[c], v.size() * sizeof(BItem)));
-            RWC_CUDA_TRY(cudaMemcpy(b->items[c], v.data(), v.size() * sizeof(BItem), cudaMemcpyHostToDevice));
+        if (!order.empty()) {
+            RWC_CUDA_TRY(balloc(b, (void **)&b->items[c], order.size() * sizeof(int32_t)));
+            RWC_CUDA_TRY(cudaMemcpy(b->items[c], order.data(), order.size() * sizeof(int32_t), cudaMemcpyHostToDevice));
         }
         b->max_n[c] = 0;
         for (int32_t g : order) b->max_n[c] = std::max(b->max_n[c], b->hgraphs[g].n);
     }
-    RWC_TRY(build_bins(b, orders, (T + b->tile - 1) / b->tile));
+    RWC_TRY(build_bins(b, orders, T));
     b->items_T = T;
-    b->items_tile = b->tile;
     b->items_split = b->split;
     drop_graph(b);
     return RWC_OK;
@@ -313,8 +299,8 @@ rwc_status enqueue(rwc_batch *b, uint64_t seed, int64_t T, double *sums, cudaStr
         ::rwc::count_launches(1);
         dispatch_nt(b->off64, b->weighted, q.nt, [&](auto kern) {
             kern<<<(unsigned)q.blocks, q.nt, q.smem, s>>>(b->base, b->graphs, b->items[q.cls] + q.begin,
-                                                          q.count * b->tile, next + i, b->tile, T, k0, k1, q.max_n,
-                                                          sums, b->spill + q.spill, err, ctr);
+                                                          q.count * T, next + i, T, k0, k1, q.max_n, sums,
+                                                          b->spill + q.spill, err, ctr);
         });
         e = cudaGetLastError();
     }
@@ -435,10 +421,10 @@ extern "C" rwc_status rwc_batch_create(int32_t G, const int64_t *voff, const int
     if ((e = balloc(b, (void **)&b->graphs, G * sizeof(BGraph))) != cudaSuccess) return fail(e);
     if ((e = cudaMemcpy(b->graphs, hg.data(), G * sizeof(BGraph), cudaMemcpyHostToDevice)) != cudaSuccess) return fail(e);
     {
-        std::vector<BItem> one(G);
-        for (int32_t g = 0; g < G; ++g) one[g] = BItem{g, 0};
-        if ((e = balloc(b, (void **)&b->single, G * sizeof(BItem))) != cudaSuccess) return fail(e);
-        if ((e = cudaMemcpy(b->single, one.data(), G * sizeof(BItem), cudaMemcpyHostToDevice)) != cudaSuccess) return fail(e);
+        std::vector<int32_t> one(G);
+        for (int32_t g = 0; g < G; ++g) one[g] = g;
+        if ((e = balloc(b, (void **)&b->single, G * sizeof(int32_t))) != cudaSuccess) return fail(e);
+        if ((e = cudaMemcpy(b->single, one.data(), G * sizeof(int32_t), cudaMemcpyHostToDevice)) != cudaSuccess) return fail(e);
     }
     if ((e = balloc(b, &b->scratch, 256)) != cudaSuccess) return fail(e);
     if ((e = cudaMallocHost((void **)&b->host, 64)) != cudaSuccess) return fail(e);
@@ -497,7 +483,7 @@ extern "C" rwc_status rwc_batch_sample(rwc_batch_t *b, uint64_t seed, int64_t T,
             ::rwc::count_launches(1);
             dispatch_nt(b->off64, b->weighted, nt, [&](auto kern) {
                 kern<<<(unsigned)blocks[g], nt, batch_tree_smem(n, nt), st>>>(
-                    b->base, b->graphs, b->single + g, T, nullptr, T, T, k0, k1, n, sums, sp, err, ctr);
+                    b->base, b->graphs, b->single + g, T, nullptr, T, k0, k1, n, sums, sp, err, ctr);
             });
         }
         cudaFreeAsync(sp, st);

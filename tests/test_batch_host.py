@@ -1,0 +1,30 @@
+"""Host logic of the batched sampler on a stand-in for the CUDA runtime
+(batch_host.cpp), linked with the library's own object files."""
+import os
+import subprocess
+
+import pytest
+
+from paper_2510_20604_gb300 import _build
+
+HERE = os.path.dirname(os.path.abspath(__file__))
+
+
+@pytest.fixture(scope="module")
+def driver(tmp_path_factory):
+    _build.build()
+    exe = str(tmp_path_factory.mktemp("batch") / "batch_host")
+    inc = os.path.join(os.path.dirname(os.path.dirname(_build.nvcc())), "include")
+    objs = [os.path.join(_build.BUILD, o) for o in ("batch.o", "graph.o")]
+    subprocess.run(["g++", "-std=c++17", "-O1", "-I", _build.INCLUDE, "-I", inc, "-o", exe,
+                    os.path.join(HERE, "batch_host.cpp")] + objs, check=True)
+    return exe
+
+
+@pytest.mark.parametrize("use_graph", [0, 1])
+def test_every_pull_is_a_tree(driver, use_graph):
+    """A launch has as many pulls as trees for every remainder of the tree
+    count (a block that skips pulls passes none of a tree's barriers between
+    two writes of the shared pull number)."""
+    r = subprocess.run([driver, "-1", str(use_graph)], capture_output=True, text=True, timeout=60)
+    assert r.returncode == 0, r.stdout + r.stderr

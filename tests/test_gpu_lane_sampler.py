@@ -107,3 +107,18 @@ def test_batch_bins_and_block_sizes(sched):
         ref = ow.Sampler(g, root=int(roots[i]), seed=7, graph_id=i).sample(0, T)
         assert np.array_equal(sums[o[i]:o[i + 1]], ref["sums"]), ns[i]
     assert st.trees == T * len(gs) and st.draws == int(sums.sum()) and st.rounds > 0
+
+
+@pytest.mark.parametrize("T", [1, 2, 3, 5, 6, 7])
+def test_batch_takes_every_tree_once(T):
+    # more blocks than trees of one graph, tree counts of every remainder of
+    # the schedule's trees per item, blocks of several warps
+    gs = [synth.ba(n, 2, seed=n) for n in range(120, 190, 2)] * 5
+    B = rwc.Batch(gs)
+    B.set_schedule(512, 0, 4, 0, 1)
+    s, st = B.sample(T, seed=3)
+    sums, roots, o = s.cpu().numpy(), B.roots(), B.offsets
+    for i in range(0, len(gs), 7):
+        ref = ow.Sampler(gs[i], root=int(roots[i]), seed=3, graph_id=i).sample(0, T)
+        assert np.array_equal(sums[o[i]:o[i + 1]], ref["sums"]), i
+    assert st.draws == int(sums.sum()) and st.trees == T * len(gs)
