@@ -227,6 +227,9 @@ __device__ __forceinline__ int lane_tree(const DevGraph &g, W *word, int kb, uin
     for (;;) {
         // ---- draw
         if (total == 0 && gsp) {
+            // the other warps may still be adding up the heights written below
+            // (one that saw the new height would skip this branch and its barrier)
+            if (WARP) __syncwarp(); else __syncthreads();
             const uint32_t c = gsp < LT_STACK / 2 ? gsp : LT_STACK / 2;
             for (uint32_t i = threadIdx.x % NT; i < c; i += NT) sh.stack[0][i] = spill[gsp - c + i];
             gsp -= c;

@@ -122,3 +122,23 @@ def test_batch_takes_every_tree_once(T):
         ref = ow.Sampler(gs[i], root=int(roots[i]), seed=3, graph_id=i).sample(0, T)
         assert np.array_equal(sums[o[i]:o[i + 1]], ref["sums"]), i
     assert st.draws == int(sums.sum()) and st.trees == T * len(gs)
+
+
+@pytest.mark.parametrize("side,T", [(130, 2), (70, 160), (70, 900), (70, 1600)])
+def test_stacks_are_refilled_from_global_memory(side, T):
+    # popped cycles of a grid overflow the 192 ends of a warp's stack; once all
+    # stacks are empty the overflow comes back (blocks of 256, 256, 128 and 64
+    # threads by the trees that an SM gets)
+    _exact(synth.grid2d(side, side), T, rwc.Options(mode=rwc.MODE_SHARED))
+
+
+def test_stacks_are_refilled_in_a_batch():
+    gs = [synth.grid2d(a, b) for a, b in ((45, 47), (60, 50), (69, 70), (90, 100))]
+    for sched in ((512, 0, 4, 0, 1), (512, 2600, 4, 1, 1)):     # blocks only; the smallest by a warp
+        B = rwc.Batch(gs)
+        B.set_schedule(*sched)
+        s, _ = B.sample(6, seed=11)
+        sums, roots, o = s.cpu().numpy(), B.roots(), B.offsets
+        for i, g in enumerate(gs):
+            ref = ow.Sampler(g, root=int(roots[i]), seed=11, graph_id=i).sample(0, 6)
+            assert np.array_equal(sums[o[i]:o[i + 1]], ref["sums"]), (sched, i)
