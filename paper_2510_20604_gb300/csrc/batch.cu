@@ -250,6 +250,9 @@ rwc_status build_bins(rwc_batch *b, const std::vector<int32_t> (&order)[2], int6
 // vertices, list 1 the others; each list runs its largest graphs first.
 rwc_status build_items(rwc_batch *b, int64_t T) {
     if (b->items_T == T && b->items_split == b->split) return RWC_OK;
+    // nothing built for another T or schedule is used again, whatever fails below
+    b->items_T = -1;
+    drop_graph(b);
     std::vector<int32_t> orders[2];
     for (int c = 0; c < 2; ++c) {
         std::vector<int32_t> &order = orders[c];
@@ -271,7 +274,6 @@ rwc_status build_items(rwc_batch *b, int64_t T) {
     RWC_TRY(build_bins(b, orders, T));
     b->items_T = T;
     b->items_split = b->split;
-    drop_graph(b);
     return RWC_OK;
 }
 

@@ -28,3 +28,13 @@ def test_every_pull_is_a_tree(driver, use_graph):
     two writes of the shared pull number)."""
     r = subprocess.run([driver, "-1", str(use_graph)], capture_output=True, text=True, timeout=60)
     assert r.returncode == 0, r.stdout + r.stderr
+
+
+@pytest.mark.parametrize("use_graph", [0, 1])
+@pytest.mark.parametrize("nth", [0, 1, 2])
+def test_a_failed_rebuild_leaves_nothing_stale(driver, nth, use_graph):
+    """The nth allocation of a call with another tree count fails (the two
+    classes' items, the spill array); the next call with the first count gives
+    no freed memory to a launch."""
+    r = subprocess.run([driver, str(nth), str(use_graph)], capture_output=True, text=True, timeout=60)
+    assert r.returncode == 0, r.stdout + r.stderr
