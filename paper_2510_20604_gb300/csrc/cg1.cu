@@ -48,6 +48,7 @@ struct CgArgs {
     double *hsumd;
     double *parts;                      // [2][2][gridDim] block sums, in turn
     double tol;
+    double scale;                       // |r| of an inner solve's start (inner_scale)
     int max_outer, max_inner;
     int use_smem;                       // inline rows fit shared memory
     bool clustered;                     // the blocks are one cluster
@@ -363,7 +364,7 @@ __device__ __forceinline__ T heavy_sum(const DevGraph &g, int64_t u, const T *hs
 }
 
 // Outer loop shared by both kernels: INNER runs the conjugate gradients on R /
-// |R| and adds the correction to X; RESID fills R = B - L X and returns this
+// |R| times the scale and adds the correction to X; RESID fills R = B - L X and returns this
 // thread's share of its sum; EACH visits the thread's rows.
 template <class Resid, class Each, class Inner>
 __device__ void refine(const CgArgs &a, int &flip, Resid resid, Each each, Inner inner) {
@@ -417,8 +418,10 @@ __device__ __forceinline__ Pair normal(Pair a) {
 // inner iteration: thread 0's, the same in every block.
 struct Inner {
     Pair rz = {0.f, 0.f};
+    float stop;                             // <r, r> that ends the iteration
     float best = INFINITY;
     int since = 0;
+    __device__ explicit Inner(double scale) : stop((float)(CG_INNER_TOL * scale * (CG_INNER_TOL * scale))) {}
     __device__ float step(Pair den) const {
         den = normal(den);
         return den.s > 0.f && rz.s > 0.f ? quotient(rz, den) : 0.f;
@@ -427,7 +430,7 @@ struct Inner {
     __device__ float2 next(Pair rz1, Pair rr2) {
         rz1 = normal(rz1);
         const float rr = normal(rr2).s;
-        if (!(rr == rr) || rr <= (float)(CG_INNER_TOL * CG_INNER_TOL)) return make_float2(0.f, 1.f);
+        if (!(rr == rr) || rr <= stop) return make_float2(0.f, 1.f);
         if (rr < 0.25f * best) { best = rr; since = 0; }
         else if (++since >= CG_WINDOW) return make_float2(0.f, 1.f);
         const float beta = rz.s > 0.f ? quotient(rz1, rz) : 0.f;
@@ -466,14 +469,14 @@ __global__ void __launch_bounds__(RES ? RES_TPB : CSR_TPB, RES ? 1 : 2) cg1_csr(
     auto inner = [&](double rn) -> int {
         Pair acc[1] = {{0.f, 0.f}};
         each([&](int64_t i) {
-            const float rv = (float)(a.R[i] / rn), zv = g.dinv32[i] * rv;
+            const float rv = (float)(a.R[i] / rn * a.scale), zv = g.dinv32[i] * rv;
             a.r[i] = rv;
             a.e[i] = 0.f;
             if (FUSED) a.zp[0][i] = make_float2(zv, 0.f);
             else p1[i] = zv;
             pair_fma(acc[0], rv, zv);
         });
-        Inner s;
+        Inner s(a.scale);
         float beta = grid_sums<1, float>(acc, a.parts, flip, a.clustered, [&](const Pair *t) { s.rz = normal(t[0]); return 0.f; });
         int it = 0;
         while (it < a.max_inner) {
@@ -523,7 +526,7 @@ __global__ void __launch_bounds__(RES ? RES_TPB : CSR_TPB, RES ? 1 : 2) cg1_csr(
                 all_sync(a.clustered);
             }
         }
-        each([&](int64_t i) { a.X[i] += rn * (double)a.e[i]; });
+        each([&](int64_t i) { a.X[i] += rn / a.scale * (double)a.e[i]; });
         all_sync(a.clustered);
         return it;
     };
@@ -579,13 +582,13 @@ __global__ void __launch_bounds__(ELL_TPB, 1) cg1_ell(CgArgs a) {
             if (l < nrow) {
                 const int64_t u = row0 + l;
                 d[i] = a.d32[u];
-                r[i] = (float)(a.R[u] / rn);
+                r[i] = (float)(a.R[u] / rn * a.scale);
                 const float zv = r[i] * __fdividef(1.f, d[i]);
                 a.zp[0][u] = make_float2(zv, 0.f);
                 pair_fma(acc[0], r[i], zv);
             }
         }
-        Inner s;
+        Inner s(a.scale);
         float beta = grid_sums<1, float>(acc, a.parts, flip, a.clustered, [&](const Pair *t) { s.rz = normal(t[0]); return 0.f; });
         int it = 0;
         while (it < a.max_inner) {
@@ -624,7 +627,7 @@ __global__ void __launch_bounds__(ELL_TPB, 1) cg1_ell(CgArgs a) {
 #pragma unroll
         for (int i = 0; i < RT; ++i) {
             const int l = threadIdx.x + i * ELL_TPB;
-            if (l < nrow) a.X[row0 + l] += rn * (double)e[i];
+            if (l < nrow) a.X[row0 + l] += rn / a.scale * (double)e[i];
         }
         all_sync(a.clustered);
         return it;
@@ -691,6 +694,7 @@ rwc_status solve_one(rwc_graph *G, const double *B, double *X, double tol, int *
     a.X = X;
     a.d32 = d32;
     a.tol = tol;
+    a.scale = inner_scale(g);
     a.max_outer = 30;
     a.max_inner = (int)std::min<int64_t>(200000, std::max<int64_t>(1000, 4 * n));
     a.use_smem = smem > 0;

@@ -225,9 +225,9 @@ __global__ void __launch_bounds__(TPB) bcg_direction(int64_t n, int k4, int qt, 
     }
 }
 
-// Start of an inner solve: r = R / |R_c|, e = 0, p = z = D^-1 r, parts of
+// Start of an inner solve: r = scale R / |R_c|, e = 0, p = z = D^-1 r, parts of
 // <r, z>; columns beyond k are 0.
-__global__ void __launch_bounds__(TPB) bcg_start(int64_t n, int k, int k4, int qt, const double *__restrict__ R,
+__global__ void __launch_bounds__(TPB) bcg_start(int64_t n, int k, int k4, int qt, double scale, const double *__restrict__ R,
                                                  const double *rnrm2, const float *dinv, float4 *__restrict__ r,
                                                  float4 *__restrict__ e, float4 *__restrict__ p, double *parts) {
     const Tile t(k4, qt);
@@ -239,7 +239,7 @@ __global__ void __launch_bounds__(TPB) bcg_start(int64_t n, int k, int k4, int q
         for (int64_t u = t.u0; u < n; u += t.step) {
             float v[4];
 #pragma unroll
-            for (int i = 0; i < 4; ++i) v[i] = nr[i] > 0.0 ? (float)(R[u * k + 4 * t.q + i] / nr[i]) : 0.f;
+            for (int i = 0; i < 4; ++i) v[i] = nr[i] > 0.0 ? (float)(R[u * k + 4 * t.q + i] / nr[i] * scale) : 0.f;
             const float di = dinv[u];
             const float4 rv = {v[0], v[1], v[2], v[3]}, zv = {di * v[0], di * v[1], di * v[2], di * v[3]};
             const int64_t i = u * k4 + t.q;
@@ -252,13 +252,13 @@ __global__ void __launch_bounds__(TPB) bcg_start(int64_t n, int k, int k4, int q
     quad_parts(t, a, qt, parts);
 }
 
-// X += |R_c| e.
-__global__ void __launch_bounds__(TPB) bcg_add(int64_t n, int k, int k4, const double *rnrm2, const float *e, double *X) {
+// X += |R_c| / scale e.
+__global__ void __launch_bounds__(TPB) bcg_add(int64_t n, int k, int k4, double scale, const double *rnrm2, const float *e, double *X) {
     const int64_t tot = n * k;
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < tot; i += (int64_t)gridDim.x * blockDim.x) {
         const int64_t u = i / k;
         const int c = (int)(i - u * k);
-        X[i] += sqrt(rnrm2[c]) * (double)e[u * 4 * k4 + c];
+        X[i] += sqrt(rnrm2[c]) / scale * (double)e[u * 4 * k4 + c];
     }
 }
 
@@ -367,7 +367,7 @@ rwc_status solve_nodemajor(rwc_graph *G, int k, const double *B, double *X, doub
     const int64_t nk = n * k;
     const int max_inner = (int)std::min<int64_t>(200000, std::max<int64_t>(1000, 4 * n));
     const int max_outer = 30;
-    const double inner_tol = 1e-5;
+    const double inner_tol = 1e-5, scale = inner_scale(g);
     const int k4 = (k + 3) / 4, kp = 4 * k4;
     // blocks: qt quads of columns x TPB / qt row slots; nb row ranges, fewer for
     // many column tiles (the parts are [kp][nb])
@@ -431,7 +431,7 @@ rwc_status solve_nodemajor(rwc_graph *G, int k, const double *B, double *X, doub
             return set_error(RWC_ERR_NOT_CONVERGED, "Laplacian solve reached %d refinements at relative residual %.3g (tol %.3g)", max_outer, worst, tol);
         // inner FP32 PCG on the normalised residual
         ::rwc::count_launches(2);
-        bcg_start<<<grid, threads, 0, st>>>(n, k, k4, qt, R, rn2, g.dinv32, r, e, p, pa);
+        bcg_start<<<grid, threads, 0, st>>>(n, k, k4, qt, scale, R, rn2, g.dinv32, r, e, p, pa);
         sum_cols<<<dim3((unsigned)kp, 1), 128, 0, st>>>(pa, nullptr, (int)nb, rz[0], nullptr);
         int it = 0;
         // iterations between looks at the residual (a host round trip each)
@@ -460,7 +460,7 @@ rwc_status solve_nodemajor(rwc_graph *G, int k, const double *B, double *X, doub
                 bad = bad || !(h[c] == h[c]);
                 w2 = std::max(w2, h[c]);
             }
-            if (std::sqrt(w2) <= inner_tol || bad) inner_done = true;
+            if (std::sqrt(w2) <= inner_tol * scale || bad) inner_done = true;
             // FP32 stagnation: the residual norm has not halved for 1024
             // iterations; CG residuals are not monotone, so the window is long
             if (w2 < 0.25 * best) { best = w2; since_best = 0; }
@@ -468,7 +468,7 @@ rwc_status solve_nodemajor(rwc_graph *G, int k, const double *B, double *X, doub
         }
         total_iters += it;
         ::rwc::count_launches(1);
-        bcg_add<<<gs, TPB, 0, st>>>(n, k, k4, rn2, (const float *)e, X);
+        bcg_add<<<gs, TPB, 0, st>>>(n, k, k4, scale, rn2, (const float *)e, X);
         RWC_CUDA_TRY(cudaGetLastError());
     }
     // final projection of X onto 1-perp
