@@ -352,6 +352,36 @@ __device__ __forceinline__ void all_rows(const DevGraph &g, Term term, F f, H h)
         if (lane == 0) h(c, u, b == rb, s);
     }
 }
+// all rows of a graph of bounded degree by their inline neighbours, one thread
+// per row, several rows in flight: f(row, sum of get(neighbour))
+template <int EW, class T, class Get, class F>
+__device__ __forceinline__ void inline_rows(const DevGraph &g, Get get, F f) {
+    constexpr int NR = EW == 4 ? 4 : 2, E4 = EW / 4;
+    const int64_t tid = blockIdx.x * (int64_t)blockDim.x + threadIdx.x, nthr = (int64_t)gridDim.x * blockDim.x;
+    for (int64_t i = tid; i < g.n; i += NR * nthr) {
+        int4 c[NR][E4];
+        T s[NR];
+#pragma unroll
+        for (int k = 0; k < NR; ++k)
+#pragma unroll
+            for (int j = 0; j < E4; ++j)
+                c[k][j] = i + k * nthr < g.n ? __ldg(g.ell + (i + k * nthr) * E4 + j) : make_int4(-1, -1, -1, -1);
+#pragma unroll
+        for (int k = 0; k < NR; ++k) {
+            s[k] = 0;
+#pragma unroll
+            for (int j = 0; j < E4; ++j) {
+                const int4 q = c[k][j];
+                const T v0 = q.x >= 0 ? get(q.x) : (T)0, v1 = q.y >= 0 ? get(q.y) : (T)0;
+                const T v2 = q.z >= 0 ? get(q.z) : (T)0, v3 = q.w >= 0 ? get(q.w) : (T)0;
+                s[k] += v0; s[k] += v1; s[k] += v2; s[k] += v3;
+            }
+        }
+#pragma unroll
+        for (int k = 0; k < NR; ++k)
+            if (i + k * nthr < g.n) f((int32_t)(i + k * nthr), s[k]);
+    }
+}
 // sum of a heavy row's chunks in chunk order
 template <bool OFF64, class T>
 __device__ __forceinline__ T heavy_sum(const DevGraph &g, int64_t u, const T *hsum) {
@@ -441,8 +471,9 @@ struct Inner {
 
 // FUSED: the direction is formed from (z, p) pairs as it is gathered; else it is
 // an array of its own with a pass and a barrier per iteration, for systems whose
-// pairs do not stay in L2 while the directions do.
-template <bool OFF64, bool W, bool RES, bool FUSED>
+// pairs do not stay in L2 while the directions do.  EW: inline rows of EW slots,
+// for graphs of bounded degree with more rows than cg1_ell holds (0: CSR).
+template <bool OFF64, bool W, bool RES, bool FUSED, int EW = 0>
 __global__ void __launch_bounds__(RES ? RES_TPB : CSR_TPB, RES ? 1 : 2) cg1_csr(CgArgs a) {
     const DevGraph &g = a.g;
     const int64_t n = g.n;
@@ -451,10 +482,12 @@ __global__ void __launch_bounds__(RES ? RES_TPB : CSR_TPB, RES ? 1 : 2) cg1_csr(
     auto each = [&](auto f) { for (int64_t i = tid; i < n; i += nthr) f(i); };
     auto resid = [&]() -> double {
         double s = 0.0;
-        all_rows<OFF64, double>(
-            g, [&](int64_t j) { return (W ? (double)g.w[j] : 1.0) * a.X[g.col[j]]; },
-            [&](int32_t u, double t) { a.R[u] = a.B[u] - (g.d[u] * a.X[u] - t); },
-            [&](int64_t c, int32_t, bool, double t) { a.hsumd[c] = t; });
+        auto row = [&](int32_t u, double t) { a.R[u] = a.B[u] - (g.d[u] * a.X[u] - t); };
+        if constexpr (EW > 0)
+            inline_rows<EW, double>(g, [&](int32_t v) { return a.X[v]; }, row);
+        else
+            all_rows<OFF64, double>(g, [&](int64_t j) { return (W ? (double)g.w[j] : 1.0) * a.X[g.col[j]]; }, row,
+                                    [&](int64_t c, int32_t, bool, double t) { a.hsumd[c] = t; });
         all_sync(a.clustered);
         each([&](int64_t i) {
             if (g.hc_n && g.hfirst[i] >= 0)
@@ -502,6 +535,7 @@ __global__ void __launch_bounds__(RES ? RES_TPB : CSR_TPB, RES ? 1 : 2) cg1_csr(
             };
             auto term = [&](int64_t j) { return (W ? g.w[j] : 1.f) * dir(g.col[j]); };
             if constexpr (RES) held.rows(g, dir, row);
+            else if constexpr (EW > 0) inline_rows<EW, float>(g, dir, row);
             else all_rows<OFF64, float>(g, term, row, chunk);
             const float al = grid_sums<1, float>(pq, a.parts, flip, a.clustered, [&](const Pair *t) { return s.step(t[0]); });
             Pair z2[2] = {{0.f, 0.f}, {0.f, 0.f}};
@@ -735,6 +769,13 @@ rwc_status solve_one(rwc_graph *G, const double *B, double *X, double tol, int *
         return g.weighted ? launch(cg1_csr<false, true, RES, FU>, tpb, 0, nb) : launch(cg1_csr<false, false, RES, FU>, tpb, 0, nb);
     };
     auto csr = [&](int64_t nb) -> cudaError_t {
+        if (g.ell) {
+            // more rows than cg1_ell's registers hold
+            if (fused) return g.ell_w == 4 ? launch(cg1_csr<false, false, false, true, 4>, CSR_TPB, 0, nb)
+                                           : launch(cg1_csr<false, false, false, true, 8>, CSR_TPB, 0, nb);
+            return g.ell_w == 4 ? launch(cg1_csr<false, false, false, false, 4>, CSR_TPB, 0, nb)
+                                : launch(cg1_csr<false, false, false, false, 8>, CSR_TPB, 0, nb);
+        }
         if (held && nb == blocks) return csr_of(std::true_type{}, std::true_type{}, RES_TPB, nb);
         if (fused) return csr_of(std::false_type{}, std::true_type{}, CSR_TPB, nb);
         return csr_of(std::false_type{}, std::false_type{}, CSR_TPB, nb);
