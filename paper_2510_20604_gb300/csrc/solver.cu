@@ -56,7 +56,7 @@ struct Tile {
         : q(blockIdx.y * qt + threadIdx.x % qt), rs(threadIdx.x / qt), slots(blockDim.x / qt) {
         u0 = (int64_t)blockIdx.x * slots + rs;
         step = (int64_t)gridDim.x * slots;
-        on = q < k4;
+        on = q < k4 && rs < slots;
     }
 };
 
@@ -97,10 +97,12 @@ __device__ __forceinline__ void dot4(Pair (&a)[4], const float4 &x, const float4
     pair_fma(a[0], x.x, y.x); pair_fma(a[1], x.y, y.y); pair_fma(a[2], x.z, y.z); pair_fma(a[3], x.w, y.w);
 }
 
-// Rows of more arcs are shared by a block's slots: one slot takes about 150 cycles
-// per arc, so the hub of a BA graph of 9000 vertices alone took longer than the
-// rest of the product.
-constexpr int WIDE_ROW = 128;
+// One slot takes about 150 cycles per arc, so a hub row alone takes longer than the
+// rest of the product.  With more than SHARE_QUADS quads of columns the rows of more
+// than WIDE_ROW arcs are shared by a block's slots.  With fewer, a warp holds several
+// arcs of a quad side by side: it takes each row of 17 to 1024 arcs (the last degree
+// bin) by itself, and a block's slots share the heavy rows.
+constexpr int WIDE_ROW = 128, SHARE_QUADS = 16, SHARE_ROW = 16;
 
 // Q = L P and the parts of <P, Q>.  Four neighbour rows are in flight.
 template <bool OFF64, bool W>
@@ -108,11 +110,20 @@ __global__ void __launch_bounds__(TPB) bcg_product(DevGraph g, int k4, int qt, c
                                                    float4 *__restrict__ Q, double *parts) {
     const Tile t(k4, qt);
     Pair a[4] = {};
+    const bool warps = qt <= SHARE_QUADS;
+    const int64_t alone = warps ? SHARE_ROW : WIDE_ROW;
+    auto finish = [&](int64_t u, const float4 &s) {
+        const float d = (float)g.d[u];
+        const float4 p = P[u * k4 + t.q];
+        const float4 q = {d * p.x - s.x, d * p.y - s.y, d * p.z - s.z, d * p.w - s.w};
+        Q[u * k4 + t.q] = q;
+        dot4(a, p, q);
+    };
     if (t.on)
         for (int64_t u = t.u0; u < g.n; u += t.step) {
             int64_t b, e;
             rowb<OFF64>(g, u, b, e);
-            if (e - b > WIDE_ROW) continue;
+            if (e - b > alone) continue;
             float4 s0 = {}, s1 = {};
             int64_t j = b;
             for (; j + 4 <= e; j += 4) {
@@ -126,44 +137,64 @@ __global__ void __launch_bounds__(TPB) bcg_product(DevGraph g, int k4, int qt, c
                 fma4(s0, w[0], v[0]); fma4(s1, w[1], v[1]); fma4(s0, w[2], v[2]); fma4(s1, w[3], v[3]);
             }
             for (; j < e; ++j) fma4(s0, W ? g.w[j] : 1.f, P[(int64_t)g.col[j] * k4 + t.q]);
-            const float d = (float)g.d[u];
-            const float4 p = P[u * k4 + t.q];
-            const float4 q = {d * p.x - (s0.x + s1.x), d * p.y - (s0.y + s1.y), d * p.z - (s0.z + s1.z),
-                              d * p.w - (s0.w + s1.w)};
-            Q[u * k4 + t.q] = q;
-            dot4(a, p, q);
+            fma4(s0, 1.f, s1);
+            finish(u, s0);
         }
-    // longer rows: the block's slots share the arcs of one
     __shared__ float4 hs[TPB];
-    for (int64_t base = (int64_t)blockIdx.x * t.slots; base < g.n; base += t.step) {
-        int64_t b = 0, e = 0;
-        if (base + t.rs < g.n) rowb<OFF64>(g, base + t.rs, b, e);
-        if (!__syncthreads_or(e - b > WIDE_ROW)) continue;
-        for (int r = 0; r < t.slots && base + r < g.n; ++r) {
-            const int64_t u = base + r;
-            rowb<OFF64>(g, u, b, e);
-            if (e - b <= WIDE_ROW) continue;
-            float4 s = {};
-            if (t.on)
+    // a row's arcs shared by the block's slots
+    auto by_block = [&](int64_t u, int64_t b, int64_t e) {
+        float4 s = {};
+        if (t.on)
 #pragma unroll 4
-                for (int64_t j = b + t.rs; j < e; j += t.slots) fma4(s, W ? g.w[j] : 1.f, P[(int64_t)g.col[j] * k4 + t.q]);
-            hs[threadIdx.x] = s;
-            int h = 1;
-            while (h < t.slots) h *= 2;
-            for (h /= 2; h > 0; h /= 2) {
-                __syncthreads();
-                if (t.rs < h && t.rs + h < t.slots) fma4(hs[threadIdx.x], 1.f, hs[threadIdx.x + h * qt]);
-            }
+            for (int64_t j = b + t.rs; j < e; j += t.slots) fma4(s, W ? g.w[j] : 1.f, P[(int64_t)g.col[j] * k4 + t.q]);
+        hs[threadIdx.x] = s;
+        int h = 1;
+        while (h < t.slots) h *= 2;
+        for (h /= 2; h > 0; h /= 2) {
             __syncthreads();
-            if (t.rs == 0 && t.on) {
-                s = hs[threadIdx.x];
-                const float d = (float)g.d[u];
-                const float4 p = P[u * k4 + t.q];
-                const float4 q = {d * p.x - s.x, d * p.y - s.y, d * p.z - s.z, d * p.w - s.w};
-                Q[u * k4 + t.q] = q;
-                dot4(a, p, q);
+            if (t.rs < h && t.rs + h < t.slots) fma4(hs[threadIdx.x], 1.f, hs[threadIdx.x + h * qt]);
+        }
+        __syncthreads();
+        if (t.rs == 0 && t.on) finish(u, hs[threadIdx.x]);
+        __syncthreads();
+    };
+    if (warps) {
+        // lanes of a warp as arcs x quads (rotated where qt does not divide 32)
+        const int lane = threadIdx.x & 31, na = 32 / qt, al = lane / qt;
+        const bool on = al < na && t.q < k4;
+        int top = 1;
+        while (top < na) top *= 2;
+        const int32_t *rows = g.bin_rows + g.bin_off[4];
+        const int64_t nrows = g.bin_off[5] - g.bin_off[4], nw = (int64_t)gridDim.x * (TPB / 32);
+        for (int64_t i = (int64_t)blockIdx.x * (TPB / 32) + (threadIdx.x >> 5); i < nrows; i += nw) {
+            const int64_t u = rows[i];
+            int64_t b, e;
+            rowb<OFF64>(g, u, b, e);
+            float4 s = {};
+            if (on)
+#pragma unroll 4
+                for (int64_t j = b + al; j < e; j += na) fma4(s, W ? g.w[j] : 1.f, P[(int64_t)g.col[j] * k4 + t.q]);
+            for (int h = top / 2; h > 0; h /= 2) {
+                const float4 o = {__shfl_down_sync(0xffffffffu, s.x, h * qt), __shfl_down_sync(0xffffffffu, s.y, h * qt),
+                                  __shfl_down_sync(0xffffffffu, s.z, h * qt), __shfl_down_sync(0xffffffffu, s.w, h * qt)};
+                if (al < h && al + h < na) fma4(s, 1.f, o);
             }
-            __syncthreads();
+            if (on && al == 0) finish(u, s);
+        }
+        for (int64_t c = blockIdx.x; c < g.hc_n; c += gridDim.x) {
+            int64_t b, e;
+            rowb<OFF64>(g, g.hc_row[c], b, e);
+            if (g.hc_beg[c] == b) by_block(g.hc_row[c], b, e);
+        }
+    } else {
+        for (int64_t base = (int64_t)blockIdx.x * t.slots; base < g.n; base += t.step) {
+            int64_t b = 0, e = 0;
+            if (t.rs < t.slots && base + t.rs < g.n) rowb<OFF64>(g, base + t.rs, b, e);
+            if (!__syncthreads_or(e - b > WIDE_ROW)) continue;
+            for (int r = 0; r < t.slots && base + r < g.n; ++r) {
+                rowb<OFF64>(g, base + r, b, e);
+                if (e - b > WIDE_ROW) by_block(base + r, b, e);
+            }
         }
     }
     quad_parts(t, a, qt, parts);
@@ -372,8 +403,11 @@ rwc_status solve_nodemajor(rwc_graph *G, int k, const double *B, double *X, doub
     // blocks: qt quads of columns x TPB / qt row slots; nb row ranges, fewer for
     // many column tiles (the parts are [kp][nb])
     const int qt = std::min(k4, 64), threads = qt * (TPB / qt), tiles = (k4 + qt - 1) / qt;
+    const int64_t rows_nb = (n + threads / qt - 1) / (threads / qt);
+    // a warp for each row that is not one slot's
+    const int64_t wide_nb = qt <= SHARE_QUADS ? (g.bin_off[5] - g.bin_off[4] + TPB / 32 - 1) / (TPB / 32) : 0;
     const unsigned nb = (unsigned)std::max<int64_t>(1, std::min<int64_t>(((int64_t)num_sms() * 6 + tiles - 1) / tiles,
-                                                                         (n + threads / qt - 1) / (threads / qt)));
+                                                                         std::max(rows_nb, wide_nb)));
     const dim3 grid(nb, (unsigned)tiles);
     const int ct = std::min(k, 128), rthreads = ct * (TPB / ct);
     const dim3 rgrid((unsigned)std::max<int64_t>(1, std::min<int64_t>((int64_t)num_sms() * 8, (n * ct + rthreads - 1) / rthreads)),
@@ -444,7 +478,7 @@ rwc_status solve_nodemajor(rwc_graph *G, int k, const double *B, double *X, doub
                 double *z0 = rz[it & 1], *z1 = rz[(it & 1) ^ 1];
                 ::rwc::count_launches(5);
                 dispatch(g, [&](auto o64, auto wt) {
-                    bcg_product<decltype(o64)::value, decltype(wt)::value><<<grid, threads, 0, st>>>(g, k4, qt, p, q, pa);
+                    bcg_product<decltype(o64)::value, decltype(wt)::value><<<grid, TPB, 0, st>>>(g, k4, qt, p, q, pa);
                 });
                 sum_cols<<<dim3((unsigned)kp, 1), 128, 0, st>>>(pa, nullptr, (int)nb, pq, nullptr);
                 bcg_residual<<<grid, threads, 0, st>>>(n, k4, qt, z0, pq, g.dinv32, q, r, pa, pb);

@@ -20,7 +20,7 @@ def _scaled(g, e):
     return synth.graphs.Graph(g.n, g.row_ptr, g.col, np.ldexp(g.w, e).astype(np.float32))
 
 
-@pytest.mark.parametrize("e", [-80, 80, 110])
+@pytest.mark.parametrize("e", [-110, -80, 80, 110])
 @pytest.mark.parametrize("k", [1, 3])
 @pytest.mark.parametrize("kind", list(GRAPHS))
 def test_solve_with_scaled_weights(kind, k, e):
