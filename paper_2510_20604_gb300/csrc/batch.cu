@@ -147,13 +147,18 @@ struct rwc_batch {
     int warp = 1;
     int tile = 4;
     int conc = 1;                      // 1: the classes run concurrently (forked streams)
-    cudaStream_t side[MAX_BINS] = {};  // the bins' streams (forked from the call's)
+    cudaStream_t side[MAX_BINS] = {};  // the bins' streams (forked from the call's), made with the bins
     cudaEvent_t fork = nullptr, join[MAX_BINS] = {};
     int32_t *items[2] = {nullptr, nullptr};   // each class's graphs, the largest first
     int max_n[2] = {0, 0};             // largest n of each class
     std::vector<Bin> bins;
     uint32_t *spill = nullptr;         // the bins' pending ends beyond shared memory
-    int32_t *single = nullptr;         // graph ids 0 .. G - 1 (one launch per graph)
+    // one launch per graph: graph ids 0 .. G - 1, each graph's resident blocks
+    // (made on first use) and their pending ends beyond shared memory
+    int32_t *single = nullptr;
+    std::vector<int64_t> single_blocks;
+    uint32_t *single_spill = nullptr;
+    int64_t single_spill_n = 0;
     int64_t items_T = -1;              // T the bins were built for
     int64_t items_split = -1;
     void *scratch = nullptr;           // [0] err, [8] rounds, [16] draws, [64..160) the bins' counters
@@ -174,6 +179,14 @@ cudaError_t balloc(rwc_batch *b, void **p, size_t bytes) {
     cudaError_t e = cudaMalloc(p, bytes ? bytes : 16);
     if (e == cudaSuccess) b->allocs.push_back(*p);
     return e;
+}
+
+template <class T>
+void bfree(rwc_batch *b, T *&p) {
+    if (!p) return;
+    cudaFree(p);
+    b->allocs.erase(std::find(b->allocs.begin(), b->allocs.end(), (void *)p));
+    p = nullptr;
 }
 
 void drop_graph(rwc_batch *b) {
@@ -203,6 +216,32 @@ size_t schedule_allowance(int max_large, int max_small, int warp) {
 }
 size_t batch_smem(const rwc_batch *b) { return schedule_allowance(b->max_n[0], b->max_n[1], b->warp); }
 
+// Blocks of nt threads and smem bytes that the device holds at once.
+rwc_status resident_blocks(const rwc_batch *b, int nt, size_t smem, int64_t *out) {
+    int per_sm = 0;
+    cudaError_t e = cudaSuccess;
+    dispatch_nt(b->off64, b->weighted, nt, [&](auto kern) {
+        // one value for all batches: other threads launch the kernel too
+        e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 96 * 1024);
+        if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, nt, smem);
+    });
+    RWC_CUDA_TRY(e);
+    if (per_sm < 1) return set_error(RWC_ERR_UNSUPPORTED, "batch block does not fit on an SM");
+    *out = (int64_t)num_sms() * per_sm;
+    return RWC_OK;
+}
+
+// Resident blocks of each graph's own launch.
+rwc_status plan_single(rwc_batch *b) {
+    std::vector<int64_t> blocks(b->G);
+    for (int32_t g = 0; g < b->G; ++g) {
+        const int n = b->hgraphs[g].n, nt = batch_threads(n);
+        RWC_TRY(resident_blocks(b, nt, batch_tree_smem(n, nt), &blocks[g]));
+    }
+    b->single_blocks = std::move(blocks);
+    return RWC_OK;
+}
+
 rwc_status build_bins(rwc_batch *b, const std::vector<int32_t> (&order)[2], int64_t T) {
     b->bins.clear();
     for (int c = 0; c < 2; ++c)
@@ -223,25 +262,19 @@ rwc_status build_bins(rwc_batch *b, const std::vector<int32_t> (&order)[2], int6
             i = j;
         }
     if (b->bins.size() > (size_t)MAX_BINS) return set_error(RWC_ERR_UNSUPPORTED, "too many size bins");
+    for (size_t i = 1; i < b->bins.size(); ++i) {
+        if (!b->fork) RWC_CUDA_TRY(cudaEventCreateWithFlags(&b->fork, cudaEventDisableTiming));
+        if (!b->side[i]) RWC_CUDA_TRY(cudaStreamCreateWithFlags(&b->side[i], cudaStreamNonBlocking));
+        if (!b->join[i]) RWC_CUDA_TRY(cudaEventCreateWithFlags(&b->join[i], cudaEventDisableTiming));
+    }
     int64_t spill = 0;
     for (Bin &q : b->bins) {
-        int per_sm = 0;
-        cudaError_t e = cudaSuccess;
-        dispatch_nt(b->off64, b->weighted, q.nt, [&](auto kern) {
-            e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)std::max<size_t>(q.smem, 96 * 1024));
-            if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, q.nt, q.smem);
-        });
-        RWC_CUDA_TRY(e);
-        if (per_sm < 1) return set_error(RWC_ERR_UNSUPPORTED, "batch block does not fit on an SM");
-        q.blocks = std::max<int64_t>(1, std::min<int64_t>(q.count * T, (int64_t)num_sms() * per_sm));
+        RWC_TRY(resident_blocks(b, q.nt, q.smem, &q.blocks));
+        q.blocks = std::max<int64_t>(1, std::min<int64_t>(q.count * T, q.blocks));
         q.spill = spill;
         spill += q.blocks * q.max_n;
     }
-    if (b->spill) {
-        cudaFree(b->spill);
-        b->allocs.erase(std::find(b->allocs.begin(), b->allocs.end(), (void *)b->spill));
-        b->spill = nullptr;
-    }
+    bfree(b, b->spill);
     RWC_CUDA_TRY(balloc(b, (void **)&b->spill, (size_t)spill * sizeof(uint32_t)));
     return RWC_OK;
 }
@@ -262,8 +295,7 @@ rwc_status build_items(rwc_batch *b, int64_t T) {
         }
         std::stable_sort(order.begin(), order.end(),
                          [&](int32_t x, int32_t y) { return b->hgraphs[x].n > b->hgraphs[y].n; });
-        if (b->items[c]) { cudaFree(b->items[c]); b->allocs.erase(std::find(b->allocs.begin(), b->allocs.end(), (void *)b->items[c])); }
-        b->items[c] = nullptr;
+        bfree(b, b->items[c]);
         if (!order.empty()) {
             RWC_CUDA_TRY(balloc(b, (void **)&b->items[c], order.size() * sizeof(int32_t)));
             RWC_CUDA_TRY(cudaMemcpy(b->items[c], order.data(), order.size() * sizeof(int32_t), cudaMemcpyHostToDevice));
@@ -430,15 +462,6 @@ extern "C" rwc_status rwc_batch_create(int32_t G, const int64_t *voff, const int
     }
     if ((e = balloc(b, &b->scratch, 256)) != cudaSuccess) return fail(e);
     if ((e = cudaMallocHost((void **)&b->host, 64)) != cudaSuccess) return fail(e);
-    e = cudaEventCreateWithFlags(&b->fork, cudaEventDisableTiming);
-    for (int i = 1; i < MAX_BINS && e == cudaSuccess; ++i) {
-        e = cudaStreamCreateWithFlags(&b->side[i], cudaStreamNonBlocking);
-        if (e == cudaSuccess) e = cudaEventCreateWithFlags(&b->join[i], cudaEventDisableTiming);
-    }
-    if (e != cudaSuccess) {
-        drop_streams(b);
-        return fail(e);
-    }
     *out = b;
     return RWC_OK;
 }
@@ -462,33 +485,25 @@ extern "C" rwc_status rwc_batch_sample(rwc_batch_t *b, uint64_t seed, int64_t T,
         int *err = (int *)b->scratch;
         unsigned long long *ctr = (unsigned long long *)((char *)b->scratch + 8);
         const uint32_t k0 = (uint32_t)seed, k1 = (uint32_t)(seed >> 32);
-        std::vector<int64_t> blocks(b->G);
+        if (b->single_blocks.empty()) RWC_TRY(plan_single(b));
         int64_t spill = 0;
-        cudaError_t e = cudaSuccess;
-        for (int32_t g = 0; g < b->G && e == cudaSuccess; ++g) {
-            const int n = b->hgraphs[g].n, nt = batch_threads(n);
-            const size_t smem = batch_tree_smem(n, nt);
-            int per_sm = 0;
-            dispatch_nt(b->off64, b->weighted, nt, [&](auto kern) {
-                e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)std::max<size_t>(smem, 96 * 1024));
-                if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, nt, smem);
-            });
-            if (e == cudaSuccess && per_sm < 1) return set_error(RWC_ERR_UNSUPPORTED, "graph %d does not fit", g);
-            blocks[g] = std::min<int64_t>(T, (int64_t)num_sms() * per_sm);
-            spill = std::max(spill, blocks[g] * n);
+        for (int32_t g = 0; g < b->G; ++g)
+            if (b->hgraphs[g].n > (int)LT_STACK)
+                spill = std::max(spill, std::min(T, b->single_blocks[g]) * b->hgraphs[g].n);
+        if (spill > b->single_spill_n) {
+            bfree(b, b->single_spill);
+            b->single_spill_n = 0;
+            RWC_CUDA_TRY(balloc(b, (void **)&b->single_spill, (size_t)spill * sizeof(uint32_t)));
+            b->single_spill_n = spill;
         }
-        RWC_CUDA_TRY(e);
-        uint32_t *sp = nullptr;
-        RWC_CUDA_TRY(cudaMallocAsync((void **)&sp, (size_t)spill * sizeof(uint32_t), st));
         for (int32_t g = 0; g < b->G; ++g) {
             const int n = b->hgraphs[g].n, nt = batch_threads(n);
             ::rwc::count_launches(1);
             dispatch_nt(b->off64, b->weighted, nt, [&](auto kern) {
-                kern<<<(unsigned)blocks[g], nt, batch_tree_smem(n, nt), st>>>(
-                    b->base, b->graphs, b->single + g, T, nullptr, T, k0, k1, n, sums, sp, err, ctr);
+                kern<<<(unsigned)std::min(T, b->single_blocks[g]), nt, batch_tree_smem(n, nt), st>>>(
+                    b->base, b->graphs, b->single + g, T, nullptr, T, k0, k1, n, sums, b->single_spill, err, ctr);
             });
         }
-        cudaFreeAsync(sp, st);
         RWC_CUDA_TRY(cudaGetLastError());
         return finish(b, stats, 3, T, st);
     }
