@@ -316,9 +316,9 @@ struct ResidentRows {
         }
     }
 };
-// Units of a graph's rows.
+// Units of a graph's rows, a heavy row's chunks among them.
 inline int64_t row_units(const DevGraph &g) {
-    int64_t t = 0;
+    int64_t t = g.hc_n;
     for (int b = 0; b < 5; ++b) t += (g.bin_off[b + 1] - g.bin_off[b] + (16 >> b) - 1) / (16 >> b);
     return t;
 }

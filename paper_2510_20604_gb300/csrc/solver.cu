@@ -404,8 +404,9 @@ rwc_status solve_nodemajor(rwc_graph *G, int k, const double *B, double *X, doub
     // many column tiles (the parts are [kp][nb])
     const int qt = std::min(k4, 64), threads = qt * (TPB / qt), tiles = (k4 + qt - 1) / qt;
     const int64_t rows_nb = (n + threads / qt - 1) / (threads / qt);
-    // a warp for each row that is not one slot's
-    const int64_t wide_nb = qt <= SHARE_QUADS ? (g.bin_off[5] - g.bin_off[4] + TPB / 32 - 1) / (TPB / 32) : 0;
+    // a warp for each row that is not one slot's, a block for each heavy row
+    const int64_t wide_nb =
+        qt <= SHARE_QUADS ? std::max((g.bin_off[5] - g.bin_off[4] + TPB / 32 - 1) / (TPB / 32), g.hc_n) : 0;
     const unsigned nb = (unsigned)std::max<int64_t>(1, std::min<int64_t>(((int64_t)num_sms() * 6 + tiles - 1) / tiles,
                                                                          std::max(rows_nb, wide_nb)));
     const dim3 grid(nb, (unsigned)tiles);

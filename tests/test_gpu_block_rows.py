@@ -42,3 +42,15 @@ def test_solve_with_hub_rows(weighted, k):
     r = b - (np.asarray(A.sum(1)).ravel() * x - (A @ x.T).T)
     # the solver's criterion, and rounding in the evaluation of r
     assert (np.linalg.norm(r, axis=1) <= 2e-10 * np.linalg.norm(b, axis=1)).all()
+
+
+@pytest.mark.parametrize("n", [1024, 1025, 1026, 1300])
+@pytest.mark.parametrize("k", [1, 3, 70])
+def test_solve_where_every_row_is_heavy(n, k):
+    # L = n I - J: x = b / n for mean-free b
+    b = np.random.default_rng(n).standard_normal((k, n))
+    b -= b.mean(1, keepdims=True)
+    x = torch.empty(k, n, dtype=torch.float64, device="cuda")
+    rwc.rwc_solve(rwc.Graph.from_synth(synth.complete(n)).handle, k, torch.as_tensor(b, device="cuda"), x, 1e-10)
+    err = np.linalg.norm(n * x.cpu().numpy() - b, axis=1)
+    assert (err <= 2e-10 * np.linalg.norm(b, axis=1)).all()
