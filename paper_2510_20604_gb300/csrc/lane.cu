@@ -65,11 +65,14 @@ __global__ void __launch_bounds__(NT) l_trees_smem(DevGraph g, uint32_t tree0, i
 }
 
 // One tree per block of NT threads, its words in global memory (zeroed by the
-// caller), `ld` words apart.
+// caller), `ld` words apart: the trees ids[0 .. B) of the call, or its first B
+// (ids = NULL).  Trees whose counts outgrow the word are listed in wide[0 ..
+// ctr[2]) and their root's word is left 0.
 template <bool OFF64, bool WT, int EW, int NT, class W>
 __global__ void __launch_bounds__(NT) l_trees(DevGraph g, uint32_t tree0, int64_t B, int64_t ld, uint32_t k0,
                                               uint32_t k1, uint32_t klim, int kb, W *words, uint32_t *spill,
-                                              int *err, unsigned long long *ctr) {
+                                              const uint32_t *ids, int *err, unsigned long long *ctr,
+                                              uint32_t *wide) {
     constexpr int S = 2;   // lanes per thread: two loads in flight
     __shared__ LaneShared<NT, S> sh;
     __shared__ unsigned long long sh_next;
@@ -80,23 +83,27 @@ __global__ void __launch_bounds__(NT) l_trees(DevGraph g, uint32_t tree0, int64_
         if (threadIdx.x == 0) word[g.root] = lt_root_word<W>(kb, NT * S);
         __syncthreads();
         uint32_t rounds = 0;
-        const int bad = lane_tree<OFF64, WT, EW, NT, S, false, W>(g, word, kb, klim, sh, sp, tree0 + (uint32_t)t, 0u,
-                                                                  k0, k1, rounds);
-        if (bad) { if (threadIdx.x == 0) atomicOr(err, bad); break; }
+        const int bad = lane_tree<OFF64, WT, EW, NT, S, false, W>(g, word, kb, klim, sh, sp,
+                                                                  tree0 + (ids ? ids[t] : (uint32_t)t), 0u, k0, k1,
+                                                                  rounds);
+        if (bad & ~LE_KREP) { if (threadIdx.x == 0) atomicOr(err, bad); break; }
+        if (bad && threadIdx.x == 0) { wide[atomicAdd(ctr + 2, 1ull)] = (uint32_t)t; word[g.root] = 0; }
         if (threadIdx.x == 0) sh_next = atomicAdd(ctr, 1ull);
         __syncthreads();
         t = (int64_t)gridDim.x + (int64_t)sh_next;
     }
 }
 
-// visits_u = k_u + 1 over the chunk's trees into sums; optional per-tree
-// output.  Nothing after an error (the chunk is then sampled again).  The trees
-// are split over gridDim.y so that small graphs fill the chip too; the sums are
+// visits_u = k_u + 1 over the chunk's trees into sums, without the listed ones
+// (root's word 0); optional per-tree output (rows ids[t]).  Nothing after an
+// error.  The trees are split over gridDim.y so that small graphs fill the chip too; the sums are
 // whole numbers, exact in any order.
 template <class W>
-__global__ void l_accum(int64_t n, int32_t root, const W *words, int64_t ld, int kb, uint32_t id0, int64_t B, double *sums,
-                        int32_t *parents, int32_t *visits, const int *err, unsigned long long *draws) {
+__global__ void l_accum(int64_t n, int32_t root, const W *words, int64_t ld, int kb, uint32_t id0, int64_t B,
+                        const uint32_t *ids, double *sums, int32_t *parents, int32_t *visits, const int *err,
+                        unsigned long long *ctr) {
     if (*err) return;
+    const bool listed = ctr[2] != 0;
     const W kmask = ((W)1 << kb) - 1, pmask = ~(W)0 >> 1;
     const int64_t t0 = B * blockIdx.y / gridDim.y, t1 = B * (blockIdx.y + 1) / gridDim.y;
     unsigned long long local = 0;
@@ -105,17 +112,21 @@ __global__ void l_accum(int64_t n, int32_t root, const W *words, int64_t ld, int
         unsigned long long acc = 0;
 #pragma unroll 4
         for (int64_t t = t0; t < t1; ++t) {
+            if (listed && words[t * ld + root] == 0) continue;
             const W w = words[t * ld + u];
             const uint32_t vis = u == root ? 0u : (uint32_t)(w & kmask) + 1u;
             acc += vis;
-            if (parents) parents[t * n + u] = u == root ? -1 : (int32_t)((uint32_t)((w & pmask) >> kb) - id0);
-            if (visits) visits[t * n + u] = (int32_t)vis;
+            if (parents || visits) {
+                const int64_t row = ids ? ids[t] : t;
+                if (parents) parents[row * n + u] = u == root ? -1 : (int32_t)((uint32_t)((w & pmask) >> kb) - id0);
+                if (visits) visits[row * n + u] = (int32_t)vis;
+            }
         }
         local += acc;
         if (sums && acc) atomicAdd(sums + u, (double)acc);
     }
     for (int o = 16; o > 0; o >>= 1) local += __shfl_xor_sync(0xffffffffu, local, o);
-    if ((threadIdx.x & 31) == 0 && local) atomicAdd(draws, local);
+    if ((threadIdx.x & 31) == 0 && local) atomicAdd(ctr + 1, local);
 }
 
 template <int V> using int_c = std::integral_constant<int, V>;
@@ -153,9 +164,14 @@ constexpr size_t SMEM_MAX = 226 * 1024;   // dynamic shared memory of one block 
 constexpr int64_t TAIL = 64;   // err @0, next tree @8, draws @16, listed trees @24, rounds @32
 constexpr int64_t WIDE_CAP = 65536;   // trees of one shared-memory launch
 
+// Trees tree0 .. tree0 + T - 1 (`only`: the T trees tree0 + only[i], a part of
+// a call whose other trees are done) with words of type W.  With 32-bit words the
+// trees whose counts outgrow them are appended to `redo`, and a chunk that lists
+// more than half of its trees is the last: *done trees have been taken.
 template <int NT, class W>
-rwc_status walker_range(rwc_graph *G, uint64_t seed, int64_t tree0, int64_t T, double *sums, int32_t *parents,
-                        int32_t *visits, const rwc_options_t &o, rwc_stats_t *st, cudaStream_t stream) {
+rwc_status walker_range(rwc_graph *G, uint64_t seed, int64_t tree0, int64_t T, const uint32_t *only, double *sums,
+                        int32_t *parents, int32_t *visits, const rwc_options_t &o, rwc_stats_t *st,
+                        std::vector<uint32_t> *redo, int64_t *done, cudaStream_t stream) {
     const DevGraph &g = G->g;
     const int64_t n = g.n, ld = (n + 3) & ~(int64_t)3;
     const uint32_t klim = (1u << 20) - 1u;
@@ -175,7 +191,6 @@ rwc_status walker_range(rwc_graph *G, uint64_t seed, int64_t tree0, int64_t T, d
         B = (int64_t)std::max<size_t>(1, budget / per_tree);
     }
     B = std::min(B, T);
-    rwc_status status = RWC_OK;
     int per_sm = 0;
     dispatch(g, [&](auto o64, auto wt, auto ew) {
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(
@@ -185,34 +200,38 @@ rwc_status walker_range(rwc_graph *G, uint64_t seed, int64_t tree0, int64_t T, d
     const int64_t slots = std::min<int64_t>(B, (int64_t)sms * per_sm);
     Buf buf(stream);
     const size_t wbytes = (size_t)B * ld * sizeof(W);
-    RWC_CUDA_TRY(cudaMallocAsync(&buf.p, wbytes + (size_t)slots * n * 4 + TAIL + 64, stream));
+    RWC_CUDA_TRY(cudaMallocAsync(&buf.p, wbytes + (size_t)slots * n * 4 + (size_t)B * 8 + TAIL + 64, stream));
     W *words = (W *)buf.p;
     uint32_t *spill = (uint32_t *)((char *)buf.p + wbytes);
-    char *tail = (char *)(spill + slots * n);
+    uint32_t *ids = spill + slots * n, *wide = ids + B;
+    char *tail = (char *)(wide + B);
     tail = (char *)(((uintptr_t)tail + 63) & ~(uintptr_t)63);
     int *err = (int *)tail;
     unsigned long long *ctr = (unsigned long long *)(tail + 8);
     Events ev(o.profile != 0);
     int64_t *h = G->host_scalars;
+    if (st) st->mode = RWC_MODE_WALKER;
     for (int64_t c0 = 0; c0 < T; c0 += B) {
-        const int64_t Bc = std::min(B, T - c0);
-        int32_t *par = parents ? parents + c0 * n : nullptr, *vis = visits ? visits + c0 * n : nullptr;
+        const int64_t Bc = std::min(B, T - c0), first = only ? 0 : c0;
+        int32_t *par = parents ? parents + first * n : nullptr, *vis = visits ? visits + first * n : nullptr;
         RWC_CUDA_TRY(cudaMemsetAsync(tail, 0, TAIL, stream));
+        if (only) RWC_CUDA_TRY(cudaMemcpyAsync(ids, only + c0, (size_t)Bc * 4, cudaMemcpyHostToDevice, stream));
+        const uint32_t *list = only ? ids : nullptr;
         ev.rec(0, stream);
         RWC_CUDA_TRY(cudaMemsetAsync(words, 0, (size_t)Bc * ld * sizeof(W), stream));
         ev.rec(1, stream);
         dispatch(g, [&](auto o64, auto wt, auto ew) {
             ::rwc::count_launches(1);
             l_trees<decltype(o64)::value, decltype(wt)::value, decltype(ew)::value, NT, W>
-                <<<(unsigned)std::min(Bc, slots), NT, 0, stream>>>(g, (uint32_t)(tree0 + c0), Bc, ld, k0, k1, klim,
-                                                                   kb, words, spill, err, ctr);
+                <<<(unsigned)std::min(Bc, slots), NT, 0, stream>>>(g, (uint32_t)(tree0 + first), Bc, ld, k0, k1, klim,
+                                                                   kb, words, spill, list, err, ctr, wide);
         });
         ev.rec(2, stream);
         const int64_t bx = std::min<int64_t>((n + 255) / 256, (int64_t)sms * 8);
         const int64_t by = std::max<int64_t>(1, std::min<int64_t>((int64_t)sms * 8 / bx, Bc / 8));
         ::rwc::count_launches(1);
-        l_accum<W><<<dim3((unsigned)bx, (unsigned)by), 256, 0, stream>>>(n, g.root, words, ld, kb, lt_id0(NL), Bc, sums, par,
-                                                                         vis, err, ctr + 1);
+        l_accum<W><<<dim3((unsigned)bx, (unsigned)by), 256, 0, stream>>>(n, g.root, words, ld, kb, lt_id0(NL), Bc, list,
+                                                                         sums, par, vis, err, ctr);
         ev.rec(3, stream);
         RWC_CUDA_TRY(cudaGetLastError());
         if (o.async_status) {
@@ -221,20 +240,14 @@ rwc_status walker_range(rwc_graph *G, uint64_t seed, int64_t tree0, int64_t T, d
             RWC_CUDA_TRY(cudaGetLastError());
             continue;
         }
-        RWC_CUDA_TRY(cudaMemcpyAsync(h, tail, 24, cudaMemcpyDeviceToHost, stream));
+        RWC_CUDA_TRY(cudaMemcpyAsync(h, tail, 32, cudaMemcpyDeviceToHost, stream));
         RWC_CUDA_TRY(cudaStreamSynchronize(stream));
         const int e = (int)(h[0] & 0xffffffff);
         if (e & LE_KOVF) return set_error(RWC_ERR_UNSUPPORTED, "a vertex was popped more than 2^20 - 1 times");
-        if (e & LE_LOOP) return set_error(RWC_ERR_CUDA, "sampler internal check failed");
-        if (e & LE_KREP) {
-            // a count outgrew the 32-bit word: this chunk again with 64-bit words
-            if (sizeof(W) == 8) return set_error(RWC_ERR_CUDA, "sampler internal check failed");
-            RWC_TRY((walker_range<NT, uint64_t>(G, seed, tree0 + c0, Bc, sums, par, vis, o, st, stream)));
-            continue;
-        }
+        if (e) return set_error(RWC_ERR_CUDA, "sampler internal check failed");
         if (st) {
             const int64_t draws = h[2];
-            st->chunks += 1;
+            if (!only) st->chunks += 1;
             st->draws += draws;
             st->marked += draws;
             st->block_threads = NL;
@@ -249,9 +262,40 @@ rwc_status walker_range(rwc_graph *G, uint64_t seed, int64_t tree0, int64_t T, d
                 st->phase_launches[RWC_PHASE_ACCUM] += 1;
             }
         }
+        if (const int64_t listed = h[3]) {
+            if (!redo) return set_error(RWC_ERR_CUDA, "sampler internal check failed");   // 64-bit words hold every allowed count
+            const size_t at = redo->size();
+            redo->resize(at + (size_t)listed);
+            RWC_CUDA_TRY(cudaMemcpyAsync(redo->data() + at, wide, (size_t)listed * 4, cudaMemcpyDeviceToHost, stream));
+            RWC_CUDA_TRY(cudaStreamSynchronize(stream));
+            for (size_t i = at; i < redo->size(); ++i) (*redo)[i] += (uint32_t)c0;
+            if (2 * listed > Bc) { *done = c0 + Bc; return RWC_OK; }
+        }
     }
-    if (st) st->mode = RWC_MODE_WALKER;
-    return status;
+    if (done) *done = T;
+    return RWC_OK;
+}
+
+// f(threads per tree) for T trees with words in global memory, by the trees that an SM
+// gets: 32 (64 lanes) when they fill it, more when few are left to it (300 x 300
+// grid, 300 trees: 572, 429 and 449 ms with 32, 128 and 512; 512 x 512, 64 trees:
+// 2.01, 1.44, 1.18 s); graphs of unbounded degree have ends for 1024 lanes (R-MAT n
+// = 262144, 2000 trees: 101, 60 and 48 ms).
+template <class F>
+rwc_status with_threads(const DevGraph &g, int64_t T, F f) {
+    const int64_t share = (T + num_sms() - 1) / num_sms();
+    if (g.ell && share >= 8) return f(int_c<32>{});
+    if (g.ell && share >= 2) return f(int_c<128>{});
+    return f(int_c<512>{});
+}
+
+// Trees of a call with 64-bit words.
+rwc_status wide_trees(rwc_graph *G, uint64_t seed, int64_t tree0, int64_t T, const uint32_t *only, double *sums,
+                      int32_t *parents, int32_t *visits, const rwc_options_t &o, rwc_stats_t *st, cudaStream_t stream) {
+    return with_threads(G->g, T, [&](auto nt) {
+        return walker_range<decltype(nt)::value, uint64_t>(G, seed, tree0, T, only, sums, parents, visits, o, st, nullptr,
+                                                           nullptr, stream);
+    });
 }
 
 }  // namespace
@@ -317,8 +361,9 @@ rwc_status smem_range(rwc_graph *G, uint64_t seed, int64_t tree0, int64_t T, dou
     *h_err = (int)(h[0] & 0xffffffff);
     if (*h_err) return RWC_OK;
     if (h[3]) {
-        redo.resize((size_t)h[3]);
-        RWC_CUDA_TRY(cudaMemcpyAsync(redo.data(), (char *)buf.p + TAIL, redo.size() * 4, cudaMemcpyDeviceToHost, stream));
+        const size_t at = redo.size();
+        redo.resize(at + (size_t)h[3]);
+        RWC_CUDA_TRY(cudaMemcpyAsync(redo.data() + at, (char *)buf.p + TAIL, (size_t)h[3] * 4, cudaMemcpyDeviceToHost, stream));
         RWC_CUDA_TRY(cudaStreamSynchronize(stream));
     }
     if (st) {
@@ -351,23 +396,21 @@ rwc_status sample_smem(rwc_graph *G, uint64_t seed, int64_t tree0, int64_t T, do
     while (NTs > 64 && NTs * std::min<int64_t>((227 * 1024) / (int64_t)(lane_smem(n, NTs) + 1024),
                                                (chunk + num_sms() - 1) / num_sms()) > 1024)
         NTs /= 2;
+    std::vector<uint32_t> redo;
     for (int64_t c0 = 0; c0 < T; c0 += chunk) {
         const int64_t Tc = std::min(chunk, T - c0);
         int32_t *par = parents ? parents + c0 * n : nullptr, *vis = visits ? visits + c0 * n : nullptr;
-        std::vector<uint32_t> redo;
+        const size_t at = redo.size();
         if (NTs == 256) RWC_TRY(smem_range<256>(G, seed, tree0 + c0, Tc, sums, par, vis, klim, o, st, redo, err, stream));
         else if (NTs == 128) RWC_TRY(smem_range<128>(G, seed, tree0 + c0, Tc, sums, par, vis, klim, o, st, redo, err, stream));
         else RWC_TRY(smem_range<64>(G, seed, tree0 + c0, Tc, sums, par, vis, klim, o, st, redo, err, stream));
         if (*err) return RWC_OK;
-        // trees whose counts outgrew 32-bit words, again with 64-bit ones
-        for (uint32_t t : redo)
-            RWC_TRY((walker_range<256, uint64_t>(G, seed, tree0 + c0 + t, 1, sums, par ? par + (int64_t)t * n : nullptr,
-                                                 vis ? vis + (int64_t)t * n : nullptr, o, st, stream)));
-        if (st) {
-            st->chunks -= (int64_t)redo.size();
-            st->block_threads = NTs;
-        }
+        for (size_t i = at; i < redo.size(); ++i) redo[i] += (uint32_t)c0;
     }
+    // trees whose counts outgrew 32-bit words, again with 64-bit ones, side by side
+    if (!redo.empty())
+        RWC_TRY(wide_trees(G, seed, tree0, (int64_t)redo.size(), redo.data(), sums, parents, visits, o, st, stream));
+    if (st) st->block_threads = NTs;
     return RWC_OK;
 }
 }  // namespace
@@ -408,24 +451,27 @@ rwc_status sample_lane_walker(rwc_graph *G, uint64_t seed, int64_t tree0, int64_
         if (st) { st->mode = RWC_MODE_WALKER; st->rounds = 0; }
         return RWC_OK;
     }
-    auto run = [&](auto nt) -> rwc_status {
+    std::vector<uint32_t> redo;
+    int64_t done = 0;
+    RWC_TRY(with_threads(G->g, T, [&](auto nt) -> rwc_status {
         constexpr int NT = decltype(nt)::value;
-        // 64-bit words at once where 32 bits leave less than 8 for the count,
-        // and for asynchronous calls unless every allowed count fits
+        // 64-bit words at once where 32 bits leave less than 8 for the count, and for
+        // asynchronous calls unless every allowed count fits.  With 8 bits (2048 x 2048
+        // grid: mean count 21, one tree in 64 beyond 255) wide words take 8% longer,
+        // a repeated tree as long as a lone one (64 trees: 20.2 s in wide words,
+        // 31.9 s with one of them repeated): narrow words for a few trees, which rarely
+        // have one to repeat, and for many, beside which it does not count.
         const int kb = n < ((int64_t)1 << 30) ? lt_kbits<uint32_t>(n, 2 * NT) : 0;
-        if (kb < (o.async_status ? 20 : 8))
-            return walker_range<NT, uint64_t>(G, seed, tree0, T, sums, parents, visits, o, st, stream);
-        return walker_range<NT, uint32_t>(G, seed, tree0, T, sums, parents, visits, o, st, stream);
-    };
-    // threads per tree by the trees that an SM gets: 32 (64 lanes) when they
-    // fill it, more when few are left to it (300 x 300 grid, 300 trees: 572, 429
-    // and 449 ms with 32, 128 and 512; 512 x 512, 64 trees: 2.01, 1.44, 1.18 s);
-    // graphs of unbounded degree have ends for 1024 lanes (R-MAT n = 262144, 2000
-    // trees: 101, 60 and 48 ms)
-    const int64_t share = (T + num_sms() - 1) / num_sms();
-    if (G->g.ell && share >= 8) return run(int_c<32>{});
-    if (G->g.ell && share >= 2) return run(int_c<128>{});
-    return run(int_c<512>{});
+        const bool some = T >= 16 && T < 4 * (int64_t)num_sms();
+        if (kb < (o.async_status ? 20 : some ? 9 : 8)) return RWC_OK;
+        return walker_range<NT, uint32_t>(G, seed, tree0, T, nullptr, sums, parents, visits, o, st, &redo, &done, stream);
+    }));
+    if (!redo.empty())
+        RWC_TRY(wide_trees(G, seed, tree0, (int64_t)redo.size(), redo.data(), sums, parents, visits, o, st, stream));
+    if (done < T)
+        RWC_TRY(wide_trees(G, seed, tree0 + done, T - done, nullptr, sums, parents ? parents + done * n : nullptr,
+                           visits ? visits + done * n : nullptr, o, st, stream));
+    return RWC_OK;
 }
 
 rwc_status sample_lane_shared(rwc_graph *G, uint64_t seed, int64_t tree0, int64_t T, double *sums,

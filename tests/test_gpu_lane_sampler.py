@@ -142,3 +142,18 @@ def test_stacks_are_refilled_in_a_batch():
         for i, g in enumerate(gs):
             ref = ow.Sampler(g, root=int(roots[i]), seed=11, graph_id=i).sample(0, 6)
             assert np.array_equal(sums[o[i]:o[i + 1]], ref["sums"]), (sched, i)
+
+
+@pytest.mark.parametrize("chunk", [0, 1, 2])
+def test_counts_beyond_global_words_repeat_only_their_trees(chunk):
+    # above the shared-memory size 32-bit words leave 15 bits for the count; one
+    # tree, a part or all of a chunk's trees are listed
+    g, hub = _heavy_pair(60000, 3e5)
+    opt = rwc.Options(mode=rwc.MODE_WALKER, trees_per_chunk=chunk)
+    G = rwc.Graph.from_synth(g, root=hub)
+    _, _, _, vis = G.sample(7, want_trees=True, opt=opt)
+    big = (vis.max(1).values > 32768).sum().item()
+    assert 0 < big < 7
+    _exact(g, 7, opt, root=hub)
+    g, hub = _heavy_pair(60000, 2e6)
+    _exact(g, 5, opt, root=hub)
