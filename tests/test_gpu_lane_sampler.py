@@ -157,3 +157,14 @@ def test_counts_beyond_global_words_repeat_only_their_trees(chunk):
     _exact(g, 7, opt, root=hub)
     g, hub = _heavy_pair(60000, 2e6)
     _exact(g, 5, opt, root=hub)
+
+
+@pytest.mark.parametrize("n", [2, 3, 33, 93, 94, 95, 222, 223, 448, 449])
+def test_small_trees_by_one_warp(n):
+    # p' takes one more bit at n + 34 = 2^b; blocks of one warp up to 448 vertices
+    for g in (synth.path(n), synth.ba(n, 2, seed=n) if n > 5 else synth.complete(n)):
+        st = _exact(g, 5)
+        _exact(g, 5, rwc.Options(mode=rwc.MODE_WALKER), tree0=9)
+        assert st.block_threads == (32 if n <= 448 else 256)
+    if n >= 3:
+        _exact(synth.cycle(n), 3)
