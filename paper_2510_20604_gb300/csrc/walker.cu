@@ -101,9 +101,11 @@ __global__ void w_init(int64_t n, int32_t root, uint64_t *word, int64_t B) {
 }
 
 // Entries of a tree's retry queue.  A walker adds one only after it has taken a
-// start, so a queue that is within two blocks of full (a block's walkers may
-// each add one, and each may still be emptying a slot) only has to hand out its
-// own entries before fresh starts.  R-MAT 20, 2000 trees: 8.4 GB less scratch to
+// start, so a queue that is half full only has to hand out its own entries before
+// fresh starts: it then holds at most half and one per walker (512), and 1536 starts
+// and more pass between a walker's taking of an entry and the next use of its slot,
+// which the walker empties at once.  Its length is read head first: the head may move
+// on in between, which makes the queue look longer, never shorter.  R-MAT 20, 2000 trees: 8.4 GB less scratch to
 // map and clear on every call, 292 -> 275 ms (281 ms with 65536 entries).
 constexpr int RETRY_CAP = 4096;
 
@@ -283,8 +285,11 @@ __global__ void __maxnreg__(RWC_WALKER_MAXNREG) w_trees(DevGraph g, WState s, in
                 // the prefetched fresh start, else a fresh one, else a requeued one
                 int idx = -1;
                 int32_t sv = -1;
-                const bool full = s.rcap < nstart &&
-                                  vread(&sh_rtail) - vread(&sh_rhead) >= s.rcap - 2 * (int)blockDim.x;
+                bool full = false;
+                if (s.rcap < nstart) {
+                    const int hd = vread(&sh_rhead);
+                    full = vread(&sh_rtail) - hd >= s.rcap / 2;
+                }
                 if (pend_idx >= 0 && !full) {
                     idx = pend_idx; sv = pend_start; pend_idx = -1;
                 } else {
