@@ -332,7 +332,9 @@ rwc_status smem_range(rwc_graph *G, uint64_t seed, int64_t tree0, int64_t T, dou
             int per_sm = 0;
             RWC_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, NT, smem));
             if (per_sm < 1) return set_error(RWC_ERR_UNSUPPORTED, "graph too large for shared mode");
-            const int64_t blocks = std::min<int64_t>(T, (int64_t)sms * per_sm);
+            int64_t blocks = std::min<int64_t>(T, (int64_t)sms * per_sm);
+            if (o.memory_budget > 0 && need_spill)
+                blocks = std::max<int64_t>(1, std::min(blocks, (o.memory_budget - TAIL - T * 4) / (n * 4)));
             RWC_CUDA_TRY(cudaMallocAsync(&buf.p, TAIL + (size_t)T * 4 + (need_spill ? (size_t)blocks * n * 4 : 0), stream));
             RWC_CUDA_TRY(cudaMemsetAsync(buf.p, 0, TAIL, stream));
             err = (int *)buf.p;
@@ -388,7 +390,9 @@ rwc_status sample_smem(rwc_graph *G, uint64_t seed, int64_t tree0, int64_t T, do
                        int32_t *visits, uint32_t klim, const rwc_options_t &o, rwc_stats_t *st, int *err,
                        cudaStream_t stream) {
     const int64_t n = G->g.n;
-    const int64_t chunk = std::min(T, o.trees_per_chunk > 0 ? std::min(o.trees_per_chunk, WIDE_CAP) : WIDE_CAP);
+    int64_t chunk = std::min(T, o.trees_per_chunk > 0 ? std::min(o.trees_per_chunk, WIDE_CAP) : WIDE_CAP);
+    // a budget is shared by the list of trees (4 bytes each) and the blocks' ends
+    if (o.memory_budget > 0) chunk = std::max<int64_t>(1, std::min(chunk, o.memory_budget / 8));
     // threads per tree: 1024 on an SM, over the trees that it holds at once (BA
     // n = 12000, 1000 trees: 1.0, 0.65 and 0.50 ms with 64, 128 and 256 threads;
     // n = 2000, 1000 trees: 0.142, 0.122 and 0.135 ms)
@@ -484,7 +488,9 @@ rwc_status sample_lane_shared(rwc_graph *G, uint64_t seed, int64_t tree0, int64_
                               int32_t *parents, int32_t *visits, const rwc_options_t &o, rwc_stats_t *st,
                               cudaStream_t stream) {
     int e = 0;
-    RWC_TRY(sample_smem(G, seed, tree0, T, sums, parents, visits, 65535u, o, st, &e, stream));
+    rwc_options_t p = o;                    // chunks and budgets are walker mode's
+    p.trees_per_chunk = p.memory_budget = 0;
+    RWC_TRY(sample_smem(G, seed, tree0, T, sums, parents, visits, 65535u, p, st, &e, stream));
     if (e & LE_KOVF) return set_error(RWC_ERR_UNSUPPORTED, "a vertex was popped more than 65535 times; use RWC_MODE_GLOBAL");
     if (e) return set_error(RWC_ERR_CUDA, "sampler internal check failed");
     if (st) st->mode = RWC_MODE_SHARED;

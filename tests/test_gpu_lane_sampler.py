@@ -168,3 +168,25 @@ def test_small_trees_by_one_warp(n):
         assert st.block_threads == (32 if n <= 448 else 256)
     if n >= 3:
         _exact(synth.cycle(n), 3)
+
+
+@pytest.mark.parametrize("n", [30000, 60000])
+def test_memory_budget_bounds_the_scratch(n):
+    # words in shared memory (the blocks' pending ends are the scratch) and in global
+    # memory; what the call takes from the device's pool
+    import ctypes
+    rt = ctypes.CDLL("libcudart.so.13")
+    pool, high, budget = ctypes.c_void_p(), ctypes.c_uint64(0), 6 << 20
+    g = synth.rgg(n, 8.0, seed=n)
+    G = rwc.Graph.from_synth(g)
+    ref, *_ = G.sample(200, seed=4, opt=rwc.Options(mode=rwc.MODE_WALKER))
+    torch.cuda.synchronize()
+    assert rt.cudaDeviceGetDefaultMemPool(ctypes.byref(pool), 0) == 0
+    used_current, used_high = 7, 8
+    before = ctypes.c_uint64()
+    assert rt.cudaMemPoolGetAttribute(pool, used_current, ctypes.byref(before)) == 0
+    assert rt.cudaMemPoolSetAttribute(pool, used_high, ctypes.byref(high)) == 0
+    s, *_ = G.sample(200, seed=4, opt=rwc.Options(mode=rwc.MODE_WALKER, memory_budget=budget))
+    assert rt.cudaMemPoolGetAttribute(pool, used_high, ctypes.byref(high)) == 0
+    assert torch.equal(s, ref)
+    assert 0 < high.value - before.value <= budget
