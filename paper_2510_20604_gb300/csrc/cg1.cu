@@ -786,11 +786,11 @@ rwc_status solve_one(rwc_graph *G, const double *B, double *X, double tol, int *
              : rt == 4 ? launch(cg1_ell<EW, 4>, ELL_TPB, smem, blocks) : launch(cg1_ell<EW, ELL_RMAX>, ELL_TPB, smem, blocks);
     };
     cudaError_t e = !ell ? csr(blocks) : g.ell_w == 4 ? inl(std::integral_constant<int, 4>{}) : inl(std::integral_constant<int, 8>{});
-    if (e != cudaSuccess && blocks > 1) {
-        // a device that refuses the cooperative launch: one block, no grid barrier
+    // a device or context that does not hold that many blocks at once: as many as it does
+    for (int64_t nb = blocks / 2; e != cudaSuccess && nb >= 1; nb /= 2) {
         (void)cudaGetLastError();
-        a.clustered = false;
-        e = csr(1);
+        a.clustered = nb > 1 && nb <= 8;
+        e = csr(nb);
     }
     RWC_CUDA_TRY(e);
     double h[3];

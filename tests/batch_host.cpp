@@ -1,7 +1,8 @@
-// Host driver of the batched sampler on a stand-in for the CUDA runtime that
-// keeps track of device allocations, fails one on request and checks that no
-// launch (direct, or replayed from a captured graph) is given freed memory and
-// that every launch has as many pulls as trees.
+// Host driver of the batched sampler and of the one-column solve on a stand-in for
+// the CUDA runtime.  Batch: it keeps track of device allocations, fails one on
+// request and checks that no launch (direct, or replayed from a captured graph) is
+// given freed memory and that every launch has as many pulls as trees.  Solve: it
+// refuses cooperative launches of more blocks than a limit.
 #include <cstdio>
 #include <cstdint>
 #include <cstdlib>
@@ -18,6 +19,7 @@ static std::map<char *, std::pair<size_t, bool>> blocks;   // address -> size, l
 static int fail_in = -1;                                    // allocations until one fails
 static int stale = 0, launches = 0;
 static int64_t pulls = 0;                                   // pulls launched
+static unsigned coop_limit = 0, coop_blocks = 0;            // solve: the limit (0: batch), blocks launched
 static bool capturing = false;
 static std::vector<char *> captured;                        // pointers of the captured launches
 
@@ -76,7 +78,15 @@ void __cudaRegisterVar(void **, char *, char *, const char *, int, size_t, int, 
 unsigned __cudaPushCallConfiguration(dim3, dim3, size_t, struct CUstream_st *) { return 0; }
 cudaError_t __cudaPopCallConfiguration(dim3 *, dim3 *, size_t *, void *) { return cudaSuccess; }
 cudaError_t __cudaGetKernel(cudaKernel_t *k, const void *f) { *k = (cudaKernel_t)f; return cudaSuccess; }
+cudaError_t cudaLaunchCooperativeKernel(const void *, dim3 grid, dim3, void **, size_t, cudaStream_t) {
+    if (grid.x > coop_limit) return cudaErrorCooperativeLaunchTooLarge;
+    coop_blocks = grid.x;
+    return cudaSuccess;
+}
+cudaError_t cudaLaunchKernel(const void *, dim3 grid, dim3, void **, size_t, cudaStream_t) { coop_blocks = grid.x; return cudaSuccess; }
+cudaError_t cudaLaunchKernelExC(const cudaLaunchConfig_t *c, const void *, void **) { coop_blocks = c->gridDim.x; return cudaSuccess; }
 cudaError_t __cudaLaunchKernel(cudaKernel_t, dim3, dim3, void **args, size_t, cudaStream_t) {
+    if (coop_limit) return cudaSuccess;
     // kernel arguments 1, 2 and 10: the graphs' records, the bin's graphs, the
     // pending ends beyond shared memory; 3: pulls
     pulls += *(int64_t *)args[3];
@@ -91,7 +101,33 @@ cudaError_t __cudaLaunchKernel(cudaKernel_t, dim3, dim3, void **args, size_t, cu
 
 #define EXPECT(c) do { if (!(c)) { printf("line %d: %s (stale %d, %s)\n", __LINE__, #c, stale, rwc_last_error()); return 1; } } while (0)
 
+// A cycle with unit weights of its own (general rows, many blocks).
+static int solve() {
+    const int n = 200000;
+    std::vector<int64_t> rp{0};
+    std::vector<int32_t> col;
+    for (int u = 0; u < n; ++u) {
+        const int a = (u + n - 1) % n, b = (u + 1) % n;
+        col.push_back(a < b ? a : b);
+        col.push_back(a < b ? b : a);
+        rp.push_back((int64_t)col.size());
+    }
+    std::vector<float> w(col.size(), 1.f);
+    std::vector<double> b(n), x(n);
+    for (unsigned limit : {1000u, 60u, 20u, 9u, 8u}) {
+        rwc_graph_t *g = nullptr;
+        coop_limit = limit;
+        EXPECT(rwc_graph_create(n, (int64_t)col.size(), rp.data(), col.data(), w.data(), -1, 0, &g) == RWC_OK);
+        EXPECT(rwc_solve(g, 1, b.data(), x.data(), 1e-10, nullptr, nullptr) == RWC_OK);
+        EXPECT(coop_blocks <= limit && coop_blocks >= (limit < 100 ? limit / 2 : 100));
+        EXPECT(rwc_graph_destroy(g) == RWC_OK);
+    }
+    printf("ok\n");
+    return 0;
+}
+
 int main(int argc, char **argv) {
+    if (argc > 1 && !strcmp(argv[1], "solve")) return solve();
     const int nth = argc > 1 ? atoi(argv[1]) : -1, use_graph = argc > 2 ? atoi(argv[2]) : 0;
     // two cycles, one for each size class
     const int ns[2] = {40, 1500};

@@ -1,4 +1,4 @@
-"""Host logic of the batched sampler on a stand-in for the CUDA runtime
+"""Host logic of the batched sampler and of the one-column solve on a stand-in for the CUDA runtime
 (batch_host.cpp), linked with the library's own object files."""
 import os
 import subprocess
@@ -15,7 +15,7 @@ def driver(tmp_path_factory):
     _build.build()
     exe = str(tmp_path_factory.mktemp("batch") / "batch_host")
     inc = os.path.join(os.path.dirname(os.path.dirname(_build.nvcc())), "include")
-    objs = [os.path.join(_build.BUILD, o) for o in ("batch.o", "graph.o")]
+    objs = [os.path.join(_build.BUILD, o) for o in ("batch.o", "graph.o", "estimate.o", "solver.o", "cg1.o")]
     subprocess.run(["g++", "-std=c++17", "-O1", "-I", _build.INCLUDE, "-I", inc, "-o", exe,
                     os.path.join(HERE, "batch_host.cpp")] + objs, check=True)
     return exe
@@ -37,4 +37,11 @@ def test_a_failed_rebuild_leaves_nothing_stale(driver, nth, use_graph):
     classes' items, the spill array); the next call with the first count gives
     no freed memory to a launch."""
     r = subprocess.run([driver, str(nth), str(use_graph)], capture_output=True, text=True, timeout=60)
+    assert r.returncode == 0, r.stdout + r.stderr
+
+
+def test_solve_takes_as_many_blocks_as_the_device_holds(driver):
+    """A context that refuses the cooperative launch gets at least half of the
+    blocks that it holds at once, not one."""
+    r = subprocess.run([driver, "solve"], capture_output=True, text=True, timeout=60)
     assert r.returncode == 0, r.stdout + r.stderr
