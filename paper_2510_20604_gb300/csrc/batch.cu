@@ -361,7 +361,7 @@ rwc_status finish(rwc_batch *b, rwc_stats_t *stats, int mode, int64_t T, cudaStr
         stats->marked = b->host[2];
         stats->chunks = 1;
         stats->mode = mode;
-        stats->block_threads = mode == 3 ? 0 : b->threads;   // the large class's block size
+        stats->block_threads = mode == 3 ? 0 : b->threads;   // the schedule's bound on the large class's blocks
     }
     return RWC_OK;
 }
@@ -605,14 +605,16 @@ extern "C" rwc_status rwc_autotune(rwc_batch_t *b, const char *cache_path, rwc_s
     RWC_CUDA_TRY(cudaMallocAsync((void **)&sums, b->N * sizeof(double), st));
     // coordinate search from the current schedule, each candidate timed on
     // 16 trees per graph: the split with the small class warp- or
-    // block-per-tree, then the large class's block size, then trees per item,
-    // then concurrent or sequential classes
+    // block-per-tree, then a smaller largest block of the large class (no block has
+    // more than 256 threads, so larger bounds are the same launches), then
+    // concurrent or sequential bins
     const int64_t Tp = 16;
     cudaEvent_t e0, e1;
     cudaEventCreate(&e0);
     cudaEventCreate(&e1);
     struct Sched { int th, sp, tl, wp, cc; };
     Sched best_s{b->threads, b->split, b->tile, b->warp, b->conc};
+    const Sched before = best_s;
     float best = 1e30f;
     rwc_status status = RWC_OK;
     auto time_one = [&](const Sched &c) -> float {
@@ -641,21 +643,20 @@ extern "C" rwc_status rwc_autotune(rwc_batch_t *b, const char *cache_path, rwc_s
         const int splits[][2] = {{0, 0}, {512, 1}, {1024, 1}, {2048, 1}, {1024, 0}, {2048, 0}, {4096, 0}};
         for (auto &sw : splits) { Sched c = best_s; c.sp = sw[0]; c.wp = sw[1]; if (!consider(c)) goto done; }
         const Sched base1 = best_s;
-        for (int th : {256, 512, 1024}) { Sched c = base1; c.th = th; if (!consider(c)) goto done; }
+        for (int th : {64, 128}) { Sched c = base1; c.th = th; if (!consider(c)) goto done; }
         const Sched base2 = best_s;
-        for (int tl : {1, 4, 16}) { Sched c = base2; c.tl = tl; if (!consider(c)) goto done; }
-        const Sched base3 = best_s;
-        for (int cc : {0, 1}) { Sched c = base3; c.cc = cc; if (!consider(c)) goto done; }
+        for (int cc : {0, 1}) { Sched c = base2; c.cc = cc; if (!consider(c)) goto done; }
     }
 done:
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
     cudaFreeAsync(sums, st);
-    RWC_CUDA_TRY(cudaStreamSynchronize(st));
-    RWC_TRY(status);
+    if (status != RWC_OK) best_s = before;
     b->threads = best_s.th; b->split = best_s.sp; b->tile = best_s.tl; b->warp = best_s.wp; b->conc = best_s.cc;
     b->items_T = -1;
     drop_graph(b);
+    RWC_CUDA_TRY(cudaStreamSynchronize(st));
+    RWC_TRY(status);
     if (cache_path) {
         FILE *f = fopen(cache_path, "w");
         if (f) {
