@@ -56,7 +56,7 @@ struct Tile {
         : q(blockIdx.y * qt + threadIdx.x % qt), rs(threadIdx.x / qt), slots(blockDim.x / qt) {
         u0 = (int64_t)blockIdx.x * slots + rs;
         step = (int64_t)gridDim.x * slots;
-        on = q < k4 && rs < slots;
+        on = q < k4;
     }
 };
 
@@ -97,12 +97,10 @@ __device__ __forceinline__ void dot4(Pair (&a)[4], const float4 &x, const float4
     pair_fma(a[0], x.x, y.x); pair_fma(a[1], x.y, y.y); pair_fma(a[2], x.z, y.z); pair_fma(a[3], x.w, y.w);
 }
 
-// One slot takes about 150 cycles per arc, so a hub row alone takes longer than the
-// rest of the product.  With more than SHARE_QUADS quads of columns the rows of more
-// than WIDE_ROW arcs are shared by a block's slots.  With fewer, a warp holds several
-// arcs of a quad side by side: it takes each row of 17 to 1024 arcs (the last degree
-// bin) by itself, and a block's slots share the heavy rows.
-constexpr int WIDE_ROW = 128, SHARE_QUADS = 16, SHARE_ROW = 16;
+// Rows of more arcs are shared by a block's slots: one slot takes about 150 cycles
+// per arc, so the hub of a BA graph of 9000 vertices alone took longer than the
+// rest of the product.
+constexpr int WIDE_ROW = 128;
 
 // Q = L P and the parts of <P, Q>.  Four neighbour rows are in flight.
 template <bool OFF64, bool W>
@@ -110,8 +108,82 @@ __global__ void __launch_bounds__(TPB) bcg_product(DevGraph g, int k4, int qt, c
                                                    float4 *__restrict__ Q, double *parts) {
     const Tile t(k4, qt);
     Pair a[4] = {};
-    const bool warps = qt <= SHARE_QUADS;
-    const int64_t alone = warps ? SHARE_ROW : WIDE_ROW;
+    if (t.on)
+        for (int64_t u = t.u0; u < g.n; u += t.step) {
+            int64_t b, e;
+            rowb<OFF64>(g, u, b, e);
+            if (e - b > WIDE_ROW) continue;
+            float4 s0 = {}, s1 = {};
+            int64_t j = b;
+            for (; j + 4 <= e; j += 4) {
+                int32_t c[4];
+                float w[4];
+                float4 v[4];
+#pragma unroll
+                for (int i = 0; i < 4; ++i) { c[i] = g.col[j + i]; w[i] = W ? g.w[j + i] : 1.f; }
+#pragma unroll
+                for (int i = 0; i < 4; ++i) v[i] = P[(int64_t)c[i] * k4 + t.q];
+                fma4(s0, w[0], v[0]); fma4(s1, w[1], v[1]); fma4(s0, w[2], v[2]); fma4(s1, w[3], v[3]);
+            }
+            for (; j < e; ++j) fma4(s0, W ? g.w[j] : 1.f, P[(int64_t)g.col[j] * k4 + t.q]);
+            const float d = (float)g.d[u];
+            const float4 p = P[u * k4 + t.q];
+            const float4 q = {d * p.x - (s0.x + s1.x), d * p.y - (s0.y + s1.y), d * p.z - (s0.z + s1.z),
+                              d * p.w - (s0.w + s1.w)};
+            Q[u * k4 + t.q] = q;
+            dot4(a, p, q);
+        }
+    // longer rows: the block's slots share the arcs of one
+    __shared__ float4 hs[TPB];
+    for (int64_t base = (int64_t)blockIdx.x * t.slots; base < g.n; base += t.step) {
+        int64_t b = 0, e = 0;
+        if (base + t.rs < g.n) rowb<OFF64>(g, base + t.rs, b, e);
+        if (!__syncthreads_or(e - b > WIDE_ROW)) continue;
+        for (int r = 0; r < t.slots && base + r < g.n; ++r) {
+            const int64_t u = base + r;
+            rowb<OFF64>(g, u, b, e);
+            if (e - b <= WIDE_ROW) continue;
+            float4 s = {};
+            if (t.on)
+#pragma unroll 4
+                for (int64_t j = b + t.rs; j < e; j += t.slots) fma4(s, W ? g.w[j] : 1.f, P[(int64_t)g.col[j] * k4 + t.q]);
+            hs[threadIdx.x] = s;
+            int h = 1;
+            while (h < t.slots) h *= 2;
+            for (h /= 2; h > 0; h /= 2) {
+                __syncthreads();
+                if (t.rs < h && t.rs + h < t.slots) fma4(hs[threadIdx.x], 1.f, hs[threadIdx.x + h * qt]);
+            }
+            __syncthreads();
+            if (t.rs == 0 && t.on) {
+                s = hs[threadIdx.x];
+                const float d = (float)g.d[u];
+                const float4 p = P[u * k4 + t.q];
+                const float4 q = {d * p.x - s.x, d * p.y - s.y, d * p.z - s.z, d * p.w - s.w};
+                Q[u * k4 + t.q] = q;
+                dot4(a, p, q);
+            }
+            __syncthreads();
+        }
+    }
+    quad_parts(t, a, qt, parts);
+}
+
+// Few columns (at most SHARE_QUADS quads): a block has up to 256 slots, so that a slot's
+// serial chain of arcs bounds the product from short rows on.  The lanes of a warp hold
+// several arcs of a quad side by side instead: a warp takes each row of 17 to 1024 arcs
+// (the last degree bin) by itself, a block's slots share each heavy row.  (Two columns:
+// dense n = 1000 7.5 -> 1.15 ms, BA 100000 7.3 -> 2.95, BA 10^6 18.5 -> 6.2; gradient of BA
+// 60000 with 34 columns 7.5 -> 5.7.)  Blocks of TPB threads; those beyond the slots
+// only help in the warps.
+constexpr int SHARE_QUADS = 16, SHARE_ROW = 16;
+
+template <bool OFF64, bool W>
+__global__ void __launch_bounds__(TPB) bcg_product_few(DevGraph g, int k4, int qt, const float4 *__restrict__ P,
+                                                       float4 *__restrict__ Q, double *parts) {
+    const Tile t(k4, qt);
+    const bool slot = t.on && t.rs < t.slots;
+    Pair a[4] = {};
     auto finish = [&](int64_t u, const float4 &s) {
         const float d = (float)g.d[u];
         const float4 p = P[u * k4 + t.q];
@@ -119,11 +191,11 @@ __global__ void __launch_bounds__(TPB) bcg_product(DevGraph g, int k4, int qt, c
         Q[u * k4 + t.q] = q;
         dot4(a, p, q);
     };
-    if (t.on)
+    if (slot)
         for (int64_t u = t.u0; u < g.n; u += t.step) {
             int64_t b, e;
             rowb<OFF64>(g, u, b, e);
-            if (e - b > alone) continue;
+            if (e - b > SHARE_ROW) continue;
             float4 s0 = {}, s1 = {};
             int64_t j = b;
             for (; j + 4 <= e; j += 4) {
@@ -140,28 +212,10 @@ __global__ void __launch_bounds__(TPB) bcg_product(DevGraph g, int k4, int qt, c
             fma4(s0, 1.f, s1);
             finish(u, s0);
         }
-    __shared__ float4 hs[TPB];
-    // a row's arcs shared by the block's slots
-    auto by_block = [&](int64_t u, int64_t b, int64_t e) {
-        float4 s = {};
-        if (t.on)
-#pragma unroll 4
-            for (int64_t j = b + t.rs; j < e; j += t.slots) fma4(s, W ? g.w[j] : 1.f, P[(int64_t)g.col[j] * k4 + t.q]);
-        hs[threadIdx.x] = s;
-        int h = 1;
-        while (h < t.slots) h *= 2;
-        for (h /= 2; h > 0; h /= 2) {
-            __syncthreads();
-            if (t.rs < h && t.rs + h < t.slots) fma4(hs[threadIdx.x], 1.f, hs[threadIdx.x + h * qt]);
-        }
-        __syncthreads();
-        if (t.rs == 0 && t.on) finish(u, hs[threadIdx.x]);
-        __syncthreads();
-    };
-    if (warps) {
+    {
         // lanes of a warp as arcs x quads (rotated where qt does not divide 32)
         const int lane = threadIdx.x & 31, na = 32 / qt, al = lane / qt;
-        const bool on = al < na && t.q < k4;
+        const bool on = al < na && t.on;
         int top = 1;
         while (top < na) top *= 2;
         const int32_t *rows = g.bin_rows + g.bin_off[4];
@@ -181,21 +235,27 @@ __global__ void __launch_bounds__(TPB) bcg_product(DevGraph g, int k4, int qt, c
             }
             if (on && al == 0) finish(u, s);
         }
-        for (int64_t c = blockIdx.x; c < g.hc_n; c += gridDim.x) {
-            int64_t b, e;
-            rowb<OFF64>(g, g.hc_row[c], b, e);
-            if (g.hc_beg[c] == b) by_block(g.hc_row[c], b, e);
+    }
+    __shared__ float4 hs[TPB];
+    for (int64_t c = blockIdx.x; c < g.hc_n; c += gridDim.x) {
+        const int64_t u = g.hc_row[c];
+        int64_t b, e;
+        rowb<OFF64>(g, u, b, e);
+        if (g.hc_beg[c] != b) continue;          // not the row's first chunk
+        float4 s = {};
+        if (slot)
+#pragma unroll 4
+            for (int64_t j = b + t.rs; j < e; j += t.slots) fma4(s, W ? g.w[j] : 1.f, P[(int64_t)g.col[j] * k4 + t.q]);
+        hs[threadIdx.x] = s;
+        int h = 1;
+        while (h < t.slots) h *= 2;
+        for (h /= 2; h > 0; h /= 2) {
+            __syncthreads();
+            if (t.rs < h && t.rs + h < t.slots) fma4(hs[threadIdx.x], 1.f, hs[threadIdx.x + h * qt]);
         }
-    } else {
-        for (int64_t base = (int64_t)blockIdx.x * t.slots; base < g.n; base += t.step) {
-            int64_t b = 0, e = 0;
-            if (t.rs < t.slots && base + t.rs < g.n) rowb<OFF64>(g, base + t.rs, b, e);
-            if (!__syncthreads_or(e - b > WIDE_ROW)) continue;
-            for (int r = 0; r < t.slots && base + r < g.n; ++r) {
-                rowb<OFF64>(g, base + r, b, e);
-                if (e - b > WIDE_ROW) by_block(base + r, b, e);
-            }
-        }
+        __syncthreads();
+        if (t.rs == 0 && t.on) finish(u, hs[threadIdx.x]);
+        __syncthreads();
     }
     quad_parts(t, a, qt, parts);
 }
@@ -479,7 +539,9 @@ rwc_status solve_nodemajor(rwc_graph *G, int k, const double *B, double *X, doub
                 double *z0 = rz[it & 1], *z1 = rz[(it & 1) ^ 1];
                 ::rwc::count_launches(5);
                 dispatch(g, [&](auto o64, auto wt) {
-                    bcg_product<decltype(o64)::value, decltype(wt)::value><<<grid, TPB, 0, st>>>(g, k4, qt, p, q, pa);
+                    constexpr bool O = decltype(o64)::value, W = decltype(wt)::value;
+                    if (qt <= SHARE_QUADS) bcg_product_few<O, W><<<grid, TPB, 0, st>>>(g, k4, qt, p, q, pa);
+                    else bcg_product<O, W><<<grid, threads, 0, st>>>(g, k4, qt, p, q, pa);
                 });
                 sum_cols<<<dim3((unsigned)kp, 1), 128, 0, st>>>(pa, nullptr, (int)nb, pq, nullptr);
                 bcg_residual<<<grid, threads, 0, st>>>(n, k4, qt, z0, pq, g.dinv32, q, r, pa, pb);
