@@ -500,9 +500,10 @@ __global__ void __launch_bounds__(RES ? RES_TPB : CSR_TPB, RES ? 1 : 2) cg1_csr(
     ResidentRows<OFF64, W> held;
     if constexpr (RES) held.load(g);
     auto inner = [&](double rn) -> int {
+        const double rs = rn / a.scale;
         Pair acc[1] = {{0.f, 0.f}};
         each([&](int64_t i) {
-            const float rv = (float)(a.R[i] / rn * a.scale), zv = g.dinv32[i] * rv;
+            const float rv = (float)(a.R[i] / rs), zv = g.dinv32[i] * rv;
             a.r[i] = rv;
             a.e[i] = 0.f;
             if (FUSED) a.zp[0][i] = make_float2(zv, 0.f);
@@ -560,7 +561,7 @@ __global__ void __launch_bounds__(RES ? RES_TPB : CSR_TPB, RES ? 1 : 2) cg1_csr(
                 all_sync(a.clustered);
             }
         }
-        each([&](int64_t i) { a.X[i] += rn / a.scale * (double)a.e[i]; });
+        each([&](int64_t i) { a.X[i] += rs * (double)a.e[i]; });
         all_sync(a.clustered);
         return it;
     };
@@ -606,6 +607,7 @@ __global__ void __launch_bounds__(ELL_TPB, 1) cg1_ell(CgArgs a) {
         return s;
     };
     auto inner = [&](double rn) -> int {
+        const double rs = rn / a.scale;
         float e[RT], r[RT], p[RT], q[RT], d[RT];
         Pair acc[1] = {{0.f, 0.f}};
 #pragma unroll
@@ -616,7 +618,7 @@ __global__ void __launch_bounds__(ELL_TPB, 1) cg1_ell(CgArgs a) {
             if (l < nrow) {
                 const int64_t u = row0 + l;
                 d[i] = a.d32[u];
-                r[i] = (float)(a.R[u] / rn * a.scale);
+                r[i] = (float)(a.R[u] / rs);
                 const float zv = r[i] * __fdividef(1.f, d[i]);
                 a.zp[0][u] = make_float2(zv, 0.f);
                 pair_fma(acc[0], r[i], zv);
@@ -661,7 +663,7 @@ __global__ void __launch_bounds__(ELL_TPB, 1) cg1_ell(CgArgs a) {
 #pragma unroll
         for (int i = 0; i < RT; ++i) {
             const int l = threadIdx.x + i * ELL_TPB;
-            if (l < nrow) a.X[row0 + l] += rn / a.scale * (double)e[i];
+            if (l < nrow) a.X[row0 + l] += rs * (double)e[i];
         }
         all_sync(a.clustered);
         return it;

@@ -326,11 +326,11 @@ __global__ void __launch_bounds__(TPB) bcg_start(int64_t n, int k, int k4, int q
     if (t.on) {
         double nr[4];
 #pragma unroll
-        for (int i = 0; i < 4; ++i) nr[i] = 4 * t.q + i < k ? sqrt(rnrm2[4 * t.q + i]) : 0.0;
+        for (int i = 0; i < 4; ++i) nr[i] = 4 * t.q + i < k ? sqrt(rnrm2[4 * t.q + i]) / scale : 0.0;
         for (int64_t u = t.u0; u < n; u += t.step) {
             float v[4];
 #pragma unroll
-            for (int i = 0; i < 4; ++i) v[i] = nr[i] > 0.0 ? (float)(R[u * k + 4 * t.q + i] / nr[i] * scale) : 0.f;
+            for (int i = 0; i < 4; ++i) v[i] = nr[i] > 0.0 ? (float)(R[u * k + 4 * t.q + i] / nr[i]) : 0.f;
             const float di = dinv[u];
             const float4 rv = {v[0], v[1], v[2], v[3]}, zv = {di * v[0], di * v[1], di * v[2], di * v[3]};
             const int64_t i = u * k4 + t.q;
@@ -343,13 +343,13 @@ __global__ void __launch_bounds__(TPB) bcg_start(int64_t n, int k, int k4, int q
     quad_parts(t, a, qt, parts);
 }
 
-// X += |R_c| / scale e.
-__global__ void __launch_bounds__(TPB) bcg_add(int64_t n, int k, int k4, double scale, const double *rnrm2, const float *e, double *X) {
+// X += |R_c| e times unscale, 1 / scale.
+__global__ void __launch_bounds__(TPB) bcg_add(int64_t n, int k, int k4, double unscale, const double *rnrm2, const float *e, double *X) {
     const int64_t tot = n * k;
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < tot; i += (int64_t)gridDim.x * blockDim.x) {
         const int64_t u = i / k;
         const int c = (int)(i - u * k);
-        X[i] += sqrt(rnrm2[c]) / scale * (double)e[u * 4 * k4 + c];
+        X[i] += sqrt(rnrm2[c]) * unscale * (double)e[u * 4 * k4 + c];
     }
 }
 
@@ -565,7 +565,7 @@ rwc_status solve_nodemajor(rwc_graph *G, int k, const double *B, double *X, doub
         }
         total_iters += it;
         ::rwc::count_launches(1);
-        bcg_add<<<gs, TPB, 0, st>>>(n, k, k4, scale, rn2, (const float *)e, X);
+        bcg_add<<<gs, TPB, 0, st>>>(n, k, k4, 1.0 / scale, rn2, (const float *)e, X);
         RWC_CUDA_TRY(cudaGetLastError());
     }
     // final projection of X onto 1-perp
