@@ -481,7 +481,7 @@ rwc_status rwc_predict_mre(rwc_graph_t *g, const double *sums, int64_t num_trees
  * tau-a).  a, b: device FP64 [n], no NaN (-0.0 equals +0.0).  out_diff:
  * device int64 scalar, written with alpha - beta (exact).  host_tau: NULL, or
  * a host double receiving K (then the call synchronises stream).  Every pair
- * is counted (sorting and inversions above 8192 elements): 0 <= n <= 2^26.
+ * is counted (sorting and inversions above 16384 elements): 0 <= n <= 2^26.
  */
 rwc_status rwc_kendall(int64_t n, const double *a, const double *b, int64_t *out_diff,
                        double *host_tau, rwc_stream_t stream);

@@ -325,9 +325,11 @@ void kendall_sorted(int64_t n, const double *a, const double *b, KeyPair *scratc
     kendall_ties<<<(unsigned)std::min<int64_t>((n + 255) / 256, (int64_t)num_sms() * 8), 256, 0, st>>>(n, src, k0, out);
 }
 
-// Below this many elements all pairs are compared: one launch (n = 262144: 24.2 ms
-// for all pairs, 0.52 ms by sorting, with rwc_mre in both).
-constexpr int64_t KENDALL_PAIRS_MAX = 8192;
+// Up to this many elements all pairs are compared: one launch in place of 9 to 11
+// passes of about 10 us (whole calls, all pairs and by sorting: n = 8300 0.353 and 0.380
+// ms, 16000 0.358 and 0.384, 20000 0.540 and 0.405, 32000 0.86 and 0.40): 16384 elements
+// are the last whose tiles are one wave of blocks.
+constexpr int64_t KENDALL_PAIRS_MAX = 16384;
 
 }  // namespace
 }  // namespace rwc

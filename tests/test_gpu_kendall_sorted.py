@@ -1,4 +1,4 @@
-"""rwc_kendall by sorting (more than 8192 elements) against all pairs compared
+"""rwc_kendall by sorting (more than 16384 elements) against all pairs compared
 one by one: run and tile edges, ties in one, in the other and in both vectors,
 signed zeros and infinities; the counts are whole numbers, so equal exactly."""
 import numpy as np
@@ -48,6 +48,23 @@ def test_sorted_equals_all_pairs(n, kind):
     ref = _all_pairs(a, b)
     assert diff == ref
     assert tau == 2.0 * ref / (n * (n - 1.0))
+
+
+# the first size that is sorted, a part tile behind an odd number of tiles, two levels
+# of runs with a part run
+@pytest.mark.parametrize("kind", ["plain", "ties", "ties_a", "equal", "reversed", "same", "special"])
+@pytest.mark.parametrize("n", [16384, 16385, 18433, 22528, 24577])
+def test_sorted_equals_all_pairs_above_the_bound(n, kind):
+    a, b = _vectors(n, kind)
+    assert rwc.rwc_kendall(a, b)[1] == _all_pairs(a, b)
+
+
+def test_one_launch_up_to_the_bound():
+    for n in (8193, 12000, 16384):
+        a, b = _vectors(n, "plain")
+        before = rwc.rwc_launch_count()
+        rwc.rwc_kendall(a, b)
+        assert rwc.rwc_launch_count() == before + 1
 
 
 def test_sorted_on_a_side_stream_and_repeated():
