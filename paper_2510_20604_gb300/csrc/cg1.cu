@@ -251,6 +251,7 @@ __device__ __forceinline__ bool few_rows(const DevGraph &g, Term term, F f) {
 // gather instead of a chain of four loads per unit, which the barrier's acquire
 // sends to L2 each time (BA 2000: 13500 -> 4700 cycles per product).
 constexpr int RES_UNITS = 4, RES_TPB = 1024;
+constexpr int64_t RES_ARCS = 80000;
 template <bool OFF64, bool W>
 struct ResidentRows {
     int32_t u[RES_UNITS], c[RES_UNITS];
@@ -697,9 +698,13 @@ rwc_status solve_one(rwc_graph *G, const double *B, double *X, double tol, int *
     int rt = 1;
     while (ell && (n + (int64_t)ELL_TPB * rt - 1) / ((int64_t)ELL_TPB * rt) > sms) rt = rt == 1 ? 2 : rt == 2 ? 4 : ELL_RMAX;
     // small systems: rows in registers, up to a cluster of blocks (the smallest
-    // take one block of half the threads: ER 100 178 against 215 us)
+    // take one block of half the threads: ER 100 178 against 215 us).  Registers hold
+    // one arc per lane, so beyond about 10000 arcs a block the rest streams through too
+    // few SMs (complete graphs of 400, 700 and 1000 vertices, weighted: 492, 582 and 736
+    // us so, 453, 504 and 526 on up to 304 blocks; ER 1000 of mean degree 40 and 80: 541 and
+    // 524 against 559 and 501).
     const int64_t units = row_units(g);
-    const bool held = !ell && g.hc_n == 0 && units > 64 && units <= 8 * (RES_TPB / 32) * RES_UNITS;
+    const bool held = !ell && g.hc_n == 0 && units > 64 && units <= 8 * (RES_TPB / 32) * RES_UNITS && g.nnz <= RES_ARCS;
     int64_t blocks = ell ? (n + (int64_t)ELL_TPB * rt - 1) / ((int64_t)ELL_TPB * rt)
                          : held ? (units <= RES_TPB / 32 * RES_UNITS ? 1 : std::min<int64_t>(8, (units + 63) / 64))
                          : units <= 64 ? 1

@@ -126,7 +126,30 @@ static int solve() {
     return 0;
 }
 
+// Complete graphs: few rows, on a cluster of blocks only while their arcs are few too.
+static int dense() {
+    for (int n : {250, 400, 900}) {
+        std::vector<int64_t> rp{0};
+        std::vector<int32_t> col;
+        for (int u = 0; u < n; ++u) {
+            for (int v = 0; v < n; ++v)
+                if (v != u) col.push_back(v);
+            rp.push_back((int64_t)col.size());
+        }
+        std::vector<double> b(n), x(n);
+        rwc_graph_t *g = nullptr;
+        coop_limit = 1000;
+        EXPECT(rwc_graph_create(n, (int64_t)col.size(), rp.data(), col.data(), nullptr, -1, 0, &g) == RWC_OK);
+        EXPECT(rwc_solve(g, 1, b.data(), x.data(), 1e-10, nullptr, nullptr) == RWC_OK);
+        EXPECT(n == 250 ? coop_blocks <= 8 : (int64_t)coop_blocks >= (int64_t)col.size() / 4096);
+        EXPECT(rwc_graph_destroy(g) == RWC_OK);
+    }
+    printf("ok\n");
+    return 0;
+}
+
 int main(int argc, char **argv) {
+    if (argc > 1 && !strcmp(argv[1], "dense")) return dense();
     if (argc > 1 && !strcmp(argv[1], "solve")) return solve();
     const int nth = argc > 1 ? atoi(argv[1]) : -1, use_graph = argc > 2 ? atoi(argv[2]) : 0;
     // two cycles, one for each size class

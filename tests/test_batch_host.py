@@ -45,3 +45,9 @@ def test_solve_takes_as_many_blocks_as_the_device_holds(driver):
     blocks that it holds at once, not one."""
     r = subprocess.run([driver, "solve"], capture_output=True, text=True, timeout=60)
     assert r.returncode == 0, r.stdout + r.stderr
+
+
+def test_dense_graphs_are_not_solved_by_a_few_blocks(driver):
+    """A graph of few rows and many arcs gets blocks for its arcs."""
+    r = subprocess.run([driver, "dense"], capture_output=True, text=True, timeout=60)
+    assert r.returncode == 0, r.stdout + r.stderr
