@@ -84,7 +84,14 @@ __global__ void __launch_bounds__(NT) l_batch(DevGraph base, const BGraph *__res
 // vertices by registers, 10 of 128 up to 5000, 2 of 256 at 20000).  512 graphs
 // of 50 to 20000 vertices, 64 trees each: 158 ms with whole-block popping
 // rounds (11 bytes per vertex, one kernel for each of two classes), 19.4 ms so.
-int batch_threads(int n) { return n <= 2500 ? 64 : n <= 5000 ? 128 : 256; }
+// Calls of at most one tree per SM take 256 threads for each, which nothing else would
+// use (one tree: BA 5000 0.154 -> 0.116 ms a call; of each of 64 weighted BA graphs of
+// 2000 vertices: 0.186 -> 0.132).  Up to 448 vertices more than a warp gains nothing.
+bool few_trees(int64_t trees) { return trees <= num_sms(); }
+int batch_threads(int n, bool few) { return few && n > 448 ? 256 : n <= 2500 ? 64 : n <= 5000 ? 128 : 256; }
+// One launch per graph: one warp up to 448 vertices, whose rounds need no block barrier
+// (30 paths of 60, 1 tree each: 18.8 ms, 22.0 with 64 threads).
+int single_threads(int n, bool few) { return n <= 448 ? 32 : batch_threads(n, few); }
 
 size_t batch_tree_smem(int n, int nt) {
     const size_t head = nt == 32 ? sizeof(LaneShared<32, 1>) : nt == 64 ? sizeof(LaneShared<64, 1>)
@@ -231,11 +238,13 @@ rwc_status resident_blocks(const rwc_batch *b, int nt, size_t smem, int64_t *out
     return RWC_OK;
 }
 
-// Resident blocks of each graph's own launch.
+// Resident blocks of each graph's own launch with many trees (with few there is a
+// block for each tree; blocks of 256 threads whose words need more than the default 48
+// KB are those of many trees too, so their kernels' limit is set here).
 rwc_status plan_single(rwc_batch *b) {
     std::vector<int64_t> blocks(b->G);
     for (int32_t g = 0; g < b->G; ++g) {
-        const int n = b->hgraphs[g].n, nt = batch_threads(n);
+        const int n = b->hgraphs[g].n, nt = single_threads(n, false);
         RWC_TRY(resident_blocks(b, nt, batch_tree_smem(n, nt), &blocks[g]));
     }
     b->single_blocks = std::move(blocks);
@@ -244,6 +253,7 @@ rwc_status plan_single(rwc_batch *b) {
 
 rwc_status build_bins(rwc_batch *b, const std::vector<int32_t> (&order)[2], int64_t T) {
     b->bins.clear();
+    const bool few = few_trees(T * b->G);
     for (int c = 0; c < 2; ++c)
         for (size_t i = 0; i < order[c].size();) {
             const int top = b->hgraphs[order[c][i]].n;
@@ -254,7 +264,7 @@ rwc_status build_bins(rwc_batch *b, const std::vector<int32_t> (&order)[2], int6
             q.begin = (int64_t)i;
             q.count = (int64_t)(j - i);
             q.max_n = top;
-            q.nt = batch_threads(top);
+            q.nt = batch_threads(top, few);
             if (c == 1 && b->warp) q.nt = 32;
             while (c == 0 && q.nt > b->threads) q.nt /= 2;
             q.smem = batch_tree_smem(top, q.nt);
@@ -486,10 +496,11 @@ extern "C" rwc_status rwc_batch_sample(rwc_batch_t *b, uint64_t seed, int64_t T,
         unsigned long long *ctr = (unsigned long long *)((char *)b->scratch + 8);
         const uint32_t k0 = (uint32_t)seed, k1 = (uint32_t)(seed >> 32);
         if (b->single_blocks.empty()) RWC_TRY(plan_single(b));
+        const bool few = few_trees(T);
+        auto blocks = [&](int32_t g) { return few ? T : std::min(T, b->single_blocks[g]); };
         int64_t spill = 0;
         for (int32_t g = 0; g < b->G; ++g)
-            if (b->hgraphs[g].n > (int)LT_STACK)
-                spill = std::max(spill, std::min(T, b->single_blocks[g]) * b->hgraphs[g].n);
+            if (b->hgraphs[g].n > (int)LT_STACK) spill = std::max(spill, blocks(g) * b->hgraphs[g].n);
         if (spill > b->single_spill_n) {
             bfree(b, b->single_spill);
             b->single_spill_n = 0;
@@ -497,10 +508,10 @@ extern "C" rwc_status rwc_batch_sample(rwc_batch_t *b, uint64_t seed, int64_t T,
             b->single_spill_n = spill;
         }
         for (int32_t g = 0; g < b->G; ++g) {
-            const int n = b->hgraphs[g].n, nt = batch_threads(n);
+            const int n = b->hgraphs[g].n, nt = single_threads(n, few);
             ::rwc::count_launches(1);
             dispatch_nt(b->off64, b->weighted, nt, [&](auto kern) {
-                kern<<<(unsigned)std::min(T, b->single_blocks[g]), nt, batch_tree_smem(n, nt), st>>>(
+                kern<<<(unsigned)blocks(g), nt, batch_tree_smem(n, nt), st>>>(
                     b->base, b->graphs, b->single + g, T, nullptr, T, k0, k1, n, sums, b->single_spill, err, ctr);
             });
         }

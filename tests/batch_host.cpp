@@ -20,6 +20,7 @@ static int fail_in = -1;                                    // allocations until
 static int stale = 0, launches = 0;
 static int64_t pulls = 0;                                   // pulls launched
 static unsigned coop_limit = 0, coop_blocks = 0;            // solve: the limit (0: batch), blocks launched
+static unsigned last_grid = 0, last_block = 0;              // the last launch
 static bool capturing = false;
 static std::vector<char *> captured;                        // pointers of the captured launches
 
@@ -75,7 +76,11 @@ void __cudaRegisterFatBinaryEnd(void **) {}
 void __cudaUnregisterFatBinary(void **) {}
 void __cudaRegisterFunction(void **, const char *, char *, const char *, int, uint3 *, uint3 *, dim3 *, dim3 *, int *) {}
 void __cudaRegisterVar(void **, char *, char *, const char *, int, size_t, int, int) {}
-unsigned __cudaPushCallConfiguration(dim3, dim3, size_t, struct CUstream_st *) { return 0; }
+unsigned __cudaPushCallConfiguration(dim3 grid, dim3 block, size_t, struct CUstream_st *) {
+    last_grid = grid.x;
+    last_block = block.x;
+    return 0;
+}
 cudaError_t __cudaPopCallConfiguration(dim3 *, dim3 *, size_t *, void *) { return cudaSuccess; }
 cudaError_t __cudaGetKernel(cudaKernel_t *k, const void *f) { *k = (cudaKernel_t)f; return cudaSuccess; }
 cudaError_t cudaLaunchCooperativeKernel(const void *, dim3 grid, dim3, void **, size_t, cudaStream_t) {
@@ -148,7 +153,34 @@ static int dense() {
     return 0;
 }
 
+// One cycle of n vertices, T trees: threads and blocks of the launch.
+static int few() {
+    const struct { int n, T, per_graph; unsigned threads, blocks; } want[] = {
+        {40, 1, 0, 32, 1}, {40, 1, 1, 32, 1}, {40, 9000, 1, 32, 152}, {448, 5, 1, 32, 5}, {449, 5, 1, 256, 5},
+        {1500, 1, 0, 256, 1}, {1500, 152, 0, 256, 152}, {1500, 153, 0, 64, 152}, {1500, 152, 1, 256, 152},
+        {1500, 153, 1, 64, 152}, {20000, 1, 1, 256, 1}, {20000, 1000, 1, 256, 152}};
+    for (const auto &q : want) {
+        std::vector<int64_t> voff{0, q.n}, rp{0};
+        std::vector<int32_t> col;
+        for (int u = 0; u < q.n; ++u) {
+            const int a = (u + q.n - 1) % q.n, b = (u + 1) % q.n;
+            col.push_back(a < b ? a : b);
+            col.push_back(a < b ? b : a);
+            rp.push_back((int64_t)col.size());
+        }
+        std::vector<double> sums(q.n);
+        rwc_batch_t *b = nullptr;
+        EXPECT(rwc_batch_create(1, voff.data(), rp.data(), col.data(), nullptr, &b) == RWC_OK);
+        EXPECT(rwc_batch_sample(b, 1, q.T, sums.data(), 0, q.per_graph, nullptr, nullptr) == RWC_OK);
+        EXPECT(last_block == q.threads && last_grid == q.blocks);
+        EXPECT(rwc_batch_destroy(b) == RWC_OK);
+    }
+    printf("ok\n");
+    return 0;
+}
+
 int main(int argc, char **argv) {
+    if (argc > 1 && !strcmp(argv[1], "few")) return few();
     if (argc > 1 && !strcmp(argv[1], "dense")) return dense();
     if (argc > 1 && !strcmp(argv[1], "solve")) return solve();
     const int nth = argc > 1 ? atoi(argv[1]) : -1, use_graph = argc > 2 ? atoi(argv[2]) : 0;

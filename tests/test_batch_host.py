@@ -51,3 +51,10 @@ def test_dense_graphs_are_not_solved_by_a_few_blocks(driver):
     """A graph of few rows and many arcs gets blocks for its arcs."""
     r = subprocess.run([driver, "dense"], capture_output=True, text=True, timeout=60)
     assert r.returncode == 0, r.stdout + r.stderr
+
+
+def test_few_trees_take_wide_blocks(driver):
+    """A tree that has an SM to itself is run by 256 threads, one of at most 448
+    vertices by a warp."""
+    r = subprocess.run([driver, "few"], capture_output=True, text=True, timeout=60)
+    assert r.returncode == 0, r.stdout + r.stderr

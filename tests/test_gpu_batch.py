@@ -111,3 +111,19 @@ def test_weighted_batch_matches_oracle():
         ref = ow.Sampler(g, root=int(roots[i]), seed=4, graph_id=i).sample(0, T)
         o = B.offsets
         assert np.array_equal(sums[o[i]:o[i + 1]], ref["sums"]), i
+
+
+@pytest.mark.parametrize("T", [1, 50, 51, 152, 153])
+def test_few_and_many_trees_match_oracle(T):
+    """Block sizes change with the call's trees (one per SM, 152 of them) and the
+    graph's size; one launch per graph counts the trees of each graph."""
+    gs = [synth.batch_graph(i, n, "ba", seed=3) for i, n in enumerate((448, 449, 2600))]
+    B = rwc.Batch(gs)
+    B.set_schedule(512, 300, 4, 1, 1)          # all graphs in the large class
+    s, _ = B.sample(T, seed=6, use_graph=0)
+    one, _ = B.sample(T, seed=6, per_graph_launch=1)
+    assert torch.equal(s, one)
+    sums, roots, o = s.cpu().numpy(), B.roots(), B.offsets
+    for i, g in enumerate(gs):
+        ref = ow.Sampler(g, root=int(roots[i]), seed=6, graph_id=i).sample(0, T)
+        assert np.array_equal(sums[o[i]:o[i + 1]], ref["sums"]), i
