@@ -260,32 +260,20 @@ __global__ void __launch_bounds__(TPB) bcg_product_few(DevGraph g, int k4, int q
     quad_parts(t, a, qt, parts);
 }
 
-// A column whose residual is a tenth of the inner tolerance stands still while the
-// others go on.  Iterated further its residual is soon the rounding errors along the
-// constant vector, on which L is 0: <p, q> is noise, the step is huge and the column
-// diverges, and all of them go on for hundreds or thousands of iterations (weighted
-// complete graph of 1500 vertices, 7 columns 254 -> 2.7 ms; star of 300, 16 columns 43
-// -> 1.05; gradient of the 100 x 100 grid, 64 columns 169 -> 56; a hundredth of the
-// tolerance is too late for that grid).
-constexpr double STILL = 0.01;   // (1/10)^2: of squares
-
-// Step length of a column whose residual's square is rr.
-__device__ __forceinline__ float step_of(double num, double den, double rr, double still) {
-    return den > 0.0 && num > 0.0 && rr > still ? (float)(num / den) : 0.f;
+__device__ __forceinline__ float step_of(double num, double den) {
+    return den > 0.0 && num > 0.0 ? (float)(num / den) : 0.f;
 }
 
 // r -= alpha q; parts of <r, z> (z = D^-1 r) and <r, r>.  Every parts array is
 // [4 k4][gridDim.x].
 __global__ void __launch_bounds__(TPB) bcg_residual(int64_t n, int k4, int qt, const double *rz, const double *pq,
-                                                    const double *rr, double still, const float *dinv,
-                                                    const float4 *__restrict__ Q,
+                                                    const float *dinv, const float4 *__restrict__ Q,
                                                     float4 *__restrict__ r, double *parts, double *parts2) {
     const Tile t(k4, qt);
     Pair a[4] = {}, b[4] = {};
     if (t.on) {
-        const double *z = rz + 4 * t.q, *d = pq + 4 * t.q, *s = rr + 4 * t.q;
-        const float4 al = {step_of(z[0], d[0], s[0], still), step_of(z[1], d[1], s[1], still),
-                           step_of(z[2], d[2], s[2], still), step_of(z[3], d[3], s[3], still)};
+        const double *z = rz + 4 * t.q, *d = pq + 4 * t.q;
+        const float4 al = {step_of(z[0], d[0]), step_of(z[1], d[1]), step_of(z[2], d[2]), step_of(z[3], d[3])};
         for (int64_t u = t.u0; u < n; u += t.step) {
             const int64_t i = u * k4 + t.q;
             const float4 q = Q[i];
@@ -303,17 +291,17 @@ __global__ void __launch_bounds__(TPB) bcg_residual(int64_t n, int k4, int qt, c
 
 // e += alpha p; p = D^-1 r + beta p.
 __global__ void __launch_bounds__(TPB) bcg_direction(int64_t n, int k4, int qt, const double *rz0, const double *pq,
-                                                     const double *rz1, const double *rr, double still, const float *dinv,
+                                                     const double *rz1, const float *dinv,
                                                      const float4 *__restrict__ r, float4 *__restrict__ e,
                                                      float4 *__restrict__ p) {
     const Tile t(k4, qt);
     if (!t.on) return;
-    const double *z = rz0 + 4 * t.q, *d = pq + 4 * t.q, *z1 = rz1 + 4 * t.q, *s = rr + 4 * t.q;
+    const double *z = rz0 + 4 * t.q, *d = pq + 4 * t.q, *z1 = rz1 + 4 * t.q;
     float al[4], be[4];
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
-        al[i] = step_of(z[i], d[i], s[i], still);
-        be[i] = z[i] > 0.0 && s[i] > still ? (float)(z1[i] / z[i]) : 0.f;
+        al[i] = step_of(z[i], d[i]);
+        be[i] = z[i] > 0.0 ? (float)(z1[i] / z[i]) : 0.f;
     }
     for (int64_t u = t.u0; u < n; u += t.step) {
         const int64_t i = u * k4 + t.q;
@@ -421,16 +409,28 @@ __global__ void __launch_bounds__(TPB) col_parts(int64_t n, int k, const double 
     }
 }
 
-// out[c] = sum over b of parts[c * nb + b] in order of b; one block per column
-// (blockIdx.y = 1: the second set of parts, into out2).
+// A column whose residual is a tenth of the inner tolerance stands still while the
+// others go on.  Iterated further its residual is soon the rounding errors along the
+// constant vector, on which L is 0: <p, q> is noise, the step is huge and the column
+// diverges, and all of them go on for hundreds or thousands of iterations (weighted
+// complete graph of 1500 vertices, 7 columns 254 -> 2.7 ms; star of 300, 16 columns 43
+// -> 1.05; gradient of the 100 x 100 grid, 64 columns 169 -> 56; a hundredth of the
+// tolerance is too late for that grid).
+// The step is 0 because sum_cols gives it a <p, q> of 0: the passes over the rows,
+// whose FP64 quotients count, know nothing of it.
+constexpr double STILL = 0.01;   // (1/10)^2: of squares
+
+// out[c] = sum over b of parts[c * nb + b] in order of b, or 0 for a column whose rr[c]
+// is at most `still` (rr = NULL: none); one block per column (blockIdx.y = 1: the
+// second set of parts, into out2).
 __global__ void __launch_bounds__(128) sum_cols(const double *parts, const double *parts2, int nb, double *out,
-                                                double *out2) {
+                                                double *out2, const double *rr = nullptr, double still = 0.0) {
     const int c = blockIdx.x;
     const double *p = (blockIdx.y ? parts2 : parts) + (int64_t)c * nb;
     double s = 0.0;
     for (int b = threadIdx.x; b < nb; b += blockDim.x) s += p[b];
     s = block_sum_fixed(s);
-    if (threadIdx.x == 0) (blockIdx.y ? out2 : out)[c] = s;
+    if (threadIdx.x == 0) (blockIdx.y ? out2 : out)[c] = rr && rr[c] <= still ? 0.0 : s;
 }
 
 // V[u][c] -= colsum[c] / n (FP64).
@@ -490,7 +490,7 @@ rwc_status solve_nodemajor(rwc_graph *G, int k, const double *B, double *X, doub
     Buf buf(st);
     const size_t fbytes = (size_t)n * kp * sizeof(float);
     const size_t nparts = (size_t)kp * std::max(nb, nbc);
-    const size_t bytes = (size_t)nk * 8 + 4 * fbytes + 2 * nparts * 8 + (size_t)8 * kp * 8 + 17 * 256;
+    const size_t bytes = (size_t)nk * 8 + 4 * fbytes + 2 * nparts * 8 + (size_t)8 * kp * 8 + 16 * 256;
     RWC_CUDA_TRY(cudaMallocAsync(&buf.p, bytes, st));
     char *at = (char *)buf.p;
     auto take = [&](size_t b) { char *r = at; at += (b + 255) & ~(size_t)255; return r; };
@@ -498,8 +498,7 @@ rwc_status solve_nodemajor(rwc_graph *G, int k, const double *B, double *X, doub
     float4 *r = (float4 *)take(fbytes), *e = (float4 *)take(fbytes), *p = (float4 *)take(fbytes), *q = (float4 *)take(fbytes);
     double *pa = (double *)take(nparts * 8), *pb = (double *)take(nparts * 8);
     double *colsum = (double *)take((size_t)kp * 8), *rn2 = (double *)take((size_t)kp * 8);
-    double *pq = (double *)take((size_t)kp * 8);
-    double *rr[2] = {(double *)take((size_t)kp * 8), (double *)take((size_t)kp * 8)};
+    double *pq = (double *)take((size_t)kp * 8), *rr = (double *)take((size_t)kp * 8);
     double *rz[2] = {(double *)take((size_t)kp * 8), (double *)take((size_t)kp * 8)};
     const unsigned gs = grid_for(nk);
     auto col_sum = [&](auto square, const double *A, double *out) {
@@ -542,7 +541,7 @@ rwc_status solve_nodemajor(rwc_graph *G, int k, const double *B, double *X, doub
         ::rwc::count_launches(2);
         bcg_start<<<grid, threads, 0, st>>>(n, k, k4, qt, scale, R, rn2, g.dinv32, r, e, p, pa);
         sum_cols<<<dim3((unsigned)kp, 1), 128, 0, st>>>(pa, nullptr, (int)nb, rz[0], nullptr);
-        RWC_CUDA_TRY(cudaMemsetAsync(rr[0], 0x7f, (size_t)kp * 8, st));   // 1e306: every column starts
+        RWC_CUDA_TRY(cudaMemsetAsync(rr, 0x7f, (size_t)kp * 8, st));   // 1e306: every column starts
         int it = 0;
         // iterations between looks at the residual (a host round trip each)
         const int check = (int64_t)n * kp >= 1000000 ? 4 : 8;
@@ -551,20 +550,20 @@ rwc_status solve_nodemajor(rwc_graph *G, int k, const double *B, double *X, doub
         int since_best = 0;
         while (!inner_done && it < max_inner) {
             for (int j = 0; j < check && it < max_inner; ++j, ++it) {
-                double *z0 = rz[it & 1], *z1 = rz[(it & 1) ^ 1], *r0 = rr[it & 1], *r1 = rr[(it & 1) ^ 1];
+                double *z0 = rz[it & 1], *z1 = rz[(it & 1) ^ 1];
                 ::rwc::count_launches(5);
                 dispatch(g, [&](auto o64, auto wt) {
                     constexpr bool O = decltype(o64)::value, W = decltype(wt)::value;
                     if (qt <= SHARE_QUADS) bcg_product_few<O, W><<<grid, TPB, 0, st>>>(g, k4, qt, p, q, pa);
                     else bcg_product<O, W><<<grid, threads, 0, st>>>(g, k4, qt, p, q, pa);
                 });
-                sum_cols<<<dim3((unsigned)kp, 1), 128, 0, st>>>(pa, nullptr, (int)nb, pq, nullptr);
-                bcg_residual<<<grid, threads, 0, st>>>(n, k4, qt, z0, pq, r0, still, g.dinv32, q, r, pa, pb);
-                sum_cols<<<dim3((unsigned)kp, 2), 128, 0, st>>>(pa, pb, (int)nb, z1, r1);
-                bcg_direction<<<grid, threads, 0, st>>>(n, k4, qt, z0, pq, z1, r0, still, g.dinv32, r, e, p);
+                sum_cols<<<dim3((unsigned)kp, 1), 128, 0, st>>>(pa, nullptr, (int)nb, pq, nullptr, rr, still);
+                bcg_residual<<<grid, threads, 0, st>>>(n, k4, qt, z0, pq, g.dinv32, q, r, pa, pb);
+                sum_cols<<<dim3((unsigned)kp, 2), 128, 0, st>>>(pa, pb, (int)nb, z1, rr);
+                bcg_direction<<<grid, threads, 0, st>>>(n, k4, qt, z0, pq, z1, g.dinv32, r, e, p);
             }
             RWC_CUDA_TRY(cudaGetLastError());
-            RWC_CUDA_TRY(cudaMemcpyAsync(h.data(), rr[it & 1], (size_t)k * 8, cudaMemcpyDeviceToHost, st));
+            RWC_CUDA_TRY(cudaMemcpyAsync(h.data(), rr, (size_t)k * 8, cudaMemcpyDeviceToHost, st));
             RWC_CUDA_TRY(cudaStreamSynchronize(st));
             double w2 = 0.0;
             bool bad = false;
