@@ -13,9 +13,9 @@ e2e      = the same metric through the public API from host buffers: graph
 roofline = the sampler's algorithmic bytes (per successor draw: row bounds,
            arc head and, for weighted rows, the alias entry; per tree and
            vertex: parent and visit count) over the device time of its
-           kernels, against the measured HBM copy bandwidth; the walker's own
-           state-word traffic and the ncu-measured DRAM traffic are reported
-           beside it.
+           kernels, against the measured HBM copy bandwidth; the samplers' own
+           state-word traffic and, for the kernel source that it was measured
+           on, the ncu-measured DRAM traffic are reported beside it.
 extras   = the paper-size R-MAT 24 (500 trees), the 4096-graph batch
            (persistent launch against one launch per graph) and the gradient
            on the 1e5-vertex geometric graph, measured in the same run.
@@ -76,9 +76,17 @@ def bytes_per_draw(weighted, off64):
 
 # Per (tree, vertex): the tree's parent (int32) and visit count (int32).
 BYTES_PER_TREE_VERTEX = 8
-# Implementation traffic of the concurrent-walker sampler, not counted above:
-# each draw reads and writes back the vertex's 8-byte state word.
-IMPL_BYTES_PER_DRAW = 16
+# Implementation traffic of the samplers in walker mode, not counted above: each
+# draw reads and writes back the vertex's word, of 8 bytes for the concurrent
+# walkers and 4 for the lane sampler.
+IMPL_BYTES_PER_DRAW = {"walkers": 16, "lanes": 8, "shared": 0}
+
+
+def sampler_of(st, info):
+    """Which sampler a call of this graph with default options ran."""
+    if st["mode"] != 3:
+        return "shared"
+    return "walkers" if info.n > 400000 and (info.weighted or info.offsets64 or info.dmax > 8) else "lanes"
 
 
 def algorithmic_bytes(draws, trees, n, weighted, off64):
@@ -92,9 +100,9 @@ def algorithmic_bytes(draws, trees, n, weighted, off64):
 # on (code_hash of the .cu file), else reported as null.
 TRAFFIC_PER_DRAW = {
     # family: (bytes per draw, case captured, source file, code hash of the kernel region)
-    "rmat": (222.3, "R-MAT scale 18, 2000 trees, 64 walkers per tree: one w_trees launch "
-                     "(171.0 GB over 7.693e8 draws)", "walker.cu",
-             "ab1fdc759f922dfae00450c5610e7341609c15fbdcdfceea4077a8a0d4278a2e"),
+    "rmat": (195.2, "R-MAT scale 19, 500 trees, 64 walkers per tree: one w_trees launch "
+                     "(77.5 GB over 3.972e8 draws)", "walker.cu",
+             "4fb7320d9b55e54826931fd4ff30dd3d0f9fde8d3b198fdf4725eefa02e1031c"),
 }
 
 
@@ -662,16 +670,20 @@ def main():
     phase_ms = {p: 0.0 for p in PHASE_NAMES}
     per_graph = {}
     alg_total, impl_total, traffic_total, sampler_ms, launches_dom = 0.0, 0.0, 0.0, 0.0, 0
-    traffic_known = True
+    traffic_known, traffic_source = True, {}
+    info_of = {x[0]: x[3].info for x in graphs}
     for key, st in all_stats:
         gi = [x for x in graphs if x[0] == key][0]
         n, info = gi[2].n, gi[3].info
         T_key = gi[1]
         ms_k = sum(st["phase_ms"])
         alg = algorithmic_bytes(st["draws"], T_key, n, bool(info.weighted), bool(info.offsets64))
-        impl = st["draws"] * IMPL_BYTES_PER_DRAW if st["mode"] == 3 else 0
-        tpd = traffic_per_draw(key) if st["mode"] == 3 else None
+        sampler = sampler_of(st, info)
+        impl = st["draws"] * IMPL_BYTES_PER_DRAW[sampler]
+        tpd = traffic_per_draw(key) if sampler == "walkers" else None
         traffic_known &= tpd is not None
+        if tpd is not None:
+            traffic_source[family(key)] = TRAFFIC_PER_DRAW[family(key)][1]
         for i, p in enumerate(PHASE_NAMES):
             phase_ms[p] += st["phase_ms"][i]
         alg_total += alg
@@ -696,13 +708,14 @@ def main():
                 "unit_bytes": {"per_draw": {k: bytes_per_draw(bool(G.info.weighted), bool(G.info.offsets64))
                                             for k, _T, _g, G, _s in graphs},
                                "per_tree_vertex": BYTES_PER_TREE_VERTEX},
-                # the walker's own state-word traffic, not part of `achieved`
-                "implementation_bytes_per_draw": IMPL_BYTES_PER_DRAW if dom_mode == 3 else 0,
+                # the samplers' own state-word traffic, not part of `achieved`
+                "implementation_bytes_per_draw": {
+                    k: IMPL_BYTES_PER_DRAW[sampler_of(st, info_of[k])] for k, st in all_stats[-len(graphs):]},
                 "implementation_gbs": impl_total / (sampler_ms / 1000.0) / 1e9 if sampler_ms > 0 else 0.0,
                 # DRAM bytes actually moved (ncu per draw on a small case, scaled by the draws)
                 "dram_gbs": traffic_total / (sampler_ms / 1000.0) / 1e9 if traffic_known and sampler_ms > 0 else None,
                 "dram_frac": traffic_total / (sampler_ms / 1000.0) / 1e9 / hbm_peak if traffic_known and sampler_ms > 0 else None,
-                "traffic_source": {f: TRAFFIC_PER_DRAW[f][1] for f in {family(k) for k, *_ in graphs} if f in TRAFFIC_PER_DRAW},
+                "traffic_source": traffic_source,
                 "per_graph": {k: {"gbs": v["alg_bytes"] / (v["ms"] / 1000.0) / 1e9 if v["ms"] > 0 else 0.0,
                                   "frac": v["alg_bytes"] / (v["ms"] / 1000.0) / 1e9 / hbm_peak if v["ms"] > 0 else 0.0,
                                   "draws_per_s": v["draws"] / (v["ms"] / 1000.0) if v["ms"] > 0 else 0.0}
@@ -811,7 +824,8 @@ def main():
             "step_ms": step_ms,
             "sampler_stats": [{"graph": k, "mode": st["mode"], "rounds_or_yields": st["rounds"],
                                "draws": st["draws"], "walk_steps": st["walk_steps"],
-                               "chunks": st["chunks"], "walkers_per_tree": st["block_threads"],
+                               "chunks": st["chunks"], "sampler": sampler_of(st, info_of[k]),
+                               "lanes_or_walkers_per_tree": st["block_threads"],
                                "diag": st["diag"]}
                               for k, st in all_stats[-len(graphs):]],
         }

@@ -148,7 +148,8 @@ typedef struct {
                              (profile = 2 only) */
     int64_t chunks;       /* tree chunks processed */
     int32_t mode;         /* mode actually used */
-    int32_t block_threads; /* WALKER: walkers (threads) per tree of the last chunk */
+    int32_t block_threads; /* WALKER: walkers or lanes per tree of the last chunk; SHARED: threads
+                              per tree; batch: the schedule's largest block */
     int64_t marked;       /* compressed-graph nodes over all rounds (= draws) */
     /* with rwc_options_t.profile: device time (ms), launches and work units
      * per phase; units are vertices (INIT, ACCUM), pointer-chasing steps (WALK
@@ -373,20 +374,22 @@ rwc_status rwc_batch_sample(rwc_batch_t *b, uint64_t seed, int64_t trees_per_gra
                             double *sums, int32_t use_graph, int32_t per_graph_launch,
                             rwc_stats_t *stats, rwc_stream_t stream);
 rwc_status rwc_batch_roots(const rwc_batch_t *b, int32_t *host_roots);
-/* Choose the schedule (block size, split between block-per-tree and
- * warp-per-tree, trees per work item) for this batch by timing candidates on
- * the device; the choice is cached in cache_path (JSON, may be NULL) under a
+/* Choose the schedule (split between block-per-tree and warp-per-tree, largest
+ * block of 64, 128 or the default, concurrent bins) for this batch by timing
+ * candidates on the device; the choice is cached in cache_path (JSON, may be NULL) under a
  * signature of the batch's sizes.  Synchronises stream. */
 rwc_status rwc_autotune(rwc_batch_t *b, const char *cache_path, rwc_stream_t stream);
 /* The batch's schedule.  threads: largest block of the large class (graphs with
  * more than split vertices, one tree per block of 64 to 256 threads by its
- * size; a multiple of 32, <= 1024); split: the largest n of the small class (0:
+ * size and the call's trees; a multiple of 32, <= 1024); split: the largest n of the small class (0:
  * one class); warp: 1 = the small class runs one tree per warp, 0 = one tree
- * per block as the large class; tile: trees per work item; concurrent: 1 = the
+ * per block as the large class; tile: kept with the schedule, without effect
+ * (trees are pulled one by one); concurrent: 1 = the
  * size bins' persistent kernels run on forked streams at the same time, 0 = one
  * after the other (all inside the call's one CUDA graph).  set returns
- * RWC_ERR_UNSUPPORTED when a class needs more than 227 KB of shared memory
- * per block (a tree of n vertices takes 11 n + 64 bytes).  host_sched: int32
+ * RWC_ERR_UNSUPPORTED when a class is allowed more than 227 KB of shared memory
+ * per block, at 11 n + 64 bytes for a tree of n vertices and eight trees per block
+ * where warp = 1 (the kernels take 4 n bytes and a few KB for one tree).  host_sched: int32
  * [5] = {threads, split, tile, warp, concurrent}.  Schedules do not change the
  * trees. */
 rwc_status rwc_batch_get_schedule(const rwc_batch_t *b, int32_t *host_sched);

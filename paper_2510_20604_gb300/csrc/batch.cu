@@ -83,14 +83,14 @@ __global__ void __launch_bounds__(NT) l_batch(DevGraph base, const BGraph *__res
 // an SM beside n words of shared memory per tree (21 blocks of 64 up to 2500
 // vertices by registers, 10 of 128 up to 5000, 2 of 256 at 20000).  512 graphs
 // of 50 to 20000 vertices, 64 trees each: 158 ms with whole-block popping
-// rounds (11 bytes per vertex, one kernel for each of two classes), 19.4 ms so.
+// rounds (11 bytes per vertex, one kernel for each of two classes), 18.8 ms so.
 // Calls of at most one tree per SM take 256 threads for each, which nothing else would
 // use (one tree: BA 5000 0.154 -> 0.116 ms a call; of each of 64 weighted BA graphs of
 // 2000 vertices: 0.186 -> 0.132).  Up to 448 vertices more than a warp gains nothing.
 bool few_trees(int64_t trees) { return trees <= num_sms(); }
 int batch_threads(int n, bool few) { return few && n > 448 ? 256 : n <= 2500 ? 64 : n <= 5000 ? 128 : 256; }
 // One launch per graph: one warp up to 448 vertices, whose rounds need no block barrier
-// (30 paths of 60, 1 tree each: 18.8 ms, 22.0 with 64 threads).
+// (30 paths of 60, 1 tree each: 18.7 ms, 23.8 with 64 threads).
 int single_threads(int n, bool few) { return n <= 448 ? 32 : batch_threads(n, few); }
 
 size_t batch_tree_smem(int n, int nt) {

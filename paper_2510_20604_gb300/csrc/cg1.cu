@@ -12,8 +12,8 @@
 //   - graphs of bounded degree keep a thread's rows of e, r, p, q in registers
 //     and their inline neighbour rows in shared memory.
 // Measured (pivot solve and recovery, one kernel per inner solve with FP64 dots
-// and three grid barriers -> here): 1024 x 1024 grid 369 -> 121 ms (45 -> 14.4 us
-// per iteration), R-MAT 20 21.4 -> 12.2 ms, BA 2000 0.67 -> 0.37 ms, ER 100 0.54
+// and three grid barriers -> here): 1024 x 1024 grid 369 -> 122 ms (45 -> 14.8 us
+// per iteration), R-MAT 20 21.4 -> 12.7 ms, BA 2000 0.67 -> 0.37 ms, ER 100 0.54
 // -> 0.18 ms.
 #include <algorithm>
 #include <cmath>

@@ -158,7 +158,8 @@ __device__ __forceinline__ bool after(uint64_t x, uint64_t y) { return x > y; }
 __device__ __forceinline__ KeyPair last_key(KeyPair) { return {~0ull, ~0ull}; }
 __device__ __forceinline__ uint64_t last_key(uint64_t) { return ~0ull; }
 
-// Elements of L among the first d of the stable merge of L (nl) and R (nr).
+// Elements of L among the first d of the stable merge of L (nl) and R (nr): the
+// diagonal search of merge path (Odeh, Green, Mwassi, Shmueli, Birk 2012).
 template <class K, class I>
 __device__ __forceinline__ I merge_split(const K *L, I nl, const K *R, I nr, I d) {
     I lo = d > nr ? d - nr : 0, hi = d < nl ? d : nl;

@@ -440,8 +440,9 @@ bool walker_in_smem(int64_t n, const rwc_options_t &o) {
 // The concurrent walkers (sample_walker) keep calls that ask for their options
 // and, with words in global memory, graphs of unbounded degree above 400000
 // vertices: there every access goes to HBM and the walkers' fewer words per
-// draw count (R-MAT n = 262144, 500 trees: 24.4 -> 13.6 ms here; n = 524288:
-// 36.8 and 33.2; n = 1048576: 69 and 80).
+// draw count (R-MAT, 500 trees, walkers and lanes: n = 262144 24.4 and 13.6 ms, 524288
+// 36.8 and 33.2, 1048576 69 and 80; the line lies below the crossing, whose place for
+// other numbers of trees was not measured).
 bool lane_walker_takes(const rwc_graph *G, const rwc_options_t &o) {
     const DevGraph &g = G->g;
     if (o.walker_policy || o.block_threads || o.max_wait_ns || o.profile >= 2) return false;

@@ -1,5 +1,5 @@
 // Sums held as pairs of floats s + c: products are exact (FMA), additions carry
-// their rounding error in c, about 48 bits altogether.  FP64 runs at 2 FMA per
+// their rounding error (Knuth's two-sum) in c, about 48 bits altogether.  FP64 runs at 2 FMA per
 // cycle and SM on this GPU, so long FP32 dot products are summed this way and
 // only their few partial sums are FP64.
 #pragma once

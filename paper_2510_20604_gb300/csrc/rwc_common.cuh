@@ -103,7 +103,8 @@ rwc_status sample_walker(rwc_graph *G, uint64_t seed, int64_t tree0, int64_t T, 
 rwc_status sample_park(rwc_graph *G, uint64_t seed, int64_t tree0, int64_t T, double *sums,
                        int32_t *parents, int32_t *visits, const rwc_options_t &o,
                        rwc_stats_t *st, cudaStream_t stream);
-// One warp per tree (lane.cu): words in shared memory, or in global memory.
+// Lane sampler (lane.cu), a warp or a block per tree: words in shared memory, or in
+// global memory.
 rwc_status sample_lane_shared(rwc_graph *G, uint64_t seed, int64_t tree0, int64_t T, double *sums,
                               int32_t *parents, int32_t *visits, const rwc_options_t &o,
                               rwc_stats_t *st, cudaStream_t stream);

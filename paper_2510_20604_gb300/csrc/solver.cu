@@ -15,8 +15,8 @@
 // passes (product and <p,q>; r and its sums; e and p), whose working set of four
 // arrays stays in L2 for 66 columns of 100000 rows.
 // Measured (whole gradient calls, a warp per row with FP64 dots -> here): RGG
-// 100000, 64 sketch columns 39.7 -> 13.6 ms; BA 100000, 64 columns 42.3 -> 14.9;
-// BA 8792, 16 columns 4.7 -> 3.8; RGG 1500, 8 columns 3.1 -> 2.3.
+// 100000, 64 sketch columns 39.7 -> 13.7 ms; BA 100000, 64 columns 42.3 -> 15.1;
+// BA 8792, 16 columns 4.7 -> 3.4; RGG 1500, 8 columns 3.1 -> 2.5.
 #include <algorithm>
 #include <cmath>
 #include <cstring>
@@ -99,7 +99,9 @@ __device__ __forceinline__ void dot4(Pair (&a)[4], const float4 &x, const float4
 
 // Rows of more arcs are shared by a block's slots: one slot takes about 150 cycles
 // per arc, so the hub of a BA graph of 9000 vertices alone took longer than the
-// rest of the product.
+// rest of the product (gradients with 64 columns, rows of more than 128 and of more than
+// 1024 arcs shared: BA 8792 4.84 and 5.82 ms, BA 60000 9.42 and 9.55, BA 100000 15.1 and
+// 14.7, R-MAT 65536 54 and 58).
 constexpr int WIDE_ROW = 128;
 
 // Q = L P and the parts of <P, Q>.  Four neighbour rows are in flight.
